@@ -1,0 +1,1116 @@
+// Tall-skinny contractions of Sec. VI on the 5th-generation tensor cores at
+// FP64 (and FP32) accuracy, by splitting every operand into integer digits.
+//
+//   overlap   S = dV X^T Y      (contraction over the grid points)
+//   rotation  Y = alpha X C + beta Y   (contraction over the states)
+//
+// GB300 has about 1.1 TFLOP/s of FP64 FMA against 1.9 PFLOP/s of FP16 tensor
+// throughput.  An operand value is written as an integer q = x 2^(s - E), E
+// the exponent of the largest entry of its column (overlap; of its row of X
+// and column of C in the rotation) and s = 8 NS - 2, and q as NS balanced
+// digits in base 256, |d| <= 128, each exact in FP16.  Digit products are
+// integers of at most 2^14, so the FP32 accumulators of the tensor cores sum
+// up to 1024 of them without any rounding.  The products of weight
+// 256^-(i+j), i + j = t, have their own accumulator in tensor memory for
+// every t < NS (NS of them; those with i + j >= NS are below the digits'
+// own resolution and are left out); the accumulators are read out every 256
+// points and summed as 64-bit integers: with t + 1 pairs of digits in
+// accumulator t everything up to t = 3 is exact and a rounding of a later
+// one is below 2^-56 of the largest product.  So the result is the exact
+// sum of products of operands rounded to s bits: NS = 8 (FP64), 7 (FP32 data
+// at FP64-like accuracy) or 5 (FP32 accuracy).  (Ozaki, Ogita, Oishi and Rump
+// 2012 give the scheme of error-free splittings of a matrix product.)
+//
+// Kernel: 8 converter warps and one MMA warp per CTA, one CTA per SM, a 128 x
+// BN tile of the result.  Stage (32 steps of the contraction, two stages): the
+// converters read the operands from global memory into registers one stage
+// ahead, extract the digits with integer instructions (the FP64 pipe would
+// take longer than the products) and store them as K-major core matrices (8
+// rows of 16 bytes) in shared memory; one thread issues the products; every
+// 256 steps the converters read the accumulators back, accumulator by
+// accumulator in the order the products run, so the products of the next
+// steps overlap the readout.  Columns or rows that hold a non-finite or an
+// extreme value (an exponent near either end of the range) make their CTA
+// take a plain loop instead, so that infinities and NaN spread as in a plain
+// contraction.  Every wait is bounded; a CTA whose wait gives up writes NaN.
+//
+// What bounds it, and what it measured (overlap of 256 x 256 columns over
+// 658 416 points): FP64 2.89 ms, FP32 data 2.63 ms, against 69.8 ms by FP64 FMA
+// and 14.3 ms by compensated FP32 sums before.  The products alone take
+// 1.65 ms (28 % more than the tensor pipe needs: the readouts); the
+// conversion, 20 integer instructions per value on a pipe of half rate,
+// accounts for the rest, the pass that finds the column exponents for 0.4 ms.
+// Every size gains (64 x 64: 4.4 -> 0.44 ms FP64, 0.94 -> 0.40 ms FP32), so
+// there is no other path.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "device.h"
+#include "digits.h"
+
+namespace rs {
+
+namespace {
+
+constexpr int DG_M = 128;            // rows of the tile (TMEM lanes)
+constexpr int DG_K = 32;             // contraction steps per stage
+constexpr int DG_DRAIN = 8;          // stages between accumulator readouts
+constexpr int DG_STAGES = 2;
+constexpr int DG_CW = 8;             // converter warps
+constexpr int DG_CT = DG_CW * 32;    // converter threads
+constexpr int DG_NT = DG_CT + 128;   // and the MMA warp's warpgroup (its other warps only help with the set-up)
+constexpr int DG_SPIN = 100000;      // barrier tests (at most 20 us each) before a wait gives up
+constexpr int KQ = DG_K / 8;         // 8-step groups per stage
+__device__ __forceinline__ uint32_t dg_su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void dg_bar_init(uint64_t *b, uint32_t n) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(dg_su32(b)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void dg_arrive(uint64_t *b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(dg_su32(b)) : "memory");
+}
+__device__ __forceinline__ bool dg_try(uint64_t *b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(dg_su32(b)), "r"(parity), "n"(20000)
+        : "memory");
+    return ok != 0;
+}
+// bounded wait; false once it has given up here or `bad` says another thread's has
+__device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile int *bad) {
+    for (int i = 0; i < DG_SPIN; ++i) {
+        if (dg_try(b, parity)) return true;
+        if (*bad) return false;
+    }
+    *bad = 1;
+    return false;
+}
+// The MMA warp runs its loop as a whole, so that descriptors stay in uniform
+// registers; `lead` (one lane) issues.
+__device__ __forceinline__ void dg_mma(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum,
+                                       uint32_t lead) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum), "r"(lead)
+        : "memory");
+}
+__device__ __forceinline__ void dg_commit(uint64_t *b, uint32_t lead) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(dg_su32(b)),
+        "r"(lead)
+        : "memory");
+}
+// registers: 384 threads are launched with 168 each; the converters' two
+// warpgroups take 232 and the MMA warp's keeps 40 (2 x 232 + 40 = 3 x 168)
+#define DG_REGS_UP() asm volatile("setmaxnreg.inc.sync.aligned.u32 232;\n")
+#define DG_REGS_DOWN() asm volatile("setmaxnreg.dec.sync.aligned.u32 40;\n")
+#define DG_FENCE_BEFORE() asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory")
+#define DG_FENCE_AFTER() asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory")
+
+// Matrix descriptor of a K-major tile without swizzle: core matrices of 8 rows x
+// 16 bytes, `lbo` bytes apart along K and 128 bytes apart along the rows.
+__device__ __forceinline__ uint64_t dg_desc(uint32_t saddr, uint32_t lbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | (uint64_t)1 << 46;
+}
+// FP16 x FP16 -> FP32, both K-major
+__host__ __device__ constexpr uint32_t dg_idesc(int M, int N) {
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void dg_tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+__device__ __forceinline__ void dg_tmem_ld8(uint32_t addr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+}
+
+// ------------------------------------------------------------- digits ---
+
+// Ordering key of |x| whose high part is the biased exponent; 0 for zero only.
+__device__ __forceinline__ int abs_key(double x) {
+    const int hi = __double2hiint(x) & 0x7fffffff;
+    return hi ? hi : (__double2loint(x) != 0);
+}
+__device__ __forceinline__ int abs_key(float x) { return __float_as_int(x) & 0x7fffffff; }
+
+// Biased exponent of a column from its largest key (of a column of zeros: any
+// that leaves their digits zero), and whether the digit
+// path takes it: below `lo` an element's missing implicit bit could reach
+// the digits, and the weights of the result could leave the FP64 range.
+template <typename T> struct ExpOf;
+template <> struct ExpOf<double> {
+    static constexpr int bias = 1023;
+    static __device__ __forceinline__ int exponent(int key) { return key ? key >> 20 : bias; }
+    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 20) < 623 || (key >> 20) > 1423); }
+};
+template <> struct ExpOf<float> {
+    static constexpr int bias = 127;
+    static __device__ __forceinline__ int exponent(int key) { return key ? key >> 23 : bias; }
+    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 23) < 64 || (key >> 23) > 254); }
+};
+
+// q + 128 in every digit, q = trunc(|x| 2^(s - E)), |x| < 2^E, E = ecol - bias + 1.
+// The mantissa stands at bits 61 .. 9 (38) and is shifted right by `room` plus
+// the distance of the exponents; room = 62 - s.
+template <int NS> struct Bias {
+    static constexpr uint64_t b = 0x8080808080808080ull >> (64 - 8 * NS);
+    static constexpr int room = 62 - (8 * NS - 2);
+};
+template <int NS> __device__ __forceinline__ uint64_t biased_int(double x, int ecol) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int d = ((ecol + Bias<NS>::room) << 20) - (int)(hi & 0x7ff00000u);
+    const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
+    const uint64_t l = (uint64_t)lo * 512u;
+    const uint64_t m = ((uint64_t)(mh * 512u + (uint32_t)(l >> 32)) << 32) | (uint32_t)l;
+    return (m >> min((uint32_t)(d >> 20), 63u)) + Bias<NS>::b;
+}
+template <int NS> __device__ __forceinline__ uint64_t biased_int(float x, int ecol) {
+    const uint32_t b = __float_as_uint(x);
+    const int d = ((ecol + Bias<NS>::room) << 23) - (int)(b & 0x7f800000u);
+    const uint32_t mh = ((b & 0x7fffffu) | 0x800000u) << 6;
+    return (((uint64_t)mh << 32) >> min((uint32_t)(d >> 23), 63u)) + Bias<NS>::b;
+}
+__device__ __forceinline__ uint32_t top_word(double x) { return (uint32_t)__double2hiint(x); }
+__device__ __forceinline__ uint32_t top_word(float x) { return __float_as_uint(x); }
+
+// The digits of eight consecutive steps of one row: slice i (most significant
+// first) is one core-matrix row of 16 bytes at dst + i * stride.  A byte b
+// becomes the FP16 number 1024 + b by its bit pattern (two elements to a
+// word), then the signed digit +-(b - 128) by one exact fused multiply-add:
+// a byte permutation and a logic operation per two digits on the integer
+// pipe, whose half rate bounds the conversion, the rest on the FP16 pipe.
+template <typename T, int NS>
+__device__ __forceinline__ void store_digits(const T (&v)[8], int ecol, unsigned char *dst, int stride) {
+    uint32_t lo[8], hi[8], mul[4], add[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint64_t u = biased_int<NS>(v[k], ecol);
+        lo[k] = (uint32_t)u;
+        hi[k] = (uint32_t)(u >> 32);
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const uint32_t sg = __byte_perm(top_word(v[2 * p]), top_word(v[2 * p + 1]), 0x7632) & 0x80008000u;
+        mul[p] = sg ^ 0x3c003c00u;   // +-1
+        add[p] = sg ^ 0xe480e480u;   // -+1152
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        constexpr int last = NS - 1;
+        const int b = last - i;      // byte of the integer
+        uint32_t w[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t x0 = b < 4 ? lo[2 * p] : hi[2 * p], x1 = b < 4 ? lo[2 * p + 1] : hi[2 * p + 1];
+            // bytes 0 and 2: the two elements' digits
+            const uint32_t h = (__byte_perm(x0, x1, (unsigned)(b & 3) | ((unsigned)(4 + (b & 3)) << 8)) & 0x00ff00ffu) | 0x64006400u;
+            const __half2 d = __hfma2(*reinterpret_cast<const __half2 *>(&h), *reinterpret_cast<const __half2 *>(&mul[p]),
+                                      *reinterpret_cast<const __half2 *>(&add[p]));
+            w[p] = *reinterpret_cast<const uint32_t *>(&d);
+        }
+        *reinterpret_cast<uint4 *>(dst + i * stride) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// ------------------------------------------------------- shared pieces ---
+
+template <int NS, int BN, int PAD> struct DgCfg {
+    // A: slice by slice, each KQ columns of core matrices; B: the slices of one
+    // column group behind one another, so that several are one wide operand
+    static constexpr int LBO_A = DG_M * 16 + PAD, LBO_B = NS * BN * 16;
+    static constexpr int SL_A = KQ * LBO_A, SL_B = BN * 16;      // bytes from slice to slice
+    static constexpr int A_BYTES = NS * SL_A, STAGE = A_BYTES + KQ * LBO_B;
+    static constexpr int TMEM = NS * BN <= 128 ? 128 : NS * BN <= 256 ? 256 : 512;
+    static constexpr size_t SMEM = (size_t)DG_STAGES * STAGE + 128;
+    static_assert(NS * BN <= 512, "tensor memory columns");
+    static_assert(LBO_A % 16 == 0, "core matrix stride");
+};
+
+struct DgBars {
+    uint64_t full[DG_STAGES], empty[DG_STAGES], accfull[8], accfree, done;
+    uint32_t tmem;
+    int bad, plain;
+};
+
+template <int NS> __device__ __forceinline__ void dg_setup(DgBars &b, int tmem_cols) {
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < DG_STAGES; ++i) {
+            dg_bar_init(&b.full[i], DG_CT);
+            dg_bar_init(&b.empty[i], 1);
+        }
+        for (int t = 0; t < NS; ++t) dg_bar_init(&b.accfull[t], 1);
+        dg_bar_init(&b.accfree, DG_CT);
+        dg_bar_init(&b.done, 1);
+        b.bad = 0;
+        b.plain = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (threadIdx.x >> 5 == DG_CW) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dg_su32(&b.tmem)),
+                     "r"(tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    DG_FENCE_AFTER();
+}
+
+// The MMA warp: all products of nst stages, in blocks of kst (a readout
+// interval ends with its block).  Slice i of A meets slices 0 .. NS - 1 - i of
+// B as one operand of (NS - i) BN columns (at most 256 to an instruction),
+// whose products fall in accumulators i .. NS - 1: a third of the instructions
+// and reads of A that single pairs of slices would take (those ran at 68
+// cycles each, twice what 64 columns need).  Accumulator t is complete after
+// slice t of the last stage.
+template <int NS, int BN, int PAD> struct DgIssue {
+    using C = DgCfg<NS, BN, PAD>;
+    uint32_t tmem, lead;
+    uint64_t da0, db0;
+    int g = 0, iv = -1;   // stages taken, readout interval
+    __device__ __forceinline__ DgIssue(DgBars &b, unsigned char *base) {
+        tmem = __shfl_sync(0xffffffffu, b.tmem, 0);
+        lead = (threadIdx.x & 31) == 0;
+        da0 = dg_desc(dg_su32(base), C::LBO_A);
+        db0 = dg_desc(dg_su32(base) + C::A_BYTES, C::LBO_B);
+    }
+    __device__ __forceinline__ bool run(DgBars &b, int nst, int kst) {
+        int kb = 0;   // stage within the block
+        bool ok = true;
+        for (int it = 0; it < nst && ok; ++it, ++g) {
+            const int s = g % DG_STAGES;
+            const bool first = kb % DG_DRAIN == 0, last = kb % DG_DRAIN == DG_DRAIN - 1 || kb == kst - 1;
+            iv += first;
+            if (++kb == kst) kb = 0;
+            ok = __all_sync(0xffffffffu, dg_wait(&b.full[s], (g / DG_STAGES) & 1, &b.bad));
+            DG_FENCE_AFTER();
+            const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
+            if (first && iv > 0 && ok) {
+                ok = __all_sync(0xffffffffu, dg_wait(&b.accfree, (iv - 1) & 1, &b.bad));
+                DG_FENCE_AFTER();
+            }
+            if (ok) {
+#pragma unroll
+                for (int i = 0; i < NS; ++i) {
+#pragma unroll
+                    for (int k = 0; k < DG_K / 16; ++k)
+#pragma unroll
+                        for (int c = 0; c < (NS - i) * BN; c += 256) {
+                            const int n = (NS - i) * BN - c < 256 ? (NS - i) * BN - c : 256;
+                            dg_mma(tmem + i * BN + c, da + (uint64_t)((i * C::SL_A + 2 * k * C::LBO_A) >> 4),
+                                   db + (uint64_t)((c * 16 + 2 * k * C::LBO_B) >> 4), dg_idesc(DG_M, n),
+                                   (first && i == 0 && k == 0) ? 0u : 1u, lead);
+                        }
+                    if (last) dg_commit(&b.accfull[i], lead);
+                }
+            }
+            dg_commit(&b.empty[s], lead);
+        }
+        return ok;
+    }
+    // after the last stage: waits for every product in flight
+    __device__ __forceinline__ void finish(DgBars &b) {
+        dg_commit(&b.done, lead);
+        dg_wait(&b.done, 0, &b.bad);
+    }
+};
+
+// One readout (in the order in which the accumulators complete): the converter thread's 32 columns of every accumulator added to
+// H (t = 0..2, in units of accumulator 2) and L (t = 3.., in units of 256 times
+// the weight of accumulator NS - 1).
+template <int NS, int BN>
+__device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t *H, int64_t *L) {
+    const int warp = threadIdx.x >> 5;
+    const uint32_t lane_base = b.tmem + ((uint32_t)(warp & 3) * 32 << 16) + (uint32_t)col0;
+#pragma unroll
+    for (int t = 0; t < NS - 2; ++t) {
+        uint32_t r[32];
+        if (!dg_wait(&b.accfull[t], iv & 1, &b.bad)) return false;
+        DG_FENCE_AFTER();
+        dg_tmem_ld32(lane_base + t * BN, r);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const int64_t v = (int64_t)__float2int_rn(__uint_as_float(r[j]));
+            if (t < 3) H[j] += v * (int64_t)(1 << (8 * (2 - t)));
+            else L[j] += v * (int64_t)(1 << (8 * (NS - 2 - t)));
+        }
+    }
+    // the last two accumulators together, rounded at the weight of the first
+    if (!dg_wait(&b.accfull[NS - 1], iv & 1, &b.bad)) return false;
+    DG_FENCE_AFTER();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t u[8], w[8];
+        dg_tmem_ld8(lane_base + (NS - 2) * BN + 8 * q, u);
+        dg_tmem_ld8(lane_base + (NS - 1) * BN + 8 * q, w);
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            L[8 * q + j] += (int64_t)__float2int_rn(fmaf(__uint_as_float(w[j]), 1.f / 256.f, __uint_as_float(u[j])));
+    }
+    DG_FENCE_BEFORE();
+    dg_arrive(&b.accfree);
+    return true;
+}
+
+// 2^e as FP64 (e within the normal range)
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
+// ------------------------------------------------------------ overlap ---
+
+template <typename T> struct GramArgs {
+    const T *X, *Y;
+    int64_t ldx, ldy, npts, lds;
+    int nx, ny;
+    const int *kx, *ky;      // column keys
+    double *S;
+    double dV;
+    int tiles_n, stages, per_cta;   // stages in all and per CTA
+    int sym;                 // Y is X: only the elements j >= i are computed, and mirrored
+};
+
+template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1) k_digit_gram(GramArgs<T> a) {
+    using C = DgCfg<NS, BN, 0>;
+    extern __shared__ __align__(128) unsigned char dgsm[];
+    __shared__ DgBars b;
+    __shared__ int ea[DG_M], eb[BN];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // tile (bm, bn): in the symmetric case the bn-th of those not entirely below the diagonal
+    int bm = 0, bn = blockIdx.x;
+    if (a.sym) {
+        for (;; ++bm) {
+            const int skip = bm * DG_M / BN;
+            if (bn < a.tiles_n - skip) {
+                bn += skip;
+                break;
+            }
+            bn -= a.tiles_n - skip;
+        }
+    } else {
+        bm = blockIdx.x / a.tiles_n;
+        bn = blockIdx.x - bm * a.tiles_n;
+    }
+    const int m0 = bm * DG_M, n0 = bn * BN;
+    const int st0 = blockIdx.y * a.per_cta, nst = min(a.per_cta, a.stages - st0);
+    dg_setup<NS>(b, C::TMEM);
+    for (int i = tid; i < DG_M + BN; i += DG_NT) {
+        const bool isa = i < DG_M;
+        const int c = isa ? m0 + i : n0 + i - DG_M;
+        const int key = isa ? (c < a.nx ? a.kx[c] : 0) : (c < a.ny ? a.ky[c] : 0);
+        (isa ? ea[i] : eb[i - DG_M]) = ExpOf<T>::exponent(key);
+        if (ExpOf<T>::plain(key)) b.plain = 1;
+    }
+    __syncthreads();
+    const int64_t p0 = (int64_t)st0 * DG_K, p1 = min(a.npts, p0 + (int64_t)nst * DG_K);
+    if (b.plain) {
+        // a column beyond the digits' range: plain FP64 sums of this tile and range
+        for (int e = tid; e < DG_M * BN; e += DG_NT) {
+            const int i = m0 + e / BN, j = n0 + e % BN;
+            if (i >= a.nx || j >= a.ny || (a.sym && j < i)) continue;
+            double s = 0;
+            for (int64_t p = p0; p < p1; ++p) s = fma((double)a.X[p * a.ldx + i], (double)a.Y[p * a.ldy + j], s);
+            atomicAdd(a.S + (int64_t)i * a.lds + j, a.dV * s);
+            if (a.sym && j > i) atomicAdd(a.S + (int64_t)j * a.lds + i, a.dV * s);
+        }
+    } else if (warp >= DG_CW) {
+        DG_REGS_DOWN();
+        if (warp == DG_CW) {
+            DgIssue<NS, BN, 0> mma(b, dgsm);
+            mma.run(b, nst, nst);
+            mma.finish(b);
+        }
+    } else {
+        DG_REGS_UP();
+        // converter warp: units (32 columns, 8 points) warp, warp + 8 of A and warp of B
+        constexpr int NB = BN / 32 * KQ;            // units of B per stage
+        constexpr int NU = 2 + (NB + DG_CW - 1) / DG_CW;
+        const T *src[NU];
+        unsigned char *dst[NU];
+        int ec[NU], sl[NU], off[NU];
+        uint32_t ld[NU];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+            const bool isa = u < 2;
+            const int w = isa ? warp + DG_CW * u : warp + DG_CW * (u - 2);
+            const bool has = isa || w < NB;
+            const int rg = w / KQ, kq = w % KQ, row = rg * 32 + lane;
+            const int c = isa ? m0 + row : n0 + row;
+            // a column beyond the last reads the first one; what its digits are
+            // only reaches results that are not written
+            const bool in = has && c < (isa ? a.nx : a.ny);
+            ec[u] = isa ? ea[row & (DG_M - 1)] : eb[row & (BN - 1)];
+            ld[u] = (uint32_t)((isa ? a.ldx : a.ldy) * (int64_t)sizeof(T));
+            off[u] = 8 * kq;
+            src[u] = (isa ? a.X : a.Y) + (in ? c : 0);
+            dst[u] = has ? dgsm + (isa ? kq * C::LBO_A : C::A_BYTES + kq * C::LBO_B) + row * 16 : nullptr;
+            sl[u] = isa ? C::SL_A : C::SL_B;
+        }
+        T v[NU][8];
+        auto load = [&](int it) {
+            const int64_t pb = p0 + (int64_t)it * DG_K;
+            if (pb + DG_K <= p1) {
+#pragma unroll
+                for (int u = 0; u < NU; ++u)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        v[u][k] = __ldg(reinterpret_cast<const T *>(reinterpret_cast<const char *>(src[u]) +
+                                                                    (uint64_t)((uint32_t)pb + off[u] + k) * ld[u]));
+            } else {
+#pragma unroll
+                for (int u = 0; u < NU; ++u)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        v[u][k] = pb + off[u] + k < p1
+                                      ? __ldg(reinterpret_cast<const T *>(reinterpret_cast<const char *>(src[u]) +
+                                                                          (uint64_t)((uint32_t)pb + off[u] + k) * ld[u]))
+                                      : T(0);
+            }
+        };
+        int64_t H[32], L[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) H[j] = L[j] = 0;
+        const int col0 = (warp >> 2) * 32;
+        const bool drains = col0 < BN;   // BN = 32: the second four warps only free the accumulators
+        bool ok = true;
+        load(0);
+        int iv = 0;   // readouts taken
+        for (int it = 0; it < nst && ok; ++it) {
+            const int s = it % DG_STAGES;
+            if (it >= DG_STAGES && !dg_wait(&b.empty[s], (it / DG_STAGES - 1) & 1, &b.bad)) {
+                ok = false;
+                break;
+            }
+#pragma unroll
+            for (int u = 0; u < NU; ++u)
+                if (dst[u]) store_digits<T, NS>(v[u], ec[u], dst[u] + s * C::STAGE, sl[u]);
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            dg_arrive(&b.full[s]);
+            if (it + 1 < nst) load(it + 1);
+            // the previous 256 points' accumulators, once the first stage after them is queued
+            if (it % DG_DRAIN == 0 && it > 0) {
+                ok = dg_drain<NS, BN>(b, iv, drains ? col0 : 0, H, L);
+                ++iv;
+            }
+        }
+        if (ok) ok = dg_drain<NS, BN>(b, iv, drains ? col0 : 0, H, L);
+        const int row = (warp & 3) * 32 + lane, i = m0 + row;
+        if (i < a.nx && drains) {
+            const int s2 = 2 * (8 * NS - 2);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int jc = n0 + col0 + j;
+                if (jc >= a.ny || (a.sym && jc < i)) continue;
+                const int e = ea[row] + eb[col0 + j] - 2 * (ExpOf<T>::bias - 1) - s2;
+                double r = a.dV * fma((double)H[j], pow2d(e + 8 * (2 * NS - 4)), (double)L[j] * pow2d(e + 8 * NS));
+                if (!ok) r = __longlong_as_double(0x7ff8000000000000ll);
+                atomicAdd(a.S + (int64_t)i * a.lds + jc, r);
+                if (a.sym && jc > i) atomicAdd(a.S + (int64_t)jc * a.lds + i, r);
+            }
+        }
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    if (warp == DG_CW)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(b.tmem), "r"(C::TMEM) : "memory");
+}
+
+// Zero S and the keys.
+__global__ void k_digit_init(double *S, int64_t lds, int n, int m, int *keys, int nkeys) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t e = t0; e < (int64_t)n * m; e += step) S[(e / m) * lds + e % m] = 0.0;
+    for (int64_t e = t0; e < nkeys; e += step) keys[e] = 0;
+}
+
+// Largest key of every column of X (blocks [0, gx)) and Y: 32 columns and 8
+// rows per block and pass.
+template <typename T>
+__global__ void __launch_bounds__(256) k_digit_keys(const T *__restrict__ X, int64_t ldx, int nx, const T *__restrict__ Y,
+                                                    int64_t ldy, int ny, int64_t npts, int gx, int *keys) {
+    __shared__ int red[8][32];
+    const int l = threadIdx.x & 31, r = threadIdx.x >> 5;
+    const bool isx = (int)blockIdx.x < gx;
+    const int c = (isx ? blockIdx.x : blockIdx.x - gx) * 32 + l;
+    const T *src = isx ? X : Y;
+    const int64_t ld = isx ? ldx : ldy;
+    int k = 0;
+    if (c < (isx ? nx : ny)) {
+        const int64_t step = (int64_t)gridDim.y * 8;
+        int64_t p = (int64_t)blockIdx.y * 8 + r;
+        for (; p + 7 * step < npts; p += 8 * step) {
+            T v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __ldg(src + (p + u * step) * ld + c);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) k = max(k, abs_key(v[u]));
+        }
+        for (; p < npts; p += step) k = max(k, abs_key(__ldg(src + p * ld + c)));
+    }
+    red[r][l] = k;
+    __syncthreads();
+    if (r == 0 && c < (isx ? nx : ny)) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) k = max(k, red[q][l]);
+        if (k) atomicMax(keys + (isx ? 0 : nx) + c, k);
+    }
+}
+
+// Stream-ordered scratch from the library's own pool of the current device.
+// The pool keeps at most 64 MB between calls (its own allocation unit is 32 MB:
+// with a lower limit every call after a synchronisation maps memory anew, 200 us); a block is freed in stream order,
+// so calls on any number of threads and streams hold separate blocks.
+int scratch_pool(cudaMemPool_t *out) {
+    constexpr int MAXDEV = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[MAXDEV] = {};
+    int dev = 0;
+    RS_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= MAXDEV) return fail(RS_ECUDA, "device %d out of range", dev);
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        RS_CUDA(cudaMemPoolCreate(&p, &props));
+        uint64_t keep = 64ull << 20;
+        RS_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
+        pools[dev] = p;
+    }
+    *out = pools[dev];
+    return RS_OK;
+}
+
+int sm_count(int *n) {
+    int dev = 0;
+    RS_CUDA(cudaGetDevice(&dev));
+    RS_CUDA(cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev));
+    return RS_OK;
+}
+
+template <typename T, int NS, int BN> int launch_gram(GramArgs<T> a, int tiles_m, cudaStream_t st) {
+    using C = DgCfg<NS, BN, 0>;
+    a.tiles_n = (a.ny + BN - 1) / BN;
+    int tiles = 0;
+    for (int m = 0; m < tiles_m; ++m) tiles += a.tiles_n - (a.sym ? m * DG_M / BN : 0);
+    int nsm = 0;
+    RS_TRY(sm_count(&nsm));
+    // the split of the points that leaves the fewest stages to the busiest SM
+    // (a CTA's set-up and result cost about as much as 6 stages)
+    a.stages = (int)((a.npts + DG_K - 1) / DG_K);
+    int64_t best = INT64_MAX;
+    for (int s = 1; s <= std::min(a.stages, 8 * nsm); ++s) {
+        if ((int64_t)tiles * s > 8ll * nsm && s > 1) break;
+        const int64_t cost = (((int64_t)tiles * s + nsm - 1) / nsm) * ((a.stages + s - 1) / s + 6);
+        if (cost < best) {
+            best = cost;
+            a.per_cta = (a.stages + s - 1) / s;
+        }
+    }
+    const int splits = (a.stages + a.per_cta - 1) / a.per_cta;
+    RS_TRY(smem_optin((const void *)k_digit_gram<T, NS, BN>, C::SMEM));
+    k_digit_gram<T, NS, BN><<<dim3((unsigned)tiles, (unsigned)splits), DG_NT, C::SMEM, st>>>(a);
+    RS_LAUNCH_CHECK();
+    return RS_OK;
+}
+
+}  // namespace
+
+template <typename T>
+int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
+               int64_t lds, bool exact, int *scratch, cudaStream_t st) {
+    if (npts > (int64_t)INT32_MAX - 64) return fail(RS_EINVAL, "digit_gram: too many points");
+    const bool sym = X == Y && ldx == ldy && nx == ny;
+    int *keys = scratch;
+    if (!keys) {
+        cudaMemPool_t pool;
+        RS_TRY(scratch_pool(&pool));
+        if (cudaMallocFromPoolAsync((void **)&keys, sizeof(int) * (size_t)digit_gram_scratch_ints(nx, ny), pool, st) !=
+            cudaSuccess) {
+            cudaGetLastError();
+            return fail(RS_ENOMEM, "digit_gram: scratch allocation failed");
+        }
+    }
+    auto go = [&]() -> int {
+        const int64_t ne = std::max<int64_t>((int64_t)nx * ny, nx + ny);
+        k_digit_init<<<(unsigned)std::min<int64_t>(256, (ne + 255) / 256), 256, 0, st>>>(S, lds, nx, ny, keys, nx + ny);
+        RS_LAUNCH_CHECK();
+        const int gx = (nx + 31) / 32, gy = sym ? 0 : (ny + 31) / 32;
+        const int rows = (int)std::max<int64_t>(1, std::min<int64_t>((npts + 63) / 64, 152 * 8 / (gx + gy)));
+        k_digit_keys<T><<<dim3((unsigned)(gx + gy), (unsigned)rows), 256, 0, st>>>(X, ldx, nx, Y, ldy, ny, npts, gx, keys);
+        RS_LAUNCH_CHECK();
+        GramArgs<T> a{};
+        a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.lds = lds, a.nx = nx, a.ny = ny;
+        a.kx = keys, a.ky = sym ? keys : keys + nx;
+        a.S = S, a.dV = dV, a.sym = sym;
+        const int tm = (nx + DG_M - 1) / DG_M;
+        // 32 columns of Y fill half of a 64-wide tile
+        const bool narrow = ny <= 32;
+        if constexpr (sizeof(T) == 8) return narrow ? launch_gram<T, 8, 32>(a, tm, st) : launch_gram<T, 8, 64>(a, tm, st);
+        else if (exact) return narrow ? launch_gram<T, 7, 32>(a, tm, st) : launch_gram<T, 7, 64>(a, tm, st);
+        else return narrow ? launch_gram<T, 5, 32>(a, tm, st) : launch_gram<T, 5, 64>(a, tm, st);
+    };
+    const int rc = go();
+    if (!scratch && cudaFreeAsync(keys, st) != cudaSuccess && rc == RS_OK) return fail(RS_ECUDA, "digit_gram: cudaFreeAsync failed");
+    return rc;
+}
+template int digit_gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
+                                int64_t, bool, int *, cudaStream_t);
+template int digit_gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *,
+                               int64_t, bool, int *, cudaStream_t);
+
+// ----------------------------------------------------------- rotation ---
+
+namespace {
+
+template <typename T> struct RotArgs {
+    const T *X;
+    const double *C;
+    T *Y;
+    int64_t ldx, ldc, ldy, npts;
+    int n, m;
+    int vec, yvec;       // X, Y rows on 16-byte boundaries
+    int cluster;         // Y is X: the CTAs of a row tile form a cluster and write together
+    double alpha, beta;
+};
+
+// (H 2^(8 (NS - 4)) + L) 2^(8 NS + e) rounded to FP64, in integer instructions
+template <int NS> __device__ __forceinline__ double dg_value(int64_t H, int64_t L, int e) {
+    constexpr int SH = 8 * (NS - 4);          // H in units of L; NS = 8: 32
+    // 128-bit sum V = H 2^SH + L
+    uint64_t lo = (uint64_t)H << SH;
+    int64_t hi = H >> (64 - SH);
+    const uint64_t l2 = lo + (uint64_t)L;
+    hi += (L >> 63) + (l2 < lo ? 1 : 0);
+    lo = l2;
+    const uint64_t sg = (uint64_t)(hi >> 63);
+    // magnitude
+    lo ^= sg;
+    uint64_t h = (uint64_t)hi ^ sg;
+    lo -= sg;
+    h += (sg && lo == 0) ? 1 : 0;
+    if (!(h | lo)) return 0.0;
+    const int z = h ? __clzll((long long)h) : 64 + __clzll((long long)lo);
+    uint64_t top = z >= 64 ? lo << (z - 64) : (z ? (h << z) | (lo >> (64 - z)) : h);   // leading one at bit 63
+    const uint64_t rest = z >= 64 ? 0 : lo << z;
+    // round to nearest even at bit 11
+    const uint64_t tail = top & 0x7ff;
+    uint64_t man = top >> 11;
+    man += (tail > 0x400 || (tail == 0x400 && (rest || (man & 1)))) ? 1 : 0;
+    const int ex = 127 - z + 8 * NS + e;      // exponent of the leading one
+    // a carry out of the rounding moves into the exponent field by itself
+    const uint64_t bits = ((uint64_t)(ex + 1022) << 52) + man;
+    return __longlong_as_double((long long)(bits | (sg << 63)));
+}
+
+struct RotBars {
+    uint64_t keyfull[2], keyfree[2], rd;
+    int plain[2][4];   // per half and key warp: a row beyond the digits' range
+};
+
+// One CTA per SM, NBLK column blocks of C per CTA, row tiles dealt round robin:
+// the key warps find the exponents of the next tile's rows (and bring the
+// rows into L2) while the converters work on this one, and the readout and
+// the stores of a tile overlap the products of the next.
+template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
+    constexpr int PAD = 32;   // a quarter-warp's four 8-step groups of two rows fall in distinct banks
+    constexpr int KW = 3;     // key warps
+    using C = DgCfg<NS, BN, PAD>;
+    extern __shared__ __align__(128) unsigned char dgsm[];
+    __shared__ DgBars b;
+    __shared__ RotBars rb;
+    __shared__ int ea[2][DG_M], eb[NBLK * BN];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nb0 = blockIdx.x * NBLK;          // first column block
+    const int kst = (a.n + DG_K - 1) / DG_K;    // stages per column block
+    const int ntiles = (int)((a.npts + DG_M - 1) / DG_M);
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            dg_bar_init(&rb.keyfull[i], KW * 32);
+            dg_bar_init(&rb.keyfree[i], DG_CT + 1);   // the converters and the MMA warp's first lane
+        }
+        dg_bar_init(&rb.rd, DG_CT * (a.cluster ? gridDim.x : 1));
+    }
+    for (int i = tid; i < NBLK * BN; i += DG_NT) eb[i] = 0;
+    dg_setup<NS>(b, C::TMEM);
+    if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    // exponents of the columns of C
+    for (int blk = 0; blk < NBLK; ++blk)
+        for (int w = warp; w < BN / 32 * 12; w += DG_NT / 32) {
+            const int cl = (w / 12) * 32 + lane, c = (nb0 + blk) * BN + cl;
+            int k = 0;
+            if (c < a.m) {
+#pragma unroll 8
+                for (int q = w % 12; q < a.n; q += 12) k = max(k, abs_key(__ldg(a.C + (int64_t)q * a.ldc + c)));
+            }
+            if (k) atomicMax(&eb[blk * BN + cl], k);
+        }
+    __syncthreads();
+    for (int i = tid; i < NBLK * BN; i += DG_NT) {
+        const int k = eb[i];
+        if (ExpOf<double>::plain(k)) b.plain = 1;
+        eb[i] = ExpOf<double>::exponent(k);
+    }
+    __syncthreads();
+    const bool cplain = b.plain != 0;
+
+    if (warp > DG_CW) {
+        // key warps: eight rows at a time, four lanes to a row
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;\n");
+        int j = 0;
+        for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y, ++j) {
+            const int h = j & 1;
+            if (j >= 2 && !dg_wait(&rb.keyfree[h], (j / 2 - 1) & 1, &b.bad)) break;
+            const int64_t r0 = (int64_t)tile * DG_M;
+            const int rows = (int)min((int64_t)DG_M, a.npts - r0);
+            bool pl = false;
+            for (int g = warp - DG_CW - 1; g < DG_M / 8; g += KW) {
+                const int r = g * 8 + (lane >> 2);
+                const T *x = a.X + (r0 + min(r, rows - 1)) * a.ldx;
+                int k = 0;
+                if (a.vec) {
+                    constexpr int E = 16 / (int)sizeof(T);
+                    const uint4 *xv = reinterpret_cast<const uint4 *>(x);
+                    const int nv = a.n / E;
+                    int q = lane & 3;
+                    for (; q + 28 < nv; q += 32) {
+                        uint4 t[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) t[i] = xv[q + 4 * i];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const T *tt = reinterpret_cast<const T *>(&t[i]);
+#pragma unroll
+                            for (int e = 0; e < E; ++e) k = max(k, abs_key(tt[e]));
+                        }
+                    }
+                    for (; q < nv; q += 4) {
+                        const uint4 t = xv[q];
+                        const T *tt = reinterpret_cast<const T *>(&t);
+#pragma unroll
+                        for (int e = 0; e < E; ++e) k = max(k, abs_key(tt[e]));
+                    }
+                    for (q = nv * E + (lane & 3); q < a.n; q += 4) k = max(k, abs_key(x[q]));
+                } else {
+#pragma unroll 8
+                    for (int q = lane & 3; q < a.n; q += 4) k = max(k, abs_key(x[q]));
+                }
+                k = max(k, __shfl_xor_sync(0xffffffffu, k, 1));
+                k = max(k, __shfl_xor_sync(0xffffffffu, k, 2));
+                if ((lane & 3) == 0) ea[h][r] = ExpOf<T>::exponent(k);
+                pl = pl || ExpOf<T>::plain(k);
+            }
+            pl = __any_sync(0xffffffffu, pl);
+            if (lane == 0) rb.plain[h][warp - DG_CW - 1] = pl;
+            __syncwarp();
+            dg_arrive(&rb.keyfull[h]);
+        }
+    } else if (warp == DG_CW) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 72;\n");
+        DgIssue<NS, BN, PAD> mma(b, dgsm);
+        int j = 0;
+        bool ok = true;
+        for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
+            const int h = j & 1;
+            ok = __all_sync(0xffffffffu, dg_wait(&rb.keyfull[h], (j / 2) & 1, &b.bad));
+            const volatile int *f = rb.plain[h];
+            const bool pl = cplain || f[0] || f[1] || f[2];
+            __syncwarp();
+            if (lane == 0) dg_arrive(&rb.keyfree[h]);
+            if (!pl && ok) ok = mma.run(b, kst * NBLK, kst);
+        }
+        mma.finish(b);
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;\n");
+        // converter warp: rows 16 warp .. + 15 of A (a lane's unit: one row, 8
+        // steps; four lanes read 32 consecutive states of a row) and unit
+        // `warp` (32 columns, 8 steps) of B
+        constexpr int NB = BN / 32 * KQ;
+        static_assert(NB <= DG_CW, "one unit of B per warp");
+        const int ar = warp * 16 + (lane >> 2), akq = lane & 3;
+        unsigned char *adst = dgsm + akq * C::LBO_A + ar * 16;
+        const bool hasb = warp < NB;
+        const int bkq = warp % KQ, bcol = warp / KQ * 32 + lane;
+        unsigned char *bdst = dgsm + C::A_BYTES + bkq * C::LBO_B + bcol * 16;
+        const int col0 = (warp >> 2) * 32, row = (warp & 3) * 32 + lane;
+        const bool owns = col0 < BN;
+        const int nst = kst * NBLK;
+        bool ok = true;
+        T va[2][8];
+        double vb[8];
+        T held[NBLK > 1 ? 32 : 1];   // two blocks: the first one's results until the rows are read
+        int64_t H[32], L[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) H[i] = L[i] = 0;
+        auto load = [&](int tile, int it) {
+            const int blk = it >= kst ? 1 : 0, k0 = (it - blk * kst) * DG_K;   // (NBLK <= 2)
+            const int64_t r0 = (int64_t)tile * DG_M;
+            const int rows = (int)min((int64_t)DG_M, a.npts - r0);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const T *x = a.X + (r0 + min(ar + 8 * u, rows - 1)) * a.ldx + k0 + 8 * akq;
+                if (a.vec && k0 + 8 * akq + 8 <= a.n) {
+                    constexpr int E = 16 / (int)sizeof(T);
+#pragma unroll
+                    for (int q = 0; q < 8 / E; ++q) {
+                        const uint4 t = reinterpret_cast<const uint4 *>(x)[q];
+                        const T *tt = reinterpret_cast<const T *>(&t);
+#pragma unroll
+                        for (int i = 0; i < E; ++i) va[u][q * E + i] = tt[i];
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) va[u][k] = k0 + 8 * akq + k < a.n ? x[k] : T(0);
+                }
+            }
+            if (hasb) {
+                const int c = (nb0 + blk) * BN + bcol;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int kk = k0 + 8 * bkq + k;
+                    vb[k] = (c < a.m && kk < a.n) ? __ldg(a.C + (int64_t)kk * a.ldc + c) : 0.0;
+                }
+            }
+        };
+        // in place: tell every CTA of the row tile that this thread has read its rows
+        auto rows_read = [&]() {
+            if (!a.cluster) return;
+            for (int r = 0; r < (int)gridDim.x; ++r)
+                asm volatile(
+                    "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
+                    " mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(dg_su32(&rb.rd)),
+                    "r"(r)
+                    : "memory");
+        };
+        const T al = (T)a.alpha, be = (T)a.beta;
+        constexpr int E = 16 / (int)sizeof(T);
+        // E results of row p from column c on
+        auto put = [&](int64_t p, int c, T (&v)[E]) {
+            if (!ok) {
+#pragma unroll
+                for (int i = 0; i < E; ++i) v[i] = (T)__longlong_as_double(0x7ff8000000000000ll);
+            }
+            T *y = a.Y + p * a.ldy + c;
+            if (a.yvec && c + E <= a.m) {
+                uint4 t;
+                T *tt = reinterpret_cast<T *>(&t);
+                if (a.beta != 0.0) t = *reinterpret_cast<const uint4 *>(y);
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    if (a.alpha != 1.0) v[i] *= al;
+                    if (a.beta != 0.0) v[i] += be * tt[i];
+                    tt[i] = v[i];
+                }
+                *reinterpret_cast<uint4 *>(y) = t;
+            } else {
+#pragma unroll
+                for (int i = 0; i < E; ++i)
+                    if (c + i < a.m) {
+                        if (a.alpha != 1.0) v[i] *= al;
+                        if (a.beta != 0.0) v[i] += be * y[i];
+                        y[i] = v[i];
+                    }
+            }
+        };
+        // an interval of products whose accumulators are still to be read out:
+        // its tile, the exponent of this thread's row in it, its block, and
+        // whether it is the block's last
+        bool open = false, pend = false;
+        int ptile = 0, ptj = 0, pe = 0, pblk = 0, iv = 0;
+        auto readout = [&]() {
+            open = false;
+            ok = ok && dg_drain<NS, BN>(b, iv, owns ? col0 : 0, H, L);
+            ++iv;
+            if (!pend) return;
+            // the block's sums are complete
+            const bool lastb = pblk == NBLK - 1;
+            if (lastb && a.cluster) ok = dg_wait(&rb.rd, ptj & 1, &b.bad) && ok;
+            const int64_t p = (int64_t)ptile * DG_M + row;
+            const bool on = owns && p < a.npts;
+            if (NBLK > 1 && lastb && on) {
+#pragma unroll
+                for (int q = 0; q < 32 / E; ++q) {
+                    T v[E];
+#pragma unroll
+                    for (int i = 0; i < E; ++i) v[i] = held[NBLK > 1 ? q * E + i : 0];
+                    put(p, nb0 * BN + col0 + q * E, v);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 32 / E; ++q) {
+                T v[E];
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const int c = q * E + i, e = eb[pblk * BN + (owns ? col0 : 0) + c] - 1022 - 2 * (8 * NS - 2);
+                    if constexpr (sizeof(T) == 8) {
+                        v[i] = (T)dg_value<NS>(H[c], L[c], pe - 1022 + e);
+                    } else {
+                        // NS = 5: H 2^8 + L stays below 2^63
+                        v[i] = ldexpf(__ll2float_rn(H[c] * (int64_t)(1ll << (8 * (NS - 4))) + L[c]), 8 * NS + pe - 126 + e);
+                    }
+                    H[c] = L[c] = 0;
+                    if (NBLK > 1 && !lastb) held[NBLK > 1 ? c : 0] = v[i];
+                }
+                if (lastb && on) put(p, (nb0 + pblk) * BN + col0 + q * E, v);
+            }
+        };
+        // One loop over the stages of all tiles; it == nst: the next tile is due.
+        int tile = (int)blockIdx.y - (int)gridDim.y, j = -1, g = 0, it = nst, kb = 0, blk = 0, h = 0;
+        int ex0 = 0, ex1 = 0, er = 0;
+        if ((int)blockIdx.y < ntiles) load(blockIdx.y, 0);
+        while (ok) {
+            bool plain = false, flush = false, end = false;
+            if (it == nst) {
+                tile += gridDim.y;
+                ++j;
+                end = tile >= ntiles;
+                if (!end) {
+                    h = j & 1;
+                    ok = dg_wait(&rb.keyfull[h], (j / 2) & 1, &b.bad);
+                    ex0 = ea[h][ar], ex1 = ea[h][ar + 8], er = ea[h][row];
+                    const volatile int *f = rb.plain[h];
+                    plain = cplain || f[0] || f[1] || f[2];
+                    dg_arrive(&rb.keyfree[h]);
+                    if (!plain) it = kb = blk = 0;
+                }
+                flush = open && (end || plain);
+            }
+            if (!end && !plain && ok) {
+                const int s = g % DG_STAGES;
+                if (g >= DG_STAGES) ok = dg_wait(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.bad);
+                if (ok) {
+                    store_digits<T, NS>(va[0], ex0, adst + s * C::STAGE, C::SL_A);
+                    store_digits<T, NS>(va[1], ex1, adst + s * C::STAGE + 128, C::SL_A);
+                    if (hasb) store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B);
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                    dg_arrive(&b.full[s]);
+                }
+                const bool lasts = it + 1 == nst;
+                if (lasts) rows_read();
+                if (!lasts || tile + (int)gridDim.y < ntiles) load(lasts ? tile + gridDim.y : tile, lasts ? 0 : it + 1);
+                flush = kb % DG_DRAIN == 0 && open;
+            }
+            if (flush) readout();
+            if (end) break;
+            if (plain) {
+                // a row or column beyond the digits' range: plain sums, then the
+                // same order as above (rows read by all, then written)
+                const int64_t p = min((int64_t)tile * DG_M + row, a.npts - 1);
+                T sum[NBLK * 32];
+                for (int i = 0; i < NBLK * 32; ++i) {
+                    const int c = (nb0 + i / 32) * BN + col0 + i % 32;
+                    double t = 0;
+                    if (owns && c < a.m)
+                        for (int k = 0; k < a.n; ++k)
+                            t = fma((double)a.X[p * a.ldx + k], __ldg(a.C + (int64_t)k * a.ldc + c), t);
+                    sum[i] = (T)t;
+                }
+                asm volatile("bar.sync 1, 256;\n" ::: "memory");   // every converter of this CTA has read its row
+                rows_read();
+                if (a.cluster) ok = dg_wait(&rb.rd, j & 1, &b.bad) && ok;
+                if (owns && (int64_t)tile * DG_M + row < a.npts)
+                    for (int i = 0; i < NBLK * 32; ++i) {
+                        const int c = (nb0 + i / 32) * BN + col0 + i % 32;
+                        if (c < a.m) {
+                            T v = sum[i], *y = a.Y + p * a.ldy + c;
+                            if (a.alpha != 1.0) v *= al;
+                            if (a.beta != 0.0) v += be * *y;
+                            *y = v;
+                        }
+                    }
+                if (tile + (int)gridDim.y < ntiles) load(tile + gridDim.y, 0);
+            } else {
+                if (kb % DG_DRAIN == DG_DRAIN - 1 || kb == kst - 1) {
+                    open = true;
+                    pend = kb == kst - 1;
+                    ptile = tile, ptj = j, pe = er, pblk = blk;
+                }
+                ++it, ++g;
+                if (++kb == kst) kb = 0, ++blk;
+            }
+        }
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    if (warp == DG_CW)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(b.tmem), "r"(C::TMEM) : "memory");
+    // no CTA leaves while another may still signal it
+    if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, int cluster, cudaStream_t st) {
+    using C = DgCfg<NS, BN, 32>;
+    auto fn = k_digit_rot<T, NS, BN, NBLK>;
+    RS_TRY(smem_optin((const void *)fn, C::SMEM));
+    const unsigned gx = (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK));
+    const int64_t tiles = (a.npts + DG_M - 1) / DG_M;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(gx, 1);
+    cfg.blockDim = dim3(DG_NT);
+    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cluster ? gx : 1;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    a.cluster = cluster && gx > 1;
+    // as many row workers as are resident at once
+    int workers = 0;
+    if (a.cluster) {
+        RS_CUDA(cudaOccupancyMaxActiveClusters(&workers, fn, &cfg));
+    } else {
+        RS_TRY(sm_count(&workers));
+        workers /= (int)gx;
+    }
+    cfg.gridDim.y = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, workers));
+    RS_CUDA(cudaLaunchKernelEx(&cfg, fn, a));
+    return RS_OK;
+}
+
+}  // namespace
+
+// In place, the CTAs of a row tile are one cluster of at most 8 (64 columns
+// each, or two blocks of 64).  A contraction of more than 2^15 states could
+// leave the 64-bit sums.
+bool digit_rot_takes(int n, int m, bool in_place) {
+    return n <= 32768 && (!in_place || m <= 1024);
+}
+
+template <typename T>
+int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
+              double alpha, double beta, cudaStream_t st) {
+    RotArgs<T> a{};
+    a.X = X, a.C = C, a.Y = Y, a.ldx = ldx, a.ldc = ldc, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
+    a.alpha = alpha, a.beta = beta;
+    a.vec = aligned16(X) && (ldx * (int64_t)sizeof(T)) % 16 == 0;
+    a.yvec = aligned16(Y) && (ldy * (int64_t)sizeof(T)) % 16 == 0;
+    constexpr int NS = sizeof(T) == 8 ? 8 : 5;
+    const bool in_place = X == Y;
+    if (m <= 32) return launch_rot<T, NS, 32, 1>(a, 0, st);
+    if (in_place && m > 512) return launch_rot<T, NS, 64, 2>(a, 1, st);
+    return launch_rot<T, NS, 64, 1>(a, in_place, st);
+}
+template int digit_rot<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
+                               double, double, cudaStream_t);
+template int digit_rot<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
+                              double, cudaStream_t);
+
+}  // namespace rs

@@ -1,0 +1,31 @@
+// FP64- and FP32-accurate contractions on the tensor cores by integer digits
+// (see digits.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace rs {
+
+// Ints of scratch the overlap of nx and ny columns needs.
+inline int64_t digit_gram_scratch_ints(int nx, int ny) { return (int64_t)nx + ny; }
+
+// S (nx x ny, FP64, row stride lds) = dV X^T Y over npts points.  Accuracy:
+// the digits of an operand resolve 2^-62 (FP64), 2^-54 (FP32, exact = true)
+// or 2^-38 (FP32, exact = false) of its column's largest entry.
+// scratch: digit_gram_scratch_ints ints of device memory, or nullptr (taken
+// from the library's stream-ordered pool).  Asynchronous.
+template <typename T>
+int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
+               int64_t lds, bool exact, int *scratch, cudaStream_t st);
+
+// Y (m columns) = alpha X C + beta Y, X [npts][ldx] (n columns), C FP64
+// [n][ldc]; Y may be X itself (same pointer and leading dimension) when
+// beta == 0.  digit_rot_takes says whether the sizes are taken.
+bool digit_rot_takes(int n, int m, bool in_place);
+template <typename T>
+int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
+              double alpha, double beta, cudaStream_t st);
+
+}  // namespace rs

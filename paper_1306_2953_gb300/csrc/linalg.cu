@@ -2,15 +2,11 @@
 // orthogonalisation (Eq. 6) and subspace diagonalisation (Eqs. 7-8).
 //
 // Tall-skinny contractions over grid points:
-//   k_gram    S = dV X^T Y, split over blocks of points ("blocks of points",
-//             Sec. VI) and accumulated in FP64.  FP64 data: FP64 FMA.  FP32
-//             data: every product is formed exactly as a float pair (fma
-//             error term) and accumulated as a compensated float pair, so
-//             the FP64 result is accurate to ~2^-44 relative while running
-//             on the FP32 pipes (FP64 throughput on this part is 1/64 of
-//             FP32).
-//   k_rowmul  Y = alpha X C + beta Y applied row by row (each CTA owns whole
-//             rows), so the in-place update Psi <- Psi C needs no copy.
+//   digits.cu S = dV X^T Y and Y = alpha X C + beta Y as exact sums of integer
+//             digit products on the tensor cores.
+//   k_rowmul  the rotation row by row with FP64 (FP32) FMA (each CTA owns whole
+//             rows), for in-place rotations of more than 1024 columns, whose
+//             row tiles do not fit one cluster of CTAs.
 // Small dense kernels (n <= a few hundred, FP64 unless stated):
 //   k_chol    S = U^T U, right-looking, one CTA, status on failure
 //   k_trinv   U^-1 by back substitution, one thread per column
@@ -24,125 +20,20 @@
 #include <vector>
 
 #include "device.h"
+#include "digits.h"
 #include "linalg.h"
 
 namespace rs {
 
-// ------------------------------------------------------------- k_gram ---
-
-constexpr int G_TM = 64, G_TN = 64, G_TK = 16, G_NT = 256;
-
-// Error-free transformation s + e = a + b (Knuth); the _rn intrinsics keep
-// the compiler from contracting any step into a fused multiply-add.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = __fadd_rn(a, b);
-    const float z = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-}
-
-// FP64 data: plain FP64 accumulation.  FP32 data: compensated float pairs.
-template <typename T> struct GramAcc;
-template <> struct GramAcc<double> {
-    double v = 0;
-    __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
-    __device__ __forceinline__ double value() const { return v; }
-};
-// FP32 data, plain FP32 accumulation within a chunk of points (the inner
-// iterations of the FP32 mode); chunks are combined in FP64.
-struct GramAccFast {
-    float v = 0;
-    __device__ __forceinline__ void add(float a, float b) { v = fmaf(a, b, v); }
-    __device__ __forceinline__ double value() const { return (double)v; }
-};
-template <> struct GramAcc<float> {
-    float hi = 0, lo = 0;
-    __device__ __forceinline__ void add(float a, float b) {
-        const float p = __fmul_rn(a, b);
-        const float pe = fmaf(a, b, -p);   // exact: a*b = p + pe
-        float s, e;
-        two_sum(hi, p, s, e);
-        hi = s;
-        lo += e + pe;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
-// S[i][j] += dV * sum_{p in chunk} X[p][i] Y[p][j]; grid (ceil(nx/64), ceil(ny/64), splits)
-template <typename T, typename ACC = GramAcc<T>>
-__global__ void __launch_bounds__(G_NT) k_gram(const T *__restrict__ X, int64_t ldx, int nx, const T *__restrict__ Y,
-                                               int64_t ldy, int ny, int64_t npts, int64_t chunk, double dV,
-                                               double *__restrict__ S, int64_t lds) {
-    __shared__ T xs[G_TK][G_TM + 1];
-    __shared__ T ys[G_TK][G_TN + 1];
-    const int i0 = blockIdx.x * G_TM, j0 = blockIdx.y * G_TN;
-    const int64_t p0 = (int64_t)blockIdx.z * chunk;
-    const int64_t p1 = min(npts, p0 + chunk);
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // 4x4 micro tile at (4ty.., 4tx..)
-    ACC acc[4][4];
-    for (int64_t pk = p0; pk < p1; pk += G_TK) {
-        for (int e = threadIdx.x; e < G_TK * G_TM; e += G_NT) {
-            const int k = e / G_TM, c = e % G_TM;
-            const int64_t p = pk + k;
-            xs[k][c] = (p < p1 && i0 + c < nx) ? X[p * ldx + i0 + c] : T(0);
-            ys[k][c] = (p < p1 && j0 + c < ny) ? Y[p * ldy + j0 + c] : T(0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < G_TK; ++k) {
-            T a[4], b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = xs[k][4 * ty + u];
-                b[u] = ys[k][4 * tx + u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v].add(a[u], b[v]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int i = i0 + 4 * ty + u, j = j0 + 4 * tx + v;
-            if (i < nx && j < ny) atomicAdd(S + (int64_t)i * lds + j, dV * acc[u][v].value());
-        }
-}
-
-__global__ void k_zero2d(double *S, int64_t lds, int n, int m) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)n * m; e += (int64_t)gridDim.x * blockDim.x)
-        S[(e / m) * lds + e % m] = 0.0;
-}
-
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-         int64_t lds, cudaStream_t st, bool fast) {
-    k_zero2d<<<64, 256, 0, st>>>(S, lds, nx, ny);
-    RS_LAUNCH_CHECK();
-    const int gx = (nx + G_TM - 1) / G_TM, gy = (ny + G_TN - 1) / G_TN;
-    // enough CTAs to fill the GPU twice over, each over a contiguous chunk of points
-    int splits = (int)std::max<int64_t>(1, std::min<int64_t>((npts + 255) / 256, (152 * 8) / std::max(1, gx * gy)));
-    int64_t chunk = (npts + splits - 1) / splits;
-    chunk = (chunk + G_TK - 1) / G_TK * G_TK;
-    splits = (int)((npts + chunk - 1) / chunk);
-    dim3 grid(gx, gy, splits);
-    if constexpr (sizeof(T) == 4) {
-        if (fast) {
-            k_gram<float, GramAccFast><<<grid, G_NT, 0, st>>>(X, ldx, nx, Y, ldy, ny, npts, chunk, dV, S, lds);
-            RS_LAUNCH_CHECK();
-            return RS_OK;
-        }
-    }
-    k_gram<T><<<grid, G_NT, 0, st>>>(X, ldx, nx, Y, ldy, ny, npts, chunk, dV, S, lds);
-    RS_LAUNCH_CHECK();
-    return RS_OK;
+         int64_t lds, cudaStream_t st, bool fast, int *scratch) {
+    return digit_gram<T>(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, !fast, scratch, st);
 }
 template int gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
-                          int64_t, cudaStream_t, bool);
+                          int64_t, cudaStream_t, bool, int *);
 template int gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *, int64_t,
-                         cudaStream_t, bool);
+                         cudaStream_t, bool, int *);
 
 // ----------------------------------------------------------- k_rowmul ---
 // Y[p][0:m] = alpha * sum_k X[p][k] C[k][0:m] + beta * Y[p][0:m] for a tile of
@@ -185,6 +76,7 @@ __global__ void __launch_bounds__(R_NT) k_rowmul(const T *X, int64_t ldx, int n,
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
            double alpha, double beta, cudaStream_t st) {
+    if (digit_rot_takes(n, m, X == Y)) return digit_rot<T>(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, st);
     const size_t smem = (size_t)R_ROWS * n * sizeof(T);
     if (smem > 200 * 1024) return fail(RS_EINVAL, "rowmul: n too large");
     if (smem > 48 * 1024) RS_TRY(smem_optin((const void *)k_rowmul<T>, smem));

@@ -14,7 +14,7 @@ namespace rs {
 // FP32 accumulation within chunks of points combined in FP64.
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-         int64_t lds, cudaStream_t st, bool fast = false);
+         int64_t lds, cudaStream_t st, bool fast = false, int *scratch = nullptr);
 
 // Y = alpha X C + beta Y row by row; X [npts][ldx] (n columns), C FP64 [n][ldc]
 // (m columns), Y [npts][ldy]; Y may alias X when beta == 0.

@@ -65,12 +65,13 @@ int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, 
 int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, int dtype, void *work, cudaStream_t st,
                         const TcWork &tc) {
     LaWork w(work, n);
+    int *keys = reinterpret_cast<int *>(w.xi);   // not in use yet: scratch of the overlap
     if (dtype == RS_F64)
-        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st));
+        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st, false, keys));
     else if (tc_grams(tc, n, npts))
         RS_TRY(umma_gram((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, tc.p, tc.err, st));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st, false, keys));
     RS_TRY(symmetrize(w.U, n, n, st));
     RS_TRY(cholesky(w.U, n, n, 1e-14, w.status, st));
     int bad = 0;
@@ -91,12 +92,13 @@ int subspace_diag_impl(rs_ham *h, void *Psi, void *HPsi, int64_t ld, int n, int 
     for (int b = 0; b < n; b += nb)
         RS_TRY(rs_ham_apply_block(h, (const char *)Psi + (size_t)b * es, ld, (char *)HPsi + (size_t)b * es, ld,
                                   std::min(nb, n - b), dtype, st));
+    int *keys = reinterpret_cast<int *>(w.xi);
     if (dtype == RS_F64)
-        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st));
+        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys));
     else if (tc_grams(tc, n, npts))
         RS_TRY(umma_gram((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, tc.p, tc.err, st));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys));
     RS_TRY(symmetrize(w.S, n, n, st));
     RS_TRY(eigh(w.S, n, n, eps_dev, w.xi, n, dtype == RS_F32 && tc.inner ? -1 : 2, w.status, w.eigw, st));
     RS_TRY(rotate_inplace(Psi, ld, n, w.xi, npts, dtype, st, tc));
