@@ -9,29 +9,21 @@
 //     FP32 blocks of 32-state groups take k_project_f32 (four states per lane
 //     and four sphere entries per warp step, the atom split sized to fill the
 //     GPU).
-//  2. k_stencil: the 25-point star kinetic stencil (Sec. V.A), the local
-//     potential (Sec. V.B) and the nonlocal sum of Eq. (4), fused.  Each CTA
-//     owns a TX x TY column of lattice points (axes 2 and 1 of the point
-//     map) and one group of SG states, and marches along axis 0.  Every
-//     thread keeps a 2x2 patch of columns for one state in registers with a
-//     9-deep queue along the march axis, so the axis-0 neighbours come from
-//     registers; the current plane (interior written from the queues, the
-//     4-point x/y halos staged by cp.async three planes deep) sits in shared
-//     memory for the axis-1/axis-2 neighbours.  The nonlocal term is a
-//     gather: each output point sums over the atoms whose spheres cover it,
-//     so overlapping spheres need neither atom colouring (Sec. V.C, Fig. 10)
-//     nor atomics, and the output is written exactly once.
+//  2. k_gather: the 25-point star kinetic stencil (Sec. V.A), the local
+//     potential (Sec. V.B) and the nonlocal sum of Eq. (4), fused: every
+//     point reads its 24 neighbours' rows.  The nonlocal term is a gather too
+//     (each output point sums over the atoms whose spheres cover it), so
+//     overlapping spheres need neither atom colouring (Sec. V.C, Fig. 10) nor
+//     atomics, and the output is written exactly once.
 // Orbitals are [npts][ld] with the state index fastest (Sec. IV, Fig. 4b);
 // grid points are addressed through the int32 point map (Sec. V.A).
 // FP32 blocks whose state count is a multiple of 32 take the persistent
-// ring-buffer kernel of stencil_ring.cu for step 2 instead; k_stencil serves
+// ring-buffer kernel of stencil_ring.cu for step 2 instead; k_gather serves
 // FP64 blocks, narrower state groups and layouts that kernel cannot copy.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
 #include <new>
-#include <utility>
 #include <vector>
 
 #include "device.h"
@@ -48,10 +40,6 @@
 // before cutting them into per-CTA runs (the default: whole columns).
 #ifndef RS_RING_SLAB
 #define RS_RING_SLAB 4096
-#endif
-
-#ifndef RS_STENCIL_MINB_F32
-#define RS_STENCIL_MINB_F32 1
 #endif
 
 namespace rs {
@@ -75,21 +63,6 @@ template <typename T> struct HamDev {
 template <typename T> __device__ __forceinline__ T point_v(int4 inf);
 template <> __device__ __forceinline__ float point_v<float>(int4 inf) { return __int_as_float(inf.z); }
 template <> __device__ __forceinline__ double point_v<double>(int4 inf) { return __hiloint2double(inf.w, inf.z); }
-
-template <int BYTES> __device__ __forceinline__ void cp_async(void *smem, const void *gmem, bool valid) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    const int sz = valid ? BYTES : 0;
-    if constexpr (BYTES == 16) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(sz) : "memory");
-    } else {
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(s), "l"(gmem), "n"(BYTES), "r"(sz)
-                     : "memory");
-    }
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 
 template <typename T> struct Four { T a, b, c, d; };
 __device__ __forceinline__ Four<float> load4(const float *p) {
@@ -206,210 +179,140 @@ __global__ void __launch_bounds__(NTP4) k_project_f32(HamDev<float> d, const flo
 
 // ------------------------------------------- fused stencil + V + nonlocal ---
 
-// Maximum number of planes of one work item (the z chunk).
-constexpr int ZCHUNK = 32;
+// V states of one point, read and written as one access.
+template <typename T, int V> struct __align__(sizeof(T) * V) Pack { T v[V]; };
 
-template <typename T, int SG, int TX, int TY> struct StencilCfg {
-    static constexpr int W2 = TX + 8, W1 = TY + 8;
-    static constexpr int PLANE = W1 * W2 * SG;
-    static constexpr int NT = (TX / 2) * (TY / 2) * SG;
-    static constexpr int RING = 3;
-    static constexpr int CHB = (SG * (int)sizeof(T) >= 16) ? 16 : SG * (int)sizeof(T);
-    static constexpr int CHE = CHB / (int)sizeof(T);
-    static constexpr int CPR = SG / CHE;
-    static constexpr int NH = 8 * TY + 8 * TX;
-    static constexpr int HPT = (NH * CPR + NT - 1) / NT;     // halo copies per thread and plane
-    static constexpr int NI = TX * TY;
-    static constexpr bool STAGE = NI <= 128;                  // stage interior rows in shared memory
-    static constexpr int NROW = STAGE ? (ZCHUNK + 9) * NI : 0;
-    static constexpr size_t SMEM = (size_t)RING * PLANE * sizeof(T) + (size_t)NROW * sizeof(int);
-    static constexpr int MINB = sizeof(T) == 4 ? RS_STENCIL_MINB_F32 : 1;
+template <typename T, int V> __device__ __forceinline__ void add_to(Pack<T, V> &a, const Pack<T, V> &b) {
+    if constexpr (sizeof(T) == 4 && V % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < V; i += 2) {
+            const float2 r = __fadd2_rn(make_float2(a.v[i], a.v[i + 1]), make_float2(b.v[i], b.v[i + 1]));
+            a.v[i] = r.x;
+            a.v[i + 1] = r.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) a.v[i] += b.v[i];
+    }
+}
+template <typename T, int V> __device__ __forceinline__ void fma_to(Pack<T, V> &acc, T w, const Pack<T, V> &b) {
+    if constexpr (sizeof(T) == 4 && V % 2 == 0) {
+#pragma unroll
+        for (int i = 0; i < V; i += 2) {
+            const float2 r = __ffma2_rn(make_float2(w, w), make_float2(b.v[i], b.v[i + 1]), make_float2(acc.v[i], acc.v[i + 1]));
+            acc.v[i] = r.x;
+            acc.v[i + 1] = r.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc.v[i] = fma(w, b.v[i], acc.v[i]);
+    }
+}
+
+// A CTA takes PTS consecutive points in storage order.  First the 24 neighbour
+// indices of every point go from the point map to shared memory (four along
+// one direction at a time); then LPP lanes a point, V states a lane, read the 24
+// rows, sum the six at each distance, and add the potential and the nonlocal
+// terms.  The rows come from L1 and L2: points that follow one another in
+// storage are lattice neighbours, so a CTA's rows overlap.
+// Why no march with register queues (the kernel before this one): a march
+// needs long columns per CTA, which left most SMs without work on small grids
+// and one CTA of latency-bound steps on each of the others.  Measured, us per
+// block, march -> gather: 103 331 points, FP32 16 states 68 -> 15.7, FP64 16
+// states 699 -> 115; 654 520 points, FP32 16 states 273 -> 91, FP64 32 states
+// 2338 -> 1211 (1060 at the FP64 pipe's rate, 25 operations per value: bound
+// by that pipe; the FP32 blocks by the rows' way from L2).
+constexpr int GT_NT = 256;
+template <typename T, int V, int LPP> struct GatherCfg {
+    static constexpr int PP = GT_NT / LPP;                 // points per pass
+    static constexpr int PTS = PP > 64 ? PP : 64;
 };
 
-template <typename T, int SG, int TX, int TY>
-__global__ void __launch_bounds__(StencilCfg<T, SG, TX, TY>::NT, StencilCfg<T, SG, TX, TY>::MINB)
-    k_stencil(HamDev<T> d, const T *__restrict__ psi, int64_t ldp, T *__restrict__ hpsi, int64_t ldh,
-              const T *__restrict__ cproj, int nb, const int4 *__restrict__ work) {
-    using C = StencilCfg<T, SG, TX, TY>;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    T *sm = reinterpret_cast<T *>(smraw);
-    int *rows = reinterpret_cast<int *>(smraw + (size_t)C::RING * C::PLANE * sizeof(T));
-
+template <typename T, int V, int LPP>
+__global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__restrict__ loc, int npts,
+                                                  const T *__restrict__ psi, int64_t ldp, T *__restrict__ hpsi, int64_t ldh,
+                                                  const T *__restrict__ cproj, int nb) {
+    using C = GatherCfg<T, V, LPP>;
+    using P = Pack<T, V>;
+    __shared__ int4 nbr[6][C::PTS];
     const int tid = threadIdx.x;
-    const int s = tid % SG;
-    const int patch = tid / SG;
-    const int lx = 2 * (patch % (TX / 2));
-    const int ly = 2 * (patch / (TX / 2));
-    const int4 wk = work[blockIdx.x];
-    const int b1 = wk.x * TY, b2 = wk.y * TX;
-    const int za = wk.z, zb = wk.w;
-    const int sg0 = blockIdx.y * SG;
-    const T *psig = psi + sg0;
-
-    auto map_at = [&](int a0, int a1, int a2) -> int {
-        if ((unsigned)a0 >= (unsigned)d.d0 || (unsigned)a1 >= (unsigned)d.d1 || (unsigned)a2 >= (unsigned)d.d2)
-            return -1;
-        return __ldg(d.map + ((int64_t)a0 * d.d1 + a1) * d.d2 + a2);
-    };
-    // interior point rows of planes za-4 .. zb+4, staged once per work item
-    if constexpr (C::STAGE) {
-        const int nrow = (zb - za + 9) * C::NI;
-        for (int e = tid; e < nrow; e += C::NT) {
-            const int pl = e / C::NI, pos = e % C::NI;
-            rows[e] = map_at(za - 4 + pl, b1 + pos / TX, b2 + pos % TX);
-        }
+    const int p0 = blockIdx.x * C::PTS;
+    const int np = min(C::PTS, npts - p0);
+    const int strides[3] = {d.d1 * d.d2, d.d2, 1};
+    for (int e = tid; e < 6 * C::PTS; e += GT_NT) {
+        const int g = e / C::PTS, q = e - g * C::PTS;
+        if (q >= np) continue;
+        const int st = (g & 1) ? -strides[g >> 1] : strides[g >> 1];
+        const int32_t *m = d.map + __ldg(loc + p0 + q);
+        nbr[g][q] = make_int4(__ldg(m + st), __ldg(m + 2 * st), __ldg(m + 3 * st), __ldg(m + 4 * st));
     }
-    auto row_of = [&](int z, int iy, int ix) -> int {
-        if constexpr (C::STAGE) return rows[(z - za + 4) * C::NI + iy * TX + ix];
-        return map_at(z, b1 + iy, b2 + ix);
-    };
-    auto load_val = [&](int r) -> T { return r >= 0 ? __ldg(psig + (int64_t)r * ldp + s) : T(0); };
-
-    // this thread's halo copies j < HPT: copy index i = tid + j NT -> (hy, hx, chunk)
-    auto halo_pos = [&](int i, int &hy, int &hx, int &c) {
-        const int hh = i / C::CPR;
-        c = i % C::CPR;
-        if (hh < 8 * TY) {
-            hy = hh >> 3;
-            const int t = hh & 7;
-            hx = t < 4 ? t - 4 : TX + t - 4;
-        } else {
-            const int h2 = hh - 8 * TY;
-            hx = h2 % TX;
-            const int t = h2 / TX;
-            hy = t < 4 ? t - 4 : TY + t - 4;
-        }
-    };
-    int hr[C::HPT];
-    auto halo_rows = [&](int z) {
-#pragma unroll
-        for (int j = 0; j < C::HPT; ++j) {
-            const int i = tid + j * C::NT;
-            int hy, hx, c;
-            halo_pos(i, hy, hx, c);
-            hr[j] = i < C::NH * C::CPR ? map_at(z, b1 + hy, b2 + hx) : -1;
-        }
-    };
-    auto issue_halo = [&](int slot) {
-        T *base = sm + slot * C::PLANE;
-#pragma unroll
-        for (int j = 0; j < C::HPT; ++j) {
-            const int i = tid + j * C::NT;
-            if (i >= C::NH * C::CPR) continue;
-            int hy, hx, c;
-            halo_pos(i, hy, hx, c);
-            const T *src = hr[j] >= 0 ? psig + (int64_t)hr[j] * ldp + c * C::CHE : psig;
-            cp_async<C::CHB>(base + ((hy + 4) * C::W2 + (hx + 4)) * SG + c * C::CHE, src, hr[j] >= 0);
-        }
-    };
     __syncthreads();
-
-    T q[2][2][9];
+    const int lane = tid % LPP;
+    const T *ps = psi + lane * V;
+    for (int q = tid / LPP; q < C::PTS; q += C::PP) {
+        if (q >= np) break;
+        int id[6][4];
+        bool all = true;
 #pragma unroll
-    for (int k = 0; k < 9; ++k)
+        for (int g = 0; g < 6; ++g) {
+            const int4 n = nbr[g][q];
+            id[g][0] = n.x, id[g][1] = n.y, id[g][2] = n.z, id[g][3] = n.w;
+            all = all && (n.x | n.y | n.z | n.w) >= 0;
+        }
+        const int p = p0 + q;
+        const int4 inf = __ldg(d.pinfo + p);
+        const P c = *reinterpret_cast<const P *>(ps + (int64_t)p * ldp);
+        // from the smallest weight to the largest, so that the roundings of the
+        // large terms come last
+        P acc;
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
+        for (int i = 0; i < V; ++i) acc.v[i] = T(0);
+        if (all) {
 #pragma unroll
-            for (int dx = 0; dx < 2; ++dx) q[dy][dx][k] = load_val(row_of(za - 4 + k, ly + dy, lx + dx));
-
-    halo_rows(za);
-    issue_halo(0);
-    cp_async_commit();
-    halo_rows(za + 1);
-    if (za + 1 < zb) issue_halo(1);
-    cp_async_commit();
-    halo_rows(za + 2);
-
-    const T w0 = d.w[0], w1 = d.w[1], w2 = d.w[2], w3 = d.w[3], w4 = d.w[4];
-    int slot = 0;
-    for (int z = za; z < zb; ++z) {
-        const int pslot = slot == 0 ? 2 : slot - 1;  // (slot + 2) % 3
-        if (z + 2 < zb) issue_halo(pslot);
-        cp_async_commit();
-
-        T nq[2][2];
+            for (int j = 3; j >= 0; --j) {
+                P n[6];
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) nq[dy][dx] = load_val(row_of(z + 5, ly + dy, lx + dx));
-
-        T *P = sm + slot * C::PLANE;
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) P[((ly + dy + 4) * C::W2 + lx + dx + 4) * SG + s] = q[dy][dx][4];
-        cp_async_wait<2>();
-        __syncthreads();
-
-        // axis-0 neighbours from the register queues
-        T acc[2][2];
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) {
-                acc[dy][dx] = w0 * q[dy][dx][4] + w1 * (q[dy][dx][5] + q[dy][dx][3]) +
-                              w2 * (q[dy][dx][6] + q[dy][dx][2]) + w3 * (q[dy][dx][7] + q[dy][dx][1]) +
-                              w4 * (q[dy][dx][8] + q[dy][dx][0]);
+                for (int g = 0; g < 6; ++g) n[g] = *reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp);
+                add_to(n[0], n[1]);
+                add_to(n[2], n[3]);
+                add_to(n[4], n[5]);
+                add_to(n[0], n[2]);
+                add_to(n[0], n[4]);
+                fma_to(acc, d.w[j + 1], n[0]);
             }
-        // axis-2 neighbours: one row of 10 values per patch row (8 from shared memory)
+        } else {
+            // a neighbour off the grid contributes nothing
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy) {
-            T v[10];
+            for (int j = 3; j >= 0; --j) {
+                P n[6];
 #pragma unroll
-            for (int k = 0; k < 10; ++k)
-                if (k != 4 && k != 5) v[k] = P[((ly + dy + 4) * C::W2 + lx + k) * SG + s];
-            v[4] = q[dy][0][4];
-            v[5] = q[dy][1][4];
+                for (int g = 0; g < 6; ++g) {
 #pragma unroll
-            for (int dx = 0; dx < 2; ++dx)
-                acc[dy][dx] += w1 * (v[5 + dx] + v[3 + dx]) + w2 * (v[6 + dx] + v[2 + dx]) +
-                               w3 * (v[7 + dx] + v[1 + dx]) + w4 * (v[8 + dx] + v[0 + dx]);
-        }
-        // axis-1 neighbours: one column of 10 values per patch column
-#pragma unroll
-        for (int dx = 0; dx < 2; ++dx) {
-            T v[10];
-#pragma unroll
-            for (int k = 0; k < 10; ++k)
-                if (k != 4 && k != 5) v[k] = P[((ly + k) * C::W2 + lx + dx + 4) * SG + s];
-            v[4] = q[0][dx][4];
-            v[5] = q[1][dx][4];
-#pragma unroll
-            for (int dy = 0; dy < 2; ++dy)
-                acc[dy][dx] += w1 * (v[5 + dy] + v[3 + dy]) + w2 * (v[6 + dy] + v[2 + dy]) +
-                               w3 * (v[7 + dy] + v[1 + dy]) + w4 * (v[8 + dy] + v[0 + dy]);
-        }
-        // local potential, nonlocal gather, store
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) {
-                const int r = row_of(z, ly + dy, lx + dx);
-                if (r < 0) continue;
-                const int4 inf = __ldg(d.pinfo + r);
-                T out = acc[dy][dx] + point_v<T>(inf) * q[dy][dx][4];
-                for (int e = inf.x; e < inf.y; ++e) {
-                    const int A = __ldg(d.cov_atom + e);
-                    const Four<T> g = load4(d.cov_gam + 4 * (int64_t)e);
-                    const Four<T> c4 = load4(cproj + ((int64_t)A * nb + sg0 + s) * 4);
-                    out += g.a * c4.a + g.b * c4.b + g.c * c4.c + g.d * c4.d;
+                    for (int i = 0; i < V; ++i) n[g].v[i] = T(0);
+                    if (id[g][j] >= 0) n[g] = *reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp);
                 }
-                hpsi[(int64_t)r * ldh + sg0 + s] = out;
+                add_to(n[0], n[1]);
+                add_to(n[2], n[3]);
+                add_to(n[4], n[5]);
+                add_to(n[0], n[2]);
+                add_to(n[0], n[4]);
+                fma_to(acc, d.w[j + 1], n[0]);
             }
-
+        }
+        fma_to(acc, d.w[0], c);
+        fma_to(acc, point_v<T>(inf), c);
+        for (int e = inf.x; e < inf.y; ++e) {
+            const int A = __ldg(d.cov_atom + e);
+            const Four<T> g = load4(d.cov_gam + 4 * (int64_t)e);
+            const T *cp = cproj + ((int64_t)A * nb + lane * V) * 4;
 #pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-            for (int dx = 0; dx < 2; ++dx) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) q[dy][dx][k] = q[dy][dx][k + 1];
-                q[dy][dx][8] = nq[dy][dx];
+            for (int i = 0; i < V; ++i) {
+                const Four<T> c4 = load4(cp + 4 * i);
+                acc.v[i] += g.a * c4.a + g.b * c4.b + g.c * c4.c + g.d * c4.d;
             }
-        halo_rows(z + 3);
-        slot = slot == 2 ? 0 : slot + 1;
-        __syncthreads();
+        }
+        *reinterpret_cast<P *>(hpsi + (int64_t)p * ldh + lane * V) = acc;
     }
-    cp_async_wait<0>();
 }
 
 // ----------------------------------------------- face-neighbour filter ---
@@ -441,22 +344,6 @@ using namespace rs;
 
 // ------------------------------------------------------------ host side ---
 
-namespace {
-
-struct WorkList {
-    DevBuf buf;
-    int count = 0;
-};
-
-// Tile shapes (TX along map axis 2, TY along map axis 1) per state-group size.
-struct Shape {
-    int sg, tx, ty;
-};
-const Shape kShapes[] = {{32, 8, 8}, {16, 16, 8}, {8, 16, 16}, {4, 32, 16}, {2, 32, 32}, {1, 64, 32}};
-const int kZChunk = ZCHUNK;
-
-}  // namespace
-
 struct rs_ham {
     int64_t npts = 0;
     int32_t d[3] = {0, 0, 0};
@@ -469,7 +356,6 @@ struct rs_ham {
     double w[5] = {0, 0, 0, 0, 0};
     DevBuf pinfo64, pinfo32, map, loc, V64, V32, cov_off, cov_atom, cov_gam64, cov_gam32, sph_off, sph_idx, sph_gam64, sph_gam32, E64, E32,
         cproj, dummy, scratch;
-    std::map<std::pair<int, int>, WorkList *> work;
     RingPlan *ring = nullptr;      // tables of the ring-buffer FP32 kernel (nullptr: not usable)
     int kernel = RS_KERNEL_AUTO;   // rs_ham_select_kernel
     // optional per-launch timing (rs_ham_timing)
@@ -478,7 +364,6 @@ struct rs_ham {
     size_t n_recorded = 0;
     ~rs_ham() {
         ring_plan_destroy(ring);
-        for (auto &kv : work) delete kv.second;
         for (cudaEvent_t e : events) cudaEventDestroy(e);
     }
     // events for the next recorded call (nullptr when timing is off)
@@ -546,34 +431,6 @@ static void fd_weights(int m, double c[5]) {
         sum += c[j];
     }
     c[0] = -2.0 * sum;
-}
-
-static int build_work(rs_ham *H, const rs_grid *g, int tx, int ty) {
-    const int d0 = g->dims[0], d1 = g->dims[1], d2 = g->dims[2];
-    const int n1 = (d1 + ty - 1) / ty, n2 = (d2 + tx - 1) / tx;
-    std::vector<int> zmin((size_t)n1 * n2, d0), zmax((size_t)n1 * n2, -1);
-    for (int a = 0; a < d0; ++a)
-        for (int b = 0; b < d1; ++b)
-            for (int c = 0; c < d2; ++c)
-                if (g->map[((size_t)a * d1 + b) * d2 + c] >= 0) {
-                    const size_t t = (size_t)(b / ty) * n2 + (c / tx);
-                    zmin[t] = std::min(zmin[t], a);
-                    zmax[t] = std::max(zmax[t], a);
-                }
-    std::vector<int4> items;
-    for (int t1 = 0; t1 < n1; ++t1)
-        for (int t2 = 0; t2 < n2; ++t2) {
-            const size_t t = (size_t)t1 * n2 + t2;
-            if (zmax[t] < 0) continue;
-            for (int z = zmin[t]; z <= zmax[t]; z += kZChunk) items.push_back(make_int4(t1, t2, z, std::min(z + kZChunk, zmax[t] + 1)));
-        }
-    // raster order over (tile row, tile column, z chunk): CTAs resident at the
-    // same time are spatial neighbours, so halo rows are re-read from L2
-    WorkList *wl = new (std::nothrow) WorkList;
-    if (!wl) return fail(RS_ENOMEM, "host allocation failed");
-    H->work[{tx, ty}] = wl;
-    wl->count = (int)items.size();
-    return wl->buf.upload(items.data(), items.size() * sizeof(int4));
 }
 
 extern "C" int rs_ham_create(const rs_grid *g, const double *V_host, const rs_proj *pr, int order, rs_ham **out) {
@@ -665,8 +522,6 @@ extern "C" int rs_ham_create(const rs_grid *g, const double *V_host, const rs_pr
             (rc = H->pinfo32.upload(p32.data(), p32.size() * sizeof(int4))))
             return bail(rc);
     }
-    for (const Shape &s : kShapes)
-        if ((rc = build_work(H, g, s.tx, s.ty))) return bail(rc);
 #if RS_STENCIL_RING
     if ((rc = ring_plan_build(&H->ring, g, coff, catom, cg32, v32, (float)H->w[0], na, RS_RING_SLAB))) return bail(rc);
 #endif
@@ -679,16 +534,13 @@ extern "C" int rs_ham_destroy(rs_ham *h) {
     return RS_OK;
 }
 
-template <typename T, int SG, int TX, int TY>
-static int launch_stencil(rs_ham *H, const HamDev<T> &d, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, int nb,
-                          cudaStream_t st) {
-    using C = StencilCfg<T, SG, TX, TY>;
-    RS_TRY(smem_optin((const void *)k_stencil<T, SG, TX, TY>, C::SMEM));
-    const WorkList *wl = H->work.at({TX, TY});
-    if (wl->count == 0) return RS_OK;
-    dim3 grid((unsigned)wl->count, (unsigned)(nb / SG));
-    k_stencil<T, SG, TX, TY><<<grid, C::NT, C::SMEM, st>>>(d, psi, ldp, hpsi, ldh, H->cproj.as<T>(), nb,
-                                                            wl->buf.as<int4>());
+// nb states of the block, V to a lane (16-byte accesses where the rows allow it)
+template <typename T, int V, int LPP>
+static int launch_gather(rs_ham *H, const HamDev<T> &d, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, int nb,
+                         cudaStream_t st) {
+    constexpr int PTS = GatherCfg<T, V, LPP>::PTS;
+    k_gather<T, V, LPP><<<(unsigned)((H->npts + PTS - 1) / PTS), GT_NT, 0, st>>>(d, H->loc.as<int32_t>(), (int)H->npts, psi,
+                                                                                ldp, hpsi, ldh, H->cproj.as<T>(), nb);
     RS_LAUNCH_CHECK();
     return RS_OK;
 }
@@ -724,29 +576,26 @@ static int apply_t(rs_ham *H, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, i
         RS_LAUNCH_CHECK();
     }
     if (ev) RS_CUDA(cudaEventRecord(ev[1], st));
-    constexpr int SGMAX = 128 / (int)sizeof(T);
-    const int sg = std::min(nb, SGMAX);
-    int rc;
-    switch (sg) {
-        case 1: rc = launch_stencil<T, 1, 64, 32>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
-        case 2: rc = launch_stencil<T, 2, 32, 32>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
-        case 4: rc = launch_stencil<T, 4, 32, 16>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
-        case 8: rc = launch_stencil<T, 8, 16, 16>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
-        case 16: rc = launch_stencil<T, 16, 16, 8>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
-        default:
-            if constexpr (SGMAX >= 32) {
-                if constexpr (sizeof(T) == 4) {
-                    if (H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, nb)) {
-                        float w[5];
-                        for (int j = 0; j < 5; ++j) w[j] = (float)H->w[j];
-                        rc = ring_launch(H->ring, psi, ldp, hpsi, ldh, H->cproj.as<float>(), nb, w, st);
-                        break;
-                    }
-                }
-                rc = launch_stencil<T, 32, 8, 8>(H, d, psi, ldp, hpsi, ldh, nb, st);
-                break;
-            }
-            return fail(RS_EINVAL, "unsupported state group");
+    int rc = -1;
+    bool ring = false;
+    if constexpr (sizeof(T) == 4) {
+        ring = H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, nb);
+        if (ring) {
+            float w[5];
+            for (int j = 0; j < 5; ++j) w[j] = (float)H->w[j];
+            rc = ring_launch(H->ring, psi, ldp, hpsi, ldh, H->cproj.as<float>(), nb, w, st);
+        }
+    }
+    constexpr int E = 16 / (int)sizeof(T);   // states per 16 bytes
+    if (!ring) switch (nb) {
+        case 1: rc = launch_gather<T, 1, 1>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 2: rc = launch_gather<T, 2, 1>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 4: rc = launch_gather<T, E, 4 / E>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 8: rc = launch_gather<T, E, 8 / E>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 16: rc = launch_gather<T, E, 16 / E>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 32: rc = launch_gather<T, E, 32 / E>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        case 64: rc = launch_gather<T, E, 64 / E>(H, d, psi, ldp, hpsi, ldh, nb, st); break;
+        default: return fail(RS_EINVAL, "unsupported state group");
     }
     if (rc == RS_OK && ev) RS_CUDA(cudaEventRecord(ev[2], st));
     return rc;

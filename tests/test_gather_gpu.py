@@ -1,0 +1,55 @@
+"""The gather kernel of H psi at the edges of its pieces (64 to 256 points per
+CTA), for every block width, both types, several point orders and column
+slices that start inside a row.
+
+Tolerance: 27 + 4 k rounded terms per element (k atoms covering the point)
+of the oracle's term magnitudes, and the projection's sums (see
+test_ham_gpu), 64 roundings of the local and 512 of the nonlocal magnitude.
+"""
+import numpy as np
+import pytest
+
+import workloads as wl
+from tests.helpers import SMALL_ATOMS, SMALL_E, SMALL_H, SMALL_RADIUS, lib_to_oracle_index, oracle_system
+from tests.test_ham_gpu import _term_magnitudes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("nb", [1, 2, 4, 8, 16, 32, 64])
+@pytest.mark.parametrize("system,order,pad", [("one", 0, 0), ("box4", -1, 4), ("box5", 1, 0), ("mol", 2, 4), ("mol", 0, 0)])
+def test_gather_edges(dtype, nb, system, order, pad):
+    from paper_1306_2953_gb300 import _lib, api
+    if system == "mol":
+        params = ("atoms", (SMALL_ATOMS, SMALL_E, SMALL_RADIUS, SMALL_H))
+    else:
+        params = ("box", ({"one": 1, "box4": 4, "box5": 5}[system], 0.3, 1.0))
+    g_ora, H_ora, atoms, E = oracle_system(params[0], *params[1])
+    if system == "mol":
+        lg = api.Grid.spheres(atoms, SMALL_RADIUS, SMALL_H, order)
+        proj = api.Projectors(lg, atoms, E, 1.0, 3.0)
+    else:
+        n = params[1][0]
+        lg, proj = api.Grid.box(n, n, n, 0.3, order), None
+    idx = lib_to_oracle_index(g_ora, lg.ijk())
+    H = api.Hamiltonian(lg, H_ora.V[idx], proj)
+    H.select_kernel(_lib.RS_KERNEL_GENERIC)
+    t, u = (torch.float64, 2.0 ** -53) if dtype == "f64" else (torch.float32, 2.0 ** -24)
+    ld = nb + 2 * pad
+    full = torch.from_numpy(np.ascontiguousarray(wl.random_block(g_ora.npts, ld, 9)[idx])).to(t).cuda()
+    out = torch.full_like(full, 7.0)
+    H.apply(full[:, pad:pad + nb], out[:, pad:pad + nb], nb=nb)
+    psi = np.empty((g_ora.npts, nb))
+    psi[idx] = full[:, pad:pad + nb].double().cpu().numpy()
+    ref = H_ora.apply(psi)[idx]
+    if proj is not None:
+        m_loc, m_nl = _term_magnitudes(g_ora, H_ora, psi)
+        bound = u * (64.0 * m_loc[idx] + 512.0 * m_nl[idx])
+    else:
+        w = 9.0 * 2.85 / (2 * 0.3 ** 2)   # three axes of weights, sum of |c_j| below 3 * 2.85
+        bound = np.full_like(ref, 64.0 * u * (w + np.abs(H_ora.V).max()))
+    o = out.double().cpu().numpy()
+    assert np.all(np.abs(o[:, pad:pad + nb] - ref) <= bound)
+    assert np.all(o[:, :pad] == 7.0) and np.all(o[:, pad + nb:] == 7.0)
