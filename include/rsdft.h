@@ -599,12 +599,14 @@ int rs_solver_destroy(rs_solver *s);
  * The transforms are the library's own complex FP64 Stockham kernels. */
 typedef struct rs_poisson rs_poisson;
 
-/* Plans the cube for grid g and allocates it on the current device, with
- * the table of v(G) (24 bytes per cube element in all; blocking).  Errors:
+/* Plans the cube for grid g and allocates its work arrays on the current
+ * device, with the table of v(G) (about 8 bytes per cube element in all: only
+ * half the frequencies and the planes that hold points are kept; blocking).  Errors:
  * RS_EINVAL (empty grid, an axis above 768 points), RS_ENOMEM. */
 int rs_poisson_create(const rs_grid *g, rs_poisson **out);
 
-/* Cube shape, the cutoff radius R_c (Bohr) and the cube's bytes. */
+/* Cube shape, the cutoff radius R_c (Bohr) and the bytes of the full complex
+ * cube (what the transforms would move if none of it were left out). */
 int rs_poisson_info(const rs_poisson *p, int32_t shape[3], double *r_cut, int64_t *cube_bytes);
 
 /* vh_dev = V_H for the density n_dev (device double [npts] in grid order,
