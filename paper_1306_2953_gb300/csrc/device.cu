@@ -20,4 +20,27 @@ int smem_optin(const void *fn, size_t bytes) {
     return RS_OK;
 }
 
+int pool_of_device(cudaMemPool_t *out) {
+    constexpr int MAXDEV = 64;
+    static std::mutex mu;
+    static cudaMemPool_t pools[MAXDEV] = {};
+    int dev = 0;
+    RS_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= MAXDEV) return fail(RS_ECUDA, "device %d out of range", dev);
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        RS_CUDA(cudaMemPoolCreate(&p, &props));
+        uint64_t keep = 256ull << 20;
+        RS_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
+        pools[dev] = p;
+    }
+    *out = pools[dev];
+    return RS_OK;
+}
+
 }  // namespace rs

@@ -66,4 +66,32 @@ struct DevBuf {
     DevBuf &operator=(const DevBuf &) = delete;
 };
 
+// Stream-ordered scratch from the library's own pool of the current device:
+// freed in stream order, so calls on any number of threads and streams hold
+// separate blocks.  The pool keeps at most 256 MB between calls (mapping memory
+// anew takes 200 us a call).
+int pool_of_device(cudaMemPool_t *out);
+struct PoolBuf {
+    void *p = nullptr;
+    cudaStream_t st = nullptr;
+    int alloc(size_t n, cudaStream_t stream) {
+        cudaMemPool_t pool;
+        RS_TRY(pool_of_device(&pool));
+        st = stream;
+        if (cudaMallocFromPoolAsync(&p, n, pool, stream) != cudaSuccess) {
+            p = nullptr;
+            cudaGetLastError();
+            return fail(RS_ENOMEM, "scratch allocation of %zu bytes failed", n);
+        }
+        return RS_OK;
+    }
+    template <typename T> T *as() const { return (T *)p; }
+    ~PoolBuf() {
+        if (p) cudaFreeAsync(p, st);
+    }
+    PoolBuf() = default;
+    PoolBuf(const PoolBuf &) = delete;
+    PoolBuf &operator=(const PoolBuf &) = delete;
+};
+
 }  // namespace rs

@@ -45,7 +45,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "device.h"
 #include "digits.h"
@@ -346,7 +345,10 @@ __device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t *H
         dg_tmem_ld32(lane_base + t * BN, r);
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
-            const int64_t v = (int64_t)__float2int_rn(__uint_as_float(r[j]));
+            // accumulators 0 and 1 stay within 2^22: their integers stand in the
+            // mantissa after one addition (the conversion unit is slow)
+            const int64_t v = t < 2 ? (int64_t)((int)__float_as_uint(__fadd_rn(__uint_as_float(r[j]), 12582912.f)) - 0x4b400000)
+                                    : (int64_t)__float2int_rn(__uint_as_float(r[j]));
             if (t < 3) H[j] += v * (int64_t)(1 << (8 * (2 - t)));
             else L[j] += v * (int64_t)(1 << (8 * (NS - 2 - t)));
         }
@@ -570,33 +572,6 @@ __global__ void __launch_bounds__(256) k_digit_keys(const T *__restrict__ X, int
     }
 }
 
-// Stream-ordered scratch from the library's own pool of the current device.
-// The pool keeps at most 64 MB between calls (its own allocation unit is 32 MB:
-// with a lower limit every call after a synchronisation maps memory anew, 200 us); a block is freed in stream order,
-// so calls on any number of threads and streams hold separate blocks.
-int scratch_pool(cudaMemPool_t *out) {
-    constexpr int MAXDEV = 64;
-    static std::mutex mu;
-    static cudaMemPool_t pools[MAXDEV] = {};
-    int dev = 0;
-    RS_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= MAXDEV) return fail(RS_ECUDA, "device %d out of range", dev);
-    std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        RS_CUDA(cudaMemPoolCreate(&p, &props));
-        uint64_t keep = 64ull << 20;
-        RS_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
-        pools[dev] = p;
-    }
-    *out = pools[dev];
-    return RS_OK;
-}
-
 int sm_count(int *n) {
     int dev = 0;
     RS_CUDA(cudaGetDevice(&dev));
@@ -638,16 +613,12 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
     if (npts > (int64_t)INT32_MAX - 64) return fail(RS_EINVAL, "digit_gram: too many points");
     const bool sym = X == Y && ldx == ldy && nx == ny;
     int *keys = scratch;
+    PoolBuf own;
     if (!keys) {
-        cudaMemPool_t pool;
-        RS_TRY(scratch_pool(&pool));
-        if (cudaMallocFromPoolAsync((void **)&keys, sizeof(int) * (size_t)digit_gram_scratch_ints(nx, ny), pool, st) !=
-            cudaSuccess) {
-            cudaGetLastError();
-            return fail(RS_ENOMEM, "digit_gram: scratch allocation failed");
-        }
+        RS_TRY(own.alloc(sizeof(int) * (size_t)digit_gram_scratch_ints(nx, ny), st));
+        keys = reinterpret_cast<int *>(own.p);
     }
-    auto go = [&]() -> int {
+    {
         const int64_t ne = std::max<int64_t>((int64_t)nx * ny, nx + ny);
         k_digit_init<<<(unsigned)std::min<int64_t>(256, (ne + 255) / 256), 256, 0, st>>>(S, lds, nx, ny, keys, nx + ny);
         RS_LAUNCH_CHECK();
@@ -665,10 +636,7 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
         if constexpr (sizeof(T) == 8) return narrow ? launch_gram<T, 8, 32>(a, tm, st) : launch_gram<T, 8, 64>(a, tm, st);
         else if (exact) return narrow ? launch_gram<T, 7, 32>(a, tm, st) : launch_gram<T, 7, 64>(a, tm, st);
         else return narrow ? launch_gram<T, 5, 32>(a, tm, st) : launch_gram<T, 5, 64>(a, tm, st);
-    };
-    const int rc = go();
-    if (!scratch && cudaFreeAsync(keys, st) != cudaSuccess && rc == RS_OK) return fail(RS_ECUDA, "digit_gram: cudaFreeAsync failed");
-    return rc;
+    }
 }
 template int digit_gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
                                 int64_t, bool, int *, cudaStream_t);
@@ -690,33 +658,17 @@ template <typename T> struct RotArgs {
     double alpha, beta;
 };
 
-// (H 2^(8 (NS - 4)) + L) 2^(8 NS + e) rounded to FP64, in integer instructions
-template <int NS> __device__ __forceinline__ double dg_value(int64_t H, int64_t L, int e) {
-    constexpr int SH = 8 * (NS - 4);          // H in units of L; NS = 8: 32
-    // 128-bit sum V = H 2^SH + L
-    uint64_t lo = (uint64_t)H << SH;
-    int64_t hi = H >> (64 - SH);
-    const uint64_t l2 = lo + (uint64_t)L;
-    hi += (L >> 63) + (l2 < lo ? 1 : 0);
-    lo = l2;
-    const uint64_t sg = (uint64_t)(hi >> 63);
-    // magnitude
-    lo ^= sg;
-    uint64_t h = (uint64_t)hi ^ sg;
-    lo -= sg;
-    h += (sg && lo == 0) ? 1 : 0;
-    if (!(h | lo)) return 0.0;
-    const int z = h ? __clzll((long long)h) : 64 + __clzll((long long)lo);
-    uint64_t top = z >= 64 ? lo << (z - 64) : (z ? (h << z) | (lo >> (64 - z)) : h);   // leading one at bit 63
-    const uint64_t rest = z >= 64 ? 0 : lo << z;
-    // round to nearest even at bit 11
-    const uint64_t tail = top & 0x7ff;
-    uint64_t man = top >> 11;
-    man += (tail > 0x400 || (tail == 0x400 && (rest || (man & 1)))) ? 1 : 0;
-    const int ex = 127 - z + 8 * NS + e;      // exponent of the leading one
-    // a carry out of the rounding moves into the exponent field by itself
-    const uint64_t bits = ((uint64_t)(ex + 1022) << 52) + man;
-    return __longlong_as_double((long long)(bits | (sg << 63)));
+// (H 2^32 + L) 2^(64 + e) rounded once to FP64 (NS = 8; |H|, |L| < 2^51): H and L
+// added to the mantissas of 1.5 2^52 at their scales give two FP64 numbers by
+// one integer addition each, whose offsets cancel in two FP64 additions, the
+// first of them exact.  (Normalising the 128-bit sum in integers took ten times
+// the instructions and a third of a rotation of 48 columns.)
+// ex: (1023 + 52 + 96 + e) << 20
+__device__ __forceinline__ double dg_value(int64_t H, int64_t L, int ex) {
+    const double a = __hiloint2double((int)(H >> 32) + ex + 0x80000, (int)(uint32_t)H);
+    const double b = __hiloint2double((int)(L >> 32) + ex + 0x80000 - (32 << 20), (int)(uint32_t)L);
+    const double ab = __hiloint2double(ex + 0x80000, 0x180000);   // both offsets: 1.5 (1 + 2^-32)
+    return __dadd_rn(__dsub_rn(a, ab), b);
 }
 
 struct RotBars {
@@ -788,11 +740,10 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                     constexpr int E = 16 / (int)sizeof(T);
                     const uint4 *xv = reinterpret_cast<const uint4 *>(x);
                     const int nv = a.n / E;
-                    int q = lane & 3;
-                    for (; q + 28 < nv; q += 32) {
+                    for (int q0 = lane & 3; q0 < nv; q0 += 32) {
                         uint4 t[8];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) t[i] = xv[q + 4 * i];
+                        for (int i = 0; i < 8; ++i) t[i] = xv[min(q0 + 4 * i, nv - 1)];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const T *tt = reinterpret_cast<const T *>(&t[i]);
@@ -800,13 +751,7 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                             for (int e = 0; e < E; ++e) k = max(k, abs_key(tt[e]));
                         }
                     }
-                    for (; q < nv; q += 4) {
-                        const uint4 t = xv[q];
-                        const T *tt = reinterpret_cast<const T *>(&t);
-#pragma unroll
-                        for (int e = 0; e < E; ++e) k = max(k, abs_key(tt[e]));
-                    }
-                    for (q = nv * E + (lane & 3); q < a.n; q += 4) k = max(k, abs_key(x[q]));
+                    for (int q = nv * E + (lane & 3); q < a.n; q += 4) k = max(k, abs_key(x[q]));
                 } else {
 #pragma unroll 8
                     for (int q = lane & 3; q < a.n; q += 4) k = max(k, abs_key(x[q]));
@@ -900,32 +845,43 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         };
         const T al = (T)a.alpha, be = (T)a.beta;
         constexpr int E = 16 / (int)sizeof(T);
-        // E results of row p from column c on
-        auto put = [&](int64_t p, int c, T (&v)[E]) {
-            if (!ok) {
+        // G results of row p from column c on; when Y is added, its G values are
+        // read at once (one after another they cost a trip to memory each)
+        constexpr int G = 8;
+        auto old = [&](int64_t p, int c, T (&o)[G]) {
+            const T *y = a.Y + p * a.ldy + c;
+            if (a.yvec && c + G <= a.m) {
 #pragma unroll
-                for (int i = 0; i < E; ++i) v[i] = (T)__longlong_as_double(0x7ff8000000000000ll);
-            }
-            T *y = a.Y + p * a.ldy + c;
-            if (a.yvec && c + E <= a.m) {
-                uint4 t;
-                T *tt = reinterpret_cast<T *>(&t);
-                if (a.beta != 0.0) t = *reinterpret_cast<const uint4 *>(y);
+                for (int q = 0; q < G / E; ++q) {
+                    const uint4 t = reinterpret_cast<const uint4 *>(y)[q];
+                    const T *tt = reinterpret_cast<const T *>(&t);
 #pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    if (a.alpha != 1.0) v[i] *= al;
-                    if (a.beta != 0.0) v[i] += be * tt[i];
-                    tt[i] = v[i];
+                    for (int i = 0; i < E; ++i) o[q * E + i] = tt[i];
                 }
-                *reinterpret_cast<uint4 *>(y) = t;
             } else {
 #pragma unroll
-                for (int i = 0; i < E; ++i)
-                    if (c + i < a.m) {
-                        if (a.alpha != 1.0) v[i] *= al;
-                        if (a.beta != 0.0) v[i] += be * y[i];
-                        y[i] = v[i];
-                    }
+                for (int i = 0; i < G; ++i) o[i] = c + i < a.m ? y[i] : T(0);
+            }
+        };
+        auto put = [&](int64_t p, int c, T (&v)[G]) {
+            T *y = a.Y + p * a.ldy + c;
+            if (!ok) {
+#pragma unroll
+                for (int i = 0; i < G; ++i) v[i] = (T)__longlong_as_double(0x7ff8000000000000ll);
+            }
+            if (a.yvec && c + G <= a.m) {
+#pragma unroll
+                for (int q = 0; q < G / E; ++q) {
+                    uint4 t;
+                    T *tt = reinterpret_cast<T *>(&t);
+#pragma unroll
+                    for (int i = 0; i < E; ++i) tt[i] = v[q * E + i];
+                    reinterpret_cast<uint4 *>(y)[q] = t;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < G; ++i)
+                    if (c + i < a.m) y[i] = v[i];
             }
         };
         // an interval of products whose accumulators are still to be read out:
@@ -945,29 +901,33 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
             const bool on = owns && p < a.npts;
             if (NBLK > 1 && lastb && on) {
 #pragma unroll
-                for (int q = 0; q < 32 / E; ++q) {
-                    T v[E];
+                for (int q = 0; q < 32 / G; ++q) {
+                    T v[G];
 #pragma unroll
-                    for (int i = 0; i < E; ++i) v[i] = held[NBLK > 1 ? q * E + i : 0];
-                    put(p, nb0 * BN + col0 + q * E, v);
+                    for (int i = 0; i < G; ++i) v[i] = held[NBLK > 1 ? q * G + i : 0];
+                    put(p, nb0 * BN + col0 + q * G, v);
                 }
             }
 #pragma unroll
-            for (int q = 0; q < 32 / E; ++q) {
-                T v[E];
+            for (int q = 0; q < 32 / G; ++q) {
+                T v[G], o[G];
+                const bool add = a.beta != 0.0 && on;
+                if (add) old(p, (nb0 + pblk) * BN + col0 + q * G, o);
 #pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    const int c = q * E + i, e = eb[pblk * BN + (owns ? col0 : 0) + c] - 1022 - 2 * (8 * NS - 2);
+                for (int i = 0; i < G; ++i) {
+                    const int c = q * G + i, e = eb[pblk * BN + (owns ? col0 : 0) + c] - 1022 - 2 * (8 * NS - 2);
                     if constexpr (sizeof(T) == 8) {
-                        v[i] = (T)dg_value<NS>(H[c], L[c], pe - 1022 + e);
+                        v[i] = (T)dg_value(H[c], L[c], (1023 + 52 + 96 + pe - 1022 + e) << 20);
                     } else {
                         // NS = 5: H 2^8 + L stays below 2^63
                         v[i] = ldexpf(__ll2float_rn(H[c] * (int64_t)(1ll << (8 * (NS - 4))) + L[c]), 8 * NS + pe - 126 + e);
                     }
                     H[c] = L[c] = 0;
+                    if (a.alpha != 1.0) v[i] *= al;
+                    if (add) v[i] += be * o[i];
                     if (NBLK > 1 && !lastb) held[NBLK > 1 ? c : 0] = v[i];
                 }
-                if (lastb && on) put(p, (nb0 + pblk) * BN + col0 + q * E, v);
+                if (lastb && on) put(p, (nb0 + pblk) * BN + col0 + q * G, v);
             }
         };
         // One loop over the stages of all tiles; it == nst: the next tile is due.
@@ -1088,10 +1048,10 @@ template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, int
 }  // namespace
 
 // In place, the CTAs of a row tile are one cluster of at most 8 (64 columns
-// each, or two blocks of 64).  A contraction of more than 2^15 states could
-// leave the 64-bit sums.
+// each, or two blocks of 64).  A contraction of more than 1536 states could
+// leave the 51 bits that dg_value takes.
 bool digit_rot_takes(int n, int m, bool in_place) {
-    return n <= 32768 && (!in_place || m <= 1024);
+    return n <= 1536 && (!in_place || m <= 1024);
 }
 
 template <typename T>
