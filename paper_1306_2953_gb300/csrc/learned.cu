@@ -26,6 +26,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "device.h"
@@ -43,47 +44,169 @@ __device__ __forceinline__ float bf16_round(float x) { return __bfloat162float(_
 
 // ------------------------------------------------------------------- CG ---
 
-template <typename T>
-__global__ void k_cg_init(const T *__restrict__ B, int64_t ldb, T *__restrict__ X, int64_t ldx, T *__restrict__ R,
-                          T *__restrict__ P, int n, int64_t npts) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t p = t / n;
-    const int k = (int)(t % n);
-    if (p >= npts) return;
-    const T b = B[p * ldb + k];
-    X[p * ldx + k] = 0;
-    R[p * n + k] = b;
-    P[p * n + k] = b;
+// One iteration is four launches: AP = H P, p.Ap, the update of X and R with
+// r.r, and the update of P.  Rows are [np][n] (n a power of two, X and B with
+// their own leading dimension), LPP lanes to a row and V columns to a lane.  The
+// few FP64 units set the time as soon as every thread uses them: a coefficient
+// is divided once per CTA and column (once per element took 32 us per update of
+// 16 columns of 103 331 points, once per thread 30, so 12.9 and 4.1 for the two updates), and
+// sums meet in FP64 only once per warp.  The sums
+// of iteration it use slot it & 1 of pap and slot (it + 1) & 1 of rr, which the
+// launch before their first use clears.
+
+// An FP64-accurate sum of products: FP32 products split exactly and added as
+// an unevaluated pair with error-free additions; FP64 Kahan-compensated.
+template <typename T> struct DotSum;
+template <> struct DotSum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float a, float b) {
+        const float pr = __fmul_rn(a, b), pe = fmaf(a, b, -pr);
+        const float sum = __fadd_rn(hi, pr), bb = __fsub_rn(sum, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bb)), __fsub_rn(pr, bb)), pe));
+        hi = sum;
+    }
+    // the sum of this and the lane `o` away, still as a pair
+    __device__ __forceinline__ void merge(int o) {
+        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float sum = __fadd_rn(hi, h), bb = __fsub_rn(sum, hi);
+        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bb)), __fsub_rn(h, bb));
+        lo = __fadd_rn(__fadd_rn(lo, l), err);
+        hi = sum;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+template <> struct DotSum<double> {
+    double acc = 0.0, comp = 0.0;
+    __device__ __forceinline__ void add(double a, double b) {
+        const double v = a * b, y = v - comp, t = acc + y;
+        comp = (t - acc) - y;
+        acc = t;
+    }
+    __device__ __forceinline__ void merge(int o) { acc += __shfl_xor_sync(0xffffffffu, acc, o); }
+    __device__ __forceinline__ double value() const { return acc; }
+};
+
+template <typename T, int V> struct __align__(sizeof(T) * V) Cols { T v[V]; };
+
+constexpr int CG_NT = 256;
+
+// adds the CTA's sums of the lanes' columns to out[0 .. LPP V)
+template <typename T, int V, int LPP> __device__ __forceinline__ void cg_reduce(DotSum<T> (&d)[V], double *out) {
+    __shared__ double red[CG_NT / 32][LPP * V];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+#pragma unroll
+        for (int o = 16; o >= LPP; o >>= 1) d[i].merge(o);
+        if (lane < LPP) red[warp][lane * V + i] = d[i].value();
+    }
+    __syncthreads();
+    if (threadIdx.x < LPP * V) {
+        double t = 0;
+#pragma unroll
+        for (int w = 0; w < CG_NT / 32; ++w) t += red[w][threadIdx.x];
+        atomicAdd(out + threadIdx.x, t);
+    }
 }
 
-// X += alpha P, R -= alpha AP with alpha = rr / pAp per column
-template <typename T>
-__global__ void k_cg_update1(T *__restrict__ X, int64_t ldx, T *__restrict__ R, const T *__restrict__ P,
-                             const T *__restrict__ AP, const double *__restrict__ rr, const double *__restrict__ pap,
-                             int n, int64_t npts) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t p = t / n;
-    const int k = (int)(t % n);
-    if (p >= npts) return;
-    const T a = pap[k] != 0.0 ? (T)(rr[k] / pap[k]) : T(0);
-    X[p * ldx + k] += a * P[p * n + k];
-    R[p * n + k] -= a * AP[p * n + k];
+// num / den (0 where den is 0) of the thread's columns
+template <typename T, int V, int LPP> __device__ __forceinline__ void cg_ratio(const double *num, const double *den, T (&q)[V]) {
+    __shared__ T ratio[LPP * V];
+    if (threadIdx.x < LPP * V) ratio[threadIdx.x] = den[threadIdx.x] != 0.0 ? (T)(num[threadIdx.x] / den[threadIdx.x]) : T(0);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < V; ++i) q[i] = ratio[(threadIdx.x % LPP) * V + i];
 }
 
-// P = R + beta P with beta = rr_new / rr per column
-template <typename T>
-__global__ void k_cg_update2(const T *__restrict__ R, T *__restrict__ P, const double *__restrict__ rr,
-                             const double *__restrict__ rr_new, int n, int64_t npts) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t p = t / n;
-    const int k = (int)(t % n);
-    if (p >= npts) return;
-    const T b = rr[k] != 0.0 ? (T)(rr_new[k] / rr[k]) : T(0);
-    P[p * n + k] = R[p * n + k] + b * P[p * n + k];
+template <typename T, int V, int LPP>
+__global__ void __launch_bounds__(CG_NT) k_cg_init(const T *__restrict__ B, int64_t ldb, T *__restrict__ X, int64_t ldx,
+                                                   T *__restrict__ R, T *__restrict__ P, int64_t npts, double *rr) {
+    const int c = (threadIdx.x % LPP) * V;
+    DotSum<T> d[V];
+    for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
+        Cols<T, V> b;
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            b.v[i] = B[p * ldb + c + i];
+            X[p * ldx + c + i] = 0;
+            d[i].add(b.v[i], b.v[i]);
+        }
+        *reinterpret_cast<Cols<T, V> *>(R + p * (LPP * V) + c) = b;
+        *reinterpret_cast<Cols<T, V> *>(P + p * (LPP * V) + c) = b;
+    }
+    cg_reduce<T, V, LPP>(d, rr);
 }
 
-__global__ void k_copy_d(const double *a, double *b, int n) {
-    if (threadIdx.x < n) b[threadIdx.x] = a[threadIdx.x];
+// pap += P.AP; clears rrn
+template <typename T, int V, int LPP>
+__global__ void __launch_bounds__(CG_NT) k_cg_pap(const T *__restrict__ P, const T *__restrict__ AP, int64_t npts, double *pap,
+                                                  double *rrn) {
+    const int c = (threadIdx.x % LPP) * V;
+    if (blockIdx.x == 0 && threadIdx.x < LPP * V) rrn[threadIdx.x] = 0.0;
+    DotSum<T> d[V];
+#pragma unroll 2
+    for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
+        const Cols<T, V> x = *reinterpret_cast<const Cols<T, V> *>(P + p * (LPP * V) + c);
+        const Cols<T, V> y = *reinterpret_cast<const Cols<T, V> *>(AP + p * (LPP * V) + c);
+#pragma unroll
+        for (int i = 0; i < V; ++i) d[i].add(x.v[i], y.v[i]);
+    }
+    cg_reduce<T, V, LPP>(d, pap);
+}
+
+// X += alpha P, R -= alpha AP with alpha = rr / pap per column; rrn += R.R; clears papn
+template <typename T, int V, int LPP>
+__global__ void __launch_bounds__(CG_NT) k_cg_update1(T *__restrict__ X, int64_t ldx, int xvec, T *__restrict__ R,
+                                                      const T *__restrict__ P, const T *__restrict__ AP, int64_t npts,
+                                                      const double *__restrict__ rr, const double *__restrict__ pap, double *rrn,
+                                                      double *papn) {
+    using C = Cols<T, V>;
+    const int c = (threadIdx.x % LPP) * V;
+    if (blockIdx.x == 0 && threadIdx.x < LPP * V) papn[threadIdx.x] = 0.0;
+    T a[V];
+    cg_ratio<T, V, LPP>(rr, pap, a);
+    DotSum<T> d[V];
+    for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
+        const C pv = *reinterpret_cast<const C *>(P + p * (LPP * V) + c), ap = *reinterpret_cast<const C *>(AP + p * (LPP * V) + c);
+        C r = *reinterpret_cast<const C *>(R + p * (LPP * V) + c), x;
+        T *xp = X + p * ldx + c;
+        if (xvec) x = *reinterpret_cast<const C *>(xp);
+        else {
+#pragma unroll
+            for (int i = 0; i < V; ++i) x.v[i] = xp[i];
+        }
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            x.v[i] += a[i] * pv.v[i];
+            r.v[i] -= a[i] * ap.v[i];
+            d[i].add(r.v[i], r.v[i]);
+        }
+        if (xvec) *reinterpret_cast<C *>(xp) = x;
+        else {
+#pragma unroll
+            for (int i = 0; i < V; ++i) xp[i] = x.v[i];
+        }
+        *reinterpret_cast<C *>(R + p * (LPP * V) + c) = r;
+    }
+    cg_reduce<T, V, LPP>(d, rrn);
+}
+
+// P = R + beta P with beta = rrn / rr per column
+template <typename T, int V, int LPP>
+__global__ void __launch_bounds__(CG_NT) k_cg_update2(const T *__restrict__ R, T *__restrict__ P, int64_t npts,
+                                                      const double *__restrict__ rr, const double *__restrict__ rrn) {
+    using C = Cols<T, V>;
+    const int c = (threadIdx.x % LPP) * V;
+    T b[V];
+    cg_ratio<T, V, LPP>(rrn, rr, b);
+#pragma unroll 2
+    for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
+        const C r = *reinterpret_cast<const C *>(R + p * (LPP * V) + c);
+        C q = *reinterpret_cast<const C *>(P + p * (LPP * V) + c);
+#pragma unroll
+        for (int i = 0; i < V; ++i) q.v[i] = r.v[i] + b[i] * q.v[i];
+        *reinterpret_cast<C *>(P + p * (LPP * V) + c) = q;
+    }
 }
 
 int64_t cg_workspace_bytes(int64_t npts, int ncols, int dtype) {
@@ -91,37 +214,52 @@ int64_t cg_workspace_bytes(int64_t npts, int ncols, int dtype) {
     return 3 * npts * ncols * es + 4 * 64 * 8 + 256;
 }
 
-template <typename T>
-static int cg_t(rs_ham *h, const T *B, int64_t ldb, T *X, int64_t ldx, int n, int n_iter, void *work, cudaStream_t st) {
+template <typename T, int V, int LPP>
+static int cg_t(rs_ham *h, const T *B, int64_t ldb, T *X, int64_t ldx, int n_iter, void *work, cudaStream_t st) {
+    constexpr int n = V * LPP;
     const int64_t np = ham_npts(h);
     T *R = reinterpret_cast<T *>(work);
     T *P = R + np * n;
     T *AP = P + np * n;
-    double *rr = reinterpret_cast<double *>(AP + np * n);
-    double *pap = rr + 64, *rrn = pap + 64;
+    // the sums, 8-byte aligned behind the arrays
+    double *rr = reinterpret_cast<double *>(((uintptr_t)(AP + np * n) + 7) & ~(uintptr_t)7), *pap = rr + 128;   // two slots of 64 each
     const int dt = sizeof(T) == 8 ? RS_F64 : RS_F32;
-    const unsigned blocks = (unsigned)((np * n + 255) / 256);
-    k_cg_init<T><<<blocks, 256, 0, st>>>(B, ldb, X, ldx, R, P, n, np);
+    const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((np + CG_NT / LPP - 1) / (CG_NT / LPP), 152 * 6));
+    const int xvec = aligned16(X) && (ldx * sizeof(T)) % 16 == 0;
+    RS_CUDA(cudaMemsetAsync(rr, 0, sizeof(double) * 256, st));
+    k_cg_init<T, V, LPP><<<blocks, CG_NT, 0, st>>>(B, ldb, X, ldx, R, P, np, rr);
     RS_LAUNCH_CHECK();
-    RS_TRY(coldots(dt, R, n, R, n, n, np, rr, st));
     for (int it = 0; it < n_iter; ++it) {
+        double *r0 = rr + 64 * (it & 1), *r1 = rr + 64 * (~it & 1), *p0 = pap + 64 * (it & 1), *p1 = pap + 64 * (~it & 1);
         RS_TRY(rs_ham_apply_block(h, P, n, AP, n, n, dt, st));
-        RS_TRY(coldots(dt, P, n, AP, n, n, np, pap, st));
-        k_cg_update1<T><<<blocks, 256, 0, st>>>(X, ldx, R, P, AP, rr, pap, n, np);
-        RS_LAUNCH_CHECK();
-        RS_TRY(coldots(dt, R, n, R, n, n, np, rrn, st));
-        k_cg_update2<T><<<blocks, 256, 0, st>>>(R, P, rr, rrn, n, np);
-        k_copy_d<<<1, 64, 0, st>>>(rrn, rr, n);
+        k_cg_pap<T, V, LPP><<<blocks, CG_NT, 0, st>>>(P, AP, np, p0, r1);
+        k_cg_update1<T, V, LPP><<<blocks, CG_NT, 0, st>>>(X, ldx, xvec, R, P, AP, np, r0, p0, r1, p1);
+        k_cg_update2<T, V, LPP><<<blocks, CG_NT, 0, st>>>(R, P, np, r0, r1);
         RS_LAUNCH_CHECK();
     }
     return RS_OK;
 }
 
+template <typename T>
+static int cg_n(rs_ham *h, const T *B, int64_t ldb, T *X, int64_t ldx, int n, int n_iter, void *work, cudaStream_t st) {
+    constexpr int E = 16 / (int)sizeof(T);   // columns per 16 bytes
+    switch (n) {
+        case 1: return cg_t<T, 1, 1>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 2: return cg_t<T, 2, 1>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 4: return cg_t<T, E, 4 / E>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 8: return cg_t<T, E, 8 / E>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 16: return cg_t<T, E, 16 / E>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 32: return cg_t<T, E, 32 / E>(h, B, ldb, X, ldx, n_iter, work, st);
+        case 64: return cg_t<T, E, 64 / E>(h, B, ldb, X, ldx, n_iter, work, st);
+        default: return fail(RS_EINVAL, "shifted Poisson CG: the column count must be a power of two <= 64");
+    }
+}
+
 int shifted_poisson_cg(rs_ham *h, const void *B, int64_t ldb, void *X, int64_t ldx, int n, int n_iter, int dtype,
                        void *work, cudaStream_t st) {
     if (dtype == RS_F64)
-        return cg_t<double>(h, (const double *)B, ldb, (double *)X, ldx, n, n_iter, work, st);
-    return cg_t<float>(h, (const float *)B, ldb, (float *)X, ldx, n, n_iter, work, st);
+        return cg_n<double>(h, (const double *)B, ldb, (double *)X, ldx, n, n_iter, work, st);
+    return cg_n<float>(h, (const float *)B, ldb, (float *)X, ldx, n, n_iter, work, st);
 }
 
 // ------------------------------------------------ network on dense tiles ---
@@ -261,6 +399,22 @@ template <int CIN, int COUT> int tile_bwd_weight(const float *gout, const float 
         gout, in, ntiles, D, dW);
     RS_LAUNCH_CHECK();
     return RS_OK;
+}
+
+// count[n] = valid grid points of tile n (one CTA per tile)
+__global__ void k_tile_count(const uint8_t *__restrict__ mask, const uint8_t *__restrict__ valid, int D3, int *__restrict__ count) {
+    const uint8_t *m = mask + (int64_t)blockIdx.x * D3;
+    int c = 0;
+    for (int e = threadIdx.x; e < D3; e += blockDim.x) c += valid[e] && m[e];
+    c = __reduce_add_sync(0xffffffffu, c);
+    __shared__ int red[32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        c = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (threadIdx.x == 0) count[blockIdx.x] = c;
+    }
 }
 
 // g = d loss / d y with loss = sum_{valid} (y - t)^2 / nvalid; returns the sum in loss[0]
@@ -406,6 +560,276 @@ __global__ void k_rms(const double *ss, int n, double inv_np, double *rms) {
 
 // --------------------------------------------- inference on the grid ---
 
+// The three layers work on rows of four lattice positions along map axis 2
+// (row items: 4-aligned positions), so that an activation read once serves the
+// three outputs it touches in its row: 54 reads for four points instead of
+// 108.  A CTA takes ITEMS consecutive items (16, or 64 of up
+// to 8 columns, which would leave the CTA little work otherwise) and stages the point indices of
+// their 3 x 3 x 6 neighbourhoods in shared memory; items without a grid point
+// are skipped.  Measured on 654 520 points and 32 states (one thread per point
+// and state and FP32 FMA before): input and layer 1 910 -> 497 us, layer 2
+// 2709 -> 1295 us, layer 3 1203 -> 652 us; they wait for loads (issue active
+// 46 % in layer 2, its tensor pipe 37 %).
+constexpr int ROWN = 4, ROWP = ROWN + 2, NBH = 9 * ROWP;
+constexpr int NET_NT = 256;
+
+struct NetGrid {
+    const int32_t *map;
+    int d1, d2, n4, items;   // n4: row items per map row
+    int nb;
+};
+
+// Indices of item `it` (of the CTA): qs[it][row][i], row = 3 (a + 1) + (b + 1),
+// i = 0 .. 5 the positions from one before the item to one behind it; the
+// item's own points are qs[it][4][1 .. 4].  False when no item has a point.
+template <int ITEMS> __device__ __forceinline__ bool net_stage(const NetGrid &g, int (&qs)[ITEMS][NBH]) {
+    const int t0 = blockIdx.x * ITEMS;
+    bool any = false;
+    for (int e = threadIdx.x; e < ITEMS * ROWN; e += NET_NT) {
+        const int t = t0 + e / ROWN, o = e % ROWN;
+        if (t < g.items) {
+            const int r = t / g.n4, w = (t - r * g.n4) * ROWN + o;
+            any = any || (w < g.d2 && __ldg(g.map + (int64_t)r * g.d2 + w) >= 0);
+        }
+    }
+    if (!__syncthreads_or(any)) return false;
+    for (int e = threadIdx.x; e < ITEMS * NBH; e += NET_NT) {
+        const int it = e / NBH, k = e - it * NBH, row = k / ROWP, i = k - row * ROWP;
+        const int t = t0 + it;
+        int q = -1;
+        if (t < g.items) {
+            const int r = t / g.n4, w = (t - r * g.n4) * ROWN + i - 1;
+            // (items with points lie at least four positions inside the map)
+            const int64_t L = ((int64_t)r + (row / 3 - 1) * g.d1 + (row % 3 - 1)) * g.d2 + w;
+            if (w >= 0 && w < g.d2 && L >= 0 && L < (int64_t)g.items / g.n4 * g.d2) q = __ldg(g.map + L);
+        }
+        qs[it][k] = q;
+    }
+    __syncthreads();
+    return true;
+}
+__device__ __forceinline__ bool item_empty(const int (&q)[NBH]) {
+    return (q[4 * ROWP + 1] & q[4 * ROWP + 2] & q[4 * ROWP + 3] & q[4 * ROWP + 4]) < 0;
+}
+
+// An FP32 value cut exactly into three BF16 pieces of 8 bits; two values to a
+// word, the first in the low half.
+__device__ __forceinline__ void bf16_cut(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[k] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+        x -= __uint_as_float(__float_as_uint(x) & 0xffff0000u);
+        y -= __uint_as_float(__float_as_uint(y) & 0xffff0000u);
+    }
+}
+
+// Layer 1 (1 -> 8, relu), the input made on the way: xhat = bf16(r / rms).  One
+// thread per (item, state).  The result is stored for layer 2's tensor-core
+// operands, exactly: three BF16 pieces [point][piece][state][channel].
+template <int ITEMS>
+__global__ void __launch_bounds__(NET_NT) k_net_first(NetGrid g, const float *__restrict__ wq, const float *__restrict__ R,
+                                                      int64_t ldr, const float *__restrict__ scale, uint4 *__restrict__ out) {
+    __shared__ __align__(16) float ws[27 * NC];
+    __shared__ int qs[ITEMS][NBH];
+    for (int e = threadIdx.x; e < 27 * NC; e += NET_NT) ws[e] = __ldg(wq + W1_OFF + (e % NC) * 27 + e / NC);
+    if (!net_stage<ITEMS>(g, qs)) return;
+    for (int t = threadIdx.x; t < ITEMS * g.nb; t += NET_NT) {
+        const int it = t / g.nb, s = t - it * g.nb;
+        const int(&q)[NBH] = qs[it];
+        if (item_empty(q)) continue;
+        const float sc = __ldg(scale + s);
+        float2 acc[ROWN][NC / 2];
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o)
+#pragma unroll
+            for (int c = 0; c < NC / 2; ++c) acc[o][c] = make_float2(0.f, 0.f);
+#pragma unroll 3
+        for (int r = 0; r < 9; ++r) {
+            float x[ROWP];
+#pragma unroll
+            for (int i = 0; i < ROWP; ++i) {
+                const int n = q[r * ROWP + i];
+                x[i] = n >= 0 ? bf16_round(__ldg(R + (int64_t)n * ldr + s) * sc) : 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float4 wa = *reinterpret_cast<const float4 *>(ws + (3 * r + c) * NC);
+                const float4 wb = *reinterpret_cast<const float4 *>(ws + (3 * r + c) * NC + 4);
+                const float2 w[4] = {{wa.x, wa.y}, {wa.z, wa.w}, {wb.x, wb.y}, {wb.z, wb.w}};
+#pragma unroll
+                for (int o = 0; o < ROWN; ++o)
+#pragma unroll
+                    for (int k = 0; k < NC / 2; ++k) acc[o][k] = __ffma2_rn(w[k], make_float2(x[o + c], x[o + c]), acc[o][k]);
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o) {
+            const int p = q[4 * ROWP + 1 + o];
+            if (p < 0) continue;
+            uint32_t pc[4][3];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) bf16_cut(fmaxf(acc[o][k].x, 0.f), fmaxf(acc[o][k].y, 0.f), pc[k]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                out[((int64_t)p * 3 + k) * g.nb + s] = make_uint4(pc[0][k], pc[1][k], pc[2][k], pc[3][k]);
+        }
+    }
+}
+
+// Layer 2 (8 -> 8, relu) on the tensor cores: a warp takes 16 (item, state)
+// pairs; a tap's 16 x 8 (state, channel) activations meet its 8 x 8 weights,
+// two taps of a row in one m16n8k16 and the third in an m16n8k8 (BF16 inputs,
+// exact products, FP32 accumulation).  The tensor core truncates where it
+// accumulates, so each row of taps starts from zero and is added to the sum
+// with rounding: one chain over all taps is three times less exact.
+__device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[2], const uint32_t (&b)[2], uint32_t w0, uint32_t w1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(b[0]), "r"(b[1]), "r"(w0), "r"(w1));
+}
+__device__ __forceinline__ void mma_k8(float (&d)[4], const uint32_t (&a)[2], uint32_t w) {
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};\n"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(w));
+}
+
+// The next row's activations are loaded while the products of this one run; the
+// weights (output channel gr, input channels 2 tq and 2 tq + 1) wait in shared
+// memory, so that two CTAs fit an SM.
+// UNI: nb is a multiple of 16, so a tile's rows are one item's.
+template <int ITEMS, bool UNI>
+__global__ void __launch_bounds__(NET_NT, 2) k_net_mid(NetGrid g, const float *__restrict__ wq, const uint32_t *__restrict__ in,
+                                                       float *__restrict__ out) {
+    __shared__ int qs[ITEMS][NBH];
+    __shared__ uint32_t ws[27][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, tq = lane & 3;
+    for (int e = threadIdx.x; e < 27 * 32; e += NET_NT) {
+        const int t = e >> 5, l = e & 31;
+        const float *w = wq + W2_OFF + ((l >> 2) * NC + 2 * (l & 3)) * 27 + t;
+        ws[t][l] = __byte_perm(__float_as_uint(__ldg(w)), __float_as_uint(__ldg(w + 27)), 0x7632);
+    }
+    if (!net_stage<ITEMS>(g, qs)) return;
+    // the 16 rows of a tile: (item, state) pairs, states fastest; this lane's are
+    // row gr (a) and gr + 8 (b)
+    const int rows = ITEMS * g.nb;
+    for (int t = warp; t * 16 < rows; t += NET_NT / 32) {
+        const int ra = t * 16 + gr, rb = ra + 8;
+        const int ia = UNI ? t * 16 / g.nb : min(ra, rows - 1) / g.nb, ib = UNI ? ia : min(rb, rows - 1) / g.nb;
+        const int sa = ra - ia * g.nb, sb = rb - ib * g.nb;
+        const int(&qa)[NBH] = qs[ia], (&qb)[NBH] = qs[ib];
+        const bool ha = ra < rows && !item_empty(qa), hb = UNI ? ha : rb < rows && !item_empty(qb);
+        if (!__any_sync(0xffffffffu, ha || hb)) continue;
+        const uint32_t *ina = in + sa * 4 + tq, *inb = in + sb * 4 + tq;
+        float acc[ROWN][4];
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[o][k] = 0.f;
+        uint32_t x[2][ROWP][3][2];
+        auto load = [&](int r, uint32_t (&y)[ROWP][3][2]) {
+#pragma unroll
+            for (int i = 0; i < ROWP; ++i) {
+                const int na = UNI || ha ? qa[r * ROWP + i] : -1, nb = UNI ? na : hb ? qb[r * ROWP + i] : -1;
+                const uint32_t *pa = ina + (int64_t)na * (12 * g.nb), *pb = UNI ? pa + 32 : inb + (int64_t)nb * (12 * g.nb);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    y[i][k][0] = na >= 0 ? __ldg(pa + k * 4 * g.nb) : 0u;
+                    y[i][k][1] = nb >= 0 ? __ldg(pb + k * 4 * g.nb) : 0u;
+                }
+            }
+        };
+        load(0, x[0]);
+#pragma unroll
+        for (int r = 0; r < 9; ++r) {
+            if (r < 8) load(r + 1, x[(r + 1) & 1]);
+            const uint32_t(&y)[ROWP][3][2] = x[r & 1];
+            const uint32_t w0 = ws[3 * r][lane], w1 = ws[3 * r + 1][lane], w2 = ws[3 * r + 2][lane];
+            float row[ROWN][4];
+#pragma unroll
+            for (int o = 0; o < ROWN; ++o)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) row[o][k] = 0.f;
+            // the small pieces first
+#pragma unroll
+            for (int k = 2; k >= 0; --k)
+#pragma unroll
+                for (int o = 0; o < ROWN; ++o) {
+                    mma_k16(row[o], y[o][k], y[o + 1][k], w0, w1);
+                    mma_k8(row[o], y[o + 2][k], w2);
+                }
+#pragma unroll
+            for (int o = 0; o < ROWN; ++o)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[o][k] += row[o][k];
+        }
+        // [point][half][state][4 channels]
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o) {
+            const int pa = ha ? qa[4 * ROWP + 1 + o] : -1, pb = hb ? qb[4 * ROWP + 1 + o] : -1;
+            float *y = out + 2 * (tq & 1);
+            const int64_t half = tq >> 1;
+            if (pa >= 0)
+                *reinterpret_cast<float2 *>(y + (((int64_t)pa * 2 + half) * g.nb + sa) * 4) =
+                    make_float2(fmaxf(acc[o][0], 0.f), fmaxf(acc[o][1], 0.f));
+            if (pb >= 0)
+                *reinterpret_cast<float2 *>(y + (((int64_t)pb * 2 + half) * g.nb + sb) * 4) =
+                    make_float2(fmaxf(acc[o][2], 0.f), fmaxf(acc[o][3], 0.f));
+        }
+    }
+}
+
+// Layer 3 (8 -> 1) times the column's rms; one thread per (item, state), the
+// activations [point][half][state][4 channels] (a warp's 16-byte reads are
+// contiguous).
+template <int ITEMS>
+__global__ void __launch_bounds__(NET_NT) k_net_last(NetGrid g, const float *__restrict__ wq, const float *__restrict__ in,
+                                                     float *__restrict__ W, int64_t ldw, const double *__restrict__ rms) {
+    __shared__ __align__(16) float ws[27 * NC];
+    __shared__ int qs[ITEMS][NBH];
+    for (int e = threadIdx.x; e < 27 * NC; e += NET_NT) ws[e] = __ldg(wq + W3_OFF + (e % NC) * 27 + e / NC);
+    if (!net_stage<ITEMS>(g, qs)) return;
+    for (int t = threadIdx.x; t < ITEMS * g.nb; t += NET_NT) {
+        const int it = t / g.nb, s = t - it * g.nb;
+        const int(&q)[NBH] = qs[it];
+        if (item_empty(q)) continue;
+        float2 acc[ROWN];   // even and odd channels
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o) acc[o] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int r = 0; r < 9; ++r) {
+            float4 xa[ROWP], xb[ROWP];
+#pragma unroll
+            for (int i = 0; i < ROWP; ++i) {
+                const int n = q[r * ROWP + i];
+                const float4 *src = reinterpret_cast<const float4 *>(in) + (int64_t)n * 2 * g.nb + s;
+                xa[i] = n >= 0 ? __ldg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+                xb[i] = n >= 0 ? __ldg(src + g.nb) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float4 wa = *reinterpret_cast<const float4 *>(ws + (3 * r + c) * NC);
+                const float4 wb = *reinterpret_cast<const float4 *>(ws + (3 * r + c) * NC + 4);
+#pragma unroll
+                for (int o = 0; o < ROWN; ++o) {
+                    const float4 a = xa[o + c], bb = xb[o + c];
+                    acc[o] = __ffma2_rn(make_float2(wa.x, wa.y), make_float2(a.x, a.y), acc[o]);
+                    acc[o] = __ffma2_rn(make_float2(wa.z, wa.w), make_float2(a.z, a.w), acc[o]);
+                    acc[o] = __ffma2_rn(make_float2(wb.x, wb.y), make_float2(bb.x, bb.y), acc[o]);
+                    acc[o] = __ffma2_rn(make_float2(wb.z, wb.w), make_float2(bb.z, bb.w), acc[o]);
+                }
+            }
+        }
+        const float f = (float)rms[s];
+#pragma unroll
+        for (int o = 0; o < ROWN; ++o) {
+            const int p = q[4 * ROWP + 1 + o];
+            if (p >= 0) W[(int64_t)p * ldw + s] = (acc[o].x + acc[o].y) * f;
+        }
+    }
+}
+
+// ---- one to three columns: one thread per point and state, FP32 FMA ----
+
 // xhat = bf16(r / rms) and the per-column rms
 __global__ void k_net_input(const float *__restrict__ R, int64_t ldr, const double *__restrict__ rms, int nb,
                             int npts, float *__restrict__ x) {
@@ -415,7 +839,7 @@ __global__ void k_net_input(const float *__restrict__ R, int64_t ldr, const doub
     x[t] = bf16_round(R[(int64_t)p * ldr + s] * (float)(1.0 / rms[s]));
 }
 
-// layer on the grid: out[p][co][s] = act(sum_t sum_ci w[co][ci][t] in[nbr_t(p)][ci][s]).
+// layer on the grid, activations [point][channel][state]: out[p][co][s] = act(sum_t sum_ci w[co][ci][t] in[nbr_t(p)][ci][s]).
 // The layer's weights (BF16 values) are staged in shared memory as
 // [tap][ci][co], so one 16-byte load gives four output channels' weights
 // (a broadcast: every lane reads the same word).
@@ -466,6 +890,11 @@ __global__ void __launch_bounds__(256) k_net_layer(const int32_t *__restrict__ m
     }
 }
 
+// per-column input scale 1 / rms
+__global__ void k_net_scale(const double *rms, int nb, float *scale) {
+    if ((int)threadIdx.x < nb) scale[threadIdx.x] = (float)(1.0 / rms[threadIdx.x]);
+}
+
 }  // namespace rs
 
 using namespace rs;
@@ -494,29 +923,29 @@ extern "C" int rs_convnet_tiles(const float *w_dev, const float *x_dev, const ui
     if ((grad_dev || loss_host) && (!target_dev || !valid_dev))
         return fail(RS_EINVAL, "rs_convnet_tiles: gradients need target and valid");
     cudaStream_t st = (cudaStream_t)stream;
-    DevBuf ws, dl;
-    RS_TRY(ws.alloc(TileBufs::floats(ntiles, D) * sizeof(float)));
-    RS_TRY(dl.alloc(sizeof(double)));
+    PoolBuf ws, dl, cnt;
+    RS_TRY(ws.alloc(TileBufs::floats(ntiles, D) * sizeof(float), st));
+    RS_TRY(dl.alloc(sizeof(double), st));
     TileBufs b(ws.as<float>(), ntiles, D);
     const int64_t n = (int64_t)ntiles * D * D * D;
+    // the number of valid points, counted on the device while the forward pass is queued
+    std::vector<int> count(grad_dev || loss_host ? ntiles : 0);
+    if (!count.empty()) {
+        RS_TRY(cnt.alloc(sizeof(int) * (size_t)ntiles, st));
+        k_tile_count<<<(unsigned)ntiles, 256, 0, st>>>(mask_dev, valid_dev, D * D * D, cnt.as<int>());
+        RS_CUDA(cudaMemcpyAsync(count.data(), cnt.p, sizeof(int) * (size_t)ntiles, cudaMemcpyDeviceToHost, st));
+    }
     k_round_weights<<<9, 256, 0, st>>>(w_dev, b.wq, W_TOTAL);
     k_round_inputs<<<1024, 256, 0, st>>>(x_dev, b.x0, n);
     RS_LAUNCH_CHECK();
     RS_TRY(tile_forward(b.wq, b.x0, mask_dev, ntiles, D, b, st));
     RS_CUDA(cudaMemcpyAsync(y_dev, b.y, sizeof(float) * n, cudaMemcpyDeviceToDevice, st));
     if (grad_dev || loss_host) {
-        int nvalid = 0;
-        {
-            std::vector<uint8_t> v((size_t)D * D * D), m((size_t)n);
-            RS_CUDA(cudaMemcpyAsync(v.data(), valid_dev, v.size(), cudaMemcpyDeviceToHost, st));
-            RS_CUDA(cudaMemcpyAsync(m.data(), mask_dev, m.size(), cudaMemcpyDeviceToHost, st));
-            RS_CUDA(cudaStreamSynchronize(st));
-            const int D3 = D * D * D;
-            for (int64_t e = 0; e < n; ++e) nvalid += (v[e % D3] && m[e]);
-        }
+        int64_t nvalid = 0;
+        for (int c : count) nvalid += c;   // (the copy to pageable memory has completed)
         RS_CUDA(cudaMemsetAsync(dl.p, 0, sizeof(double), st));
         k_tile_loss<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(b.y, target_dev, mask_dev, valid_dev, ntiles, D,
-                                                                1.0 / std::max(nvalid, 1), b.g3, dl.as<double>());
+                                                                1.0 / (double)std::max<int64_t>(nvalid, 1), b.g3, dl.as<double>());
         RS_LAUNCH_CHECK();
         if (grad_dev) {
             RS_CUDA(cudaMemsetAsync(grad_dev, 0, sizeof(float) * W_TOTAL, st));
@@ -545,7 +974,6 @@ namespace rs {
 int train_tiles_impl(float *w_dev, const float *xin, const float *tgt, const uint8_t *msk, const uint8_t *dvalid,
                      int ntiles, int D, int batch, int epochs, float lr, float *loss_host, cudaStream_t st) {
     const int D3 = D * D * D;
-    const int64_t ntot = (int64_t)ntiles * D3;
     const int B = std::min(batch, ntiles);
     DevBuf ws, grad, m, v, dl;
     RS_TRY(ws.alloc(TileBufs::floats(B, D) * sizeof(float)));
@@ -558,19 +986,12 @@ int train_tiles_impl(float *w_dev, const float *xin, const float *tgt, const uin
     // number of valid points (interior grid points) of every tile, for the mean
     std::vector<int> tvalid((size_t)ntiles, 0);
     {
-        std::vector<uint8_t> hm((size_t)ntot), valid((size_t)D3);
-        RS_CUDA(cudaMemcpyAsync(hm.data(), msk, hm.size(), cudaMemcpyDeviceToHost, st));
-        RS_CUDA(cudaMemcpyAsync(valid.data(), dvalid, valid.size(), cudaMemcpyDeviceToHost, st));
+        PoolBuf cnt;
+        RS_TRY(cnt.alloc(sizeof(int) * (size_t)ntiles, st));
+        k_tile_count<<<(unsigned)ntiles, 256, 0, st>>>(msk, dvalid, D3, cnt.as<int>());
+        RS_LAUNCH_CHECK();
+        RS_CUDA(cudaMemcpyAsync(tvalid.data(), cnt.p, sizeof(int) * (size_t)ntiles, cudaMemcpyDeviceToHost, st));
         RS_CUDA(cudaStreamSynchronize(st));
-        std::vector<int> vidx;
-        for (int e = 0; e < D3; ++e)
-            if (valid[e]) vidx.push_back(e);
-        for (int n = 0; n < ntiles; ++n) {
-            const uint8_t *tm = hm.data() + (size_t)n * D3;
-            int cnt = 0;
-            for (int e : vidx) cnt += tm[e] != 0;
-            tvalid[n] = cnt;
-        }
     }
     TileBufs b(ws.as<float>(), B, D);
     int step = 0;
@@ -676,20 +1097,49 @@ int learned_apply(const rs_ham *h, const float *R, int64_t ldr, float *W, int64_
     RS_TRY(coldots(RS_F32, R, ldr, R, ldr, nb, np, ss, st));
     k_rms<<<1, 64, 0, st>>>(ss, nb, 1.0 / (double)np, rms);
     if (np * nb >= (int64_t)INT32_MAX) return fail(RS_EINVAL, "learned preconditioner: npts * nb above 2^31");
-    const int n32 = (int)np;
-    float *x = act, *a1 = x + np * nb, *a2 = a1 + np * NC * nb;
-    const unsigned blocks = (unsigned)((np * nb + 255) / 256);
-    k_net_input<<<blocks, 256, 0, st>>>(R, ldr, rms, nb, n32, x);
-    const int32_t *map = ham_map(h), *loc = ham_loc(h);
-    const int d1 = ham_dim(h, 1), d2 = ham_dim(h, 2);
-    k_net_layer<1, NC, true, false, W1_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, x, a1, 0, rms);
-    k_net_layer<NC, NC, true, false, W2_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, a1, a2, 0, rms);
-    k_net_layer<NC, 1, false, true, W3_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, a2, W, ldw, rms);
+    // (the scale array shares the activations' buffer: 64 floats ahead of them)
+    // Few columns do not fill the row kernels: us at 1 / 2 / 3 / 4 columns, row
+    // kernels 148 / 167 / 205 / 188 on 103 331 points and 454 / 541 / 663 / 726 on
+    // 654 520, thread per point and state 112 / 172 / 162 / 278 and 442 / 774 / 742 / 1396.
+    if (nb <= 3) {
+        const int n32 = (int)np;
+        float *x = act, *a1 = x + np * nb, *a2 = a1 + np * NC * nb;
+        const unsigned blocks = (unsigned)((np * nb + 255) / 256);
+        const int32_t *map = ham_map(h), *loc = ham_loc(h);
+        const int d1 = ham_dim(h, 1), d2 = ham_dim(h, 2);
+        k_net_input<<<blocks, 256, 0, st>>>(R, ldr, rms, nb, n32, x);
+        k_net_layer<1, NC, true, false, W1_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, x, a1, 0, rms);
+        k_net_layer<NC, NC, true, false, W2_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, a1, a2, 0, rms);
+        k_net_layer<NC, 1, false, true, W3_OFF><<<blocks, 256, 0, st>>>(map, loc, d1, d2, n32, nb, wq_dev, a2, W, ldw, rms);
+        RS_LAUNCH_CHECK();
+        return RS_OK;
+    }
+    float *scale = act;
+    uint32_t *a1 = reinterpret_cast<uint32_t *>(act + 64);   // three BF16 pieces of 8 channels
+    float *a2 = reinterpret_cast<float *>(a1 + np * nb * (3 * NC / 2));
+    k_net_scale<<<1, 64, 0, st>>>(rms, nb, scale);
+    NetGrid g;
+    g.map = ham_map(h);
+    g.d1 = ham_dim(h, 1), g.d2 = ham_dim(h, 2);
+    g.n4 = (g.d2 + ROWN - 1) / ROWN;
+    g.items = ham_dim(h, 0) * g.d1 * g.n4;
+    g.nb = nb;
+    auto layers = [&](auto items, auto uni) {
+        constexpr int ITEMS = decltype(items)::value;
+        const unsigned blocks = (unsigned)((g.items + ITEMS - 1) / ITEMS);
+        k_net_first<ITEMS><<<blocks, NET_NT, 0, st>>>(g, wq_dev, R, ldr, scale, reinterpret_cast<uint4 *>(a1));
+        k_net_mid<ITEMS, decltype(uni)::value><<<blocks, NET_NT, 0, st>>>(g, wq_dev, a1, a2);
+        k_net_last<ITEMS><<<blocks, NET_NT, 0, st>>>(g, wq_dev, a2, W, ldw, rms);
+    };
+    using std::integral_constant;
+    if (nb <= 8) layers(integral_constant<int, 64>{}, integral_constant<bool, false>{});
+    else if (nb % 16) layers(integral_constant<int, 16>{}, integral_constant<bool, false>{});
+    else layers(integral_constant<int, 16>{}, integral_constant<bool, true>{});
     RS_LAUNCH_CHECK();
     return RS_OK;
 }
 
-int64_t learned_act_floats(int64_t npts, int nb) { return npts * nb * (1 + 2 * NC); }
+int64_t learned_act_floats(int64_t npts, int nb) { return npts * nb * (3 * NC / 2 + NC) + 64; }
 
 int learned_round_weights(const float *w, float *wq, cudaStream_t st) {
     k_round_weights<<<9, 256, 0, st>>>(w, wq, W_TOTAL);

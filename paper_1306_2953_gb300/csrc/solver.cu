@@ -92,8 +92,13 @@ __global__ void k_residual(const T *__restrict__ X, int64_t ldx, const T *__rest
                            const double *__restrict__ num, const double *__restrict__ den, T *__restrict__ R,
                            int64_t ldr, int ncols, int64_t npts) {
     const int rows = blockDim.x / ncols, k = threadIdx.x % ncols, r = threadIdx.x / ncols;
+    // one FP64 division per column and CTA: one per thread kept the few FP64
+    // units busy for longer than the rows' traffic
+    __shared__ T lams[256];
+    if (threadIdx.x < ncols) lams[threadIdx.x] = (T)(num[threadIdx.x] / den[threadIdx.x]);
+    __syncthreads();
     if (r >= rows) return;
-    const T lam = (T)(num[k] / den[k]);
+    const T lam = lams[k];
     for (int64_t p = blockIdx.x * (int64_t)rows + r; p < npts; p += (int64_t)gridDim.x * rows)
         R[p * ldr + k] = HX[p * ldh + k] - lam * X[p * ldx + k];
 }
@@ -106,10 +111,14 @@ __global__ void k_resnorm(const double *rr, int n, double dV, double *res) {
 template <typename T>
 __global__ void k_scale_cols(T *Y, int64_t ldy, int ncols, int64_t npts, const double *nrm2, double dV) {
     const int rows = blockDim.x / ncols, k = threadIdx.x % ncols, r = threadIdx.x / ncols;
-    if (r >= rows) return;
-    const double n2 = dV * nrm2[k];
-    if (!(n2 > 0)) return;
-    const T f = (T)(1.0 / sqrt(n2));
+    __shared__ T fs[256];   // one FP64 square root and division per column and CTA
+    if (threadIdx.x < ncols) {
+        const double n2 = dV * nrm2[threadIdx.x];
+        fs[threadIdx.x] = n2 > 0 ? (T)(1.0 / sqrt(n2)) : T(0);
+    }
+    __syncthreads();
+    if (r >= rows || !(dV * nrm2[k] > 0)) return;
+    const T f = fs[k];
     for (int64_t p = blockIdx.x * (int64_t)rows + r; p < npts; p += (int64_t)gridDim.x * rows) Y[p * ldy + k] *= f;
 }
 
