@@ -239,11 +239,12 @@ int rs_overlap_block(const rs_grid *g, const void *X_dev, int64_t ldx, int nx, c
 /* Tensor-core contractions of FP32 orbitals (5th-generation tensor cores,
  * tcgen05): every FP32 operand is split exactly into three BF16 pieces and
  * the six piece products of weight >= 2^-16 are accumulated in FP32, so the
- * results carry FP32-level accumulation error (not the exactly rounded FP64
- * of rs_overlap_block).  Workspace (device, caller-owned):
+ * results carry FP32-level accumulation error (not the FP64 accuracy of
+ * rs_overlap_block).  Workspace (device, caller-owned):
  * rs_tc_workspace_bytes(rows_a, rows_b, K) bytes, where the overlap has
  * rows_a = nx, rows_b = ny, K = npts and the rotation rows_a = npts,
- * rows_b = m, K = n.  Blocking (they read a status word). */
+ * rows_b = m, K = n.  Blocking (they synchronise the stream); a kernel whose
+ * bounded pipeline wait gives up writes NaN. */
 int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K);
 
 /* S = dV X^T Y (Eq. 5) for FP32 X [npts][ldx] (nx columns) and Y (ny
@@ -253,7 +254,7 @@ int rs_overlap_block_tc(const rs_grid *g, const float *X_dev, int64_t ldx, int n
 
 /* Subspace rotation Y = X C (Eqs. 6 and 8 applied by blocks of points): X
  * FP32 [npts][ldx] (n columns), C device double [n][ldc] (m columns), Y FP32
- * [npts][ldy]; Y may be X (the operands are split before the product). */
+ * [npts][ldy]; Y may be X or overlap it (X is copied to the workspace first where needed). */
 int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const double *C_dev, int64_t ldc, int m, float *Y_dev,
                     int64_t ldy, int64_t npts, void *work_dev, void *stream);
 
@@ -370,9 +371,9 @@ int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void *Psi0_dev, 
  * eigenvalues when the schedule took that step (rs_solver_stats says which);
  * resnorm_dev the residual norms the sweep measured.  n_converged: host,
  * states with residual norm <= tol (may be NULL).  Blocking (reads the
- * residuals).  Errors: RS_ENAN (a non-finite residual), RS_ETIMEOUT (a
- * bounded wait of an H psi or tensor-core kernel gave up: the sweep's
- * result is incomplete), RS_ECUDA. */
+ * residuals).  Errors: RS_ENAN (a non-finite residual; a tensor-core kernel
+ * whose bounded wait gave up writes NaN), RS_ETIMEOUT (a bounded wait of an
+ * H psi kernel gave up: the sweep's result is incomplete), RS_ECUDA. */
 int rs_eigensolver_step(rs_solver *s, double *eps_dev, double *resnorm_dev, int *n_converged, void *stream);
 
 typedef struct {

@@ -17,8 +17,8 @@
 // points and summed as 64-bit integers: with t + 1 pairs of digits in
 // accumulator t everything up to t = 3 is exact and a rounding of a later
 // one is below 2^-56 of the largest product.  So the result is the exact
-// sum of products of operands rounded to s bits: NS = 8 (FP64), 7 (FP32 data
-// at FP64-like accuracy) or 5 (FP32 accuracy).  (Ozaki, Ogita, Oishi and Rump
+// sum of products of operands rounded to s bits: NS = 8 (FP64), 7 (overlap of
+// FP32 data at FP64-like accuracy) or 5 (rotation of FP32 data).  (Ozaki, Ogita, Oishi and Rump
 // 2012 give the scheme of error-free splittings of a matrix product.)
 //
 // Kernel: 8 converter warps and one MMA warp per CTA, one CTA per SM, a 128 x
@@ -48,6 +48,7 @@
 
 #include "device.h"
 #include "digits.h"
+#include "linalg.h"
 
 namespace rs {
 
@@ -89,6 +90,10 @@ __device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile i
 }
 // The MMA warp runs its loop as a whole, so that descriptors stay in uniform
 // registers; `lead` (one lane) issues.
+// the whole warp: true only when every lane's wait ended (no lane goes on alone)
+__device__ __forceinline__ bool dg_wait_warp(uint64_t *b, uint32_t parity, volatile int *bad) {
+    return __all_sync(0xffffffffu, dg_wait(b, parity, bad));
+}
 __device__ __forceinline__ void dg_mma(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum,
                                        uint32_t lead) {
     asm volatile(
@@ -330,34 +335,38 @@ template <int NS, int BN, int PAD> struct DgIssue {
     }
 };
 
-// One readout (in the order in which the accumulators complete): the converter thread's 32 columns of every accumulator added to
-// H (t = 0..2, in units of accumulator 2) and L (t = 3.., in units of 256 times
-// the weight of accumulator NS - 1).
-template <int NS, int BN>
-__device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t *H, int64_t *L) {
+// One readout (in the order in which the accumulators complete) of CPT columns of
+// the converter thread's row: H += accumulators 0 .. 2 in units of accumulator
+// 2, L += the later ones in units of accumulator NS - 2, the last one rounded to
+// them.
+template <int NS, int BN, int CPT>
+__device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&H)[CPT], int64_t (&L)[CPT]) {
     const int warp = threadIdx.x >> 5;
     const uint32_t lane_base = b.tmem + ((uint32_t)(warp & 3) * 32 << 16) + (uint32_t)col0;
 #pragma unroll
     for (int t = 0; t < NS - 2; ++t) {
-        uint32_t r[32];
-        if (!dg_wait(&b.accfull[t], iv & 1, &b.bad)) return false;
+        if (!dg_wait_warp(&b.accfull[t], iv & 1, &b.bad)) return false;
         DG_FENCE_AFTER();
-        dg_tmem_ld32(lane_base + t * BN, r);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            // accumulators 0 and 1 stay within 2^22: their integers stand in the
-            // mantissa after one addition (the conversion unit is slow)
-            const int64_t v = t < 2 ? (int64_t)((int)__float_as_uint(__fadd_rn(__uint_as_float(r[j]), 12582912.f)) - 0x4b400000)
-                                    : (int64_t)__float2int_rn(__uint_as_float(r[j]));
-            if (t < 3) H[j] += v * (int64_t)(1 << (8 * (2 - t)));
-            else L[j] += v * (int64_t)(1 << (8 * (NS - 2 - t)));
+        for (int c = 0; c < CPT; c += 32) {
+            uint32_t r[32];
+            dg_tmem_ld32(lane_base + t * BN + c, r);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                // accumulators 0 and 1 stay within 2^22: their integers stand in the
+                // mantissa after one addition (the conversion unit is slow)
+                const int64_t v = t < 2 ? (int64_t)((int)__float_as_uint(__fadd_rn(__uint_as_float(r[j]), 12582912.f)) - 0x4b400000)
+                                        : (int64_t)__float2int_rn(__uint_as_float(r[j]));
+                if (t < 3) H[c + j] += v * (int64_t)(1 << (8 * (2 - t)));
+                else L[c + j] += v * (int64_t)(1 << (8 * (NS - 2 - t)));
+            }
         }
     }
     // the last two accumulators together, rounded at the weight of the first
-    if (!dg_wait(&b.accfull[NS - 1], iv & 1, &b.bad)) return false;
+    if (!dg_wait_warp(&b.accfull[NS - 1], iv & 1, &b.bad)) return false;
     DG_FENCE_AFTER();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < CPT / 8; ++q) {
         uint32_t u[8], w[8];
         dg_tmem_ld8(lane_base + (NS - 2) * BN + 8 * q, u);
         dg_tmem_ld8(lane_base + (NS - 1) * BN + 8 * q, w);
@@ -484,17 +493,18 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
                                       : T(0);
             }
         };
-        int64_t H[32], L[32];
+        constexpr int CPT = 32;   // columns of the result per thread
+        int64_t H[CPT], L[CPT];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) H[j] = L[j] = 0;
-        const int col0 = (warp >> 2) * 32;
+        for (int j = 0; j < CPT; ++j) H[j] = L[j] = 0;
+        const int col0 = (warp >> 2) * CPT;
         const bool drains = col0 < BN;   // BN = 32: the second four warps only free the accumulators
         bool ok = true;
         load(0);
         int iv = 0;   // readouts taken
         for (int it = 0; it < nst && ok; ++it) {
             const int s = it % DG_STAGES;
-            if (it >= DG_STAGES && !dg_wait(&b.empty[s], (it / DG_STAGES - 1) & 1, &b.bad)) {
+            if (it >= DG_STAGES && !dg_wait_warp(&b.empty[s], (it / DG_STAGES - 1) & 1, &b.bad)) {
                 ok = false;
                 break;
             }
@@ -506,16 +516,16 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
             if (it + 1 < nst) load(it + 1);
             // the previous 256 points' accumulators, once the first stage after them is queued
             if (it % DG_DRAIN == 0 && it > 0) {
-                ok = dg_drain<NS, BN>(b, iv, drains ? col0 : 0, H, L);
+                ok = dg_drain<NS, BN, CPT>(b, iv, drains ? col0 : 0, H, L);
                 ++iv;
             }
         }
-        if (ok) ok = dg_drain<NS, BN>(b, iv, drains ? col0 : 0, H, L);
+        if (ok) ok = dg_drain<NS, BN, CPT>(b, iv, drains ? col0 : 0, H, L);
         const int row = (warp & 3) * 32 + lane, i = m0 + row;
         if (i < a.nx && drains) {
             const int s2 = 2 * (8 * NS - 2);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
+            for (int j = 0; j < CPT; ++j) {
                 const int jc = n0 + col0 + j;
                 if (jc >= a.ny || (a.sym && jc < i)) continue;
                 const int e = ea[row] + eb[col0 + j] - 2 * (ExpOf<T>::bias - 1) - s2;
@@ -609,7 +619,7 @@ template <typename T, int NS, int BN> int launch_gram(GramArgs<T> a, int tiles_m
 
 template <typename T>
 int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, bool exact, int *scratch, cudaStream_t st) {
+               int64_t lds, int *scratch, cudaStream_t st) {
     if (npts > (int64_t)INT32_MAX - 64) return fail(RS_EINVAL, "digit_gram: too many points");
     const bool sym = X == Y && ldx == ldy && nx == ny;
     int *keys = scratch;
@@ -634,14 +644,13 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
         // 32 columns of Y fill half of a 64-wide tile
         const bool narrow = ny <= 32;
         if constexpr (sizeof(T) == 8) return narrow ? launch_gram<T, 8, 32>(a, tm, st) : launch_gram<T, 8, 64>(a, tm, st);
-        else if (exact) return narrow ? launch_gram<T, 7, 32>(a, tm, st) : launch_gram<T, 7, 64>(a, tm, st);
-        else return narrow ? launch_gram<T, 5, 32>(a, tm, st) : launch_gram<T, 5, 64>(a, tm, st);
+        else return narrow ? launch_gram<T, 7, 32>(a, tm, st) : launch_gram<T, 7, 64>(a, tm, st);
     }
 }
 template int digit_gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
-                                int64_t, bool, int *, cudaStream_t);
+                                int64_t, int *, cudaStream_t);
 template int digit_gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *,
-                               int64_t, bool, int *, cudaStream_t);
+                               int64_t, int *, cudaStream_t);
 
 // ----------------------------------------------------------- rotation ---
 
@@ -803,12 +812,11 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         int64_t H[32], L[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) H[i] = L[i] = 0;
-        auto load = [&](int tile, int it) {
+        auto load = [&](int u, int tile, int it) {   // u = 0, 1: rows of X; 2: C
             const int blk = it >= kst ? 1 : 0, k0 = (it - blk * kst) * DG_K;   // (NBLK <= 2)
             const int64_t r0 = (int64_t)tile * DG_M;
             const int rows = (int)min((int64_t)DG_M, a.npts - r0);
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            if (u < 2) {
                 const T *x = a.X + (r0 + min(ar + 8 * u, rows - 1)) * a.ldx + k0 + 8 * akq;
                 if (a.vec && k0 + 8 * akq + 8 <= a.n) {
                     constexpr int E = 16 / (int)sizeof(T);
@@ -824,7 +832,7 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                     for (int k = 0; k < 8; ++k) va[u][k] = k0 + 8 * akq + k < a.n ? x[k] : T(0);
                 }
             }
-            if (hasb) {
+            if (u == 2 && hasb) {
                 const int c = (nb0 + blk) * BN + bcol;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
@@ -891,12 +899,12 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         int ptile = 0, ptj = 0, pe = 0, pblk = 0, iv = 0;
         auto readout = [&]() {
             open = false;
-            ok = ok && dg_drain<NS, BN>(b, iv, owns ? col0 : 0, H, L);
+            ok = ok && dg_drain<NS, BN, 32>(b, iv, owns ? col0 : 0, H, L);
             ++iv;
             if (!pend) return;
             // the block's sums are complete
             const bool lastb = pblk == NBLK - 1;
-            if (lastb && a.cluster) ok = dg_wait(&rb.rd, ptj & 1, &b.bad) && ok;
+            if (lastb && a.cluster) ok = dg_wait_warp(&rb.rd, ptj & 1, &b.bad) && ok;
             const int64_t p = (int64_t)ptile * DG_M + row;
             const bool on = owns && p < a.npts;
             if (NBLK > 1 && lastb && on) {
@@ -933,7 +941,10 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         // One loop over the stages of all tiles; it == nst: the next tile is due.
         int tile = (int)blockIdx.y - (int)gridDim.y, j = -1, g = 0, it = nst, kb = 0, blk = 0, h = 0;
         int ex0 = 0, ex1 = 0, er = 0;
-        if ((int)blockIdx.y < ntiles) load(blockIdx.y, 0);
+        if ((int)blockIdx.y < ntiles) {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) load(u, blockIdx.y, 0);
+        }
         while (ok) {
             bool plain = false, flush = false, end = false;
             if (it == nst) {
@@ -942,7 +953,7 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                 end = tile >= ntiles;
                 if (!end) {
                     h = j & 1;
-                    ok = dg_wait(&rb.keyfull[h], (j / 2) & 1, &b.bad);
+                    ok = dg_wait_warp(&rb.keyfull[h], (j / 2) & 1, &b.bad);
                     ex0 = ea[h][ar], ex1 = ea[h][ar + 8], er = ea[h][row];
                     const volatile int *f = rb.plain[h];
                     plain = cplain || f[0] || f[1] || f[2];
@@ -953,17 +964,20 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
             }
             if (!end && !plain && ok) {
                 const int s = g % DG_STAGES;
-                if (g >= DG_STAGES) ok = dg_wait(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.bad);
+                if (g >= DG_STAGES) ok = dg_wait_warp(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.bad);
+                const bool lasts = it + 1 == nst, more = !lasts || tile + (int)gridDim.y < ntiles;
+                const int nt = lasts ? tile + gridDim.y : tile, ni = lasts ? 0 : it + 1;
                 if (ok) {
                     store_digits<T, NS>(va[0], ex0, adst + s * C::STAGE, C::SL_A);
+                    if (more) load(0, nt, ni);
                     store_digits<T, NS>(va[1], ex1, adst + s * C::STAGE + 128, C::SL_A);
+                    if (more) load(1, nt, ni);
                     if (hasb) store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B);
+                    if (more) load(2, nt, ni);
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     dg_arrive(&b.full[s]);
                 }
-                const bool lasts = it + 1 == nst;
                 if (lasts) rows_read();
-                if (!lasts || tile + (int)gridDim.y < ntiles) load(lasts ? tile + gridDim.y : tile, lasts ? 0 : it + 1);
                 flush = kb % DG_DRAIN == 0 && open;
             }
             if (flush) readout();
@@ -983,7 +997,7 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                 }
                 asm volatile("bar.sync 1, 256;\n" ::: "memory");   // every converter of this CTA has read its row
                 rows_read();
-                if (a.cluster) ok = dg_wait(&rb.rd, j & 1, &b.bad) && ok;
+                if (a.cluster) ok = dg_wait_warp(&rb.rd, j & 1, &b.bad) && ok;
                 if (owns && (int64_t)tile * DG_M + row < a.npts)
                     for (int i = 0; i < NBLK * 32; ++i) {
                         const int c = (nb0 + i / 32) * BN + col0 + i % 32;
@@ -994,7 +1008,10 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                             *y = v;
                         }
                     }
-                if (tile + (int)gridDim.y < ntiles) load(tile + gridDim.y, 0);
+                if (tile + (int)gridDim.y < ntiles) {
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) load(u, tile + gridDim.y, 0);
+                }
             } else {
                 if (kb % DG_DRAIN == DG_DRAIN - 1 || kb == kst - 1) {
                     open = true;
@@ -1014,25 +1031,22 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
     if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, int cluster, cudaStream_t st) {
-    using C = DgCfg<NS, BN, 32>;
-    auto fn = k_digit_rot<T, NS, BN, NBLK>;
-    RS_TRY(smem_optin((const void *)fn, C::SMEM));
-    const unsigned gx = (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK));
-    const int64_t tiles = (a.npts + DG_M - 1) / DG_M;
+// Launches a rotation kernel: gx column blocks, as many row workers as are
+// resident at once; in place the column blocks of a row tile are a cluster.
+template <typename Fn, typename Args>
+int launch_rows(Fn fn, Args a, unsigned gx, size_t smem, bool in_place, cudaStream_t st) {
+    a.cluster = in_place && gx > 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(gx, 1);
     cfg.blockDim = dim3(DG_NT);
-    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cluster ? gx : 1;
+    at.val.clusterDim.x = a.cluster ? gx : 1;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    a.cluster = cluster && gx > 1;
-    // as many row workers as are resident at once
     int workers = 0;
     if (a.cluster) {
         RS_CUDA(cudaOccupancyMaxActiveClusters(&workers, fn, &cfg));
@@ -1040,8 +1054,492 @@ template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, int
         RS_TRY(sm_count(&workers));
         workers /= (int)gx;
     }
+    const int64_t tiles = (a.npts + DG_M - 1) / DG_M;
     cfg.gridDim.y = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, workers));
     RS_CUDA(cudaLaunchKernelEx(&cfg, fn, a));
+    return RS_OK;
+}
+
+template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, bool in_place, cudaStream_t st) {
+    using C = DgCfg<NS, BN, 32>;
+    auto fn = k_digit_rot<T, NS, BN, NBLK>;
+    RS_TRY(smem_optin((const void *)fn, C::SMEM));
+    return launch_rows(fn, a, (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK)), C::SMEM, in_place, st);
+}
+
+// ------------------------------------- FP32 rotation by BF16 pieces ---
+// Y = alpha X C + beta Y to FP32 accuracy, for the eigensolver's inner steps
+// and rs_rotate_block: every operand is the exact sum of three BF16 pieces
+// (8 + 8 + 8 bits), and the six piece products of weight 2^-16 and up are
+// summed in FP32 by the tensor core, the leading one apart from the others.
+// The pieces need no exponent pass and a quarter of the digits' instructions.
+//
+// One CTA per SM, row tiles of 128 dealt round robin, one column block of BN per
+// CTA; eight converter warps cut X into pieces, the pieces of C (made once by
+// k_piece_c) come by bulk copies, four stages of 32 states ahead; two
+// accumulator sets let the products of a tile run while the last one's are
+// stored.  In place the CTAs of a row tile are a cluster, as in k_digit_rot.
+// What it measured (658 416 rows, 256 -> 256 / 256 -> 64 columns): 678 / 303 us,
+// 943 / 564 us for a split pass and a product kernel before.
+
+struct PieceArgs {
+    const float *X;
+    const uint4 *Cp;     // [block][stage][8-step group][piece][column][8 steps] BF16
+    float *Y;
+    int64_t ldx, ldy, npts;
+    int n, m;
+    int vec, yvec, cluster;
+    float alpha, beta;
+};
+
+constexpr int PC_ST = 4;   // stages
+
+template <int BN> struct PcCfg {
+    static constexpr int LBO_A = DG_M * 16 + 32, SL_A = KQ * LBO_A, A_BYTES = 3 * SL_A;
+    static constexpr int SL_B = BN * 16, LBO_B = 3 * SL_B, B_BYTES = KQ * LBO_B;
+    static constexpr int STAGE = A_BYTES + B_BYTES;
+    static constexpr int TMEM = 4 * BN;   // two sets of (leading, other) products
+    static constexpr size_t SMEM = (size_t)PC_ST * STAGE + 128;
+};
+
+// two values to one word per piece, the first in the low half
+__device__ __forceinline__ void bf16_pieces(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(p[k]) : "f"(y), "f"(x));
+        x -= __uint_as_float(p[k] << 16);
+        y -= __uint_as_float(p[k] & 0xffff0000u);
+    }
+}
+
+template <int BN> __global__ void k_piece_c(const double *__restrict__ C, int64_t ldc, int n, int m, int kst, uint4 *__restrict__ P) {
+    // one thread per (block, stage, group, column)
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int col = t % BN, g = t / BN, kq = g % KQ, st = g / KQ % kst, blk = g / KQ / kst;
+    const int c = blk * BN + col, k0 = st * DG_K + kq * 8;
+    if (blk >= (m + BN - 1) / BN) return;
+    uint32_t w[4][3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = k0 + 2 * i;
+        const float x = c < m && k < n ? (float)__ldg(C + (int64_t)k * ldc + c) : 0.f;
+        const float y = c < m && k + 1 < n ? (float)__ldg(C + (int64_t)(k + 1) * ldc + c) : 0.f;
+        bf16_pieces(x, y, w[i]);
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) P[((int64_t)g * 3 + p) * BN + col] = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+}
+
+template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceArgs a) {
+    using C = PcCfg<BN>;
+    extern __shared__ __align__(128) unsigned char dgsm[];
+    __shared__ uint64_t full[PC_ST], empty[PC_ST], accfull[2], accfree[2], rd, done;
+    __shared__ uint32_t tmem_s;
+    __shared__ int bad;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int kst = (a.n + DG_K - 1) / DG_K;
+    const int ntiles = (int)((a.npts + DG_M - 1) / DG_M);
+    if (tid == 0) {
+        for (int i = 0; i < PC_ST; ++i) {
+            dg_bar_init(&full[i], DG_CT + 1);
+            dg_bar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            dg_bar_init(&accfull[i], 1);
+            dg_bar_init(&accfree[i], DG_CT);
+        }
+        dg_bar_init(&rd, DG_CT * (a.cluster ? gridDim.x : 1));
+        dg_bar_init(&done, 1);
+        bad = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == DG_CW) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dg_su32(&tmem_s)), "r"(C::TMEM)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    DG_FENCE_AFTER();
+    if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+
+    if (warp == DG_CW + 1) {
+        // the pieces of C, stage by stage
+        if (lane == 0) {
+            int g = 0;
+            bool ok = true;
+            for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y)
+                for (int it = 0; it < kst; ++it, ++g) {
+                    const int s = g % PC_ST;
+                    if (g >= PC_ST && !dg_wait(&empty[s], (g / PC_ST - 1) & 1, &bad)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(dg_su32(&full[s])), "r"(C::B_BYTES)
+                                 : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                            dg_su32(dgsm + s * C::STAGE + C::A_BYTES)),
+                        "l"(a.Cp + ((int64_t)blockIdx.x * kst + it) * (C::B_BYTES / 16)), "r"(C::B_BYTES), "r"(dg_su32(&full[s]))
+                        : "memory");
+                }
+            // no copy is in flight when the CTA ends
+            for (int q = g < PC_ST ? 0 : g - PC_ST; q < g; ++q)
+                for (int i = 0; i < (*(volatile int *)&bad ? 64 : DG_SPIN) && !dg_try(&full[q % PC_ST], (q / PC_ST) & 1); ++i) {
+                }
+        }
+    } else if (warp == DG_CW) {
+        const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_s, 0), lead = lane == 0;
+        const uint64_t da0 = dg_desc(dg_su32(dgsm), C::LBO_A), db0 = dg_desc(dg_su32(dgsm) + C::A_BYTES, C::LBO_B);
+        constexpr uint32_t BF = (1u << 7) | (1u << 10);   // both operands BF16
+        int g = 0, j = 0;
+        bool ok = true;
+        for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
+            const uint32_t acc = tmem + (j & 1) * 2 * BN;
+            if (j >= 2) ok = __all_sync(0xffffffffu, dg_wait(&accfree[j & 1], (j / 2 - 1) & 1, &bad));
+            DG_FENCE_AFTER();
+            for (int it = 0; it < kst && ok; ++it, ++g) {
+                const int s = g % PC_ST;
+                ok = __all_sync(0xffffffffu, dg_wait(&full[s], (g / PC_ST) & 1, &bad));
+                DG_FENCE_AFTER();
+                const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
+                if (ok) {
+#pragma unroll
+                    for (int k = 0; k < DG_K / 16; ++k) {
+                        const uint64_t ka = (uint64_t)(2 * k * C::LBO_A >> 4), kb = (uint64_t)(2 * k * C::LBO_B >> 4);
+                        auto A = [&](int i) { return da + ka + (uint64_t)(i * C::SL_A >> 4); };
+                        auto B = [&](int i) { return db + kb + (uint64_t)(i * C::SL_B >> 4); };
+                        const uint32_t on = it > 0 || k > 0;
+                        // leading product and A0 B1 side by side, then the rest onto the latter
+                        dg_mma(acc, A(0), B(0), dg_idesc(DG_M, 2 * BN) | BF, on, lead);
+                        dg_mma(acc + BN, A(0), B(2), dg_idesc(DG_M, BN) | BF, 1u, lead);
+                        dg_mma(acc + BN, A(1), B(0), dg_idesc(DG_M, BN) | BF, 1u, lead);
+                        dg_mma(acc + BN, A(1), B(1), dg_idesc(DG_M, BN) | BF, 1u, lead);
+                        dg_mma(acc + BN, A(2), B(0), dg_idesc(DG_M, BN) | BF, 1u, lead);
+                    }
+                }
+                dg_commit(&empty[s], lead);
+            }
+            dg_commit(&accfull[j & 1], lead);
+        }
+        dg_commit(&done, lead);
+        dg_wait(&done, 0, &bad);
+    } else if (warp < DG_CW) {
+        const int ar = warp * 16 + (lane >> 2), akq = lane & 3;
+        unsigned char *adst = dgsm + akq * C::LBO_A + ar * 16;
+        constexpr int CPT = BN / 2;   // columns per thread in the readout
+        const int col0 = (warp >> 2) * CPT, row = (warp & 3) * 32 + lane;
+        bool ok = true;
+        float va[2][8];
+        auto load = [&](int u, int tile, int it) {
+            const int64_t r0 = (int64_t)tile * DG_M;
+            const int rows = (int)min((int64_t)DG_M, a.npts - r0), k0 = it * DG_K + 8 * akq;
+            {
+                const float *x = a.X + (r0 + min(ar + 8 * u, rows - 1)) * a.ldx + k0;
+                if (a.vec && k0 + 8 <= a.n) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        const float4 t = reinterpret_cast<const float4 *>(x)[q];
+                        va[u][4 * q] = t.x, va[u][4 * q + 1] = t.y, va[u][4 * q + 2] = t.z, va[u][4 * q + 3] = t.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) va[u][k] = k0 + k < a.n ? x[k] : 0.f;
+                }
+            }
+        };
+        auto readout = [&](int tile, int j) {
+            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &bad);
+            if (a.cluster) ok = dg_wait_warp(&rd, j & 1, &bad) && ok;
+            DG_FENCE_AFTER();
+            const int64_t p = (int64_t)tile * DG_M + row;
+            const uint32_t t0 = tmem_s + ((uint32_t)(warp & 3) * 32 << 16) + (j & 1) * 2 * BN + col0;
+            const int cb = blockIdx.x * BN + col0;
+            float *y = a.Y + p * a.ldy + cb;
+#pragma unroll
+            for (int c = 0; c < CPT; c += 32) {
+                uint32_t r[32];
+                float v[32];
+                dg_tmem_ld32(t0 + BN + c, r);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+                dg_tmem_ld32(t0 + c, r);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = ok ? a.alpha * (__uint_as_float(r[i]) + v[i]) : __int_as_float(0x7fffffff);
+                if (c + 32 >= CPT) {
+                    DG_FENCE_BEFORE();
+                    dg_arrive(&accfree[j & 1]);
+                }
+                if (p >= a.npts) continue;
+                if (a.yvec && cb + c + 32 <= a.m) {
+                    float4 *y4 = reinterpret_cast<float4 *>(y + c);
+                    if (a.beta != 0.f) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 o = y4[q];
+                            v[4 * q] += a.beta * o.x, v[4 * q + 1] += a.beta * o.y, v[4 * q + 2] += a.beta * o.z, v[4 * q + 3] += a.beta * o.w;
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) y4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (cb + c + i < a.m) y[c + i] = a.beta != 0.f ? v[i] + a.beta * y[c + i] : v[i];
+                }
+            }
+        };
+        int j = 0, g = 0, ptile = -1;
+        if ((int)blockIdx.y < ntiles) {
+            load(0, blockIdx.y, 0);
+            load(1, blockIdx.y, 0);
+        }
+        for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
+            for (int it = 0; it < kst && ok; ++it, ++g) {
+                const int s = g % PC_ST;
+                if (g >= PC_ST) ok = dg_wait_warp(&empty[s], (g / PC_ST - 1) & 1, &bad);
+                if (!ok) break;
+                const bool last = it + 1 == kst;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    uint32_t w[4][3];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) bf16_pieces(va[u][2 * i], va[u][2 * i + 1], w[i]);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+                        *reinterpret_cast<uint4 *>(adst + s * C::STAGE + u * 128 + p * C::SL_A) =
+                            make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+                    if (!last || tile + (int)gridDim.y < ntiles) load(u, last ? tile + gridDim.y : tile, last ? 0 : it + 1);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                dg_arrive(&full[s]);
+                if (last && a.cluster)
+                    for (int r = 0; r < (int)gridDim.x; ++r)
+                        asm volatile(
+                            "{\n .reg .b32 ra;\n mapa.shared::cluster.u32 ra, %0, %1;\n"
+                            " mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(dg_su32(&rd)),
+                            "r"(r)
+                            : "memory");
+                if (it == 0 && ptile >= 0) readout(ptile, j - 1);
+            }
+            ptile = tile;
+        }
+        if (ptile >= 0) readout(ptile, j - 1);
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    if (warp == DG_CW)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_s), "r"(C::TMEM) : "memory");
+    // no CTA leaves while another may still signal it
+    if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+template <int BN> int launch_piece(PieceArgs a, const double *C, int64_t ldc, void *work, bool in_place, cudaStream_t st) {
+    using P = PcCfg<BN>;
+    auto fn = k_piece_rot<BN>;
+    RS_TRY(smem_optin((const void *)fn, P::SMEM));
+    const int kst = (a.n + DG_K - 1) / DG_K;
+    const unsigned gx = (unsigned)((a.m + BN - 1) / BN);
+    const int64_t nc = (int64_t)gx * kst * KQ * BN;
+    k_piece_c<BN><<<(unsigned)((nc + 127) / 128), 128, 0, st>>>(C, ldc, a.n, a.m, kst, (uint4 *)work);
+    RS_LAUNCH_CHECK();
+    a.Cp = (const uint4 *)work;
+    return launch_rows(fn, a, gx, P::SMEM, in_place, st);
+}
+
+// ------------------------------------- FP32 overlap by BF16 pieces ---
+// S += dV X^T Y to FP32 accuracy: the six piece products of a chunk of at most
+// 2048 points are summed in FP32 by the tensor core, chunks meet in FP64.  The
+// converters cut both operands into pieces on the way to shared memory, so that
+// an FP32 value is read once per tile and no pieces are written.  Work items (chunk,
+// tile), tiles fastest, are dealt round robin to one CTA per SM; the readout of
+// an item overlaps the products of the next.
+// Measured (658 416 points): 256 x 64 columns 338 us, 256 x 256 787 us; 800 and
+// 1382 us with a separate pass that wrote the pieces to memory.
+
+struct PieceGramArgs {
+    const float *X, *Y;
+    int64_t ldx, ldy, npts, lds;
+    int nx, ny;
+    double *S;
+    double dV;
+    int tiles_n, tiles, chunks, kb;   // kb: 64-point stages per chunk
+};
+
+constexpr int PG_K = 64, PG_KQ = PG_K / 8, PG_ST = 2;
+
+template <int BN> struct PgCfg {
+    static constexpr int LBO_A = DG_M * 16, SL_A = PG_KQ * LBO_A, A_BYTES = 3 * SL_A;
+    static constexpr int LBO_B = BN * 16, SL_B = PG_KQ * LBO_B, STAGE = A_BYTES + 3 * SL_B;
+    static constexpr int TMEM = 2 * BN;
+    static constexpr size_t SMEM = (size_t)PG_ST * STAGE + 128;
+};
+
+template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(PieceGramArgs a) {
+    using C = PgCfg<BN>;
+    extern __shared__ __align__(128) unsigned char dgsm[];
+    __shared__ uint64_t full[PG_ST], empty[PG_ST], accfull[2], accfree[2], done;
+    __shared__ uint32_t tmem_s;
+    __shared__ int bad;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int items = a.tiles * a.chunks, nkb = (int)((a.npts + PG_K - 1) / PG_K);
+    if (tid == 0) {
+        for (int i = 0; i < PG_ST; ++i) {
+            dg_bar_init(&full[i], DG_CT);
+            dg_bar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            dg_bar_init(&accfull[i], 1);
+            dg_bar_init(&accfree[i], DG_CT);
+        }
+        dg_bar_init(&done, 1);
+        bad = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == DG_CW) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dg_su32(&tmem_s)), "r"(C::TMEM)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    DG_FENCE_AFTER();
+    auto stages_of = [&](int item) { return min(a.kb, nkb - item / a.tiles * a.kb); };
+
+    if (warp == DG_CW) {
+        const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_s, 0), lead = lane == 0;
+        const uint64_t da0 = dg_desc(dg_su32(dgsm), C::LBO_A), db0 = dg_desc(dg_su32(dgsm) + C::A_BYTES, C::LBO_B);
+        constexpr uint32_t idesc = dg_idesc(DG_M, BN) | (1u << 7) | (1u << 10);   // both operands BF16
+        int g = 0, j = 0;
+        bool ok = true;
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++j) {
+            const uint32_t acc = tmem + (j & 1) * BN;
+            const int nst = stages_of(item);
+            if (j >= 2) ok = dg_wait_warp(&accfree[j & 1], (j / 2 - 1) & 1, &bad);
+            DG_FENCE_AFTER();
+            for (int it = 0; it < nst && ok; ++it, ++g) {
+                const int s = g % PG_ST;
+                ok = dg_wait_warp(&full[s], (g / PG_ST) & 1, &bad);
+                DG_FENCE_AFTER();
+                const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
+                if (ok) {
+                    // pieces (0,0) (0,1) (1,0) (0,2) (1,1) (2,0), each over the stage's four steps of 16
+#pragma unroll
+                    for (int pr = 0; pr < 6; ++pr) {
+                        constexpr int pa[6] = {0, 0, 1, 0, 1, 2}, pb[6] = {0, 1, 0, 2, 1, 0};
+#pragma unroll
+                        for (int k = 0; k < PG_K / 16; ++k)
+                            dg_mma(acc, da + (uint64_t)((pa[pr] * C::SL_A + 2 * k * C::LBO_A) >> 4),
+                                   db + (uint64_t)((pb[pr] * C::SL_B + 2 * k * C::LBO_B) >> 4), idesc,
+                                   (it > 0 || pr > 0 || k > 0) ? 1u : 0u, lead);
+                    }
+                }
+                dg_commit(&empty[s], lead);
+            }
+            dg_commit(&accfull[j & 1], lead);
+        }
+        dg_commit(&done, lead);
+        dg_wait(&done, 0, &bad);
+    } else if (warp < DG_CW) {
+        // units (32 columns, 8 points): 4 x 8 of X, BN / 32 x 8 of Y; warp w takes
+        // the points 8 w .. of every column group
+        constexpr int NA = DG_M / 32, NU = NA + BN / 32;
+        float v[NU][8];
+        bool ok = true;
+        auto column = [&](int tile, int u) {
+            const int m0 = tile / a.tiles_n * DG_M, n0 = tile % a.tiles_n * BN;
+            return u < NA ? m0 + u * 32 + lane : n0 + (u - NA) * 32 + lane;
+        };
+        auto load = [&](int item, int it) {
+            const int tile = item % a.tiles;
+            const int64_t p = ((int64_t)(item / a.tiles) * a.kb + it) * PG_K + 8 * warp;
+#pragma unroll
+            for (int u = 0; u < NU; ++u) {
+                const bool isx = u < NA;
+                const int c = column(tile, u);
+                const bool in = c < (isx ? a.nx : a.ny);
+                const int64_t ld = isx ? a.ldx : a.ldy;
+                const float *src = (isx ? a.X : a.Y) + p * ld + c;
+                // columns beyond the last are zero
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[u][k] = in && p + k < a.npts ? __ldg(src + k * ld) : 0.f;
+            }
+        };
+        constexpr int CPT = BN / 2;
+        const int col0 = (warp >> 2) * CPT, row = (warp & 3) * 32 + lane;
+        auto readout = [&](int item, int j) {
+            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &bad);
+            DG_FENCE_AFTER();
+            const int tile = item % a.tiles, i = tile / a.tiles_n * DG_M + row, c0 = tile % a.tiles_n * BN + col0;
+            const uint32_t t0 = tmem_s + ((uint32_t)(warp & 3) * 32 << 16) + (j & 1) * BN + col0;
+            double *srow = a.S + (int64_t)i * a.lds + c0;
+#pragma unroll
+            for (int c = 0; c < CPT; c += 32) {
+                uint32_t r[32];
+                dg_tmem_ld32(t0 + c, r);
+                if (c + 32 >= CPT) {
+                    DG_FENCE_BEFORE();
+                    dg_arrive(&accfree[j & 1]);
+                }
+                if (i < a.nx) {
+#pragma unroll
+                    for (int q = 0; q < 32; ++q)
+                        if (c0 + c + q < a.ny)
+                            atomicAdd(srow + c + q, ok ? a.dV * (double)__uint_as_float(r[q]) : __longlong_as_double(0x7ff8000000000000ll));
+                }
+            }
+        };
+        int j = 0, g = 0, pitem = -1;
+        if ((int)blockIdx.x < items) load(blockIdx.x, 0);
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++j) {
+            const int nst = stages_of(item);
+            for (int it = 0; it < nst && ok; ++it, ++g) {
+                const int s = g % PG_ST;
+                if (g >= PG_ST) ok = dg_wait_warp(&empty[s], (g / PG_ST - 1) & 1, &bad);
+                if (!ok) break;
+                unsigned char *st = dgsm + s * C::STAGE + lane * 16;
+#pragma unroll
+                for (int u = 0; u < NU; ++u) {
+                    uint32_t w[4][3];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) bf16_pieces(v[u][2 * i], v[u][2 * i + 1], w[i]);
+                    unsigned char *d = u < NA ? st + warp * C::LBO_A + u * 512 : st + C::A_BYTES + warp * C::LBO_B + (u - NA) * 512;
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+                        *reinterpret_cast<uint4 *>(d + p * (u < NA ? C::SL_A : C::SL_B)) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                dg_arrive(&full[s]);
+                const bool last = it + 1 == nst;
+                const int ni = last ? item + gridDim.x : item;
+                if (ni < items) load(ni, last ? 0 : it + 1);
+                if (it == 0 && pitem >= 0) readout(pitem, j - 1);
+            }
+            pitem = item;
+        }
+        if (pitem >= 0) readout(pitem, j - 1);
+    }
+    DG_FENCE_BEFORE();
+    __syncthreads();
+    if (warp == DG_CW)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_s), "r"(C::TMEM) : "memory");
+}
+
+template <int BN> int launch_piece_gram(PieceGramArgs a, cudaStream_t st) {
+    using C = PgCfg<BN>;
+    RS_TRY(smem_optin((const void *)k_piece_gram<BN>, C::SMEM));
+    a.tiles_n = (a.ny + BN - 1) / BN;
+    a.tiles = (a.nx + DG_M - 1) / DG_M * a.tiles_n;
+    // chunks: enough for every SM, of at most 2048 points
+    const int64_t nkb = (a.npts + PG_K - 1) / PG_K;
+    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(nkb, (148 + a.tiles - 1) / a.tiles));
+    a.kb = (int)std::min<int64_t>((nkb + want - 1) / want, 2048 / PG_K);
+    a.chunks = (int)((nkb + a.kb - 1) / a.kb);
+    int nsm = 0;
+    RS_TRY(sm_count(&nsm));
+    if ((int64_t)a.tiles * a.chunks > INT32_MAX) return fail(RS_EINVAL, "piece_gram: too many tiles");
+    k_piece_gram<BN><<<(unsigned)std::min(nsm, a.tiles * a.chunks), DG_NT, C::SMEM, st>>>(a);
+    RS_LAUNCH_CHECK();
     return RS_OK;
 }
 
@@ -1064,8 +1562,8 @@ int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int 
     a.yvec = aligned16(Y) && (ldy * (int64_t)sizeof(T)) % 16 == 0;
     constexpr int NS = sizeof(T) == 8 ? 8 : 5;
     const bool in_place = X == Y;
-    if (m <= 32) return launch_rot<T, NS, 32, 1>(a, 0, st);
-    if (in_place && m > 512) return launch_rot<T, NS, 64, 2>(a, 1, st);
+    if (m <= 32) return launch_rot<T, NS, 32, 1>(a, false, st);
+    if (in_place && m > 512) return launch_rot<T, NS, 64, 2>(a, true, st);
     return launch_rot<T, NS, 64, 1>(a, in_place, st);
 }
 template int digit_rot<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
@@ -1074,3 +1572,67 @@ template int digit_rot<float>(const float *, int64_t, int, const double *, int64
                               double, cudaStream_t);
 
 }  // namespace rs
+
+namespace rs {
+
+int64_t piece_rot_bytes(int n, int m) {
+    const int64_t BN = m <= 64 ? 64 : 128;
+    return (m + BN - 1) / BN * BN * ((n + DG_K - 1) / DG_K) * DG_K * 6;
+}
+
+int piece_gram(const float *X, int64_t ldx, int nx, const float *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
+               int64_t lds, cudaStream_t st) {
+    k_digit_init<<<(unsigned)std::min<int64_t>(256, ((int64_t)nx * ny + 255) / 256), 256, 0, st>>>(S, lds, nx, ny, nullptr, 0);
+    RS_LAUNCH_CHECK();
+    PieceGramArgs a{};
+    a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.lds = lds, a.nx = nx, a.ny = ny, a.S = S, a.dV = dV;
+    return ny <= 64 ? launch_piece_gram<64>(a, st) : launch_piece_gram<128>(a, st);
+}
+
+int piece_rot(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
+              double alpha, double beta, void *work, cudaStream_t st) {
+    PieceArgs a{};
+    a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
+    a.vec = aligned16(X) && ldx % 4 == 0;
+    a.yvec = aligned16(Y) && ldy % 4 == 0;
+    a.alpha = (float)alpha, a.beta = (float)beta;
+    if (m <= 64) return launch_piece<64>(a, C, ldc, work, X == Y, st);
+    return launch_piece<128>(a, C, ldc, work, X == Y, st);
+}
+
+}  // namespace rs
+
+// ---------------------------------------------------------------- C ABI ---
+
+using namespace rs;
+
+namespace {
+int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+}  // namespace
+
+extern "C" int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K) {
+    if (rows_a < 1 || rows_b < 1 || K < 1) return -1;
+    return 6 * (round_up(rows_a, 128) + round_up(rows_b, 128)) * round_up(K, 64) + 4352;
+}
+
+extern "C" int rs_overlap_block_tc(const rs_grid *g, const float *X_dev, int64_t ldx, int nx, const float *Y_dev,
+                                   int64_t ldy, int ny, double *S_dev, int64_t lds, void *work_dev, void *stream) {
+    if (!g || !X_dev || !Y_dev || !S_dev) return fail(RS_EINVAL, "rs_overlap_block_tc: null argument");
+    if (nx < 1 || ny < 1 || ldx < nx || ldy < ny || lds < ny) return fail(RS_EINVAL, "rs_overlap_block_tc: bad sizes");
+    if (!work_dev) return fail(RS_EINVAL, "tensor-core call: null workspace");
+    cudaStream_t st = (cudaStream_t)stream;
+    RS_TRY(piece_gram(X_dev, ldx, nx, Y_dev, ldy, ny, g->npts, g->h * g->h * g->h, S_dev, lds, st));
+    RS_CUDA(cudaStreamSynchronize(st));
+    return RS_OK;
+}
+
+extern "C" int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const double *C_dev, int64_t ldc, int m,
+                               float *Y_dev, int64_t ldy, int64_t npts, void *work_dev, void *stream) {
+    if (!X_dev || !C_dev || !Y_dev) return fail(RS_EINVAL, "rs_rotate_block: null argument");
+    if (n < 1 || m < 1 || npts < 1 || ldx < n || ldy < m || ldc < m) return fail(RS_EINVAL, "rs_rotate_block: bad sizes");
+    if (!work_dev) return fail(RS_EINVAL, "tensor-core call: null workspace");
+    cudaStream_t st = (cudaStream_t)stream;
+    RS_TRY(rotate_any(X_dev, ldx, n, C_dev, ldc, m, Y_dev, ldy, npts, 1.0, 0.0, work_dev, st));
+    RS_CUDA(cudaStreamSynchronize(st));
+    return RS_OK;
+}

@@ -12,13 +12,13 @@ namespace rs {
 inline int64_t digit_gram_scratch_ints(int nx, int ny) { return (int64_t)nx + ny; }
 
 // S (nx x ny, FP64, row stride lds) = dV X^T Y over npts points.  Accuracy:
-// the digits of an operand resolve 2^-62 (FP64), 2^-54 (FP32, exact = true)
-// or 2^-38 (FP32, exact = false) of its column's largest entry.
+// the digits of an operand resolve 2^-62 (FP64) or 2^-54 (FP32) of its
+// column's largest entry.
 // scratch: digit_gram_scratch_ints ints of device memory, or nullptr (taken
 // from the library's stream-ordered pool).  Asynchronous.
 template <typename T>
 int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, bool exact, int *scratch, cudaStream_t st);
+               int64_t lds, int *scratch, cudaStream_t st);
 
 // Y (m columns) = alpha X C + beta Y, X [npts][ldx] (n columns), C FP64
 // [n][ldc]; Y may be X itself (same pointer and leading dimension) when
@@ -27,5 +27,17 @@ bool digit_rot_takes(int n, int m, bool in_place);
 template <typename T>
 int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
               double alpha, double beta, cudaStream_t st);
+
+// S = dV X^T Y of FP32 data to FP32 accuracy by BF16 pieces, FP32 sums over at
+// most 2048 points.  Asynchronous.
+int piece_gram(const float *X, int64_t ldx, int nx, const float *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
+               int64_t lds, cudaStream_t st);
+
+// FP32 rotation to FP32 accuracy by BF16 pieces (Y may be X itself, same leading
+// dimension, for m <= 1024 and beta == 0).  work: piece_rot_bytes(n, m) bytes,
+// 16-byte aligned.  Asynchronous.
+int64_t piece_rot_bytes(int n, int m);
+int piece_rot(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
+              double alpha, double beta, void *work, cudaStream_t st);
 
 }  // namespace rs

@@ -28,7 +28,9 @@ namespace rs {
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
          int64_t lds, cudaStream_t st, bool fast, int *scratch) {
-    return digit_gram<T>(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, !fast, scratch, st);
+    if constexpr (sizeof(T) == 4)
+        if (fast) return piece_gram(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, st);
+    return digit_gram<T>(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, scratch, st);
 }
 template int gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
                           int64_t, cudaStream_t, bool, int *);
@@ -89,6 +91,27 @@ template int rowmul<double>(const double *, int64_t, int, const double *, int64_
                             double, double, cudaStream_t);
 template int rowmul<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
                            double, cudaStream_t);
+
+// FP32 rotation to FP32 accuracy for any placement of Y: where Y overlaps X and
+// cannot be written in place by one launch, X is copied first.
+int64_t rotate_work_bytes(int n, int m, int64_t copy_rows) { return piece_rot_bytes(n, m) + copy_rows * n * (int64_t)sizeof(float); }
+
+int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
+               double alpha, double beta, void *work, cudaStream_t st) {
+    const bool apart = X + (npts - 1) * ldx + n <= Y || Y + (npts - 1) * ldy + m <= X;
+    const bool inplace = X == Y && ldx == ldy && beta == 0.0 && m <= 1024;
+    // column slices of one array, side by side
+    const int64_t off = X > Y ? (X - Y) % ldx : (Y - X) % ldx;
+    const bool beside = ldx == ldy && off >= (X > Y ? m : n) && off + (X > Y ? n : m) <= ldx;
+    if (!apart && !inplace && !beside) {
+        float *copy = reinterpret_cast<float *>((char *)work + piece_rot_bytes(n, m));
+        RS_CUDA(cudaMemcpy2DAsync(copy, sizeof(float) * n, X, sizeof(float) * ldx, sizeof(float) * n, (size_t)npts,
+                                  cudaMemcpyDeviceToDevice, st));
+        X = copy;
+        ldx = n;
+    }
+    return piece_rot(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, work, st);
+}
 
 // ----------------------------------------------------- small dense FP64 ---
 

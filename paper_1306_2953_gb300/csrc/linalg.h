@@ -10,17 +10,24 @@
 namespace rs {
 
 // S = dV X^T Y (nx x ny, FP64, row stride lds); X, Y are [npts][ld] of T.
-// FP32 data: exact products with compensated accumulation, or (fast) plain
-// FP32 accumulation within chunks of points combined in FP64.
+// FP32 data: accurate like FP64, or (fast) to FP32 level; scratch: nx + ny ints or
+// nullptr (see digits.h).
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
          int64_t lds, cudaStream_t st, bool fast = false, int *scratch = nullptr);
 
-// Y = alpha X C + beta Y row by row; X [npts][ldx] (n columns), C FP64 [n][ldc]
+// Y = alpha X C + beta Y; X [npts][ldx] (n columns), C FP64 [n][ldc]
 // (m columns), Y [npts][ldy]; Y may alias X when beta == 0.
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
            double alpha, double beta, cudaStream_t st);
+
+// FP32 rotation to FP32 accuracy for any placement of Y relative to X.  work:
+// rotate_work_bytes(n, m, npts) bytes; copy_rows = 0 serves when Y is apart from
+// X, beside it in the same array, or X itself with m <= 1024.
+int64_t rotate_work_bytes(int n, int m, int64_t copy_rows);
+int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
+               double alpha, double beta, void *work, cudaStream_t st);
 
 // out[k] = sum_p A[p][k] B[p][k] (FP64, exact products, compensated sum), k < ncols <= 256.
 int coldots(int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, int ncols, int64_t npts, double *out,
@@ -68,20 +75,18 @@ struct LaWork {
     static size_t bytes(int n) { return sizeof(double) * ((size_t)4 * n * n + n + 8) + eigh_work_bytes(n) + 256; }
 };
 
-// Tensor-core workspace for FP32 contractions (optional): base pointer,
-// its size, and a device status word set when a tensor-core wait times out.
+// How the eigensolver calls the steps of Sec. VI.
 struct TcWork {
+    // workspace of rotate_any for FP32 rotations to FP32 accuracy; nullptr: the
+    // digits' FP64-like sums, rounded once
     void *p = nullptr;
-    int64_t bytes = 0;
-    int *err = nullptr;
-    // inner iterations of the FP32 eigensolver: the full overlaps of Sec. VI
-    // on the tensor cores as well, and the subspace eigenvectors from FP32
-    // Jacobi alone (the closing FP64 Rayleigh-Ritz fixes the final accuracy)
+    // inner iterations of the FP32 eigensolver: overlaps at FP32 accuracy, and the
+    // subspace eigenvectors from FP32 Jacobi alone (the closing FP64
+    // Rayleigh-Ritz fixes the final accuracy)
     bool inner = false;
 };
 
-// Psi (n columns) <- Psi C in place (C FP64 n x n); FP32 data on the tensor
-// cores when tc.p is set and large enough.
+// Psi (n columns) <- Psi C in place (C FP64 n x n).
 int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, cudaStream_t st,
                    const TcWork &tc = TcWork());
 // Psi <- Psi U^-1 with <Psi|Psi> = U^T U; w.Ui keeps U^-1.  Blocking; RS_ENOTSPD on failure.

@@ -32,7 +32,6 @@
 #include "linalg.h"
 #include "precond.h"
 #include "solver_view.h"
-#include "umma.h"
 
 using namespace rs;
 
@@ -445,9 +444,8 @@ struct rs_solver {
     double dV = 0;
     int es = 8;
     int nblk = 0;
-    DevBuf psi, hpsi, P, Z, HZ, R, small, la, eig, res, tcbuf, psi64, hpsi64, rr64, gs_tbuf, gs_nbuf;
+    DevBuf psi, hpsi, P, Z, HZ, R, small, la, eig, res, tcbuf, psi64, hpsi64, rr64;
     TcWork tc;
-    UmmaSplitCache gs_t, gs_n;   // FP32 mode: splits of Psi[:, :(b+1) nb] within a block step
     std::vector<char> has_p;
     Precond *pc = nullptr;
     // learned preconditioner: the FP32 weights last set or trained
@@ -488,27 +486,20 @@ int copy_cols(int dtype, const void *S, int64_t lds, void *D, int64_t ldd, int n
     return RS_OK;
 }
 
-// inner-iteration contractions: FP32 mode on the tensor cores (FP32-level
-// accuracy), FP64 mode on the FP64 pipes
+// inner-iteration contractions: FP32 mode to FP32-level accuracy
 int gram_any(int dtype, const void *X, int64_t ldx, int nx, const void *Y, int64_t ldy, int ny, int64_t npts, double dV,
-             double *S, int64_t lds, cudaStream_t st, const TcWork &tc, UmmaSplitCache *xcache = nullptr) {
+             double *S, int64_t lds, cudaStream_t st) {
     if (dtype == RS_F64)
         return gram<double>((const double *)X, ldx, nx, (const double *)Y, ldy, ny, npts, dV, S, lds, st);
-    if (tc.p && tc.bytes >= umma_work_bytes(nx, ny, npts))
-        return umma_gram((const float *)X, ldx, nx, (const float *)Y, ldy, ny, npts, dV, S, lds, tc.p, tc.err, st,
-                         xcache);
     return gram<float>((const float *)X, ldx, nx, (const float *)Y, ldy, ny, npts, dV, S, lds, st, true);
 }
 
+// (X and Y are different arrays, or column slices of one)
 int rowmul_any(int dtype, const void *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, void *Y, int64_t ldy,
-               int64_t npts, double alpha, double beta, cudaStream_t st, const TcWork &tc,
-               UmmaSplitCache *xcache = nullptr) {
+               int64_t npts, double alpha, double beta, cudaStream_t st, const TcWork &tc) {
     if (dtype == RS_F64)
         return rowmul<double>((const double *)X, ldx, n, C, ldc, m, (double *)Y, ldy, npts, alpha, beta, st);
-    if (tc.p && tc.bytes >= umma_work_bytes(npts, m, n))
-        return umma_rowmul((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, tc.p, tc.err, st,
-                           xcache);
-    return rowmul<float>((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, st);
+    return rotate_any((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, tc.p, st);
 }
 
 const char *off(const DevBuf &b, int64_t elems, int es) { return (const char *)b.p + (size_t)elems * es; }
@@ -563,13 +554,10 @@ int block_step(rs_solver *S, int b, cudaStream_t st) {
     void *Y = offw(S->Z, nb, es);
 
     // 3. classical Gram-Schmidt, twice, against Psi[:, :(b+1) nb]
-    // (Psi does not change between the passes: its two BF16x3 splits, one per
-    // contraction layout, are made in the first pass and reused in the second)
     const int nq = (b + 1) * nb;
-    S->gs_t.valid = S->gs_n.valid = false;
     for (int pass = 0; pass < 2; ++pass) {
-        RS_TRY(gram_any(dt, S->psi.p, nst, nq, Y, ldz, ny, np, S->dV, S->M, ny, st, S->tc, &S->gs_t));
-        RS_TRY(rowmul_any(dt, S->psi.p, nst, nq, S->M, ny, ny, Y, ldz, np, -1.0, 1.0, st, S->tc, &S->gs_n));
+        RS_TRY(gram_any(dt, S->psi.p, nst, nq, Y, ldz, ny, np, S->dV, S->M, ny, st));
+        RS_TRY(rowmul_any(dt, S->psi.p, nst, nq, S->M, ny, ny, Y, ldz, np, -1.0, 1.0, st, S->tc));
     }
     RS_TRY(coldots(dt, Y, ldz, Y, ldz, ny, np, nrm, st));
     if (dt == RS_F64)
@@ -584,8 +572,8 @@ int block_step(rs_solver *S, int b, cudaStream_t st) {
 
     // 5. Rayleigh-Ritz on Z = [X, Y]
     int n = nb + ny;
-    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->Z.p, ldz, n, np, S->dV, S->G, n, st, S->tc));
-    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->HZ.p, ldz, n, np, S->dV, S->A, n, st, S->tc));
+    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->Z.p, ldz, n, np, S->dV, S->G, n, st));
+    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->HZ.p, ldz, n, np, S->dV, S->A, n, st));
     RS_TRY(symmetrize(S->G, n, n, st));
     RS_TRY(symmetrize(S->A, n, n, st));
     int bad = 1;
@@ -1039,20 +1027,11 @@ extern "C" int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void 
                 (rc = S->rmm_small.alloc(sizeof(double) * 64 * (MD_MAX + 2 * RMM_MAXK * RMM_MAXK + RMM_MAXK + 2)))))
         return bail(rc);
     if (c.dtype == RS_F32) {
-        const int64_t need = std::max({umma_work_bytes(c.nst, 2 * c.nb, S->npts), umma_work_bytes(S->npts, c.nst, c.nst),
-                                       umma_work_bytes(3 * c.nb, 3 * c.nb, S->npts),
-                                       umma_work_bytes(c.nst, c.nst, S->npts)});
-        if ((rc = S->tcbuf.alloc((size_t)need + 256))) return bail(rc);
-        // the Gram-Schmidt splits of Psi, one per contraction layout
-        if ((rc = S->gs_tbuf.alloc((size_t)umma_split_cache_bytes(true, S->npts, c.nst)))) return bail(rc);
-        if ((rc = S->gs_nbuf.alloc((size_t)umma_split_cache_bytes(false, S->npts, c.nst)))) return bail(rc);
-        S->gs_t.buf = S->gs_tbuf.p;
-        S->gs_n.buf = S->gs_nbuf.p;
+        const int64_t need = std::max({rotate_work_bytes(c.nst, c.nst, c.nst > 1024 ? S->npts : 0), rotate_work_bytes(c.nst, 2 * c.nb, 0),
+                                       rotate_work_bytes(3 * c.nb, c.nb, 0)});
+        if ((rc = S->tcbuf.alloc((size_t)need))) return bail(rc);
         S->tc.p = S->tcbuf.p;
-        S->tc.bytes = need;
-        S->tc.err = reinterpret_cast<int *>((char *)S->tcbuf.p + need);
         S->tc.inner = true;
-        if (cudaMemset(S->tc.err, 0, sizeof(int)) != cudaSuccess) return bail(fail(RS_ECUDA, "cudaMemset failed"));
     }
     const int n3 = 3 * c.nb;
     const size_t smallbytes = sizeof(double) * (512 + (size_t)c.nst * 2 * c.nb + 7 * (size_t)n3 * n3 + n3 + (size_t)n3 * c.nb) +
@@ -1104,13 +1083,11 @@ extern "C" int rs_eigensolver_step(rs_solver *S, double *eps_dev, double *resnor
     if (resnorm_dev) RS_CUDA(cudaMemcpyAsync(resnorm_dev, S->res.p, sizeof(double) * c.nst, cudaMemcpyDeviceToDevice, st));
     std::vector<double> res(c.nst);
     RS_CUDA(cudaMemcpyAsync(res.data(), S->res.p, sizeof(double) * c.nst, cudaMemcpyDeviceToHost, st));
-    // status words of the bounded device waits: the tensor-core pipeline and
-    // the H psi ring (a wait that gave up leaves that launch's result incomplete)
-    int tcerr = 0, ringerr = 0;
-    if (S->tc.err) RS_CUDA(cudaMemcpyAsync(&tcerr, S->tc.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    // status word of the H psi ring's bounded waits (one that gave up leaves that
+    // launch's result incomplete; the contractions write NaN, found in the residuals)
+    int ringerr = 0;
     if (int *rw = ham_status_word(S->h)) RS_CUDA(cudaMemcpyAsync(&ringerr, rw, sizeof(int), cudaMemcpyDeviceToHost, st));
     RS_CUDA(cudaStreamSynchronize(st));
-    if (tcerr) return fail(RS_ETIMEOUT, "eigensolver: a tensor-core pipeline wait timed out");
     if (ringerr) return fail(RS_ETIMEOUT, "eigensolver: an H psi pipeline wait timed out");
     ++S->sweeps;
     const int nw = c.n_wanted > 0 ? c.n_wanted : c.nst;

@@ -8,7 +8,6 @@
 #include "device.h"
 #include "ham.h"
 #include "linalg.h"
-#include "umma.h"
 
 using namespace rs;
 
@@ -47,17 +46,10 @@ extern "C" int64_t rs_linalg_workspace_bytes(int nst) {
 
 namespace rs {
 
-namespace {
-bool tc_grams(const TcWork &tc, int n, int64_t npts) {
-    return tc.inner && tc.p && tc.bytes >= umma_work_bytes(n, n, npts);
-}
-}  // namespace
-
 int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, cudaStream_t st,
                    const TcWork &tc) {
     if (dtype == RS_F64) return rowmul<double>((const double *)Psi, ld, n, C, n, n, (double *)Psi, ld, npts, 1.0, 0.0, st);
-    if (tc.p && tc.bytes >= umma_work_bytes(npts, n, n))
-        return umma_rowmul((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, tc.p, tc.err, st);
+    if (tc.p) return rotate_any((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, tc.p, st);
     return rowmul<float>((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, st);
 }
 
@@ -68,10 +60,8 @@ int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, i
     int *keys = reinterpret_cast<int *>(w.xi);   // not in use yet: scratch of the overlap
     if (dtype == RS_F64)
         RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st, false, keys));
-    else if (tc_grams(tc, n, npts))
-        RS_TRY(umma_gram((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, tc.p, tc.err, st));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st, false, keys));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st, tc.inner, keys));
     RS_TRY(symmetrize(w.U, n, n, st));
     RS_TRY(cholesky(w.U, n, n, 1e-14, w.status, st));
     int bad = 0;
@@ -95,10 +85,8 @@ int subspace_diag_impl(rs_ham *h, void *Psi, void *HPsi, int64_t ld, int n, int 
     int *keys = reinterpret_cast<int *>(w.xi);
     if (dtype == RS_F64)
         RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys));
-    else if (tc_grams(tc, n, npts))
-        RS_TRY(umma_gram((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, tc.p, tc.err, st));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, tc.inner, keys));
     RS_TRY(symmetrize(w.S, n, n, st));
     RS_TRY(eigh(w.S, n, n, eps_dev, w.xi, n, dtype == RS_F32 && tc.inner ? -1 : 2, w.status, w.eigw, st));
     RS_TRY(rotate_inplace(Psi, ld, n, w.xi, npts, dtype, st, tc));

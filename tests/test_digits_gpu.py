@@ -88,3 +88,51 @@ def test_values_beyond_the_digits(dtype):
     err = np.abs(P.double().cpu().numpy() - ref)
     u = 2.0 ** -52 if dtype == "f64" else 2.0 ** -23
     assert np.all(err <= 64 * u * (np.abs(x) @ np.abs(C)))
+
+
+@pytest.mark.parametrize("npts,n,m,where", [(1, 1, 1, "out"), (127, 31, 64, "out"), (129, 33, 65, "out"), (300, 40, 40, "in"),
+                                            (260, 64, 130, "in"), (515, 256, 256, "in"), (200, 130, 300, "wide"),
+                                            (200, 64, 64, "beside"), (300, 96, 96, "shifted"), (140, 20, 1100, "in")])
+def test_piece_rotation_edges(npts, n, m, where):
+    """rs_rotate_block out of place, in place (m up to and above the cluster's
+    1024 columns), beside X in one array, and partly over X.  Tolerance: six of
+    nine piece products (the rest below 3 * 2^-24), C rounded to FP32, and at
+    most n / 16 + 6 FP32 accumulations."""
+    import ctypes
+    from paper_1306_2953_gb300 import _lib, api
+    rng = np.random.default_rng(n + m)
+    ld = {"out": n + 3, "in": max(n, m) + 1, "wide": max(n, m), "beside": n + m, "shifted": n + m}[where]
+    buf = torch.from_numpy(rng.uniform(-1, 1, (npts, ld)).astype(np.float32)).cuda()
+    x = buf[:, :n].double().cpu().numpy()
+    C = torch.from_numpy(rng.standard_normal((n, m))).cuda()
+    if where == "out":
+        Y = torch.full((npts, m + 1), 7.0, device="cuda")[:, :m]
+    elif where in ("in", "wide"):
+        Y = buf[:, :m]
+    elif where == "beside":
+        Y = buf[:, n:]
+    else:
+        Y = buf[:, 5:5 + m]
+    work = api.tc_workspace(npts, m, n)
+    _lib.call("rs_rotate_block", ctypes.c_void_p(buf.data_ptr()), buf.stride(0), n, ctypes.c_void_p(C.data_ptr()), m, m,
+              ctypes.c_void_p(Y.data_ptr()), Y.stride(0), npts, ctypes.c_void_p(work.data_ptr()), api._stream())
+    c = C.cpu().numpy()
+    ref, mag = x @ c, np.abs(x) @ np.abs(c)
+    u = 2.0 ** -24
+    assert np.all(np.abs(Y.double().cpu().numpy() - ref) <= (2 * (n / 16 + 6) + 4) * u * mag)
+
+
+@pytest.mark.parametrize("box", [(5, 3, 2), (8, 8, 4), (41, 40, 17)])
+@pytest.mark.parametrize("nx,ny,pad", [(1, 1, 0), (127, 31, 1), (128, 64, 0), (129, 65, 3), (257, 130, 0)])
+def test_piece_overlap_edges(box, nx, ny, pad):
+    """rs_overlap_block_tc.  Tolerance: six of nine piece products (the rest
+    below 3 * 2^-24), one FP32 accumulation (2^-23 where truncated) per product
+    and 16 of at most 2048 points."""
+    from paper_1306_2953_gb300 import api
+    g = api.Grid.box(*box, 0.3)
+    X, Y = _block(g.npts, nx, 4, torch.float32, pad), _block(g.npts, ny, 5, torch.float32, pad)
+    for A, B in ((X, Y), (X, X)):
+        S = api.overlap_tc(g, A, B).cpu().numpy()
+        a, b = A.double().cpu().numpy(), B.double().cpu().numpy()
+        steps = 6 * (min(g.npts, 2048) // 16 + 4)
+        assert np.all(np.abs(S - g.dV * (a.T @ b)) <= g.dV * (2 * steps + 4) * 2.0 ** -24 * (np.abs(a).T @ np.abs(b)))
