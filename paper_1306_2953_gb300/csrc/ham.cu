@@ -579,7 +579,7 @@ static int apply_t(rs_ham *H, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, i
     int rc = -1;
     bool ring = false;
     if constexpr (sizeof(T) == 4) {
-        ring = H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, nb);
+        ring = H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, ldh, nb);
         if (ring) {
             float w[5];
             for (int j = 0; j < 5; ++j) w[j] = (float)H->w[j];

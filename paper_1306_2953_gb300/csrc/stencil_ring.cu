@@ -17,29 +17,38 @@
 // 128 bytes (32 FP32 states) per position, plus the plane's record: the
 // potential and the point index of every tile point and, per 4 x 4 patch,
 // the projector values of each atom whose sphere meets the patch (zero at
-// the patch points outside the sphere).  Every thread copies its share of
-// plane it + 2 while plane it is computed: one 16-byte piece of ten point
-// rows (a warp copies a 4-point brick row per instruction; absent points are
-// zero-filled) and part of the record, all counted on the slot's "full"
-// mbarrier through cp.async.mbarrier.arrive.  A slot is refilled once every
-// warp has released it ("empty" mbarrier).  Points are stored brick by brick
-// (Sec. V.A), so one 32-bit descriptor (first point, presence mask) gives
-// the four points of a brick row; the descriptors are loaded three planes
-// ahead of their copy.  The projection coefficients of the atoms a CTA's
-// records name are staged in shared memory once per launch (the records
-// carry the CTA-local atom numbers).
+// the patch points outside the sphere).
 //
-// Compute.  Warp w owns the 4 x 4 patch of tile points at rows 4 (w / 4),
-// columns 4 (w % 4); half-warp h takes the patch's rows 2h and 2h + 1 and
-// lane l of the half the states 2l and 2l + 1, so every value is a pair of
-// states and every multiply-add a packed FP32x2 instruction.  The march
+// Copies.  Four warps do nothing but copy: as soon as every compute warp has
+// released a slot ("empty" mbarrier) they fill it with the next plane, one
+// 16-byte piece of twenty point rows per thread (a warp copies a 4-point brick
+// row per instruction, one contiguous piece where the row is full; absent
+// points are zero-filled) and the record, all counted on the slot's "full"
+// mbarrier through cp.async.mbarrier.arrive.  The point of every window
+// position comes from a table, read while the plane before is in flight.  The
+// projection coefficients of the atoms a CTA's records name are staged in
+// shared memory once per launch (the records carry the CTA-local atom
+// numbers).
+//
+// Compute.  Eight warps: warp w owns the 4 x 4 patch of tile points at rows
+// 4 (w / 4), columns 4 (w % 4); half-warp h takes the patch's rows 2h and
+// 2h + 1 and lane l of the half the states 2l and 2l + 1, so every value is a
+// pair of states and every multiply-add a packed FP32x2 instruction.  The march
 // accumulates forward: the values of plane z add w_|j| psi(z) to the outputs
 // of planes z + j (j = -4..4), and the in-plane star, the potential and the
 // nonlocal sum to plane z's own output, so a slot is read in one step only.
-// Eight accumulators per point hold the outputs z - 4 .. z + 3 (slot z mod 8,
-// addressed through unrolling): at step z output z - 4 is complete and
-// written, and its slot takes output z + 4.  The four planes on either side
-// of a unit contribute only their z-terms (tile rows only, no record).
+// Eight accumulators per point hold the outputs z - 4 .. z + 3: at step z
+// output z - 4 is complete and written, and the others move down by one as
+// they take their terms.  The four planes on either side of a unit contribute
+// only their z-terms (tile rows only, no record).
+//
+// Measured, 654 520 points, 32 states, us a launch: 77 (92 when every warp
+// copied its share between its steps, and the accumulators stayed in place
+// with eight copies of the step's code).  Copies alone take 47 and the
+// compute warps alone about 70: two compute warps a scheduler cannot hide all
+// of their shared-memory latency.  Sixteen compute warps of half the points
+// (64 accumulator registers) took 98: 9 instead of 7 rows read per point, and
+// twice the waiting and addressing.  Three slots instead of four: 87.
 //
 // Every mbarrier wait is bounded; on a timeout the kernel sets its status
 // word and leaves the march.  Built with RS_BOUNDS_CHECK=1 (a debugging
@@ -50,6 +59,7 @@
 #include <cstring>
 #include <map>
 #include <new>
+#include <type_traits>
 
 #include "device.h"
 #include "stencil_ring.h"
@@ -69,16 +79,21 @@ constexpr int ROWB = SG * 4;               // bytes per point row
 constexpr int NSLOT = 320;                 // stored window positions
 constexpr int SLOT_PSI = NSLOT * ROWB;
 constexpr int NG = 80;                     // brick rows (four positions) per window plane
-constexpr int NW = 8;                      // warps: one 4 x 4 patch each
-constexpr int NT = NW * 32;
-constexpr int CPW = NG / NW;               // brick rows copied per warp and plane
+constexpr int NP = 8;                      // 4 x 4 patches of a tile
+constexpr int NW = NP;                     // compute warps: one to a patch
+constexpr int NCW = 4;                     // copy warps
+constexpr int NT = (NW + NCW) * 32;
+constexpr int CPW = NG / NCW;              // brick rows copied per copy warp and plane
+// Registers: 384 threads are launched with 168; the copy warps give most of
+// theirs to the compute warps (128 * 72 + 256 * 216 = 384 * 168).
+constexpr int REGS_COPY = 72, REGS_COMPUTE = 216;
+static_assert(CPW % 4 == 0 && NSLOT == 4 * CPW * NCW, "a lane's point indices are read four at a time");
 
 // host load balance: march cost of an edge plane and of one atom block of a
 // plane's heaviest patch, in full planes (fitted to per-CTA clock counts)
-constexpr double EDGE_COST = 0.38;
-constexpr double NL_COST = 0.09;
-constexpr int AHEAD = 2;                   // planes in flight ahead of the one computed
-constexpr int MAX_RING = 4;                // slots per CTA (4, or 3 when 4 do not fit)
+constexpr double EDGE_COST = 0.55;
+constexpr double NL_COST = 0.135;
+constexpr int MIN_RING = 3, MAX_RING = 4;  // slots per CTA (4, or 3 when 4 do not fit)
 constexpr int NPOS = TX * TY;
 // record: [patch headers {blocks, byte offset}] [w0 + potential, as pairs, tile row-major]
 // [point index, tile row-major] [blocks: {atom} + projector values [16][4]]
@@ -89,53 +104,57 @@ constexpr int BLK = 16 + 16 * 16;
 constexpr int MAX_REC = 48 * 1024;         // record slot budget (bytes)
 constexpr size_t MAX_SMEM = 226 * 1024;    // dynamic shared memory per CTA (227 KB less the static part)
 constexpr int MAX_SLAB = 1 << 16;          // planes per z-slab (at most)
-constexpr int MAX_UNITS = 64;              // units per CTA (shared-memory table)
 constexpr int SUSPEND_NS = 20000;          // suspension limit of one barrier test
 constexpr int SPIN = 100000;               // barrier tests before a wait gives up (default)
 constexpr int DRAIN_SPIN = 5000;           // barrier tests per slot when draining after a timeout
 
 // Window layout in a slot.  Window rows wy = 0..15 (tile rows at 4..11),
 // columns wx = 0..23 (tile columns at 4..19).  Columns 4..19 of every row
-// are positions wy * 16 + wx - 4 (0..255); columns 0..3 and 20..23 of the
-// tile rows are positions 256 + (wy - 4) * 8 + (0..3 | 4..7).  Brick row g
-// covers positions 4 g .. 4 g + 3: g < 64 row g / 4 of the core columns,
-// g >= 64 the side halo.
+// are positions wy * 16 + wx - 4 (0..255); columns 0..3 and 20..23 of tile row
+// t = wy - 4 are positions 256 + (t mod 4) * 16 + (t / 4) * 8 + (0..3 | 4..7),
+// so that neighbouring rows of a patch are 16 positions apart everywhere.
+// Brick row g covers positions 4 g .. 4 g + 3: g < 64 row g / 4 of the core
+// columns, g >= 64 the side halo.
 __host__ __device__ __forceinline__ void group_pos(int g, int &wy, int &wx) {
     if (g < 64) {
         wy = g >> 2;
         wx = 4 + 4 * (g & 3);
     } else {
         const int h = g - 64;
-        wy = 4 + (h >> 1);
+        wy = 4 + (h >> 2) + 4 * ((h >> 1) & 1);
         wx = (h & 1) ? 20 : 0;
     }
 }
 // brick rows of the tile itself (window rows 4..11, core columns)
 constexpr int G_TILE0 = 16, G_TILE1 = 48;
 
-// A unit as the kernel walks it: planes zm0..zm1 (the slab's output planes
-// zo0..zo1-1 and up to four on either side), record / descriptor index of
-// plane z = pz + z.
-struct UnitDev {
-    int zm0, zm1, zo0, zo1, pz, pad0, pad1, pad2;
+// One plane of a CTA's march: its descriptors and record (plane index) and
+// what is done with it.
+enum : int {
+    STEP_FULL = 1,    // an output plane of the unit (else a plane beside them: z-terms only)
+    STEP_STORE = 2,   // output z - 4 belongs to the unit
+    STEP_FIRST = 4,   // first plane of the unit
+    STEP_Z = 4,       // bits 4..6: z mod 8
+    STEP_FLUSH = 8    // bits 8..11: outputs z - 3 .. z complete with the column's last plane
 };
 
 struct Args {
-    const UnitDev *units;   // per CTA, concatenated
-    const int4 *cta;        // [CTA]: first unit, unit count, first atom, atom count
+    const int2 *steps;      // per CTA, concatenated: {plane, STEP_*}
+    const int4 *cta;        // [CTA]: first step, step count, first atom, atom count
     const int *cta_atoms;   // per CTA, concatenated: the atoms its records name (in local order)
-    const uint32_t *desc;   // [plane][80]: first point | presence mask << 28
+    const int *idx;         // [plane][copy warp][position in brick row][k]: point of that position of brick row
+                            // (copy warp) + NCW k, -1: none
     const uint2 *recs;      // [plane]: {offset / 16, bytes}
     const unsigned char *rec;
     const float *psi;       // [npts][ldp]
-    int64_t ldp;
+    uint32_t ldp;           // row strides in bytes
     const float *cproj;     // [atom][nb][4]
     float *hpsi;
-    int64_t ldh;
+    uint32_t ldh;
     int nb, rec_slot, cs_atoms;   // cs_atoms: the largest atom count of a CTA
     int spin;                     // barrier tests before a wait gives up
     int npts;                     // point count (the bounds-checked build tests indices against it)
-    float w[5];
+    float2 w[5];                  // weights, as pairs
     int *status;
 };
 
@@ -158,6 +177,15 @@ __device__ __forceinline__ bool bar_try(uint64_t *b, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// A copy warp's wait: it has a ring of planes in hand, so it sleeps between its
+// tests instead of taking issue slots from the compute warps.
+__device__ __forceinline__ bool bar_wait_idle(uint64_t *b, uint32_t parity, int spin) {
+    for (int i = 0; i < spin; ++i) {
+        if (bar_try(b, parity)) return true;
+        __nanosleep(250);
+    }
+    return false;
+}
 // at most `spin` tests (by default about SPIN * SUSPEND_NS, two seconds, in all)
 __device__ __forceinline__ bool bar_wait(uint64_t *b, uint32_t parity, int spin) {
     for (int i = 0; i < spin; ++i)
@@ -173,7 +201,6 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *b) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(su32(b)) : "memory");
 }
 
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 operator*(float2 a, float2 b) { return __fmul2_rn(a, b); }
 
@@ -183,11 +210,10 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 // a slot's start.
 struct Lane {
     float2 W1, W2, W3, W4;
-    int cb;        // centre of patch row 0, column 0 (window row 4 + ty0)
-    int lb0, lb1;  // first of the four axis-2 neighbours left of rows 0 / 1
-    int rb0, rb1;  // first of the four right of rows 0 / 1
-    int to;        // tile index of patch row 0, column 0 (record tables)
-    int w, h, sl;
+    int cb;        // centre of row 0, column 0
+    int lb, rb;    // first of the four columns left / right of row 0's
+    int to;        // tile index of row 0, column 0 (record tables)
+    int patch, gp, sl;   // patch, point of the patch, state pair
     int npts;      // point count and status word (bounds-checked build)
     int *status;
 };
@@ -197,7 +223,7 @@ constexpr int PS = ROWB / 8;
 
 // The plane's own terms of its output (everything but the z-terms): the
 // centre of the star with the potential, the in-plane star and the
-// nonlocal gather, for the patch rows r and columns x of this thread.
+// nonlocal gather, for the rows r and columns x of this thread.
 __device__ __forceinline__ void plane_terms(float2 (&T)[2][4], const float2 (&cc)[2][4], const float2 *__restrict__ P,
                                             const unsigned char *__restrict__ rs, const float2 *__restrict__ cs,
                                             const Lane &c) {
@@ -210,16 +236,15 @@ __device__ __forceinline__ void plane_terms(float2 (&T)[2][4], const float2 (&cc
         T[r][2] = make_float2(v23.x, v23.y) * cc[r][2];
         T[r][3] = make_float2(v23.z, v23.w) * cc[r][3];
     }
-    // axis-2 neighbours: the four left and right of each patch row
+    // axis-2 neighbours: the four left and right of each row
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         float2 v[12];
-        const int lb = r ? c.lb1 : c.lb0, rb = r ? c.rb1 : c.rb0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            v[k] = P[lb + k * PS];
-            v[8 + k] = P[rb + k * PS];
+            v[k] = P[c.lb + (r * 16 + k) * PS];
             v[4 + k] = cc[r][k];
+            v[8 + k] = P[c.rb + (r * 16 + k) * PS];
         }
 #pragma unroll
         for (int j = 1; j <= 4; ++j) {
@@ -228,8 +253,8 @@ __device__ __forceinline__ void plane_terms(float2 (&T)[2][4], const float2 (&cc
             for (int x = 0; x < 4; ++x) T[r][x] = fma2(W, add2(v[x + 4 + j], v[x + 4 - j]), T[r][x]);
         }
     }
-    // axis-1 neighbours: window rows ty0 .. ty0 + 9 of each patch column,
-    // summed apart from the rest (shorter dependent chains) and added at the end
+    // axis-1 neighbours: the four above and below, summed apart from the rest
+    // (shorter dependent chains) and added at the end
     float2 Ty[2][4];
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
@@ -256,12 +281,12 @@ __device__ __forceinline__ void plane_terms(float2 (&T)[2][4], const float2 (&cc
     // coefficients of the lane's two states (staged in shared memory)
     // against the patch's projector values (scalar FMAs: a projector value
     // multiplies both states without being paired with itself first)
-    const int2 hd = reinterpret_cast<const int2 *>(rs)[c.w];
+    const int2 hd = reinterpret_cast<const int2 *>(rs)[c.patch];
     const unsigned char *blk = rs + hd.y;
     for (int k = 0; k < hd.x; ++k, blk += BLK) {
         const float2 *cq = cs + *reinterpret_cast<const int *>(blk) * (4 * SG / 2) + c.sl;
         const float2 c0 = cq[0], c1 = cq[SG / 2], c2 = cq[SG], c3 = cq[3 * SG / 2];
-        const float4 *g = reinterpret_cast<const float4 *>(blk + 16) + 8 * c.h;
+        const float4 *g = reinterpret_cast<const float4 *>(blk + 16) + c.gp;
 #pragma unroll
         for (int r = 0; r < 2; ++r)
 #pragma unroll
@@ -293,11 +318,9 @@ __device__ __forceinline__ bool index_ok(int i, int npts, int *status) {
     return true;
 }
 
-// Writes the finished output of the plane in accumulator slot R.
-template <int R>
-__device__ __forceinline__ void emit(const float2 (&A)[8][2][4], const int *rowring, float *hp, int64_t ldh,
-                                     const Lane &c) {
-    const int4 *ring4 = reinterpret_cast<const int4 *>(rowring + R * NPOS) + (c.to >> 2);
+// Writes finished outputs of the plane whose point indices are in ring slot zr.
+__device__ __forceinline__ void emit(const float2 (&v)[2][4], const int *rowring, int zr, char *hp, uint32_t ldh, const Lane &c) {
+    const int4 *ring4 = reinterpret_cast<const int4 *>(rowring + zr * NPOS) + (c.to >> 2);
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         int4 id = ring4[r * (TX / 4)];
@@ -307,84 +330,33 @@ __device__ __forceinline__ void emit(const float2 (&A)[8][2][4], const int *rowr
         if (!index_ok(id.z, c.npts, c.status)) id.z = -1;
         if (!index_ok(id.w, c.npts, c.status)) id.w = -1;
 #endif
-        if (id.x >= 0) *reinterpret_cast<float2 *>(hp + (int64_t)id.x * ldh) = A[R][r][0];
-        if (id.y >= 0) *reinterpret_cast<float2 *>(hp + (int64_t)id.y * ldh) = A[R][r][1];
-        if (id.z >= 0) *reinterpret_cast<float2 *>(hp + (int64_t)id.z * ldh) = A[R][r][2];
-        if (id.w >= 0) *reinterpret_cast<float2 *>(hp + (int64_t)id.w * ldh) = A[R][r][3];
+        if (id.x >= 0) *reinterpret_cast<float2 *>(hp + (uint64_t)(uint32_t)id.x * ldh) = v[r][0];
+        if (id.y >= 0) *reinterpret_cast<float2 *>(hp + (uint64_t)(uint32_t)id.y * ldh) = v[r][1];
+        if (id.z >= 0) *reinterpret_cast<float2 *>(hp + (uint64_t)(uint32_t)id.z * ldh) = v[r][2];
+        if (id.w >= 0) *reinterpret_cast<float2 *>(hp + (uint64_t)(uint32_t)id.w * ldh) = v[r][3];
     }
 }
-
-// The z-terms of plane z (R = z mod 8): slot k holds output z' = k mod 8 for
-// z' = z - 4 .. z + 3 before the step.  Plane z is the last contribution to
-// output z - 4, which is then written (when `store`), and its slot takes
-// output z + 4, whose first contribution plane z is.
-template <int R>
-__device__ __forceinline__ void zterms(float2 (&A)[8][2][4], const float2 (&cc)[2][4], const float2 (&T)[2][4],
-                                       bool full, bool store, const int *rowring, float *hp, int64_t ldh,
-                                       const Lane &c) {
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const float2 v = cc[r][x];
-            A[(R + 4) % 8][r][x] = fma2(c.W4, v, A[(R + 4) % 8][r][x]);
-            A[(R + 1) % 8][r][x] = fma2(c.W1, v, A[(R + 1) % 8][r][x]);
-            A[(R + 7) % 8][r][x] = fma2(c.W1, v, A[(R + 7) % 8][r][x]);
-            A[(R + 2) % 8][r][x] = fma2(c.W2, v, A[(R + 2) % 8][r][x]);
-            A[(R + 6) % 8][r][x] = fma2(c.W2, v, A[(R + 6) % 8][r][x]);
-            A[(R + 3) % 8][r][x] = fma2(c.W3, v, A[(R + 3) % 8][r][x]);
-            A[(R + 5) % 8][r][x] = fma2(c.W3, v, A[(R + 5) % 8][r][x]);
-            if (full) A[R][r][x] = add2(A[R][r][x], T[r][x]);
-        }
-    if (store) emit<(R + 4) % 8>(A, rowring, hp, ldh, c);
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) A[(R + 4) % 8][r][x] = c.W4 * cc[r][x];
-}
-
-__device__ __forceinline__ void emit_any(int r, const float2 (&A)[8][2][4], const int *rowring, float *hp,
-                                         int64_t ldh, const Lane &c) {
-    switch (r) {
-        case 0: emit<0>(A, rowring, hp, ldh, c); break;
-        case 1: emit<1>(A, rowring, hp, ldh, c); break;
-        case 2: emit<2>(A, rowring, hp, ldh, c); break;
-        case 3: emit<3>(A, rowring, hp, ldh, c); break;
-        case 4: emit<4>(A, rowring, hp, ldh, c); break;
-        case 5: emit<5>(A, rowring, hp, ldh, c); break;
-        case 6: emit<6>(A, rowring, hp, ldh, c); break;
-        default: emit<7>(A, rowring, hp, ldh, c); break;
-    }
-}
-
-// Position of the CTA in its unit list: unit k (a copy in U), plane z.
-struct Cursor {
-    int k, z;
-    UnitDev U;
-};
 
 template <int RING>
 __global__ void __launch_bounds__(NT, 1) k_hpsi_ring(Args a) {
-    static_assert(AHEAD < RING, "copy distance must leave a slot to compute on");
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ uint64_t fullb[RING], emptyb[RING];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int grp = blockIdx.y;
-    const int4 mine = a.cta[blockIdx.x];   // first unit, units, first atom, atoms
-    const int nu = min(mine.y, MAX_UNITS);
+    const int4 mine = a.cta[blockIdx.x];   // first step, steps, first atom, atoms
+    const int ns = mine.y;
+    const int2 *steps = a.steps + mine.x;
     unsigned char *psi_ring = smraw;                                       // [RING] windows
     unsigned char *rec_ring = smraw + (size_t)RING * SLOT_PSI;            // [RING] records
     float *cs = reinterpret_cast<float *>(rec_ring + (size_t)RING * a.rec_slot);   // [atom][4][32]
-    UnitDev *ut = reinterpret_cast<UnitDev *>(cs + (size_t)a.cs_atoms * 4 * SG);   // [MAX_UNITS]
-    int *rowring = reinterpret_cast<int *>(ut + MAX_UNITS);               // [8][NPOS] output rows
+    int *rowring = reinterpret_cast<int *>(cs + (size_t)a.cs_atoms * 4 * SG);      // [8][NPOS] output rows
     if (tid == 0) {
         for (int i = 0; i < RING; ++i) {
-            bar_init(&fullb[i], NT);    // every thread's copy completions
-            bar_init(&emptyb[i], NW);   // every warp's release
+            bar_init(&fullb[i], NCW * 32);   // every copy thread's completions
+            bar_init(&emptyb[i], NW);        // every compute warp's release
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    for (int k = tid; k < nu; k += NT) ut[k] = a.units[mine.x + k];
     // projection coefficients of the CTA's atoms, [local atom][projector][state]
     for (int e = tid; e < mine.w * 4 * SG; e += NT) {
         const int la = e >> 7, q = (e >> 5) & 3, st = e & 31;
@@ -392,176 +364,179 @@ __global__ void __launch_bounds__(NT, 1) k_hpsi_ring(Args a) {
         cs[e] = __ldg(a.cproj + ((int64_t)at * a.nb + grp * SG + st) * 4 + q);
     }
     __syncthreads();
-    if (nu == 0) return;
+    if (ns == 0) return;
 
-    // ---- copies: plane qi into slot j % RING.  Lane l of warp w copies
-    // bytes 16 (l % 8) .. of position l / 8 of brick rows w + 8 k.  The
-    // descriptors of the next three planes to copy are held by lane groups
-    // 0..9, 10..19, 20..29 (plane j in group j mod 3, brick row w + 8 (lane
-    // mod 10)), their record addresses by lanes 0, 10, 20; a group is
-    // reloaded, for plane j + 3 (cursor qd), as soon as plane j is issued.
     bool ok = true;
-    const float *src0 = a.psi + grp * SG + 4 * (lane & 7);
-    const int doff = (4 * warp + (lane >> 3)) * ROWB + 16 * (lane & 7);   // + k * 32 * ROWB
-    const uint32_t rbit = 1u << (lane >> 3);
-    const int lgrp = lane < 30 ? lane / 10 : -1, lsub = lane % 10;
-    uint32_t dq = 0u;
-    uint2 rq = make_uint2(0u, 0u);
-    auto advance = [&](Cursor &q) {
-        if (++q.z > q.U.zm1) {
-            ++q.k;
-            if (q.k < nu) {
-                q.U = ut[q.k];
-                q.z = q.U.zm0;
-            }
-        }
-    };
-    auto load_desc = [&](const Cursor &q, int g) {
-        if (q.k < nu && lgrp == g) {
-            const int64_t pt = (int64_t)q.U.pz + q.z;
-            dq = __ldg(a.desc + pt * NG + warp + NW * lsub);
-            if (lsub == 0) rq = (q.z >= q.U.zo0 && q.z < q.U.zo1) ? __ldg(a.recs + pt) : make_uint2(0u, 0u);
-        }
-    };
-    Cursor qi{0, ut[0].zm0, ut[0]}, qc = qi, qd = qi;
-    for (int g = 0; g < 3; ++g) {
-        load_desc(qd, g);
-        if (qd.k < nu) advance(qd);
-    }
-    int j = 0;   // planes issued
-    auto issue = [&]() {
-        const int slot = j % RING, g = j % 3;
-        if (!__all_sync(0xffffffffu, j < RING || bar_wait(&emptyb[slot], ((j / RING) - 1) & 1, a.spin))) {
-            ok = false;
-            return;
-        }
-        const bool pfull = qi.z >= qi.U.zo0 && qi.z < qi.U.zo1;
-        unsigned char *dst = psi_ring + (size_t)slot * SLOT_PSI + doff;
+    if (warp >= NW) {
+        // ---- copies: step j into slot j % RING as soon as every compute warp
+        // has released it.  Lane l of copy warp w copies bytes 16 (l % 8) .. of
+        // position l / 8 of brick rows w + NCW k; the points of a step are read
+        // while the one before it is in flight.
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(REGS_COPY));
+        const int cw = warp - NW, ct = tid - NW * 32;
+        const char *src0 = reinterpret_cast<const char *>(a.psi + grp * SG + 4 * (lane & 7));
+        const int doff = (4 * cw + (lane >> 3)) * ROWB + 16 * (lane & 7);   // + k * NCW * 4 * ROWB
+        const int4 *idx0 = reinterpret_cast<const int4 *>(a.idx) + (cw * 4 + (lane >> 3)) * (CPW / 4);
+        int4 q[CPW / 4];
+        uint2 rq;
+        int2 step = __ldg(steps);
+        auto load = [&]() {
+            const int4 *src = idx0 + (size_t)(uint32_t)step.x * (NSLOT / 4);
+            const bool full = step.y & STEP_FULL;
 #pragma unroll
-        for (int k = 0; k < CPW; ++k) {
-            // edge planes: the tile's own brick rows only (16 .. 47)
-            if (!pfull && (k < G_TILE0 / NW || k >= G_TILE1 / NW)) continue;
-            const uint32_t d = __shfl_sync(0xffffffffu, dq, 10 * g + k);
-            const uint32_t mask = d >> 28;
-            const bool has = (mask & rbit) != 0;
-            const int pnt = (int)(d & 0x0fffffffu) + __popc(mask & (rbit - 1u));
-            const bool use = has && index_ok(pnt, a.npts, a.status);
-            cp_async16(dst + k * (NW * 4 * ROWB), use ? src0 + (int64_t)pnt * a.ldp : src0, use);
+            for (int i = 0; i < CPW / 4; ++i)
+                if (full || (i >= G_TILE0 / NCW / 4 && i < G_TILE1 / NCW / 4)) q[i] = __ldg(src + i);
+            if (full) rq = __ldg(a.recs + step.x);
+        };
+        load();
+        int j = 0, slot = 0, phase = 1;
+        for (; j < ns; ++j) {
+            if (!__all_sync(0xffffffffu, j < RING || bar_wait_idle(&emptyb[slot], phase, a.spin))) {
+                ok = false;
+                break;
+            }
+            const bool full = step.y & STEP_FULL;
+            unsigned char *dst = psi_ring + (size_t)slot * SLOT_PSI + doff;
+            if (j + 1 < ns) step = __ldg(steps + j + 1);
+#pragma unroll
+            for (int i = 0; i < CPW / 4; ++i) {
+                // planes beside the outputs: the tile's own brick rows only (16 .. 47)
+                if (!full && (i < G_TILE0 / NCW / 4 || i >= G_TILE1 / NCW / 4)) continue;
+                const int p4[4] = {q[i].x, q[i].y, q[i].z, q[i].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const bool use = p4[k] >= 0 && index_ok(p4[k], a.npts, a.status);
+                    cp_async16(dst + (4 * i + k) * (NCW * 4 * ROWB), src0 + (uint64_t)(uint32_t)(use ? p4[k] : 0) * a.ldp, use);
+                }
+            }
+            if (full) {
+                const unsigned char *rsrc = a.rec + (size_t)rq.x * 16;
+                unsigned char *rdst = rec_ring + (size_t)slot * a.rec_slot;
+                for (int o = ct * 16; o < (int)rq.y; o += NCW * 32 * 16) cp_async16(rdst + o, rsrc + o, true);
+            }
+            cp_async_arrive(&fullb[slot]);
+            if (++slot == RING) slot = 0, phase ^= 1;
+            if (j + 1 < ns) load();
         }
-        if (pfull) {
-            const uint32_t rx = __shfl_sync(0xffffffffu, rq.x, 10 * g), ry = __shfl_sync(0xffffffffu, rq.y, 10 * g);
-            const unsigned char *rsrc = a.rec + (size_t)rx * 16;
-            unsigned char *rdst = rec_ring + (size_t)slot * a.rec_slot;
-            for (int o = tid * 16; o < (int)ry; o += NT * 16) cp_async16(rdst + o, rsrc + o, true);
-        }
-        cp_async_arrive(&fullb[slot]);
-        ++j;
-        advance(qi);
-        load_desc(qd, g);
-        if (qd.k < nu) advance(qd);
-    };
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        if (!ok && lane == 0) atomicExch(a.status, 1);
+        // The arrivals of the last planes may still be pending (the compute
+        // warps need not have waited for them when a wait gave up); no
+        // asynchronous arrival may reach shared memory after the CTA exits.
+        for (int i = max(0, j - RING); i < j; ++i) bar_wait(&fullb[i % RING], (i / RING) & 1, DRAIN_SPIN);
+        return;
+    }
 
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(REGS_COMPUTE));
     Lane c;
-    c.W1 = f2(a.w[1]);
-    c.W2 = f2(a.w[2]);
-    c.W3 = f2(a.w[3]);
-    c.W4 = f2(a.w[4]);
-    c.w = warp;
-    c.h = lane >> 4;
+    c.W1 = a.w[1], c.W2 = a.w[2], c.W3 = a.w[3], c.W4 = a.w[4];
+    c.patch = warp;
     c.sl = lane & 15;
     c.npts = a.npts;
     c.status = a.status;
     {
-        const int px = warp & 3, ty0 = 4 * (warp >> 2) + 2 * c.h, sl = c.sl;
-        const int tx0 = 4 * px;
-        c.cb = ((ty0 + 4) * 16 + tx0) * PS + sl;
-        c.to = ty0 * TX + tx0;
-        // left / right neighbours: core columns, or the side halo at the tile's edges
-        c.lb0 = (px == 0 ? 256 + ty0 * 8 : (ty0 + 4) * 16 + tx0 - 4) * PS + sl;
-        c.lb1 = (px == 0 ? 256 + (ty0 + 1) * 8 : (ty0 + 5) * 16 + tx0 - 4) * PS + sl;
-        c.rb0 = (px == 3 ? 256 + ty0 * 8 + 4 : (ty0 + 4) * 16 + tx0 + 4) * PS + sl;
-        c.rb1 = (px == 3 ? 256 + (ty0 + 1) * 8 + 4 : (ty0 + 5) * 16 + tx0 + 4) * PS + sl;
+        const int pr = 2 * (lane >> 4);   // first row in the patch
+        const int ty = 4 * (c.patch >> 2) + pr, tx = 4 * (c.patch & 3);
+        c.gp = 4 * pr;
+        c.to = ty * TX + tx;
+        // columns outside the tile: the side halo
+        const int side = 256 + (ty & 3) * 16 + (ty >> 2) * 8;
+        c.cb = ((ty + 4) * 16 + tx) * PS + c.sl;
+        c.lb = tx == 0 ? side * PS + c.sl : c.cb - 4 * PS;
+        c.rb = tx == TX - 4 ? (side + 4) * PS + c.sl : c.cb + 4 * PS;
     }
     const float2 *cs2 = reinterpret_cast<const float2 *>(cs);
-    float *hp = a.hpsi + grp * SG + 2 * c.sl;
-    float2 A[8][2][4];
-
-    while (j < AHEAD && qi.k < nu && ok) issue();
-    int it = 0;   // planes consumed
-    for (; qc.k < nu && ok; ++it) {
-        if (qi.k < nu) {
-            issue();
-            if (!ok) break;
-        }
-        const int slot = it % RING;
-        if (!__all_sync(0xffffffffu, bar_wait(&fullb[slot], (it / RING) & 1, a.spin))) {
+    char *hp = reinterpret_cast<char *>(a.hpsi + grp * SG + 2 * c.sl);
+    float2 S[8][2][4];   // outputs z - 4 .. z + 3 before plane z
+    auto clear = [&]() {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) S[k][r][x] = make_float2(0.f, 0.f);
+    };
+    clear();
+    int fnext = __ldg(&steps->y);
+    for (int it = 0, slot = 0, phase = 0; it < ns; ++it) {
+        if (!__all_sync(0xffffffffu, bar_wait(&fullb[slot], phase, a.spin))) {
             ok = false;
             break;
         }
-        const UnitDev &U = qc.U;
-        const int z = qc.z;
-        if (z == U.zm0) {
+        const int f = fnext;
+        if (it + 1 < ns) fnext = __ldg(&steps[it + 1].y);
+        if (f & STEP_FIRST) clear();
+        const int zr = (f >> STEP_Z) & 7;
+        const float2 *P = reinterpret_cast<const float2 *>(psi_ring + (size_t)slot * SLOT_PSI);
+        const unsigned char *rs = rec_ring + (size_t)slot * a.rec_slot;
+        uint64_t *release = &emptyb[slot];
+        if (++slot == RING) slot = 0, phase ^= 1;
+        // One plane.  Plane z is the last contribution to output z - 4; the other
+        // outputs take their terms and move down by one (a multiply-add writes
+        // its sum one slot lower, so the moves cost nothing); output z + 4 is new.
+        auto plane = [&](auto full) {
+            float2 cc[2][4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) cc[r][x] = P[c.cb + (r * 16 + x) * PS];
+            if constexpr (decltype(full)::value) {
+                float2 T[2][4];
+                plane_terms(T, cc, P, rs, cs2, c);
+                // the plane's point indices to the output ring (one lane per half-warp)
+                if (c.sl == 0) {
+                    const int4 *I4 = reinterpret_cast<const int4 *>(rs + REC_IDX) + (c.to >> 2);
+                    int4 *ring4 = reinterpret_cast<int4 *>(rowring + zr * NPOS) + (c.to >> 2);
+                    ring4[0] = I4[0];
+                    ring4[TX / 4] = I4[TX / 4];
+                }
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) A[k][r][x] = make_float2(0.f, 0.f);
-        }
-        const bool full = z >= U.zo0 && z < U.zo1;
-        const float2 *P = reinterpret_cast<const float2 *>(psi_ring + (size_t)slot * SLOT_PSI);
-        const unsigned char *rs = rec_ring + (size_t)slot * a.rec_slot;
-        float2 cc[2][4], T[2][4];
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) cc[r][x] = P[c.cb + (r * 16 + x) * PS];
-        if (full) {
-            plane_terms(T, cc, P, rs, cs2, c);
-            // the plane's point indices to the output ring (one lane per half-warp)
-            if (c.sl == 0) {
-                const int4 *I4 = reinterpret_cast<const int4 *>(rs + REC_IDX) + (c.to >> 2);
-                int4 *ring4 = reinterpret_cast<int4 *>(rowring + (z & 7) * NPOS) + (c.to >> 2);
-                ring4[0] = I4[0];
-                ring4[TX / 4] = I4[TX / 4];
+                    for (int x = 0; x < 4; ++x) S[4][r][x] = add2(S[4][r][x], T[r][x]);
             }
+            __syncwarp();
+            if (lane == 0) bar_arrive(release);   // the slot is no longer read by this warp
+            if (f & STEP_STORE) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) S[0][r][x] = fma2(c.W4, cc[r][x], S[0][r][x]);
+                emit(S[0], rowring, zr ^ 4, hp, a.ldh, c);
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float2 v = cc[r][x];
+                    S[0][r][x] = fma2(c.W3, v, S[1][r][x]);
+                    S[1][r][x] = fma2(c.W2, v, S[2][r][x]);
+                    S[2][r][x] = fma2(c.W1, v, S[3][r][x]);
+                    S[3][r][x] = S[4][r][x];
+                    S[4][r][x] = fma2(c.W1, v, S[5][r][x]);
+                    S[5][r][x] = fma2(c.W2, v, S[6][r][x]);
+                    S[6][r][x] = fma2(c.W3, v, S[7][r][x]);
+                    S[7][r][x] = c.W4 * v;
+                }
+        };
+        if (f & STEP_FULL) plane(std::true_type{});
+        else plane(std::false_type{});
+        // the column's last plane: planes beyond it are empty, so the outputs
+        // z - 3 .. z still open are complete
+        const int fl = f >> STEP_FLUSH;
+        if (fl) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (fl >> k & 1) emit(S[k], rowring, (zr + 5 + k) & 7, hp, a.ldh, c);
         }
-        __syncwarp();
-        if (lane == 0) bar_arrive(&emptyb[slot]);   // the slot is no longer read by this warp
-        const bool st = z - 4 >= U.zo0 && z - 4 < U.zo1;
-        switch (z & 7) {
-            case 0: zterms<0>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 1: zterms<1>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 2: zterms<2>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 3: zterms<3>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 4: zterms<4>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 5: zterms<5>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            case 6: zterms<6>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-            default: zterms<7>(A, cc, T, full, st, rowring, hp, a.ldh, c); break;
-        }
-        // last plane of the column inside the unit: planes beyond it are
-        // empty, so the outputs still open are complete
-        if (z == U.zm1 && z < U.zo1 + 3) {
-            for (int o = z - 3; o <= z; ++o)
-                if (o >= U.zo0 && o < U.zo1) emit_any(o & 7, A, rowring, hp, a.ldh, c);
-        }
-        advance(qc);
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    if (!ok) {
-        if (lane == 0) atomicExch(a.status, 1);
-        // A wait gave up.  The planes this thread issued but did not consume
-        // (at most RING, in distinct slots) may still have arrivals pending
-        // from its copies; wait for their phases, with a fixed bound, so that
-        // no asynchronous arrival reaches shared memory after the CTA exits.
-        for (int q = it; q < j; ++q) bar_wait(&fullb[q % RING], (q / RING) & 1, DRAIN_SPIN);
-    }
+    if (!ok && lane == 0) atomicExch(a.status, 1);
 }
 
 }  // namespace
 
 struct RingPlan {
-    DevBuf units, cta, cta_atoms, desc, recs, rec, status;
+    DevBuf steps, cta, cta_atoms, idx, recs, rec, status;
     int n_cta = 0, rec_slot = 0, cs_atoms = 0, ring = MAX_RING, spin = SPIN;
     int64_t nplanes = 0;
     float w0 = 0.f;
@@ -575,8 +550,7 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                     const std::vector<float> &cg32, const std::vector<float> &v32, float w0, int n_atoms, int slab) {
     (void)n_atoms;
     *out = nullptr;
-    // the descriptors describe four consecutive points per brick row: the
-    // kernel needs the order of bricks of 4^3 points
+    // the order of bricks of 4^3 points: a brick row's points follow one another
     if (g->order != 4 || g->npts >= (1 << 28) || slab < 1 || slab > MAX_SLAB) return RS_OK;
     const int d0 = g->dims[0], d1 = g->dims[1], d2 = g->dims[2];
     auto at = [&](int a0, int a1, int a2) -> int32_t {
@@ -589,7 +563,7 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
         int64_t p0;   // record / descriptor index of plane zmin
     };
     std::vector<Col> cols;
-    std::vector<uint32_t> desc;
+    std::vector<int32_t> idx;
     std::vector<uint2> recs;
     std::vector<double> pcost;   // march cost of each full plane (planes of the nonlocal-heaviest patch cost more)
     std::vector<int32_t> blob;   // 4-byte words; records start on 16-byte boundaries
@@ -615,20 +589,13 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                 if (zmax < 0) continue;
                 cols.push_back({zmin, zmax, nplanes});
                 for (int z = zmin; z <= zmax; ++z) {
+                    const size_t i0 = idx.size();
+                    idx.resize(i0 + NSLOT);
                     for (int gi = 0; gi < NG; ++gi) {
                         int wy, wx;
                         group_pos(gi, wy, wx);
-                        uint32_t mask = 0;
-                        int32_t first = -1, prev = -1;
-                        for (int i = 0; i < 4; ++i) {
-                            const int32_t m = at(z, b1 + wy - 4, b2 + wx - 4 + i);
-                            if (m < 0) continue;
-                            if (first < 0) first = m;
-                            else if (m != prev + 1) return fail(RS_EINVAL, "stencil plan: brick row not consecutive");
-                            prev = m;
-                            mask |= 1u << i;
-                        }
-                        desc.push_back((mask << 28) | (uint32_t)(first < 0 ? 0 : first));
+                        for (int i = 0; i < 4; ++i)
+                            idx[i0 + ((gi % NCW) * 4 + i) * CPW + gi / NCW] = at(z, b1 + wy - 4, b2 + wx - 4 + i);
                     }
                     // record of plane z
                     const size_t off = blob.size();
@@ -642,7 +609,7 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                             vv[2 * (iy * TX + ix)] = vv[2 * (iy * TX + ix) + 1] = word(vw);
                             ii[iy * TX + ix] = m;
                         }
-                    for (int w = 0; w < NW; ++w) {
+                    for (int w = 0; w < NP; ++w) {
                         const int py = w >> 2, px = w & 3;
                         // atom -> projector values of the 16 patch points
                         std::map<int32_t, std::vector<float>> per_atom;
@@ -675,7 +642,7 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                     if (off / 4 > UINT32_MAX) return RS_OK;
                     recs.push_back(make_uint2((uint32_t)(off / 4), (uint32_t)bytes));
                     int maxblk = 0;
-                    for (int w = 0; w < NW; ++w) maxblk = std::max(maxblk, hdr[2 * w]);
+                    for (int w = 0; w < NP; ++w) maxblk = std::max(maxblk, hdr[2 * w]);
                     pcost.push_back(1.0 + NL_COST * maxblk);
                     ++nplanes;
                 }
@@ -713,7 +680,11 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
         // Greedy fill of runs up to a cost T (a run takes whole planes while
         // it stays within T; a plane that fits no run alone opens one); the
         // smallest T that needs at most G runs, by bisection.
-        std::vector<std::vector<UnitDev>> per;
+        // a unit: output planes zo0 .. zo1 - 1, marched planes zm0 .. zm1
+        struct Unit {
+            int zm0, zm1, zo0, zo1, pz;
+        };
+        std::vector<std::vector<Unit>> per;
         auto fill = [&](double T, bool keep) -> int {
             if (keep) per.assign(1, {});
             int runs = 1;
@@ -736,7 +707,7 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                         ++b;
                     }
                     if (keep) {
-                        UnitDev d{};
+                        Unit d{};
                         d.zo0 = a;
                         d.zo1 = b;
                         d.zm0 = std::max(u.zmin, a - 4);
@@ -769,18 +740,17 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
         // per CTA: the atoms its records name, renumbered in the records to
         // the CTA's local order (a record belongs to the one unit whose
         // output planes hold it)
-        std::vector<UnitDev> flat;
+        std::vector<int2> flat;
         std::vector<int4> cta(G);
         std::vector<int32_t> cta_atoms;
         int cs_atoms = 0;
         for (int k = 0; k < G; ++k) {
-            if (per[k].size() > (size_t)MAX_UNITS) return RS_OK;
             std::map<int32_t, int32_t> local;
             const int first_atom = (int)cta_atoms.size();
-            for (const UnitDev &u : per[k])
+            for (const Unit &u : per[k])
                 for (int z = u.zo0; z < u.zo1; ++z) {
                     const size_t w0 = (size_t)recs[(size_t)((int64_t)u.pz + z)].x * 4;
-                    for (int w = 0; w < NW; ++w) {
+                    for (int w = 0; w < NP; ++w) {
                         const int cnt = blob[w0 + 2 * w], b0 = blob[w0 + 2 * w + 1];
                         for (int q = 0; q < cnt; ++q) {
                             int32_t &aw = blob[w0 + (size_t)(b0 + q * BLK) / 4];
@@ -794,10 +764,21 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
                     }
                 }
             cs_atoms = std::max(cs_atoms, (int)local.size());
-            cta[k] = make_int4((int)flat.size(), (int)per[k].size(), first_atom, (int)local.size());
-            flat.insert(flat.end(), per[k].begin(), per[k].end());
+            const size_t first_step = flat.size();
+            for (const Unit &u : per[k])
+                for (int z = u.zm0; z <= u.zm1; ++z) {
+                    int f = (z >= u.zo0 && z < u.zo1 ? STEP_FULL : 0) | (z - 4 >= u.zo0 && z - 4 < u.zo1 ? STEP_STORE : 0) |
+                            (z == u.zm0 ? STEP_FIRST : 0) | (z & 7) << STEP_Z;
+                    // planes beyond the column's last are empty: what is open is complete
+                    if (z == u.zm1 && z < u.zo1 + 3)
+                        for (int o = std::max(u.zo0, z - 3); o <= z && o < u.zo1; ++o) f |= 1 << (STEP_FLUSH + o - (z - 3));
+                    flat.push_back(make_int2(u.pz + z, f));
+                }
+            if (flat.size() > (size_t)INT32_MAX) return RS_OK;
+            cta[k] = make_int4((int)first_step, (int)(flat.size() - first_step), first_atom, (int)local.size());
         }
         if (cta_atoms.empty()) cta_atoms.push_back(0);
+        if (flat.empty()) return RS_OK;
         RingPlan *P = new (std::nothrow) RingPlan;
         if (!P) return fail(RS_ENOMEM, "host allocation failed");
         auto bail = [&](int rc) {
@@ -805,10 +786,10 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
             return rc;
         };
         int rc;
-        if ((rc = P->units.upload(flat.data(), flat.size() * sizeof(UnitDev))) ||
+        if ((rc = P->steps.upload(flat.data(), flat.size() * sizeof(int2))) ||
             (rc = P->cta.upload(cta.data(), cta.size() * sizeof(int4))) ||
             (rc = P->cta_atoms.upload(cta_atoms.data(), cta_atoms.size() * sizeof(int32_t))) ||
-            (rc = P->desc.upload(desc.data(), desc.size() * sizeof(uint32_t))) ||
+            (rc = P->idx.upload(idx.data(), idx.size() * sizeof(int32_t))) ||
             (rc = P->recs.upload(recs.data(), recs.size() * sizeof(uint2))) ||
             (rc = P->rec.upload(blob.data(), blob.size() * sizeof(int32_t))) || (rc = P->status.alloc(sizeof(int))))
             return bail(rc);
@@ -819,8 +800,8 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
         P->rec_slot = (max_rec + 127) & ~127;
         P->cs_atoms = cs_atoms;
         P->npts = g->npts;
-        const size_t fixed = (size_t)cs_atoms * 4 * SG * sizeof(float) + MAX_UNITS * sizeof(UnitDev) + 8 * NPOS * sizeof(int);
-        for (P->ring = MAX_RING; P->ring > AHEAD; --P->ring) {
+        const size_t fixed = (size_t)cs_atoms * 4 * SG * sizeof(float) + 8 * NPOS * sizeof(int);
+        for (P->ring = MAX_RING; P->ring >= MIN_RING; --P->ring) {
             P->smem = (size_t)P->ring * (SLOT_PSI + P->rec_slot) + fixed;
             if (P->smem <= MAX_SMEM) break;
         }
@@ -832,30 +813,31 @@ int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t>
     return RS_OK;
 }
 
-bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int nb) {
-    return p && nb % SG == 0 && ldp % 4 == 0 && aligned16(psi);
+bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int64_t ldh, int nb) {
+    // row strides in bytes are 32-bit numbers
+    return p && nb % SG == 0 && ldp % 4 == 0 && aligned16(psi) && ldp < (1 << 30) && ldh < (1 << 30);
 }
 
 int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t ldh, const float *cproj, int nb,
                 const float w[5], cudaStream_t st) {
     Args a;
-    a.units = p->units.as<UnitDev>();
+    a.steps = p->steps.as<int2>();
     a.cta = p->cta.as<int4>();
     a.cta_atoms = p->cta_atoms.as<int>();
     a.cs_atoms = p->cs_atoms;
-    a.desc = p->desc.as<uint32_t>();
+    a.idx = p->idx.as<int>();
     a.recs = p->recs.as<uint2>();
     a.rec = p->rec.as<unsigned char>();
     a.psi = psi;
-    a.ldp = ldp;
+    a.ldp = (uint32_t)(4 * ldp);
     a.cproj = cproj;
     a.hpsi = hpsi;
-    a.ldh = ldh;
+    a.ldh = (uint32_t)(4 * ldh);
     a.nb = nb;
     a.rec_slot = p->rec_slot;
     a.spin = p->spin;
     a.npts = (int)p->npts;
-    for (int j = 0; j < 5; ++j) a.w[j] = w[j];
+    for (int j = 0; j < 5; ++j) a.w[j] = make_float2(w[j], w[j]);
     a.status = p->status.as<int>();
     const dim3 grid((unsigned)p->n_cta, (unsigned)(nb / SG));
     const int r4 = p->ring == 4 ? 1 : 0;

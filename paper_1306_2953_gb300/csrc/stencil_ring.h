@@ -18,15 +18,15 @@ struct RingPlan;
 // per entry), the FP32 potential, the FP32 centre weight of the star, the
 // number of atoms and the z-slab height
 // of a work unit.  Returns RS_OK with *out == nullptr when the grid cannot
-// use the kernel (2^28 points or more, a plane record or a CTA's unit list
-// above the shared-memory budget).
+// use the kernel (2^28 points or more, not in bricks of 4^3 points, or plane
+// records or atom coefficients above the shared-memory budget).
 int ring_plan_build(RingPlan **out, const rs_grid *g, const std::vector<int32_t> &coff, const std::vector<int32_t> &catom,
                     const std::vector<float> &cg32, const std::vector<float> &v32, float w0, int n_atoms, int slab);
 void ring_plan_destroy(RingPlan *p);
 
 // True when the kernel takes this block: nb a multiple of 32 and 16-byte
-// copies of psi rows (16-byte aligned base, ld a multiple of 4).
-bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int nb);
+// copies of psi rows (16-byte aligned base, ld a multiple of 4; ld below 2^30).
+bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int64_t ldh, int nb);
 
 // Hpsi = (T + V + V_nl) psi for nb states (w: kinetic weights, cproj: the
 // projection coefficients [atom][nb][4] of this block, already computed).

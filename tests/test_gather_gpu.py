@@ -53,3 +53,24 @@ def test_gather_edges(dtype, nb, system, order, pad):
     o = out.double().cpu().numpy()
     assert np.all(np.abs(o[:, pad:pad + nb] - ref) <= bound)
     assert np.all(o[:, :pad] == 7.0) and np.all(o[:, pad + nb:] == 7.0)
+
+
+@pytest.mark.parametrize("box", [(1, 1, 1), (3, 2, 5), (4, 8, 16), (5, 9, 17), (23, 7, 33), (70, 12, 40)])
+def test_ring_march_edges(box):
+    """FP32 blocks of 32 states (the ring kernel): columns shorter than the
+    star, ragged tiles, runs that are cut inside a column.  Against the FP64
+    gather of the same values; tolerance 64 roundings of the terms' magnitude,
+    the sum of the weights and the potential times the largest value."""
+    from paper_1306_2953_gb300 import api
+    g = api.Grid.box(*box, 0.3)
+    rng = np.random.default_rng(sum(box))
+    V = rng.uniform(-2, 2, g.npts)
+    H = api.Hamiltonian(g, V, None)
+    psi = torch.from_numpy(rng.uniform(-1, 1, (g.npts, 64)).astype(np.float32)).cuda()
+    bound = 64 * 2.0 ** -24 * (9.0 * 2.85 / (2 * 0.3 ** 2) + 2)
+    for c0, nb in ((0, 32), (32, 32), (0, 64)):
+        out = torch.full_like(psi, 7.0)
+        H.apply(psi[:, c0:c0 + nb], out[:, c0:c0 + nb], nb=nb)
+        ref = H.apply(psi[:, c0:c0 + nb].double().contiguous(), nb=nb)
+        assert (out[:, c0:c0 + nb].double() - ref).abs().max().item() <= bound
+    assert H.status() == 0
