@@ -94,4 +94,32 @@ struct PoolBuf {
     PoolBuf &operator=(const PoolBuf &) = delete;
 };
 
+// Launch whose start may overlap the end of the kernel before it in the stream:
+// the kernel calls pdl_wait() before it reads or writes anything that the
+// stream's earlier work touches.
+template <typename... P, typename... A>
+int launch_overlapped(void (*fn)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    RS_CUDA(cudaLaunchKernelEx(&cfg, fn, P(args)...));
+    return RS_OK;
+}
+#ifdef __CUDACC__
+// All earlier work of the stream is complete and visible (at once when the
+// kernel was launched without overlap).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// The next kernel of the stream may be started (it waits in pdl_wait).  Only where
+// its CTAs fill every SM anyway: a small grid that starts in a tail is packed
+// on the few SMs that are free.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+#endif
+
 }  // namespace rs

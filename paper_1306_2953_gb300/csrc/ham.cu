@@ -4,7 +4,7 @@
 //  1. k_project: the Kleinman-Bylander projection integrals of Eq. (4),
 //     c[A,q,s] = E[A,q] dV sum_{p in S_A} gamma_Aq(p) psi(p,s), PSPLIT CTAs
 //     per (atom, state group), each a block-wide tree reduction over its share
-//     of the sphere points added to the zeroed coefficients; stored
+//     of the sphere points; the last of them adds the shares up; stored
 //     [atom][state][q] so that one 16-byte load gives a state's four.
 //     FP32 blocks of 32-state groups take k_project_f32 (four states per lane
 //     and four sphere entries per warp step, the atom split sized to fill the
@@ -77,21 +77,38 @@ __device__ __forceinline__ Four<double> load4(const double *p) {
 
 // ------------------------------------------------- projection integrals ---
 
-// Grid (atoms * PSPLIT, state groups): each CTA sums 1/PSPLIT of an atom's
-// sphere points and adds its partial sums to the (zeroed) coefficients.
+// Grid (atoms * split, state groups): each CTA sums 1 / split of an atom's
+// sphere points and writes its partial sums to `part` [atom, group][split][n];
+// the CTA that comes last (`count`, which returns to zero) adds the parts in
+// their order and writes the group's coefficients.
+// (Atomic additions to zeroed coefficients needed a memset before each block and
+// gave sums that depended on the order.)
 constexpr int PSPLIT = 8;
+
+// True in the whole CTA that is the last of the `split` of its atom and group;
+// the parts of the others are visible to it.
+__device__ __forceinline__ bool last_part(unsigned *count, int split) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(count, (unsigned)split - 1) == (unsigned)split - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
 
 template <typename T, int SGP, int NT>
 __global__ void __launch_bounds__(NT) k_project(HamDev<T> d, const T *__restrict__ psi, int64_t ldp, int nb,
-                                                T *__restrict__ cproj) {
+                                                T *part, unsigned *count, T *__restrict__ cproj) {
     constexpr int R = NT / SGP;
     __shared__ T red[4][NT];
-    const int A = blockIdx.x / PSPLIT, part = blockIdx.x % PSPLIT;
+    const int A = blockIdx.x / PSPLIT, piece = blockIdx.x % PSPLIT;
     const int sg0 = blockIdx.y * SGP;
     const int s = threadIdx.x % SGP, r = threadIdx.x / SGP;
     const int o = __ldg(d.sph_off + A), e = __ldg(d.sph_off + A + 1);
     const int len = e - o, per = (len + PSPLIT - 1) / PSPLIT;
-    const int i0 = o + part * per, i1 = min(e, i0 + per);
+    const int i0 = o + piece * per, i1 = min(e, i0 + per);
+    pdl_wait();
     const T *ps = psi + sg0 + s;
     T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
 #pragma unroll 8
@@ -116,46 +133,75 @@ __global__ void __launch_bounds__(NT) k_project(HamDev<T> d, const T *__restrict
         }
         __syncthreads();
     }
-    if (r == 0 && i0 < i1) {
+    const int slot = A * gridDim.y + blockIdx.y;
+    part += (int64_t)slot * PSPLIT * 4 * SGP;
+    if (threadIdx.x < 4 * SGP) part[piece * 4 * SGP + threadIdx.x] = red[threadIdx.x % 4][threadIdx.x / 4];
+    if (last_part(count + slot, PSPLIT) && threadIdx.x < 4 * SGP) {
+        T t = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            atomicAdd(cproj + ((int64_t)A * nb + sg0 + s) * 4 + q, __ldg(d.E + 4 * A + q) * d.dV * red[q][s]);
+        for (int k = 0; k < PSPLIT; ++k) t += __ldcg(part + k * 4 * SGP + threadIdx.x);
+        cproj[((int64_t)A * nb + sg0) * 4 + threadIdx.x] = __ldg(d.E + 4 * A + threadIdx.x % 4) * d.dV * t;
     }
 }
 
 #ifndef RS_PROJ_CTAS
-#define RS_PROJ_CTAS 5
+#define RS_PROJ_CTAS 4
 #endif
 
 // FP32 blocks of 32-state groups: lane l of a warp takes sphere entry
 // l / 8 of the warp's four and the states 4 (l % 8) .. + 3 (one 16-byte
-// load of the psi row), so a warp reads four psi rows per step; the grid is
-// (atoms * split, state groups) with the split sized to fill the GPU.
+// load of the psi row), so a warp reads four psi rows per step, four steps
+// at a time; the point indices are read one round ahead of their rows.  The
+// grid is (atoms * split,
+// state groups) with the split sized to fill the GPU.  SUM: the last part adds
+// them up; else (the ring kernel, whose CTAs read few atoms each) the reader
+// does, which spares the fences at the kernel's end, 2.3 us a block.
 constexpr int NTP4 = 256;
 
-__global__ void __launch_bounds__(NTP4) k_project_f32(HamDev<float> d, const float *__restrict__ psi, int64_t ldp,
-                                                     int nb, int split, float *__restrict__ cproj) {
+template <bool SUM>
+__global__ void __launch_bounds__(NTP4, RS_PROJ_CTAS) k_project_f32(HamDev<float> d, const float *__restrict__ psi, int64_t ldp, int nb,
+                                                     int split, float *part, unsigned *count, float *__restrict__ cproj) {
+    constexpr int STEP = 4 * (NTP4 / 32), UN = 4;
     __shared__ float red[NTP4 / 32][8][16];
-    const int A = blockIdx.x / split, part = blockIdx.x - A * split;
+    const int A = blockIdx.x / split, piece = blockIdx.x - A * split;
     const int sg0 = blockIdx.y * 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane & 7;
     const int o = __ldg(d.sph_off + A), e = __ldg(d.sph_off + A + 1);
     const int per = (e - o + split - 1) / split;
-    const int i0 = o + part * per, i1 = min(e, i0 + per);
+    const int i0 = o + piece * per, i1 = min(e, i0 + per);
     const float *ps = psi + sg0 + 4 * q;
     float acc[16];   // [projector][state]
 #pragma unroll
     for (int k = 0; k < 16; ++k) acc[k] = 0.f;
-#pragma unroll 4
-    for (int i = i0 + 4 * warp + (lane >> 3); i < i1; i += 4 * (NTP4 / 32)) {
-        const int p = __ldg(d.sph_idx + i);
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(ps + (int64_t)p * ldp));
-        const float4 g = __ldg(reinterpret_cast<const float4 *>(d.sph_gam) + i);
-        const float gv[4] = {g.x, g.y, g.z, g.w}, vv[4] = {v.x, v.y, v.z, v.w};
+    int i = i0 + 4 * warp + (lane >> 3);
+    int p[UN];
 #pragma unroll
-        for (int l = 0; l < 4; ++l)
+    for (int u = 0; u < UN; ++u) p[u] = i + u * STEP < i1 ? __ldg(d.sph_idx + i + u * STEP) : -1;
+    pdl_wait();
+    pdl_launch();
+    for (; i < i1; i += UN * STEP) {
+        float4 v[UN], g[UN];
 #pragma unroll
-            for (int st = 0; st < 4; ++st) acc[4 * l + st] = fmaf(gv[l], vv[st], acc[4 * l + st]);
+        for (int u = 0; u < UN; ++u) {
+            v[u] = g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (p[u] >= 0) {
+                v[u] = __ldg(reinterpret_cast<const float4 *>(ps + (int64_t)p[u] * ldp));
+                g[u] = __ldg(reinterpret_cast<const float4 *>(d.sph_gam) + i + u * STEP);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const int n = i + (UN + u) * STEP;
+            p[u] = n < i1 ? __ldg(d.sph_idx + n) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const float gv[4] = {g[u].x, g[u].y, g[u].z, g[u].w}, vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+            for (int l = 0; l < 4; ++l)
+#pragma unroll
+                for (int st = 0; st < 4; ++st) acc[4 * l + st] = fmaf(gv[l], vv[st], acc[4 * l + st]);
+        }
     }
     // the four entries of a warp, then the warps
 #pragma unroll
@@ -168,13 +214,21 @@ __global__ void __launch_bounds__(NTP4) k_project_f32(HamDev<float> d, const flo
         for (int k = 0; k < 16; ++k) red[warp][q][k] = acc[k];
     }
     __syncthreads();
-    if (threadIdx.x < 128 && i0 < i1) {
-        const int qq = threadIdx.x >> 4, k = threadIdx.x & 15, l = k >> 2, st = k & 3;
+    // thread t < 128: state t / 4 of the group, projector t % 4
+    const int slot = A * gridDim.y + blockIdx.y, l = threadIdx.x & 3, st = threadIdx.x >> 2;
+    part += (int64_t)slot * split * 128;
+    if (threadIdx.x < 128) {
         float t = 0.f;
 #pragma unroll
-        for (int w = 0; w < NTP4 / 32; ++w) t += red[w][qq][k];
-        atomicAdd(cproj + ((int64_t)A * nb + sg0 + 4 * qq + st) * 4 + l, __ldg(d.E + 4 * A + l) * d.dV * t);
+        for (int w = 0; w < NTP4 / 32; ++w) t += red[w][st >> 2][4 * l + (st & 3)];
+        part[piece * 128 + threadIdx.x] = __ldg(d.E + 4 * A + l) * d.dV * t;
     }
+    if constexpr (SUM)
+        if (last_part(count + slot, split) && threadIdx.x < 128) {
+            float t = 0.f;
+            for (int k = 0; k < split; ++k) t += __ldcg(part + k * 128 + threadIdx.x);
+            cproj[((int64_t)A * nb + sg0) * 4 + threadIdx.x] = t;
+        }
 }
 
 // ------------------------------------------- fused stencil + V + nonlocal ---
@@ -247,6 +301,7 @@ __global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__
         nbr[g][q] = make_int4(__ldg(m + st), __ldg(m + 2 * st), __ldg(m + 3 * st), __ldg(m + 4 * st));
     }
     __syncthreads();
+    pdl_wait();
     const int lane = tid % LPP;
     const T *ps = psi + lane * V;
     for (int q = tid / LPP; q < C::PTS; q += C::PP) {
@@ -355,7 +410,7 @@ struct rs_ham {
     int n_sm = 1;                  // SMs of the device (grid sizing)
     double w[5] = {0, 0, 0, 0, 0};
     DevBuf pinfo64, pinfo32, map, loc, V64, V32, cov_off, cov_atom, cov_gam64, cov_gam32, sph_off, sph_idx, sph_gam64, sph_gam32, E64, E32,
-        cproj, dummy, scratch;
+        cproj, cpart, ccount, dummy, scratch;
     RingPlan *ring = nullptr;      // tables of the ring-buffer FP32 kernel (nullptr: not usable)
     int kernel = RS_KERNEL_AUTO;   // rs_ham_select_kernel
     // optional per-launch timing (rs_ham_timing)
@@ -379,6 +434,9 @@ struct rs_ham {
         return &events[3 * n_recorded++];
     }
     template <typename T> HamDev<T> view() const;
+    // parts of an atom's sphere in k_project_f32: one wave of at most
+    // RS_PROJ_CTAS CTAs of 256 threads per SM in all
+    int proj_split() const { return std::max(1, std::min(64, RS_PROJ_CTAS * n_sm / std::max(1, n_atoms))); }
 };
 
 template <> HamDev<double> rs_ham::view<double>() const {
@@ -509,6 +567,16 @@ extern "C" int rs_ham_create(const rs_grid *g, const double *V_host, const rs_pr
         return bail(rc);
     if ((rc = H->cproj.alloc((size_t)std::max(na, 1) * 4 * 64 * sizeof(double)))) return bail(rc);
     {
+        // partial sums: PSPLIT parts of 64 FP64 states, or as many FP32 parts as proj_split allows
+        const size_t a64 = (size_t)std::max(na, 1) * PSPLIT * 4 * 64 * sizeof(double);
+        const size_t a32 = (size_t)std::max(na, 1) * H->proj_split() * 4 * 64 * sizeof(float);
+        if ((rc = H->cpart.alloc(std::max(a64, a32)))) return bail(rc);
+        // one count per atom and state group (at most two groups)
+        if ((rc = H->ccount.alloc((size_t)std::max(na, 1) * 2 * sizeof(unsigned)))) return bail(rc);
+        if (cudaMemset(H->ccount.p, 0, (size_t)std::max(na, 1) * 2 * sizeof(unsigned)) != cudaSuccess)
+            return bail(fail(RS_ECUDA, "cudaMemset failed"));
+    }
+    {
         std::vector<int4> p64((size_t)np), p32((size_t)np);
         for (int64_t p = 0; p < np; ++p) {
             int64_t bits;
@@ -539,10 +607,8 @@ template <typename T, int V, int LPP>
 static int launch_gather(rs_ham *H, const HamDev<T> &d, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, int nb,
                          cudaStream_t st) {
     constexpr int PTS = GatherCfg<T, V, LPP>::PTS;
-    k_gather<T, V, LPP><<<(unsigned)((H->npts + PTS - 1) / PTS), GT_NT, 0, st>>>(d, H->loc.as<int32_t>(), (int)H->npts, psi,
-                                                                                ldp, hpsi, ldh, H->cproj.as<T>(), nb);
-    RS_LAUNCH_CHECK();
-    return RS_OK;
+    return launch_overlapped(k_gather<T, V, LPP>, dim3((unsigned)((H->npts + PTS - 1) / PTS)), GT_NT, 0, st, d,
+                             H->loc.as<int32_t>(), (int)H->npts, psi, ldp, hpsi, ldh, H->cproj.as<T>(), nb);
 }
 
 template <typename T>
@@ -550,42 +616,39 @@ static int apply_t(rs_ham *H, const T *psi, int64_t ldp, T *hpsi, int64_t ldh, i
     const HamDev<T> d = H->view<T>();
     cudaEvent_t *ev = H->next_events();
     if (ev) RS_CUDA(cudaEventRecord(ev[0], st));
+    bool ring = false;
+    if constexpr (sizeof(T) == 4) ring = H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, ldh, nb);
     if (H->n_atoms > 0) {
         const int sgp = std::min(nb, 32);
-        dim3 grid((unsigned)(H->n_atoms * PSPLIT), (unsigned)(nb / sgp));
-        T *cp = H->cproj.as<T>();
-        RS_CUDA(cudaMemsetAsync(cp, 0, sizeof(T) * (size_t)H->n_atoms * 4 * nb, st));
+        const dim3 grid((unsigned)(H->n_atoms * PSPLIT), (unsigned)(nb / sgp));
+        T *cp = H->cproj.as<T>(), *part = H->cpart.as<T>();
+        unsigned *cnt = H->ccount.as<unsigned>();
         bool done = false;
         if constexpr (sizeof(T) == 4) {
             if (nb % 32 == 0 && ldp % 4 == 0 && aligned16(psi)) {
-                // one wave: at most RS_PROJ_CTAS CTAs of 256 threads per SM in all
-                const int split = std::max(1, std::min(64, RS_PROJ_CTAS * H->n_sm / H->n_atoms));
-                k_project_f32<<<dim3((unsigned)(H->n_atoms * split), (unsigned)(nb / 32)), NTP4, 0, st>>>(d, psi, ldp, nb,
-                                                                                                        split, cp);
+                const int split = H->proj_split();
+                RS_TRY(launch_overlapped(ring ? k_project_f32<false> : k_project_f32<true>, dim3((unsigned)(H->n_atoms * split), (unsigned)(nb / 32)), NTP4, 0, st,
+                                         d, psi, ldp, nb, split, part, cnt, cp));
                 done = true;
             }
         }
         if (!done) switch (sgp) {
-            case 1: k_project<T, 1, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
-            case 2: k_project<T, 2, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
-            case 4: k_project<T, 4, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
-            case 8: k_project<T, 8, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
-            case 16: k_project<T, 16, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
-            default: k_project<T, 32, 512><<<grid, 512, 0, st>>>(d, psi, ldp, nb, cp); break;
+            case 1: RS_TRY(launch_overlapped(k_project<T, 1, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
+            case 2: RS_TRY(launch_overlapped(k_project<T, 2, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
+            case 4: RS_TRY(launch_overlapped(k_project<T, 4, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
+            case 8: RS_TRY(launch_overlapped(k_project<T, 8, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
+            case 16: RS_TRY(launch_overlapped(k_project<T, 16, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
+            default: RS_TRY(launch_overlapped(k_project<T, 32, 512>, grid, 512, 0, st, d, psi, ldp, nb, part, cnt, cp)); break;
         }
-        RS_LAUNCH_CHECK();
     }
     if (ev) RS_CUDA(cudaEventRecord(ev[1], st));
     int rc = -1;
-    bool ring = false;
-    if constexpr (sizeof(T) == 4) {
-        ring = H->kernel == RS_KERNEL_AUTO && ring_usable(H->ring, psi, ldp, ldh, nb);
+    if constexpr (sizeof(T) == 4)
         if (ring) {
             float w[5];
             for (int j = 0; j < 5; ++j) w[j] = (float)H->w[j];
-            rc = ring_launch(H->ring, psi, ldp, hpsi, ldh, H->cproj.as<float>(), nb, w, st);
+            rc = ring_launch(H->ring, psi, ldp, hpsi, ldh, H->cpart.as<float>(), H->proj_split(), nb, w, st);
         }
-    }
     constexpr int E = 16 / (int)sizeof(T);   // states per 16 bytes
     if (!ring) switch (nb) {
         case 1: rc = launch_gather<T, 1, 1>(H, d, psi, ldp, hpsi, ldh, nb, st); break;

@@ -148,10 +148,11 @@ struct Args {
     const unsigned char *rec;
     const float *psi;       // [npts][ldp]
     uint32_t ldp;           // row strides in bytes
-    const float *cproj;     // [atom][nb][4]
+    const float *part;      // [atom][state group][split][32][4]: parts of the projection coefficients
+    int split;
     float *hpsi;
     uint32_t ldh;
-    int nb, rec_slot, cs_atoms;   // cs_atoms: the largest atom count of a CTA
+    int rec_slot, cs_atoms;   // cs_atoms: the largest atom count of a CTA
     int spin;                     // barrier tests before a wait gives up
     int npts;                     // point count (the bounds-checked build tests indices against it)
     float2 w[5];                  // weights, as pairs
@@ -357,11 +358,17 @@ __global__ void __launch_bounds__(NT, 1) k_hpsi_ring(Args a) {
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    // projection coefficients of the CTA's atoms, [local atom][projector][state]
+    pdl_wait();
+    pdl_launch();
+    // projection coefficients of the CTA's atoms, [local atom][projector][state]: the sum of their parts
     for (int e = tid; e < mine.w * 4 * SG; e += NT) {
-        const int la = e >> 7, q = (e >> 5) & 3, st = e & 31;
+        const int la = e >> 7, q = e & 3, st = (e >> 2) & 31;
         const int at = __ldg(a.cta_atoms + mine.z + la);
-        cs[e] = __ldg(a.cproj + ((int64_t)at * a.nb + grp * SG + st) * 4 + q);
+        const float *part = a.part + (((int64_t)at * gridDim.y + grp) * a.split * SG + st) * 4 + q;
+        float t = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < a.split; ++k) t += __ldg(part + k * 4 * SG);
+        cs[(4 * la + q) * SG + st] = t;
     }
     __syncthreads();
     if (ns == 0) return;
@@ -818,8 +825,8 @@ bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int64_t ldh, 
     return p && nb % SG == 0 && ldp % 4 == 0 && aligned16(psi) && ldp < (1 << 30) && ldh < (1 << 30);
 }
 
-int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t ldh, const float *cproj, int nb,
-                const float w[5], cudaStream_t st) {
+int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t ldh, const float *part, int split,
+                int nb, const float w[5], cudaStream_t st) {
     Args a;
     a.steps = p->steps.as<int2>();
     a.cta = p->cta.as<int4>();
@@ -830,10 +837,10 @@ int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t
     a.rec = p->rec.as<unsigned char>();
     a.psi = psi;
     a.ldp = (uint32_t)(4 * ldp);
-    a.cproj = cproj;
+    a.part = part;
+    a.split = split;
     a.hpsi = hpsi;
     a.ldh = (uint32_t)(4 * ldh);
-    a.nb = nb;
     a.rec_slot = p->rec_slot;
     a.spin = p->spin;
     a.npts = (int)p->npts;
@@ -842,10 +849,7 @@ int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t
     const dim3 grid((unsigned)p->n_cta, (unsigned)(nb / SG));
     const int r4 = p->ring == 4 ? 1 : 0;
     RS_TRY(smem_optin(r4 ? (const void *)k_hpsi_ring<4> : (const void *)k_hpsi_ring<3>, p->smem));
-    if (r4) k_hpsi_ring<4><<<grid, NT, p->smem, st>>>(a);
-    else k_hpsi_ring<3><<<grid, NT, p->smem, st>>>(a);
-    RS_LAUNCH_CHECK();
-    return RS_OK;
+    return launch_overlapped(r4 ? k_hpsi_ring<4> : k_hpsi_ring<3>, grid, NT, p->smem, st, a);
 }
 
 int ring_status(const RingPlan *p, int *flag) {

@@ -28,10 +28,11 @@ void ring_plan_destroy(RingPlan *p);
 // copies of psi rows (16-byte aligned base, ld a multiple of 4; ld below 2^30).
 bool ring_usable(const RingPlan *p, const float *psi, int64_t ldp, int64_t ldh, int nb);
 
-// Hpsi = (T + V + V_nl) psi for nb states (w: kinetic weights, cproj: the
-// projection coefficients [atom][nb][4] of this block, already computed).
-int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t ldh, const float *cproj, int nb,
-                const float w[5], cudaStream_t st);
+// Hpsi = (T + V + V_nl) psi for nb states (w: kinetic weights, part: the
+// projection coefficients of this block as sums of `split` parts, [atom][nb /
+// 32][split][32][4], already computed).
+int ring_launch(RingPlan *p, const float *psi, int64_t ldp, float *hpsi, int64_t ldh, const float *part, int split,
+                int nb, const float w[5], cudaStream_t st);
 
 // Status word of the kernel's bounded waits (0 = none timed out); blocking.
 int ring_status(const RingPlan *p, int *flag);

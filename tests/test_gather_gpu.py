@@ -74,3 +74,37 @@ def test_ring_march_edges(box):
         ref = H.apply(psi[:, c0:c0 + nb].double().contiguous(), nb=nb)
         assert (out[:, c0:c0 + nb].double() - ref).abs().max().item() <= bound
     assert H.status() == 0
+
+
+def test_projection_parts_repeat():
+    """The projections' parts are added in a fixed order, so a block gives the
+    same bits again after blocks of other widths and types on the same handle,
+    one after the other without a pause, and in a replayed graph."""
+    from paper_1306_2953_gb300 import _lib, api
+    g_ora, H_ora, atoms, E = oracle_system("atoms", SMALL_ATOMS, SMALL_E, SMALL_RADIUS, SMALL_H)
+    lg = api.Grid.spheres(atoms, SMALL_RADIUS, SMALL_H)
+    H = api.Hamiltonian(lg, H_ora.V[lib_to_oracle_index(g_ora, lg.ijk())], api.Projectors(lg, atoms, E, 1.0, 3.0))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    blocks = [(t, nb, k) for k in (_lib.RS_KERNEL_AUTO, _lib.RS_KERNEL_GENERIC) for t in (torch.float32, torch.float64)
+              for nb in (1, 4, 16, 32, 64)]
+    psi = {b: torch.rand((lg.npts, b[1]), generator=gen, device="cuda", dtype=b[0]) - 0.5 for b in blocks}
+
+    def run(out):
+        for b in blocks:
+            H.select_kernel(b[2])
+            H.apply(psi[b], out[b], nb=b[1])
+
+    first, again, graph = ({b: torch.empty_like(psi[b]) for b in blocks} for _ in range(3))
+    run(first)
+    for _ in range(3):
+        run(again)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    cg = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(cg, stream=s):
+        run(graph)
+    for _ in range(3):
+        cg.replay()
+    torch.cuda.synchronize()
+    for b in blocks:
+        assert torch.equal(first[b], again[b]) and torch.equal(first[b], graph[b]), b
