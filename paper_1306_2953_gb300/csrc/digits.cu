@@ -80,10 +80,13 @@ __device__ __forceinline__ bool dg_try(uint64_t *b, uint32_t parity) {
     return ok != 0;
 }
 // bounded wait; false once it has given up here or `bad` says another thread's has
-__device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile int *bad) {
+// (sleep: nanoseconds between tests, for warps that wait most of the time and
+// would take issue slots from the converters)
+__device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile int *bad, unsigned sleep = 0) {
     for (int i = 0; i < DG_SPIN; ++i) {
         if (dg_try(b, parity)) return true;
-        if (*bad) return false;
+        if ((i & 7) == 7 && *bad) return false;
+        if (sleep) __nanosleep(sleep);
     }
     *bad = 1;
     return false;
@@ -138,6 +141,14 @@ __device__ __forceinline__ void dg_tmem_ld32(uint32_t addr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
+__device__ __forceinline__ void dg_tmem_ld16(uint32_t addr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(addr));
+}
 __device__ __forceinline__ void dg_tmem_ld8(uint32_t addr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -302,7 +313,7 @@ template <int NS, int BN, int PAD> struct DgIssue {
             const bool first = kb % DG_DRAIN == 0, last = kb % DG_DRAIN == DG_DRAIN - 1 || kb == kst - 1;
             iv += first;
             if (++kb == kst) kb = 0;
-            ok = __all_sync(0xffffffffu, dg_wait(&b.full[s], (g / DG_STAGES) & 1, &b.bad));
+            ok = __all_sync(0xffffffffu, dg_wait(&b.full[s], (g / DG_STAGES) & 1, &b.bad, 40));
             DG_FENCE_AFTER();
             const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
             if (first && iv > 0 && ok) {
@@ -340,7 +351,7 @@ template <int NS, int BN, int PAD> struct DgIssue {
 // 2, L += the later ones in units of accumulator NS - 2, the last one rounded to
 // them.
 template <int NS, int BN, int CPT>
-__device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&H)[CPT], int64_t (&L)[CPT]) {
+__device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&H)[CPT], int64_t (&L)[CPT], bool release = true) {
     const int warp = threadIdx.x >> 5;
     const uint32_t lane_base = b.tmem + ((uint32_t)(warp & 3) * 32 << 16) + (uint32_t)col0;
 #pragma unroll
@@ -348,11 +359,13 @@ __device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&
         if (!dg_wait_warp(&b.accfull[t], iv & 1, &b.bad)) return false;
         DG_FENCE_AFTER();
 #pragma unroll
-        for (int c = 0; c < CPT; c += 32) {
-            uint32_t r[32];
-            dg_tmem_ld32(lane_base + t * BN + c, r);
+        for (int c = 0; c < CPT; c += CPT < 32 ? CPT : 32) {
+            constexpr int W = CPT < 32 ? CPT : 32;
+            uint32_t r[W];
+            if constexpr (W == 32) dg_tmem_ld32(lane_base + t * BN + c, r);
+            else dg_tmem_ld16(lane_base + t * BN + c, r);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
+            for (int j = 0; j < W; ++j) {
                 // accumulators 0 and 1 stay within 2^22: their integers stand in the
                 // mantissa after one addition (the conversion unit is slow)
                 const int64_t v = t < 2 ? (int64_t)((int)__float_as_uint(__fadd_rn(__uint_as_float(r[j]), 12582912.f)) - 0x4b400000)
@@ -375,8 +388,10 @@ __device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&
         for (int j = 0; j < 8; ++j)
             L[8 * q + j] += (int64_t)__float2int_rn(fmaf(__uint_as_float(w[j]), 1.f / 256.f, __uint_as_float(u[j])));
     }
-    DG_FENCE_BEFORE();
-    dg_arrive(&b.accfree);
+    if (release) {
+        DG_FENCE_BEFORE();
+        dg_arrive(&b.accfree);
+    }
     return true;
 }
 
@@ -689,7 +704,11 @@ struct RotBars {
 // the key warps find the exponents of the next tile's rows (and bring the
 // rows into L2) while the converters work on this one, and the readout and
 // the stores of a tile overlap the products of the next.
-template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
+// ONE: at most 256 states, so that a block is one readout and its sums need no
+// registers while the operands are converted (with them the converters spill:
+// 5.5 ms instead of 4.7 for 658 416 rows of 256 FP64 states).
+template <typename T, int NS, int BN, int NBLK, bool ONE>
+__global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
     constexpr int PAD = 32;   // a quarter-warp's four 8-step groups of two rows fall in distinct banks
     constexpr int KW = 3;     // key warps
     using C = DgCfg<NS, BN, PAD>;
@@ -737,7 +756,7 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         int j = 0;
         for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y, ++j) {
             const int h = j & 1;
-            if (j >= 2 && !dg_wait(&rb.keyfree[h], (j / 2 - 1) & 1, &b.bad)) break;
+            if (j >= 2 && !dg_wait(&rb.keyfree[h], (j / 2 - 1) & 1, &b.bad, 50 * kst)) break;
             const int64_t r0 = (int64_t)tile * DG_M;
             const int rows = (int)min((int64_t)DG_M, a.npts - r0);
             bool pl = false;
@@ -800,6 +819,9 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         const int ar = warp * 16 + (lane >> 2), akq = lane & 3;
         unsigned char *adst = dgsm + akq * C::LBO_A + ar * 16;
         const bool hasb = warp < NB;
+        // one or two stages a block: a stage's buffer meets the same digits of C in
+        // every tile, so they are written once
+        const int bstages = NBLK == 1 && kst <= DG_STAGES ? DG_STAGES : INT32_MAX;
         const int bkq = warp % KQ, bcol = warp / KQ * 32 + lane;
         unsigned char *bdst = dgsm + C::A_BYTES + bkq * C::LBO_B + bcol * 16;
         const int col0 = (warp >> 2) * 32, row = (warp & 3) * 32 + lane;
@@ -809,9 +831,10 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         T va[2][8];
         double vb[8];
         T held[NBLK > 1 ? 32 : 1];   // two blocks: the first one's results until the rows are read
-        int64_t H[32], L[32];
+        constexpr int HC = ONE ? 16 : 32;   // columns summed at a time
+        int64_t H[ONE ? 1 : HC], L[ONE ? 1 : HC];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) H[i] = L[i] = 0;
+        for (int i = 0; i < (ONE ? 1 : HC); ++i) H[i] = L[i] = 0;
         auto load = [&](int u, int tile, int it) {   // u = 0, 1: rows of X; 2: C
             const int blk = it >= kst ? 1 : 0, k0 = (it - blk * kst) * DG_K;   // (NBLK <= 2)
             const int64_t r0 = (int64_t)tile * DG_M;
@@ -897,11 +920,36 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
         // whether it is the block's last
         bool open = false, pend = false;
         int ptile = 0, ptj = 0, pe = 0, pblk = 0, iv = 0;
+        // HC finished sums from the thread's column c0 on: scaled and stored
+        auto finish = [&](const int64_t (&h)[HC], const int64_t (&l)[HC], int c0, int64_t p, bool on, bool lastb) {
+#pragma unroll
+            for (int q = 0; q < HC / G; ++q) {
+                T v[G], o[G];
+                const bool add = a.beta != 0.0 && on;
+                if (add) old(p, (nb0 + pblk) * BN + col0 + c0 + q * G, o);
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    const int c = q * G + i, e = eb[pblk * BN + (owns ? col0 : 0) + c0 + c] - 1022 - 2 * (8 * NS - 2);
+                    if constexpr (sizeof(T) == 8) {
+                        v[i] = (T)dg_value(h[c], l[c], (1023 + 52 + 96 + pe - 1022 + e) << 20);
+                    } else {
+                        // NS = 5: H 2^8 + L stays below 2^63
+                        v[i] = ldexpf(__ll2float_rn(h[c] * (int64_t)(1ll << (8 * (NS - 4))) + l[c]), 8 * NS + pe - 126 + e);
+                    }
+                    if (a.alpha != 1.0) v[i] *= al;
+                    if (add) v[i] += be * o[i];
+                    if (NBLK > 1 && !lastb) held[NBLK > 1 ? c0 + c : 0] = v[i];
+                }
+                if (lastb && on) put(p, (nb0 + pblk) * BN + col0 + c0 + q * G, v);
+            }
+        };
         auto readout = [&]() {
             open = false;
-            ok = ok && dg_drain<NS, BN, 32>(b, iv, owns ? col0 : 0, H, L);
-            ++iv;
-            if (!pend) return;
+            if constexpr (!ONE) {
+                ok = ok && dg_drain<NS, BN, HC>(b, iv, owns ? col0 : 0, H, L);
+                ++iv;
+                if (!pend) return;
+            }
             // the block's sums are complete
             const bool lastb = pblk == NBLK - 1;
             if (lastb && a.cluster) ok = dg_wait_warp(&rb.rd, ptj & 1, &b.bad) && ok;
@@ -916,26 +964,20 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                     put(p, nb0 * BN + col0 + q * G, v);
                 }
             }
+            if constexpr (ONE) {
 #pragma unroll
-            for (int q = 0; q < 32 / G; ++q) {
-                T v[G], o[G];
-                const bool add = a.beta != 0.0 && on;
-                if (add) old(p, (nb0 + pblk) * BN + col0 + q * G, o);
+                for (int c0 = 0; c0 < 32; c0 += HC) {
+                    int64_t h[HC], l[HC];
 #pragma unroll
-                for (int i = 0; i < G; ++i) {
-                    const int c = q * G + i, e = eb[pblk * BN + (owns ? col0 : 0) + c] - 1022 - 2 * (8 * NS - 2);
-                    if constexpr (sizeof(T) == 8) {
-                        v[i] = (T)dg_value(H[c], L[c], (1023 + 52 + 96 + pe - 1022 + e) << 20);
-                    } else {
-                        // NS = 5: H 2^8 + L stays below 2^63
-                        v[i] = ldexpf(__ll2float_rn(H[c] * (int64_t)(1ll << (8 * (NS - 4))) + L[c]), 8 * NS + pe - 126 + e);
-                    }
-                    H[c] = L[c] = 0;
-                    if (a.alpha != 1.0) v[i] *= al;
-                    if (add) v[i] += be * o[i];
-                    if (NBLK > 1 && !lastb) held[NBLK > 1 ? c : 0] = v[i];
+                    for (int i = 0; i < HC; ++i) h[i] = l[i] = 0;
+                    ok = ok && dg_drain<NS, BN, HC>(b, iv, owns ? col0 + c0 : 0, h, l, c0 + HC == 32);
+                    finish(h, l, c0, p, on, lastb);
                 }
-                if (lastb && on) put(p, (nb0 + pblk) * BN + col0 + q * G, v);
+                ++iv;
+            } else {
+                finish(H, L, 0, p, on, lastb);
+#pragma unroll
+                for (int i = 0; i < HC; ++i) H[i] = L[i] = 0;
             }
         };
         // One loop over the stages of all tiles; it == nst: the next tile is due.
@@ -972,8 +1014,8 @@ template <typename T, int NS, int BN, int NBLK> __global__ void __launch_bounds_
                     if (more) load(0, nt, ni);
                     store_digits<T, NS>(va[1], ex1, adst + s * C::STAGE + 128, C::SL_A);
                     if (more) load(1, nt, ni);
-                    if (hasb) store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B);
-                    if (more) load(2, nt, ni);
+                    if (hasb && g < bstages) store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B);
+                    if (more && g + 1 < bstages) load(2, nt, ni);
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     dg_arrive(&b.full[s]);
                 }
@@ -1060,9 +1102,9 @@ int launch_rows(Fn fn, Args a, unsigned gx, size_t smem, bool in_place, cudaStre
     return RS_OK;
 }
 
-template <typename T, int NS, int BN, int NBLK> int launch_rot(RotArgs<T> a, bool in_place, cudaStream_t st) {
+template <typename T, int NS, int BN, int NBLK, bool ONE> int launch_rot(RotArgs<T> a, bool in_place, cudaStream_t st) {
     using C = DgCfg<NS, BN, 32>;
-    auto fn = k_digit_rot<T, NS, BN, NBLK>;
+    auto fn = k_digit_rot<T, NS, BN, NBLK, ONE>;
     RS_TRY(smem_optin((const void *)fn, C::SMEM));
     return launch_rows(fn, a, (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK)), C::SMEM, in_place, st);
 }
@@ -1562,9 +1604,10 @@ int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int 
     a.yvec = aligned16(Y) && (ldy * (int64_t)sizeof(T)) % 16 == 0;
     constexpr int NS = sizeof(T) == 8 ? 8 : 5;
     const bool in_place = X == Y;
-    if (m <= 32) return launch_rot<T, NS, 32, 1>(a, false, st);
-    if (in_place && m > 512) return launch_rot<T, NS, 64, 2>(a, true, st);
-    return launch_rot<T, NS, 64, 1>(a, in_place, st);
+    const bool one = n <= DG_DRAIN * DG_K;
+    if (m <= 32) return one ? launch_rot<T, NS, 32, 1, true>(a, false, st) : launch_rot<T, NS, 32, 1, false>(a, false, st);
+    if (in_place && m > 512) return launch_rot<T, NS, 64, 2, false>(a, true, st);
+    return one ? launch_rot<T, NS, 64, 1, true>(a, in_place, st) : launch_rot<T, NS, 64, 1, false>(a, in_place, st);
 }
 template int digit_rot<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
                                double, double, cudaStream_t);
