@@ -9,8 +9,9 @@
 //             row tiles do not fit one cluster of CTAs.
 // Small dense kernels (n <= a few hundred, FP64 unless stated):
 //   k_chol    S = U^T U, right-looking, one CTA, status on failure
-//   k_trinv   U^-1 by back substitution, one thread per column
-//   k_gemm_nn small C = alpha op(A) op(B) + beta C, tiled over many CTAs
+//   k_trinv_rows  U^-1, one warp per row (n <= 256); k_trinv, one warp per
+//             column, above
+//   k_gemm_small  small C = alpha op(A) op(B) + beta C, tiled over many CTAs
 //   k_jacobi  cyclic Jacobi with the parallel (round-robin) ordering, one
 //             CTA, FP32 or FP64
 //   RefSyEv   FP64 refinement of FP32 eigenvectors by the iterative
@@ -118,59 +119,84 @@ int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc,
 // Right-looking Cholesky of the leading n x n block of A (in place): the
 // upper triangle receives U with A = U^T U, the strict lower triangle is
 // zeroed.  status[0] = 0, or j+1 if pivot j is not finite or not larger
-// than rel * (original A_jj).  One CTA; the matrix is worked on in shared
-// memory when it fits (IN_SMEM, the path cholesky takes up to
-// CHOL_SMEM_MAX), else in global memory (L1/L2 resident).
-// Rows are spread over warps and columns over lanes, so no index division.
-constexpr int CHOL_MAX = 2048;
+// than rel * (original A_jj).  One CTA, the matrix in shared memory (n up to
+// CHOL_SMEM_MAX).
 constexpr int CHOL_SMEM_MAX = 160;   // n x n FP64 in 200 KB
-template <bool IN_SMEM>
-__global__ void __launch_bounds__(1024) k_chol(double *Ag, int lda, int n, double rel, int *status) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ double diag0[CHOL_MAX];
-    __shared__ double piv;
-    __shared__ int bad;
-    double *A = IN_SMEM ? reinterpret_cast<double *>(smraw) : Ag;
-    const int ld = IN_SMEM ? n : lda;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    if (IN_SMEM)
-        for (int r = warp; r < n; r += nw)
-            for (int c = lane; c < n; c += 32) A[r * ld + c] = Ag[(int64_t)r * lda + c];
-    __syncthreads();
-    for (int j = tid; j < n; j += blockDim.x) diag0[j] = A[(int64_t)j * ld + j];
-    if (tid == 0) bad = 0;
-    __syncthreads();
-    for (int j = 0; j < n; ++j) {
-        if (tid == 0) {
-            const double d = A[(int64_t)j * ld + j];
-            if (!isfinite(d) || !(d > 0.0) || !(d > rel * diag0[j])) {
-                bad = j + 1;
-                piv = 1.0;
-            } else {
-                piv = sqrt(d);
-            }
-            A[(int64_t)j * ld + j] = piv;
+
+// The factorisation inside one CTA, rows over warps and columns over lanes.
+// The loop runs on unscaled rows (A = U^T U with U = D^-1/2 W: the update takes
+// g_r W_jc, g = W_j / d_j), so that a column waits for one division and one
+// barrier: warp 0 updates row j + 1 first, divides for the next pivot and makes
+// the next g while the other warps update the rest; the square roots come at
+// the end, row by row.  FP64 instructions (64 cycles each on a quarter of an SM,
+// however few their lanes) are what it waits for.
+// orig(j): the original diagonal; g: [2][n].  Returns through *bad (0, or j+1 of the
+// failing pivot; the rows are then not scaled).
+// (With the root, the division, the scaled row and three barriers in each
+// step: 61 us for n = 48 and 100 us for a block of 64, now 46 and 68.)
+template <typename Orig>
+__device__ __forceinline__ void chol_cta(double *A, int ld, int n, double rel, Orig orig, double *g, int *bad) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // warp 0: pivot j, whose value is lane 0's d, and its g
+    auto pivot = [&](int j, double d) {
+        double t = 0.0;
+        if (lane == 0) {
+            if (!(isfinite(d) && d > 0.0 && d > rel * orig(j))) *bad = j + 1;
+            t = 1.0 / d;
         }
-        __syncthreads();
-        if (bad) break;
-        const double inv = 1.0 / piv;
-        double *uj = A + (int64_t)j * ld;
-        for (int c = j + 1 + tid; c < n; c += blockDim.x) uj[c] *= inv;
-        __syncthreads();
-        // trailing update A[r][c] -= U[j][r] U[j][c] on the upper triangle, r, c > j
-        for (int r = j + 1 + warp; r < n; r += nw) {
-            const double ujr = uj[r];
-            double *ar = A + (int64_t)r * ld;
-            for (int c = r + lane; c < n; c += 32) ar[c] -= ujr * uj[c];
+        t = __shfl_sync(0xffffffffu, t, 0);
+        for (int c = j + 1 + lane; c < n; c += 32) g[(j & 1) * n + c] = A[(int64_t)j * ld + c] * t;
+    };
+    if (warp == 0) pivot(0, A[0]);
+    __syncthreads();
+    // (pivot j + 1 may fail while a slow warp still tests for pivot j)
+    for (int j = 0; j + 1 < n && (*(volatile int *)bad == 0 || *(volatile int *)bad > j + 1); ++j) {
+        const double *wj = A + (int64_t)j * ld, *gj = g + (j & 1) * n;
+        if (warp == 0) {
+            const int r = j + 1;
+            double *ar = A + (int64_t)r * ld, d = 0.0;
+            const double f = gj[r];
+            for (int c = r + lane; c < n; c += 32) {
+                const double v = fma(-f, wj[c], ar[c]);
+                ar[c] = v;
+                if (c == r) d = v;
+            }
+            __syncwarp();
+            pivot(r, d);
+        } else {
+            for (int r = j + 1 + warp; r < n; r += nw - 1) {
+                const double f = gj[r];
+                double *ar = A + (int64_t)r * ld;
+                for (int c = r + lane; c < n; c += 32) ar[c] = fma(-f, wj[c], ar[c]);
+            }
         }
         __syncthreads();
     }
+    if (*bad) return;
+    for (int r = warp; r < n; r += nw) {
+        double *ar = A + (int64_t)r * ld;
+        const double s = sqrt(ar[r]), inv = 1.0 / s;
+        __syncwarp();
+        for (int c = r + lane; c < n; c += 32) ar[c] = c == r ? s : ar[c] * inv;
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(1024) k_chol(double *Ag, int lda, int n, double rel, int *status) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ double diag0[CHOL_SMEM_MAX], g[2 * CHOL_SMEM_MAX];
+    __shared__ int bad;
+    double *A = reinterpret_cast<double *>(smraw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     for (int r = warp; r < n; r += nw)
-        for (int c = lane; c < n; c += 32) {
-            const double v = c < r ? 0.0 : A[(int64_t)r * ld + c];
-            if (IN_SMEM) Ag[(int64_t)r * lda + c] = v;
-            else if (c < r) Ag[(int64_t)r * lda + c] = 0.0;
-        }
+        for (int c = lane; c < n; c += 32) A[r * n + c] = Ag[(int64_t)r * lda + c];
+    __syncthreads();
+    for (int j = tid; j < n; j += blockDim.x) diag0[j] = A[j * n + j];
+    if (tid == 0) bad = 0;
+    __syncthreads();
+    chol_cta(A, n, n, rel, [&](int j) { return diag0[j]; }, g, &bad);
+    for (int r = warp; r < n; r += nw)
+        for (int c = lane; c < n; c += 32) Ag[(int64_t)r * lda + c] = c < r ? 0.0 : A[r * n + c];
     if (tid == 0) status[0] = bad;
 }
 
@@ -193,6 +219,61 @@ __global__ void __launch_bounds__(256) k_trinv(const double *__restrict__ U, int
         __syncwarp();
     }
     for (int i = lane; i < n; i += 32) X[(int64_t)i * ldx + j] = i <= j ? x[i] : 0.0;
+}
+
+// a / u from r = 1 / u: the quotient with one correction of its remainder
+__device__ __forceinline__ double div_by(double a, double u, double r) {
+    const double q = a * r;
+    return fma(fma(-q, u, a), r, q);
+}
+
+// The same for n <= 32 Q, a warp to a row i of X: X U = I gives x_ij from the
+// diagonal to the right, x_ij = (delta_ij - sum_{k<j} x_ik U_kj) / U_jj, and each
+// x_ij is taken from the sums of all later columns at once.  No sum crosses the
+// lanes and the divisions use the diagonal's reciprocals: FP64 instructions,
+// 64 cycles each on a quarter of an SM, are what a step waits for (n = 256: 90 us,
+// 423 for the kernel above; n = 48: 13 and 56).
+template <int Q>
+__global__ void __launch_bounds__(64) k_trinv_rows(const double *__restrict__ U, int ldu, int n, double *__restrict__ X,
+                                                   int ldx) {
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 2 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    double acc[Q], u[Q], dg[Q], dr[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int l = 32 * q + lane;
+        acc[q] = l == i ? 1.0 : 0.0;
+        u[q] = l < n ? U[(int64_t)i * ldu + l] : 0.0;
+        dg[q] = l < n ? U[(int64_t)l * ldu + l] : 1.0;
+        dr[q] = 1.0 / dg[q];
+    }
+#pragma unroll
+    for (int b = 0; b < Q; ++b) {
+        if (32 * b + 31 < i) continue;
+        for (int j = max(i, 32 * b); j < min(n, 32 * b + 32); ++j) {
+            const int src = j & 31;
+            const double x = div_by(__shfl_sync(0xffffffffu, acc[b], src), __shfl_sync(0xffffffffu, dg[b], src),
+                                    __shfl_sync(0xffffffffu, dr[b], src));
+            // row j + 1 of U while row j is used
+            double un[Q];
+#pragma unroll
+            for (int q = b; q < Q; ++q) {
+                const int l = 32 * q + lane;
+                un[q] = l < n && j + 1 < n ? U[(int64_t)(j + 1) * ldu + l] : 0.0;
+            }
+            if (lane == src) acc[b] = x;
+            if (lane > src) acc[b] = fma(-x, u[b], acc[b]);
+#pragma unroll
+            for (int q = b + 1; q < Q; ++q) acc[q] = fma(-x, u[q], acc[q]);
+#pragma unroll
+            for (int q = b; q < Q; ++q) u[q] = un[q];
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int l = 32 * q + lane;
+        if (l < n) X[(int64_t)i * ldx + l] = acc[q];
+    }
 }
 
 // C = alpha op(A) op(B) + beta C for small dense FP64 matrices (row-major),
@@ -248,43 +329,20 @@ __global__ void k_chol_save_diag(double *A, int lda, int n) {
 
 // factor the bk x bk diagonal block at (k, k) in shared memory
 __global__ void __launch_bounds__(1024) k_chol_diag(double *Ag, int lda, int k, int bk, double rel, int *status) {
-    __shared__ double A[CHOL_NB * CHOL_NB];
-    __shared__ double piv;
+    __shared__ double A[CHOL_NB * CHOL_NB], diag0[CHOL_NB], g[2 * CHOL_NB];
     __shared__ int bad;
     if (*(volatile int *)status) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     double *blk = Ag + (int64_t)k * lda + k;
     for (int r = warp; r < bk; r += nw)
         for (int c = lane; c < bk; c += 32) A[r * bk + c] = blk[(int64_t)r * lda + c];
+    // the original diagonal (saved; the first entry is still in place)
+    if (tid < bk) diag0[tid] = k + tid == 0 ? Ag[0] : Ag[(int64_t)(k + tid) * lda];
     if (tid == 0) bad = 0;
     __syncthreads();
-    for (int j = 0; j < bk; ++j) {
-        if (tid == 0) {
-            const int g = k + j;
-            const double d0 = g == 0 ? A[0] : Ag[(int64_t)g * lda];   // original diagonal (saved)
-            const double d = A[j * bk + j];
-            if (!isfinite(d) || !(d > 0.0) || !(d > rel * d0)) {
-                bad = g + 1;
-                piv = 1.0;
-            } else {
-                piv = sqrt(d);
-            }
-            A[j * bk + j] = piv;
-        }
-        __syncthreads();
-        if (bad) break;
-        const double inv = 1.0 / piv;
-        double *uj = A + j * bk;
-        for (int c = j + 1 + tid; c < bk; c += blockDim.x) uj[c] *= inv;
-        __syncthreads();
-        for (int r = j + 1 + warp; r < bk; r += nw) {
-            const double ujr = uj[r];
-            for (int c = r + lane; c < bk; c += 32) A[r * bk + c] -= ujr * uj[c];
-        }
-        __syncthreads();
-    }
+    chol_cta(A, bk, bk, rel, [&](int j) { return diag0[j]; }, g, &bad);
     if (bad) {
-        if (tid == 0) atomicCAS(status, 0, bad);
+        if (tid == 0) atomicCAS(status, 0, k + bad);
         return;
     }
     for (int r = warp; r < bk; r += nw)
@@ -292,29 +350,43 @@ __global__ void __launch_bounds__(1024) k_chol_diag(double *Ag, int lda, int k, 
 }
 
 // panel: rows k..k+bk-1, columns c >= k+bk, x = U_kk^-T a by forward
-// substitution, x_i = (a_i - sum_{l<i} U_li x_l) / U_ii, in place
+// substitution, x_i = (a_i - sum_{l<i} U_li x_l) / U_ii, in place.  Four lanes to
+// a column, lane s holding x_l for l = s mod 4: a warp's FP64 instruction takes
+// the same time for any number of its lanes' columns, so the sums are split
+// rather than the columns packed (n = 256: 48 us a panel, 115 with a column a lane).
 __global__ void __launch_bounds__(128) k_chol_panel(double *Ag, int lda, int n, int k, int bk, const int *status) {
-    __shared__ double U[CHOL_NB * CHOL_NB];
+    constexpr int LD = CHOL_NB + 1;
+    __shared__ double U[CHOL_NB * LD], inv[CHOL_NB];
     if (*(volatile const int *)status) return;
     const int tid = threadIdx.x;
     const double *blk = Ag + (int64_t)k * lda + k;
-    for (int e = tid; e < bk * bk; e += blockDim.x) U[e] = blk[(int64_t)(e / bk) * lda + e % bk];
+    for (int e = tid; e < bk * bk; e += blockDim.x) U[e / bk * LD + e % bk] = blk[(int64_t)(e / bk) * lda + e % bk];
     __syncthreads();
-    const int c = k + bk + blockIdx.x * blockDim.x + tid;
-    if (c >= n) return;
-    double *col = Ag + (int64_t)k * lda + c;
-    double x[CHOL_NB];   // the column's solution, in registers (fully unrolled loops)
+    if (tid < bk) inv[tid] = 1.0 / U[tid * LD + tid];
+    __syncthreads();
+    const int s = tid & 3, c = k + bk + blockIdx.x * (blockDim.x / 4) + (tid >> 2);
+    double *col = Ag + (int64_t)k * lda + min(c, n - 1);
+    double x[CHOL_NB / 4];   // a, then the solution
+#pragma unroll
+    for (int m = 0; m < CHOL_NB / 4; ++m) x[m] = 4 * m + s < bk ? col[(int64_t)(4 * m + s) * lda] : 0.0;
+    __syncwarp();
 #pragma unroll
     for (int i = 0; i < CHOL_NB; ++i) {
         if (i < bk) {
-            double t = col[(int64_t)i * lda];
+            double t = 0.0;
 #pragma unroll
-            for (int l = 0; l < i; ++l) t -= U[l * bk + i] * x[l];
-            t /= U[i * bk + i];
-            x[i] = t;
-            col[(int64_t)i * lda] = t;
+            for (int m = 0; 4 * m < i; ++m)
+                if (4 * m + s < i) t = fma(U[(4 * m + s) * LD + i], x[m], t);
+            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            t += __shfl_xor_sync(0xffffffffu, t, 2);
+            const double v = div_by(x[i / 4] - t, U[i * LD + i], inv[i]);
+            if (s == i % 4) x[i / 4] = v;
         }
     }
+    if (c >= n) return;
+#pragma unroll
+    for (int m = 0; m < CHOL_NB / 4; ++m)
+        if (4 * m + s < bk) col[(int64_t)(4 * m + s) * lda] = x[m];
 }
 
 __global__ void k_zero_lower(double *A, int lda, int n) {
@@ -328,8 +400,8 @@ __global__ void k_zero_lower(double *A, int lda, int n) {
 int cholesky(double *A, int lda, int n, double rel, int *status_dev, cudaStream_t st) {
     if (n <= CHOL_SMEM_MAX) {
         const size_t sm = sizeof(double) * (size_t)n * n;
-        RS_TRY(smem_optin((const void *)k_chol<true>, sm));
-        k_chol<true><<<1, 1024, sm, st>>>(A, lda, n, rel, status_dev);
+        RS_TRY(smem_optin((const void *)k_chol, sm));
+        k_chol<<<1, 1024, sm, st>>>(A, lda, n, rel, status_dev);
         RS_LAUNCH_CHECK();
         return RS_OK;
     }
@@ -341,7 +413,7 @@ int cholesky(double *A, int lda, int n, double rel, int *status_dev, cudaStream_
         k_chol_diag<<<1, 1024, 0, st>>>(A, lda, k, bk, rel, status_dev);
         RS_LAUNCH_CHECK();
         if (m == 0) break;
-        k_chol_panel<<<(m + 127) / 128, 128, 0, st>>>(A, lda, n, k, bk, status_dev);
+        k_chol_panel<<<(m + 31) / 32, 128, 0, st>>>(A, lda, n, k, bk, status_dev);
         RS_LAUNCH_CHECK();
         double *Xk = A + (int64_t)k * lda + k + bk, *C = A + (int64_t)(k + bk) * lda + k + bk;
         RS_TRY(gemm_small(m, m, bk, -1.0, Xk, lda, true, Xk, lda, false, 1.0, C, lda, st));
@@ -352,6 +424,15 @@ int cholesky(double *A, int lda, int n, double rel, int *status_dev, cudaStream_
 }
 
 int tri_inv(const double *U, int ldu, int n, double *X, int ldx, cudaStream_t st) {
+    const unsigned rows2 = (unsigned)(n + 1) / 2;
+    if (n <= 32) k_trinv_rows<1><<<rows2, 64, 0, st>>>(U, ldu, n, X, ldx);
+    else if (n <= 64) k_trinv_rows<2><<<rows2, 64, 0, st>>>(U, ldu, n, X, ldx);
+    else if (n <= 128) k_trinv_rows<4><<<rows2, 64, 0, st>>>(U, ldu, n, X, ldx);
+    else if (n <= 256) k_trinv_rows<8><<<rows2, 64, 0, st>>>(U, ldu, n, X, ldx);
+    if (n <= 256) {
+        RS_LAUNCH_CHECK();
+        return RS_OK;
+    }
     constexpr int WPB = 8;   // columns (warps) per CTA
     const size_t sm = sizeof(double) * (size_t)WPB * n;
     if (sm > 48 * 1024) RS_TRY(smem_optin((const void *)k_trinv, sm));

@@ -136,3 +136,31 @@ def test_piece_overlap_edges(box, nx, ny, pad):
         a, b = A.double().cpu().numpy(), B.double().cpu().numpy()
         steps = 6 * (min(g.npts, 2048) // 16 + 4)
         assert np.all(np.abs(S - g.dV * (a.T @ b)) <= g.dV * (2 * steps + 4) * 2.0 ** -24 * (np.abs(a).T @ np.abs(b)))
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 129, 160, 161, 257])
+def test_factor_and_inverse_edges(n):
+    """The triangular factor's inverse at the edges of its kernels (32, 64, 128
+    and 256 columns; one CTA up to 160): C^T S C = 1 and C upper triangular.
+    Tolerance: n rounded terms in each of the factor, the inverse and numpy's
+    products, times the condition of S (below 2)."""
+    from paper_1306_2953_gb300 import api
+    g = api.Grid.box(24, 24, 24, 0.3)
+    rng = np.random.default_rng(n)
+    P = torch.from_numpy(rng.standard_normal((g.npts, n))).cuda()
+    p = P.cpu().numpy()
+    S = g.dV * (p.T @ p)
+    assert n == 1 or np.linalg.cond(S) < 2
+    C = api.orthonormalize(g, P).cpu().numpy()
+    assert np.array_equal(C, np.triu(C))
+    assert np.abs(C.T @ S @ C - np.eye(n)).max() <= 16 * (n + 8) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("n,bad", [(5, 3), (48, 47), (130, 64), (200, 130)])
+def test_dependent_column_is_refused(n, bad):
+    from paper_1306_2953_gb300 import api
+    g = api.Grid.box(12, 12, 12, 0.3)
+    P = torch.from_numpy(np.random.default_rng(n).standard_normal((g.npts, n))).cuda()
+    P[:, bad] = 0.0
+    with pytest.raises(Exception):
+        api.orthonormalize(g, P)
