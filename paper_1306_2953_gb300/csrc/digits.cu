@@ -18,8 +18,9 @@
 // accumulator t everything up to t = 3 is exact and a rounding of a later
 // one is below 2^-56 of the largest product.  So the result is the exact
 // sum of products of operands rounded to s bits: NS = 8 (FP64), 7 (overlap of
-// FP32 data at FP64-like accuracy) or 5 (rotation of FP32 data).  (Ozaki, Ogita, Oishi and Rump
-// 2012 give the scheme of error-free splittings of a matrix product.)
+// FP32 data at FP64-like accuracy) or 5 (rotation of FP32 data).  (Ozaki,
+// Ogita, Oishi and Rump 2012 give the scheme of error-free splittings of a
+// matrix product.)
 //
 // Kernel: 8 converter warps and one MMA warp per CTA, one CTA per SM, a 128 x
 // BN tile of the result.  Stage (32 steps of the contraction, two stages): the
@@ -35,12 +36,12 @@
 // contraction.  Every wait is bounded; a CTA whose wait gives up writes NaN.
 //
 // What bounds it, and what it measured (overlap of 256 x 256 columns over
-// 658 416 points): FP64 2.89 ms, FP32 data 2.63 ms, against 69.8 ms by FP64 FMA
+// 658 416 points): FP64 2.95 ms, FP32 data 2.64 ms, against 69.8 ms by FP64 FMA
 // and 14.3 ms by compensated FP32 sums before.  The products alone take
 // 1.65 ms (28 % more than the tensor pipe needs: the readouts); the
 // conversion, 20 integer instructions per value on a pipe of half rate,
 // accounts for the rest, the pass that finds the column exponents for 0.4 ms.
-// Every size gains (64 x 64: 4.4 -> 0.44 ms FP64, 0.94 -> 0.40 ms FP32), so
+// Every size gains (64 x 64: 4.4 -> 0.45 ms FP64, 0.94 -> 0.41 ms FP32), so
 // there is no other path.
 #include <cuda_fp16.h>
 
@@ -1121,7 +1122,7 @@ template <typename T, int NS, int BN, int NBLK, bool ONE> int launch_rot(RotArgs
 // k_piece_c) come by bulk copies, four stages of 32 states ahead; two
 // accumulator sets let the products of a tile run while the last one's are
 // stored.  In place the CTAs of a row tile are a cluster, as in k_digit_rot.
-// What it measured (658 416 rows, 256 -> 256 / 256 -> 64 columns): 678 / 303 us,
+// What it measured (658 416 rows, 256 -> 256 / 256 -> 64 columns): 685 / 302 us,
 // 943 / 564 us for a split pass and a product kernel before.
 
 struct PieceArgs {
@@ -1396,7 +1397,7 @@ template <int BN> int launch_piece(PieceArgs a, const double *C, int64_t ldc, vo
 // an FP32 value is read once per tile and no pieces are written.  Work items (chunk,
 // tile), tiles fastest, are dealt round robin to one CTA per SM; the readout of
 // an item overlaps the products of the next.
-// Measured (658 416 points): 256 x 64 columns 338 us, 256 x 256 787 us; 800 and
+// Measured (658 416 points): 256 x 64 columns 340 us, 256 x 256 790 us; 800 and
 // 1382 us with a separate pass that wrote the pieces to memory.
 
 struct PieceGramArgs {
