@@ -1110,7 +1110,12 @@ int learned_apply(const rs_ham *h, const float *R, int64_t ldr, float *W, int64_
     // Few columns do not fill the row kernels: us at 1 / 2 / 3 / 4 columns, row
     // kernels 148 / 167 / 205 / 188 on 103 331 points and 454 / 541 / 663 / 726 on
     // 654 520, thread per point and state 112 / 172 / 162 / 278 and 442 / 774 / 742 / 1396.
-    if (nb <= 3) {
+    // Nor do 5 or 7, or 9 to 11 (a CTA's rows leave its last round half empty), until
+    // the grid has rounds enough: 5 / 7 columns 156 / 161 against 113 / 142 on 41 625 points, 250 / 309
+    // against 230 / 287 on 120 681, 283 / 348 against 285 / 354 on 154 249; 9 / 11
+    // columns 176 / 185 against 167 / 178 on 41 625, 221 / 243 against 239 / 275 on 71 387.
+    const bool per_point = nb <= 3 || (np < 150000 && (nb == 5 || nb == 7)) || (np < 50000 && nb >= 5 && nb <= 11);
+    if (per_point) {
         const int n32 = (int)np;
         float *x = act, *a1 = x + np * nb, *a2 = a1 + np * NC * nb;
         const unsigned blocks = (unsigned)((np * nb + 255) / 256);
