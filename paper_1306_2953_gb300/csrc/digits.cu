@@ -94,9 +94,13 @@ __device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile i
 }
 // The MMA warp runs its loop as a whole, so that descriptors stay in uniform
 // registers; `lead` (one lane) issues.
-// the whole warp: true only when every lane's wait ended (no lane goes on alone)
+// the whole warp: true only when every lane's wait ended (no lane goes on alone).
+// The lanes leave it together, as the warp-wide loads of tensor memory need
+// (they run apart in the loop, and in stores and atomics of ragged tiles before it).
 __device__ __forceinline__ bool dg_wait_warp(uint64_t *b, uint32_t parity, volatile int *bad) {
-    return __all_sync(0xffffffffu, dg_wait(b, parity, bad));
+    const bool all = __all_sync(0xffffffffu, dg_wait(b, parity, bad));
+    __syncwarp();
+    return all;
 }
 __device__ __forceinline__ void dg_mma(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum,
                                        uint32_t lead) {
@@ -1303,6 +1307,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
             for (int c = 0; c < CPT; c += 32) {
                 uint32_t r[32];
                 float v[32];
+                __syncwarp();   // rows beyond the last skipped the stores of the round before
                 dg_tmem_ld32(t0 + BN + c, r);
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
@@ -1519,6 +1524,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
 #pragma unroll
             for (int c = 0; c < CPT; c += 32) {
                 uint32_t r[32];
+                __syncwarp();   // rows beyond the last skipped the sums of the round before
                 dg_tmem_ld32(t0 + c, r);
                 if (c + 32 >= CPT) {
                     DG_FENCE_BEFORE();
