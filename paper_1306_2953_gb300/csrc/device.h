@@ -96,7 +96,7 @@ struct PoolBuf {
 
 // Launch whose start may overlap the end of the kernel before it in the stream:
 // the kernel calls pdl_wait() before it reads or writes anything that the
-// stream's earlier work touches.
+// stream's earlier work touches, and reads what that work wrote by ld_fresh().
 template <typename... P, typename... A>
 int launch_overlapped(void (*fn)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg{};
@@ -116,6 +116,27 @@ int launch_overlapped(void (*fn)(P...), dim3 grid, unsigned threads, size_t smem
 // All earlier work of the stream is complete and visible (at once when the
 // kernel was launched without overlap).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+// Load, behind pdl_wait(), of what an earlier kernel of the stream wrote.  That
+// kernel may still be running when this one starts, so such data is not
+// read-only for this kernel's life, as the loads that the compiler makes of
+// const __restrict__ pointers and of __ldg require; and an ordinary load of such a pointer
+// may be moved ahead of the wait.  This one is neither.
+template <typename T> __device__ __forceinline__ T ld_fresh(const T *p) {
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one access");
+    if constexpr (sizeof(T) == 4) {
+        uint32_t r;
+        asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(r) : "l"(p));
+        return *reinterpret_cast<const T *>(&r);
+    } else if constexpr (sizeof(T) == 8) {
+        unsigned long long r;
+        asm volatile("ld.global.b64 %0, [%1];\n" : "=l"(r) : "l"(p));
+        return *reinterpret_cast<const T *>(&r);
+    } else {
+        uint4 r;
+        asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+        return *reinterpret_cast<const T *>(&r);
+    }
+}
 // The next kernel of the stream may be started (it waits in pdl_wait).  Only where
 // its CTAs fill every SM anyway: a small grid that starts in a tail is packed
 // on the few SMs that are free.

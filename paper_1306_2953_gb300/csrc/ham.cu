@@ -75,6 +75,15 @@ __device__ __forceinline__ Four<double> load4(const double *p) {
     return {u.x, u.y, v.x, v.y};
 }
 
+__device__ __forceinline__ Four<float> fresh4(const float *p) {
+    const float4 v = ld_fresh(reinterpret_cast<const float4 *>(p));
+    return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Four<double> fresh4(const double *p) {
+    const double2 u = ld_fresh(reinterpret_cast<const double2 *>(p)), v = ld_fresh(reinterpret_cast<const double2 *>(p) + 1);
+    return {u.x, u.y, v.x, v.y};
+}
+
 // ------------------------------------------------- projection integrals ---
 
 // Grid (atoms * split, state groups): each CTA sums 1 / split of an atom's
@@ -114,7 +123,7 @@ __global__ void __launch_bounds__(NT) k_project(HamDev<T> d, const T *__restrict
 #pragma unroll 8
     for (int i = i0 + r; i < i1; i += R) {
         const int p = __ldg(d.sph_idx + i);
-        const T v = __ldg(ps + (int64_t)p * ldp);
+        const T v = ld_fresh(ps + (int64_t)p * ldp);
         const Four<T> g = load4(d.sph_gam + 4 * (int64_t)i);
         a0 += g.a * v;
         a1 += g.b * v;
@@ -185,7 +194,7 @@ __global__ void __launch_bounds__(NTP4, RS_PROJ_CTAS) k_project_f32(HamDev<float
         for (int u = 0; u < UN; ++u) {
             v[u] = g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (p[u] >= 0) {
-                v[u] = __ldg(reinterpret_cast<const float4 *>(ps + (int64_t)p[u] * ldp));
+                v[u] = ld_fresh(reinterpret_cast<const float4 *>(ps + (int64_t)p[u] * ldp));
                 g[u] = __ldg(reinterpret_cast<const float4 *>(d.sph_gam) + i + u * STEP);
             }
         }
@@ -315,8 +324,8 @@ __global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__
             all = all && (n.x | n.y | n.z | n.w) >= 0;
         }
         const int p = p0 + q;
-        const int4 inf = __ldg(d.pinfo + p);
-        const P c = *reinterpret_cast<const P *>(ps + (int64_t)p * ldp);
+        const int4 inf = ld_fresh(d.pinfo + p);
+        const P c = ld_fresh(reinterpret_cast<const P *>(ps + (int64_t)p * ldp));
         // from the smallest weight to the largest, so that the roundings of the
         // large terms come last
         P acc;
@@ -327,7 +336,7 @@ __global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__
             for (int j = 3; j >= 0; --j) {
                 P n[6];
 #pragma unroll
-                for (int g = 0; g < 6; ++g) n[g] = *reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp);
+                for (int g = 0; g < 6; ++g) n[g] = ld_fresh(reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp));
                 add_to(n[0], n[1]);
                 add_to(n[2], n[3]);
                 add_to(n[4], n[5]);
@@ -344,7 +353,7 @@ __global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__
                 for (int g = 0; g < 6; ++g) {
 #pragma unroll
                     for (int i = 0; i < V; ++i) n[g].v[i] = T(0);
-                    if (id[g][j] >= 0) n[g] = *reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp);
+                    if (id[g][j] >= 0) n[g] = ld_fresh(reinterpret_cast<const P *>(ps + (int64_t)id[g][j] * ldp));
                 }
                 add_to(n[0], n[1]);
                 add_to(n[2], n[3]);
@@ -362,7 +371,7 @@ __global__ void __launch_bounds__(GT_NT) k_gather(HamDev<T> d, const int32_t *__
             const T *cp = cproj + ((int64_t)A * nb + lane * V) * 4;
 #pragma unroll
             for (int i = 0; i < V; ++i) {
-                const Four<T> c4 = load4(cp + 4 * i);
+                const Four<T> c4 = fresh4(cp + 4 * i);
                 acc.v[i] += g.a * c4.a + g.b * c4.b + g.c * c4.c + g.d * c4.d;
             }
         }

@@ -112,7 +112,10 @@ template <typename T, int V, int LPP> __device__ __forceinline__ void cg_reduce(
 // num / den (0 where den is 0) of the thread's columns
 template <typename T, int V, int LPP> __device__ __forceinline__ void cg_ratio(const double *num, const double *den, T (&q)[V]) {
     __shared__ T ratio[LPP * V];
-    if (threadIdx.x < LPP * V) ratio[threadIdx.x] = den[threadIdx.x] != 0.0 ? (T)(num[threadIdx.x] / den[threadIdx.x]) : T(0);
+    if (threadIdx.x < LPP * V) {
+        const double b = ld_fresh(den + threadIdx.x);
+        ratio[threadIdx.x] = b != 0.0 ? (T)(ld_fresh(num + threadIdx.x) / b) : T(0);
+    }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < V; ++i) q[i] = ratio[(threadIdx.x % LPP) * V + i];
@@ -148,8 +151,8 @@ __global__ void __launch_bounds__(CG_NT) k_cg_pap(const T *__restrict__ P, const
     DotSum<T> d[V];
 #pragma unroll 2
     for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
-        const Cols<T, V> x = *reinterpret_cast<const Cols<T, V> *>(P + p * (LPP * V) + c);
-        const Cols<T, V> y = *reinterpret_cast<const Cols<T, V> *>(AP + p * (LPP * V) + c);
+        const Cols<T, V> x = ld_fresh(reinterpret_cast<const Cols<T, V> *>(P + p * (LPP * V) + c));
+        const Cols<T, V> y = ld_fresh(reinterpret_cast<const Cols<T, V> *>(AP + p * (LPP * V) + c));
 #pragma unroll
         for (int i = 0; i < V; ++i) d[i].add(x.v[i], y.v[i]);
     }
@@ -171,7 +174,8 @@ __global__ void __launch_bounds__(CG_NT) k_cg_update1(T *__restrict__ X, int64_t
     cg_ratio<T, V, LPP>(rr, pap, a);
     DotSum<T> d[V];
     for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
-        const C pv = *reinterpret_cast<const C *>(P + p * (LPP * V) + c), ap = *reinterpret_cast<const C *>(AP + p * (LPP * V) + c);
+        const C pv = ld_fresh(reinterpret_cast<const C *>(P + p * (LPP * V) + c));
+        const C ap = ld_fresh(reinterpret_cast<const C *>(AP + p * (LPP * V) + c));
         C r = *reinterpret_cast<const C *>(R + p * (LPP * V) + c), x;
         T *xp = X + p * ldx + c;
         if (xvec) x = *reinterpret_cast<const C *>(xp);
@@ -207,7 +211,7 @@ __global__ void __launch_bounds__(CG_NT) k_cg_update2(const T *__restrict__ R, T
     cg_ratio<T, V, LPP>(rrn, rr, b);
 #pragma unroll 2
     for (int64_t p = blockIdx.x * (int64_t)(CG_NT / LPP) + threadIdx.x / LPP; p < npts; p += (int64_t)gridDim.x * (CG_NT / LPP)) {
-        const C r = *reinterpret_cast<const C *>(R + p * (LPP * V) + c);
+        const C r = ld_fresh(reinterpret_cast<const C *>(R + p * (LPP * V) + c));
         C q = *reinterpret_cast<const C *>(P + p * (LPP * V) + c);
 #pragma unroll
         for (int i = 0; i < V; ++i) q.v[i] = r.v[i] + b[i] * q.v[i];

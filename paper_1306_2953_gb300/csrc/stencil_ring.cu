@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(NT, 1) k_hpsi_ring(Args a) {
         const float *part = a.part + (((int64_t)at * gridDim.y + grp) * a.split * SG + st) * 4 + q;
         float t = 0.f;
 #pragma unroll 8
-        for (int k = 0; k < a.split; ++k) t += __ldg(part + k * 4 * SG);
+        for (int k = 0; k < a.split; ++k) t += ld_fresh(part + k * 4 * SG);
         cs[(4 * la + q) * SG + st] = t;
     }
     __syncthreads();
