@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             for (int u = 0; u < 3; ++u) load(u, blockIdx.y, 0);
         }
         while (ok) {
-            bool plain = false, flush = false, end = false;
+            bool plain = false, flush = false, end = false, told = false;
             if (it == nst) {
                 tile += gridDim.y;
                 ++j;
@@ -1024,10 +1024,14 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     dg_arrive(&b.full[s]);
                 }
-                if (lasts) rows_read();
+                told = lasts;
                 flush = kb % DG_DRAIN == 0 && open;
             }
             if (flush) readout();
+            // behind the readout of the tile before, whose rows_read it waits for: a
+            // thread that signalled twice without that wait (a tile of one stage)
+            // would stand in for one that has not read its rows yet
+            if (told) rows_read();
             if (end) break;
             if (plain) {
                 // a row or column beyond the digits' range: plain sums, then the
@@ -1361,6 +1365,10 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
                 }
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 dg_arrive(&full[s]);
+                // the readout waits for rd of the tile before: ahead of this tile's
+                // arrival, or a thread would count twice in one phase (n <= 32: the
+                // first stage is the last) and rows be overwritten before a peer reads them
+                if (it == 0 && ptile >= 0) readout(ptile, j - 1);
                 if (last && a.cluster)
                     for (int r = 0; r < (int)gridDim.x; ++r)
                         asm volatile(
@@ -1368,7 +1376,6 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
                             " mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(dg_su32(&rd)),
                             "r"(r)
                             : "memory");
-                if (it == 0 && ptile >= 0) readout(ptile, j - 1);
             }
             ptile = tile;
         }
