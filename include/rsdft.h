@@ -408,7 +408,9 @@ int64_t rs_cg_workspace_bytes(int64_t npts, int ncols, int dtype);
 /* Training targets: exactly n_iter conjugate-gradient iterations from X = 0
  * on (-1/2 Lap + sigma) X = B, one independent system per column.  h must be
  * a Hamiltonian built with V = sigma everywhere and no projectors; B_dev, X_dev
- * [npts][ld] (ncols columns, a power of two <= 64).  Asynchronous. */
+ * [npts][ld] (ncols columns, a power of two <= 64).  work_dev starts on a
+ * boundary of 16 bytes, or of one row of ncols values where that is less.
+ * Asynchronous. */
 int rs_shifted_poisson_cg(rs_ham *h, const void *B_dev, void *X_dev, int64_t ld, int ncols, int n_iter, int dtype,
                           void *work_dev, void *stream);
 

@@ -925,6 +925,15 @@ extern "C" int rs_shifted_poisson_cg(rs_ham *h, const void *B_dev, void *X_dev, 
     if (ncols < 1 || ncols > 64 || (ncols & (ncols - 1))) return fail(RS_EINVAL, "rs_shifted_poisson_cg: ncols must be a power of two <= 64");
     if (ld < ncols || n_iter < 0) return fail(RS_EINVAL, "rs_shifted_poisson_cg: bad ld or n_iter");
     if (dtype != RS_F64 && dtype != RS_F32) return fail(RS_EINVAL, "rs_shifted_poisson_cg: bad dtype");
+    // the rows in the workspace are read and written 16 bytes (or a row) at a time,
+    // as the H psi kernels need them
+    const int es = dtype == RS_F64 ? 8 : 4, need = std::min(ncols * es, 16);
+    if ((uintptr_t)work_dev % need) {
+        if (n_iter > 0) return fail(RS_EINVAL, "rs_shifted_poisson_cg: misaligned workspace");
+        // no iteration, no workspace: X = 0
+        RS_CUDA(cudaMemset2DAsync(X_dev, (size_t)ld * es, 0, (size_t)ncols * es, (size_t)ham_npts(h), (cudaStream_t)stream));
+        return RS_OK;
+    }
     return shifted_poisson_cg(h, B_dev, ld, X_dev, ld, ncols, n_iter, dtype, work_dev, (cudaStream_t)stream);
 }
 
