@@ -243,7 +243,7 @@ int rs_overlap_block(const rs_grid *g, const void *X_dev, int64_t ldx, int nx, c
  * rs_overlap_block).  Workspace (device, caller-owned):
  * rs_tc_workspace_bytes(rows_a, rows_b, K) bytes, where the overlap has
  * rows_a = nx, rows_b = ny, K = npts and the rotation rows_a = npts,
- * rows_b = m, K = n.  Blocking (they synchronise the stream); a kernel whose
+ * rows_b = m, K = n, on a 16-byte boundary.  Blocking (they synchronise the stream); a kernel whose
  * bounded pipeline wait gives up writes NaN. */
 int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K);
 

@@ -1665,6 +1665,13 @@ using namespace rs;
 
 namespace {
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+
+// the pieces of C are stored and copied 16 bytes at a time
+int check_work(const void *work) {
+    if (!work) return fail(RS_EINVAL, "tensor-core call: null workspace");
+    if (!aligned16(work)) return fail(RS_EINVAL, "tensor-core call: workspace not on a 16-byte boundary");
+    return RS_OK;
+}
 }  // namespace
 
 extern "C" int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K) {
@@ -1676,7 +1683,7 @@ extern "C" int rs_overlap_block_tc(const rs_grid *g, const float *X_dev, int64_t
                                    int64_t ldy, int ny, double *S_dev, int64_t lds, void *work_dev, void *stream) {
     if (!g || !X_dev || !Y_dev || !S_dev) return fail(RS_EINVAL, "rs_overlap_block_tc: null argument");
     if (nx < 1 || ny < 1 || ldx < nx || ldy < ny || lds < ny) return fail(RS_EINVAL, "rs_overlap_block_tc: bad sizes");
-    if (!work_dev) return fail(RS_EINVAL, "tensor-core call: null workspace");
+    RS_TRY(check_work(work_dev));
     cudaStream_t st = (cudaStream_t)stream;
     RS_TRY(piece_gram(X_dev, ldx, nx, Y_dev, ldy, ny, g->npts, g->h * g->h * g->h, S_dev, lds, st));
     RS_CUDA(cudaStreamSynchronize(st));
@@ -1687,7 +1694,7 @@ extern "C" int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const dou
                                float *Y_dev, int64_t ldy, int64_t npts, void *work_dev, void *stream) {
     if (!X_dev || !C_dev || !Y_dev) return fail(RS_EINVAL, "rs_rotate_block: null argument");
     if (n < 1 || m < 1 || npts < 1 || ldx < n || ldy < m || ldc < m) return fail(RS_EINVAL, "rs_rotate_block: bad sizes");
-    if (!work_dev) return fail(RS_EINVAL, "tensor-core call: null workspace");
+    RS_TRY(check_work(work_dev));
     cudaStream_t st = (cudaStream_t)stream;
     RS_TRY(rotate_any(X_dev, ldx, n, C_dev, ldc, m, Y_dev, ldy, npts, 1.0, 0.0, work_dev, st));
     RS_CUDA(cudaStreamSynchronize(st));
