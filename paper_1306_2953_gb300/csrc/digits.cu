@@ -701,7 +701,7 @@ __device__ __forceinline__ double dg_value(int64_t H, int64_t L, int ex) {
 }
 
 struct RotBars {
-    uint64_t keyfull[2], keyfree[2], rd;
+    uint64_t keyfull[2], keyfree[2], rd, sums;
     int plain[2][4];   // per half and key warp: a row beyond the digits' range
 };
 
@@ -731,6 +731,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             dg_bar_init(&rb.keyfree[i], DG_CT + 1);   // the converters and the MMA warp's first lane
         }
         dg_bar_init(&rb.rd, DG_CT * (a.cluster ? gridDim.x : 1));
+        dg_bar_init(&rb.sums, DG_CT);
     }
     for (int i = tid; i < NBLK * BN; i += DG_NT) eb[i] = 0;
     dg_setup<NS>(b, C::TMEM);
@@ -987,7 +988,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
         };
         // One loop over the stages of all tiles; it == nst: the next tile is due.
         int tile = (int)blockIdx.y - (int)gridDim.y, j = -1, g = 0, it = nst, kb = 0, blk = 0, h = 0;
-        int ex0 = 0, ex1 = 0, er = 0;
+        int ex0 = 0, ex1 = 0, er = 0, nplain = 0;
         if ((int)blockIdx.y < ntiles) {
 #pragma unroll
             for (int u = 0; u < 3; ++u) load(u, blockIdx.y, 0);
@@ -1046,7 +1047,10 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                             t = fma((double)a.X[p * a.ldx + k], __ldg(a.C + (int64_t)k * a.ldc + c), t);
                     sum[i] = (T)t;
                 }
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");   // every converter of this CTA has read its row
+                // every converter of this CTA has read its row (a bounded wait: a warp
+                // whose own wait has given up does not come)
+                dg_arrive(&rb.sums);
+                ok = dg_wait_warp(&rb.sums, nplain++ & 1, &b.bad);
                 rows_read();
                 if (a.cluster) ok = dg_wait_warp(&rb.rd, j & 1, &b.bad) && ok;
                 if (owns && (int64_t)tile * DG_M + row < a.npts)
@@ -1056,7 +1060,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                             T v = sum[i], *y = a.Y + p * a.ldy + c;
                             if (a.alpha != 1.0) v *= al;
                             if (a.beta != 0.0) v += be * *y;
-                            *y = v;
+                            *y = ok ? v : (T)__longlong_as_double(0x7ff8000000000000ll);
                         }
                     }
                 if (tile + (int)gridDim.y < ntiles) {

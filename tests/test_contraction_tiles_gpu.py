@@ -49,3 +49,28 @@ def test_digit_rotation_in_place_many_tiles(dtype, n):
     tol = ((n + 8) * 2.0 ** -53 * (x.abs() @ C.abs()) +
            8 * n * 2.0 ** -s * x.abs().amax(1)[:, None] * C.abs().amax(0)[None, :] + 2 * u * ref.abs())
     assert bool(((P.double() - ref).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("n", [40, 130, 300])
+def test_rows_beyond_the_digits_in_many_tiles(dtype, n):
+    """Rows that the digits cannot hold in some of the row tiles (one that follows
+    another, the first and the last among them): those tiles take plain sums, in
+    one CTA (n = 40) and in clusters.  Tolerance: a plain sum of n products in
+    FP64, rounded once to the type."""
+    from paper_1306_2953_gb300 import api
+    t, tiny, u = (torch.float64, 1e-200, 2.0 ** -53) if dtype == "f64" else (torch.float32, 1e-30, 2.0 ** -24)
+    g = api.Grid.box(31, 31, 32, 0.3)
+    rng = np.random.default_rng(n)
+    P = torch.from_numpy(rng.uniform(-1, 1, (g.npts, n))).to(t).cuda()
+    tiles = [0, 1, 7, 100, 101, 155, 200, (g.npts - 1) // 128]
+    for k in tiles:
+        P[min(128 * k + 17, g.npts - 1)] *= tiny
+    x = P.double().clone()
+    C = api.orthonormalize(g, P)
+    ref, mag = x @ C, x.abs() @ C.abs()
+    err = (P.double() - ref).abs()
+    for k in tiles:
+        r = slice(128 * k, min(128 * k + 128, g.npts))
+        assert bool((err[r] <= (2 * (n + 8) * 2.0 ** -53 + 2 * u) * mag[r]).all())
+    assert bool((err <= 64 * n * u * x.abs().amax(1)[:, None] * C.abs().amax(0)[None, :]).all())
