@@ -243,8 +243,10 @@ int rs_overlap_block(const rs_grid *g, const void *X_dev, int64_t ldx, int nx, c
  * rs_overlap_block).  Workspace (device, caller-owned):
  * rs_tc_workspace_bytes(rows_a, rows_b, K) bytes, where the overlap has
  * rows_a = nx, rows_b = ny, K = npts and the rotation rows_a = npts,
- * rows_b = m, K = n, on a 16-byte boundary.  Blocking (they synchronise the stream); a kernel whose
- * bounded pipeline wait gives up writes NaN. */
+ * rows_b = m, K = n, on a 16-byte boundary.  Blocking (they
+ * read a status word in the workspace); a kernel whose bounded pipeline wait
+ * gives up writes NaN where it has not stored its results, and the call
+ * returns RS_ETIMEOUT. */
 int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K);
 
 /* S = dV X^T Y (Eq. 5) for FP32 X [npts][ldx] (nx columns) and Y (ny
@@ -257,6 +259,14 @@ int rs_overlap_block_tc(const rs_grid *g, const float *X_dev, int64_t ldx, int n
  * [npts][ldy]; Y may be X or overlap it (X is copied to the workspace first where needed). */
 int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const double *C_dev, int64_t ldc, int m, float *Y_dev,
                     int64_t ldy, int64_t npts, void *work_dev, void *stream);
+
+/* Test hook of the failure detection: barrier tests after which a bounded wait
+ * inside a contraction kernel gives up, for the overlaps and for the rotations of
+ * the calling host thread's calls from now on (< 0: the default, 100000, about two seconds; 0:
+ * at once).  A kernel whose wait has given up writes NaN in all the results that
+ * it has not stored.  rs_overlap_block_tc, rs_rotate_block and the eigensolver's sweeps then
+ * return RS_ETIMEOUT; of the other calls the NaN are the sign. */
+int rs_contraction_wait_limit(int overlap_tests, int rotation_tests);
 
 /* Device workspace (bytes) that rs_orthonormalize / rs_subspace_diag need
  * for nst states. */
@@ -371,9 +381,9 @@ int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void *Psi0_dev, 
  * eigenvalues when the schedule took that step (rs_solver_stats says which);
  * resnorm_dev the residual norms the sweep measured.  n_converged: host,
  * states with residual norm <= tol (may be NULL).  Blocking (reads the
- * residuals).  Errors: RS_ENAN (a non-finite residual; a tensor-core kernel
- * whose bounded wait gave up writes NaN), RS_ETIMEOUT (a bounded wait of an
- * H psi kernel gave up: the sweep's result is incomplete), RS_ECUDA. */
+ * residuals).  Errors: RS_ENAN (a non-finite residual), RS_ETIMEOUT (a
+ * bounded wait of an H psi kernel or of a contraction gave up: the sweep's
+ * result is incomplete), RS_ECUDA. */
 int rs_eigensolver_step(rs_solver *s, double *eps_dev, double *resnorm_dev, int *n_converged, void *stream);
 
 typedef struct {

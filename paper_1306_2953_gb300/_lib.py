@@ -92,6 +92,7 @@ SIGNATURES = {
     "rs_ham_reset_status": (None, [P]),
     "rs_ham_select_kernel": (None, [P, I32]),
     "rs_ham_set_wait_limit": (None, [P, I32]),
+    "rs_contraction_wait_limit": (None, [I32, I32]),
     "rs_ham_timing": (None, [P, I32]),
     "rs_ham_timing_read": (None, [P, P, P, P]),
     "rs_ham_launch_bytes": (None, [P, I32, I32, P, P]),

@@ -33,7 +33,9 @@
 // steps overlap the readout.  Columns or rows that hold a non-finite or an
 // extreme value (an exponent near either end of the range) make their CTA
 // take a plain loop instead, so that infinities and NaN spread as in a plain
-// contraction.  Every wait is bounded; a CTA whose wait gives up writes NaN.
+// contraction.  Every wait is bounded; a CTA whose wait gives up writes
+// NaN in every result that it has not stored, and sets the call's status word
+// where it has one.
 //
 // What bounds it, and what it measured (overlap of 256 x 256 columns over
 // 658 416 points): FP64 2.95 ms, FP32 data 2.64 ms, against 69.8 ms by FP64 FMA
@@ -80,11 +82,17 @@ __device__ __forceinline__ bool dg_try(uint64_t *b, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// What a CTA's bounded waits share: whether one has given up, and after how many tests.
+struct DgGive {
+    int bad, spin;
+};
 // bounded wait; false once it has given up here or `bad` says another thread's has
 // (sleep: nanoseconds between tests, for warps that wait most of the time and
 // would take issue slots from the converters)
-__device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile int *bad, unsigned sleep = 0) {
-    for (int i = 0; i < DG_SPIN; ++i) {
+__device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, DgGive *give, unsigned sleep = 0) {
+    volatile int *bad = &give->bad;
+    const int spin = give->spin;
+    for (int i = 0; i < spin; ++i) {
         if (dg_try(b, parity)) return true;
         if ((i & 7) == 7 && *bad) return false;
         if (sleep) __nanosleep(sleep);
@@ -92,13 +100,19 @@ __device__ __forceinline__ bool dg_wait(uint64_t *b, uint32_t parity, volatile i
     *bad = 1;
     return false;
 }
+// The wait for products in flight, whatever has given up: nothing may write shared or
+// tensor memory after the CTA has left.
+__device__ __forceinline__ void dg_settle(uint64_t *b, uint32_t parity) {
+    for (int i = 0; i < DG_SPIN && !dg_try(b, parity); ++i) {
+    }
+}
 // The MMA warp runs its loop as a whole, so that descriptors stay in uniform
 // registers; `lead` (one lane) issues.
 // the whole warp: true only when every lane's wait ended (no lane goes on alone).
 // The lanes leave it together, as the warp-wide loads of tensor memory need
 // (they run apart in the loop, and in stores and atomics of ragged tiles before it).
-__device__ __forceinline__ bool dg_wait_warp(uint64_t *b, uint32_t parity, volatile int *bad) {
-    const bool all = __all_sync(0xffffffffu, dg_wait(b, parity, bad));
+__device__ __forceinline__ bool dg_wait_warp(uint64_t *b, uint32_t parity, DgGive *give) {
+    const bool all = __all_sync(0xffffffffu, dg_wait(b, parity, give));
     __syncwarp();
     return all;
 }
@@ -265,10 +279,11 @@ template <int NS, int BN, int PAD> struct DgCfg {
 struct DgBars {
     uint64_t full[DG_STAGES], empty[DG_STAGES], accfull[8], accfree, done;
     uint32_t tmem;
-    int bad, plain;
+    DgGive give;
+    int plain;
 };
 
-template <int NS> __device__ __forceinline__ void dg_setup(DgBars &b, int tmem_cols) {
+template <int NS> __device__ __forceinline__ void dg_setup(DgBars &b, int tmem_cols, int spin) {
     if (threadIdx.x == 0) {
         for (int i = 0; i < DG_STAGES; ++i) {
             dg_bar_init(&b.full[i], DG_CT);
@@ -277,7 +292,7 @@ template <int NS> __device__ __forceinline__ void dg_setup(DgBars &b, int tmem_c
         for (int t = 0; t < NS; ++t) dg_bar_init(&b.accfull[t], 1);
         dg_bar_init(&b.accfree, DG_CT);
         dg_bar_init(&b.done, 1);
-        b.bad = 0;
+        b.give = {0, spin};
         b.plain = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -318,11 +333,11 @@ template <int NS, int BN, int PAD> struct DgIssue {
             const bool first = kb % DG_DRAIN == 0, last = kb % DG_DRAIN == DG_DRAIN - 1 || kb == kst - 1;
             iv += first;
             if (++kb == kst) kb = 0;
-            ok = __all_sync(0xffffffffu, dg_wait(&b.full[s], (g / DG_STAGES) & 1, &b.bad, 40));
+            ok = __all_sync(0xffffffffu, dg_wait(&b.full[s], (g / DG_STAGES) & 1, &b.give, 40));
             DG_FENCE_AFTER();
             const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
             if (first && iv > 0 && ok) {
-                ok = __all_sync(0xffffffffu, dg_wait(&b.accfree, (iv - 1) & 1, &b.bad));
+                ok = __all_sync(0xffffffffu, dg_wait(&b.accfree, (iv - 1) & 1, &b.give));
                 DG_FENCE_AFTER();
             }
             if (ok) {
@@ -347,7 +362,7 @@ template <int NS, int BN, int PAD> struct DgIssue {
     // after the last stage: waits for every product in flight
     __device__ __forceinline__ void finish(DgBars &b) {
         dg_commit(&b.done, lead);
-        dg_wait(&b.done, 0, &b.bad);
+        dg_settle(&b.done, 0);
     }
 };
 
@@ -361,7 +376,7 @@ __device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&
     const uint32_t lane_base = b.tmem + ((uint32_t)(warp & 3) * 32 << 16) + (uint32_t)col0;
 #pragma unroll
     for (int t = 0; t < NS - 2; ++t) {
-        if (!dg_wait_warp(&b.accfull[t], iv & 1, &b.bad)) return false;
+        if (!dg_wait_warp(&b.accfull[t], iv & 1, &b.give)) return false;
         DG_FENCE_AFTER();
 #pragma unroll
         for (int c = 0; c < CPT; c += CPT < 32 ? CPT : 32) {
@@ -381,7 +396,7 @@ __device__ __forceinline__ bool dg_drain(DgBars &b, int iv, int col0, int64_t (&
         }
     }
     // the last two accumulators together, rounded at the weight of the first
-    if (!dg_wait_warp(&b.accfull[NS - 1], iv & 1, &b.bad)) return false;
+    if (!dg_wait_warp(&b.accfull[NS - 1], iv & 1, &b.give)) return false;
     DG_FENCE_AFTER();
 #pragma unroll
     for (int q = 0; q < CPT / 8; ++q) {
@@ -414,6 +429,8 @@ template <typename T> struct GramArgs {
     double dV;
     int tiles_n, stages, per_cta;   // stages in all and per CTA
     int sym;                 // Y is X: only the elements j >= i are computed, and mirrored
+    int spin;                // barrier tests before a wait gives up
+    int *err;                // status word (or nullptr): 1 once one has
 };
 
 template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1) k_digit_gram(GramArgs<T> a) {
@@ -439,7 +456,7 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
     }
     const int m0 = bm * DG_M, n0 = bn * BN;
     const int st0 = blockIdx.y * a.per_cta, nst = min(a.per_cta, a.stages - st0);
-    dg_setup<NS>(b, C::TMEM);
+    dg_setup<NS>(b, C::TMEM, a.spin);
     for (int i = tid; i < DG_M + BN; i += DG_NT) {
         const bool isa = i < DG_M;
         const int c = isa ? m0 + i : n0 + i - DG_M;
@@ -524,7 +541,7 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
         int iv = 0;   // readouts taken
         for (int it = 0; it < nst && ok; ++it) {
             const int s = it % DG_STAGES;
-            if (it >= DG_STAGES && !dg_wait_warp(&b.empty[s], (it / DG_STAGES - 1) & 1, &b.bad)) {
+            if (it >= DG_STAGES && !dg_wait_warp(&b.empty[s], (it / DG_STAGES - 1) & 1, &b.give)) {
                 ok = false;
                 break;
             }
@@ -558,6 +575,7 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
     }
     DG_FENCE_BEFORE();
     __syncthreads();
+    if (tid == 0 && a.err && b.give.bad) atomicExch(a.err, 1);
     if (warp == DG_CW)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(b.tmem), "r"(C::TMEM) : "memory");
 }
@@ -602,6 +620,10 @@ __global__ void __launch_bounds__(256) k_digit_keys(const T *__restrict__ X, int
     }
 }
 
+// Barrier tests before a wait of a contraction gives up, for the calls of this host
+// thread (rs_contraction_wait_limit).
+thread_local int t_gram_spin = DG_SPIN, t_rot_spin = DG_SPIN;
+
 int sm_count(int *n) {
     int dev = 0;
     RS_CUDA(cudaGetDevice(&dev));
@@ -639,7 +661,7 @@ template <typename T, int NS, int BN> int launch_gram(GramArgs<T> a, int tiles_m
 
 template <typename T>
 int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, int *scratch, cudaStream_t st) {
+               int64_t lds, int *scratch, cudaStream_t st, int *err) {
     if (npts > (int64_t)INT32_MAX - 64) return fail(RS_EINVAL, "digit_gram: too many points");
     const bool sym = X == Y && ldx == ldy && nx == ny;
     int *keys = scratch;
@@ -659,7 +681,7 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
         GramArgs<T> a{};
         a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.lds = lds, a.nx = nx, a.ny = ny;
         a.kx = keys, a.ky = sym ? keys : keys + nx;
-        a.S = S, a.dV = dV, a.sym = sym;
+        a.S = S, a.dV = dV, a.sym = sym, a.spin = t_gram_spin, a.err = err;
         const int tm = (nx + DG_M - 1) / DG_M;
         // 32 columns of Y fill half of a 64-wide tile
         const bool narrow = ny <= 32;
@@ -668,9 +690,9 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
     }
 }
 template int digit_gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
-                                int64_t, int *, cudaStream_t);
+                                int64_t, int *, cudaStream_t, int *);
 template int digit_gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *,
-                               int64_t, int *, cudaStream_t);
+                               int64_t, int *, cudaStream_t, int *);
 
 // ----------------------------------------------------------- rotation ---
 
@@ -684,6 +706,7 @@ template <typename T> struct RotArgs {
     int n, m;
     int vec, yvec;       // X, Y rows on 16-byte boundaries
     int cluster;         // Y is X: the CTAs of a row tile form a cluster and write together
+    int spin, *err;      // as in GramArgs
     double alpha, beta;
 };
 
@@ -734,7 +757,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
         dg_bar_init(&rb.sums, DG_CT);
     }
     for (int i = tid; i < NBLK * BN; i += DG_NT) eb[i] = 0;
-    dg_setup<NS>(b, C::TMEM);
+    dg_setup<NS>(b, C::TMEM, a.spin);
     if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     // exponents of the columns of C
     for (int blk = 0; blk < NBLK; ++blk)
@@ -762,7 +785,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
         int j = 0;
         for (int tile = blockIdx.y; tile < ntiles; tile += gridDim.y, ++j) {
             const int h = j & 1;
-            if (j >= 2 && !dg_wait(&rb.keyfree[h], (j / 2 - 1) & 1, &b.bad, 50 * kst)) break;
+            if (j >= 2 && !dg_wait(&rb.keyfree[h], (j / 2 - 1) & 1, &b.give, 50 * kst)) break;
             const int64_t r0 = (int64_t)tile * DG_M;
             const int rows = (int)min((int64_t)DG_M, a.npts - r0);
             bool pl = false;
@@ -807,7 +830,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
         bool ok = true;
         for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
             const int h = j & 1;
-            ok = __all_sync(0xffffffffu, dg_wait(&rb.keyfull[h], (j / 2) & 1, &b.bad));
+            ok = __all_sync(0xffffffffu, dg_wait(&rb.keyfull[h], (j / 2) & 1, &b.give));
             const volatile int *f = rb.plain[h];
             const bool pl = cplain || f[0] || f[1] || f[2];
             __syncwarp();
@@ -958,7 +981,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             }
             // the block's sums are complete
             const bool lastb = pblk == NBLK - 1;
-            if (lastb && a.cluster) ok = dg_wait_warp(&rb.rd, ptj & 1, &b.bad) && ok;
+            if (lastb && a.cluster) ok = dg_wait_warp(&rb.rd, ptj & 1, &b.give) && ok;
             const int64_t p = (int64_t)ptile * DG_M + row;
             const bool on = owns && p < a.npts;
             if (NBLK > 1 && lastb && on) {
@@ -1001,7 +1024,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                 end = tile >= ntiles;
                 if (!end) {
                     h = j & 1;
-                    ok = dg_wait_warp(&rb.keyfull[h], (j / 2) & 1, &b.bad);
+                    ok = dg_wait_warp(&rb.keyfull[h], (j / 2) & 1, &b.give);
                     ex0 = ea[h][ar], ex1 = ea[h][ar + 8], er = ea[h][row];
                     const volatile int *f = rb.plain[h];
                     plain = cplain || f[0] || f[1] || f[2];
@@ -1012,7 +1035,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             }
             if (!end && !plain && ok) {
                 const int s = g % DG_STAGES;
-                if (g >= DG_STAGES) ok = dg_wait_warp(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.bad);
+                if (g >= DG_STAGES) ok = dg_wait_warp(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.give);
                 const bool lasts = it + 1 == nst, more = !lasts || tile + (int)gridDim.y < ntiles;
                 const int nt = lasts ? tile + gridDim.y : tile, ni = lasts ? 0 : it + 1;
                 if (ok) {
@@ -1050,9 +1073,9 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                 // every converter of this CTA has read its row (a bounded wait: a warp
                 // whose own wait has given up does not come)
                 dg_arrive(&rb.sums);
-                ok = dg_wait_warp(&rb.sums, nplain++ & 1, &b.bad);
+                ok = dg_wait_warp(&rb.sums, nplain++ & 1, &b.give) && ok;
                 rows_read();
-                if (a.cluster) ok = dg_wait_warp(&rb.rd, j & 1, &b.bad) && ok;
+                if (a.cluster) ok = dg_wait_warp(&rb.rd, j & 1, &b.give) && ok;
                 if (owns && (int64_t)tile * DG_M + row < a.npts)
                     for (int i = 0; i < NBLK * 32; ++i) {
                         const int c = (nb0 + i / 32) * BN + col0 + i % 32;
@@ -1077,9 +1100,23 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                 if (++kb == kst) kb = 0, ++blk;
             }
         }
+        if (!ok) {
+            // a wait gave up: NaN in the tile before this one, which may not have been
+            // stored, and in all that follow
+            for (int t = max((int)blockIdx.y, tile - (int)gridDim.y); t < ntiles; t += gridDim.y) {
+                const int64_t p = (int64_t)t * DG_M + row;
+                if (!owns || p >= a.npts) continue;
+#pragma unroll 1
+                for (int i = 0; i < NBLK * 32; ++i) {
+                    const int c = (nb0 + i / 32) * BN + col0 + i % 32;
+                    if (c < a.m) a.Y[p * a.ldy + c] = (T)__longlong_as_double(0x7ff8000000000000ll);
+                }
+            }
+        }
     }
     DG_FENCE_BEFORE();
     __syncthreads();
+    if (tid == 0 && a.err && b.give.bad) atomicExch(a.err, 1);
     if (warp == DG_CW)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(b.tmem), "r"(C::TMEM) : "memory");
     // no CTA leaves while another may still signal it
@@ -1144,6 +1181,7 @@ struct PieceArgs {
     int64_t ldx, ldy, npts;
     int n, m;
     int vec, yvec, cluster;
+    int spin, *err;      // as in GramArgs
     float alpha, beta;
 };
 
@@ -1190,7 +1228,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
     extern __shared__ __align__(128) unsigned char dgsm[];
     __shared__ uint64_t full[PC_ST], empty[PC_ST], accfull[2], accfree[2], rd, done;
     __shared__ uint32_t tmem_s;
-    __shared__ int bad;
+    __shared__ DgGive give;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int kst = (a.n + DG_K - 1) / DG_K;
     const int ntiles = (int)((a.npts + DG_M - 1) / DG_M);
@@ -1205,7 +1243,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
         }
         dg_bar_init(&rd, DG_CT * (a.cluster ? gridDim.x : 1));
         dg_bar_init(&done, 1);
-        bad = 0;
+        give = {0, a.spin};
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == DG_CW) {
@@ -1226,7 +1264,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
             for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y)
                 for (int it = 0; it < kst; ++it, ++g) {
                     const int s = g % PC_ST;
-                    if (g >= PC_ST && !dg_wait(&empty[s], (g / PC_ST - 1) & 1, &bad)) {
+                    if (g >= PC_ST && !dg_wait(&empty[s], (g / PC_ST - 1) & 1, &give)) {
                         ok = false;
                         break;
                     }
@@ -1240,7 +1278,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
                 }
             // no copy is in flight when the CTA ends
             for (int q = g < PC_ST ? 0 : g - PC_ST; q < g; ++q)
-                for (int i = 0; i < (*(volatile int *)&bad ? 64 : DG_SPIN) && !dg_try(&full[q % PC_ST], (q / PC_ST) & 1); ++i) {
+                for (int i = 0; i < (*(volatile int *)&give.bad ? 64 : DG_SPIN) && !dg_try(&full[q % PC_ST], (q / PC_ST) & 1); ++i) {
                 }
         }
     } else if (warp == DG_CW) {
@@ -1251,11 +1289,11 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
         bool ok = true;
         for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
             const uint32_t acc = tmem + (j & 1) * 2 * BN;
-            if (j >= 2) ok = __all_sync(0xffffffffu, dg_wait(&accfree[j & 1], (j / 2 - 1) & 1, &bad));
+            if (j >= 2) ok = __all_sync(0xffffffffu, dg_wait(&accfree[j & 1], (j / 2 - 1) & 1, &give));
             DG_FENCE_AFTER();
             for (int it = 0; it < kst && ok; ++it, ++g) {
                 const int s = g % PC_ST;
-                ok = __all_sync(0xffffffffu, dg_wait(&full[s], (g / PC_ST) & 1, &bad));
+                ok = __all_sync(0xffffffffu, dg_wait(&full[s], (g / PC_ST) & 1, &give));
                 DG_FENCE_AFTER();
                 const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
                 if (ok) {
@@ -1278,7 +1316,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
             dg_commit(&accfull[j & 1], lead);
         }
         dg_commit(&done, lead);
-        dg_wait(&done, 0, &bad);
+        dg_settle(&done, 0);
     } else if (warp < DG_CW) {
         const int ar = warp * 16 + (lane >> 2), akq = lane & 3;
         unsigned char *adst = dgsm + akq * C::LBO_A + ar * 16;
@@ -1304,8 +1342,8 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
             }
         };
         auto readout = [&](int tile, int j) {
-            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &bad);
-            if (a.cluster) ok = dg_wait_warp(&rd, j & 1, &bad) && ok;
+            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &give);
+            if (a.cluster) ok = dg_wait_warp(&rd, j & 1, &give) && ok;
             DG_FENCE_AFTER();
             const int64_t p = (int64_t)tile * DG_M + row;
             const uint32_t t0 = tmem_s + ((uint32_t)(warp & 3) * 32 << 16) + (j & 1) * 2 * BN + col0;
@@ -1353,7 +1391,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
         for (int tile = blockIdx.y; tile < ntiles && ok; tile += gridDim.y, ++j) {
             for (int it = 0; it < kst && ok; ++it, ++g) {
                 const int s = g % PC_ST;
-                if (g >= PC_ST) ok = dg_wait_warp(&empty[s], (g / PC_ST - 1) & 1, &bad);
+                if (g >= PC_ST) ok = dg_wait_warp(&empty[s], (g / PC_ST - 1) & 1, &give);
                 if (!ok) break;
                 const bool last = it + 1 == kst;
 #pragma unroll
@@ -1384,9 +1422,18 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_rot(PieceA
             ptile = tile;
         }
         if (ptile >= 0) readout(ptile, j - 1);
+        if (!ok)   // as in k_digit_rot
+            for (int t = max((int)blockIdx.y, ptile - (int)gridDim.y); t < ntiles; t += gridDim.y) {
+                const int64_t p = (int64_t)t * DG_M + row;
+                const int cb = blockIdx.x * BN + col0;
+                if (p >= a.npts) continue;
+#pragma unroll 1
+                for (int i = 0; i < CPT && cb + i < a.m; ++i) a.Y[p * a.ldy + cb + i] = __int_as_float(0x7fffffff);
+            }
     }
     DG_FENCE_BEFORE();
     __syncthreads();
+    if (tid == 0 && a.err && give.bad) atomicExch(a.err, 1);
     if (warp == DG_CW)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_s), "r"(C::TMEM) : "memory");
     // no CTA leaves while another may still signal it
@@ -1423,6 +1470,7 @@ struct PieceGramArgs {
     double *S;
     double dV;
     int tiles_n, tiles, chunks, kb;   // kb: 64-point stages per chunk
+    int spin, *err;                   // as in GramArgs
 };
 
 constexpr int PG_K = 64, PG_KQ = PG_K / 8, PG_ST = 2;
@@ -1439,7 +1487,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
     extern __shared__ __align__(128) unsigned char dgsm[];
     __shared__ uint64_t full[PG_ST], empty[PG_ST], accfull[2], accfree[2], done;
     __shared__ uint32_t tmem_s;
-    __shared__ int bad;
+    __shared__ DgGive give;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int items = a.tiles * a.chunks, nkb = (int)((a.npts + PG_K - 1) / PG_K);
     if (tid == 0) {
@@ -1452,7 +1500,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
             dg_bar_init(&accfree[i], DG_CT);
         }
         dg_bar_init(&done, 1);
-        bad = 0;
+        give = {0, a.spin};
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == DG_CW) {
@@ -1474,11 +1522,11 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++j) {
             const uint32_t acc = tmem + (j & 1) * BN;
             const int nst = stages_of(item);
-            if (j >= 2) ok = dg_wait_warp(&accfree[j & 1], (j / 2 - 1) & 1, &bad);
+            if (j >= 2) ok = dg_wait_warp(&accfree[j & 1], (j / 2 - 1) & 1, &give);
             DG_FENCE_AFTER();
             for (int it = 0; it < nst && ok; ++it, ++g) {
                 const int s = g % PG_ST;
-                ok = dg_wait_warp(&full[s], (g / PG_ST) & 1, &bad);
+                ok = dg_wait_warp(&full[s], (g / PG_ST) & 1, &give);
                 DG_FENCE_AFTER();
                 const uint64_t da = da0 + (uint64_t)(s * (C::STAGE >> 4)), db = db0 + (uint64_t)(s * (C::STAGE >> 4));
                 if (ok) {
@@ -1498,7 +1546,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
             dg_commit(&accfull[j & 1], lead);
         }
         dg_commit(&done, lead);
-        dg_wait(&done, 0, &bad);
+        dg_settle(&done, 0);
     } else if (warp < DG_CW) {
         // units (32 columns, 8 points): 4 x 8 of X, BN / 32 x 8 of Y; warp w takes
         // the points 8 w .. of every column group
@@ -1527,7 +1575,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
         constexpr int CPT = BN / 2;
         const int col0 = (warp >> 2) * CPT, row = (warp & 3) * 32 + lane;
         auto readout = [&](int item, int j) {
-            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &bad);
+            ok = ok && dg_wait_warp(&accfull[j & 1], (j / 2) & 1, &give);
             DG_FENCE_AFTER();
             const int tile = item % a.tiles, i = tile / a.tiles_n * DG_M + row, c0 = tile % a.tiles_n * BN + col0;
             const uint32_t t0 = tmem_s + ((uint32_t)(warp & 3) * 32 << 16) + (j & 1) * BN + col0;
@@ -1555,7 +1603,7 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
             const int nst = stages_of(item);
             for (int it = 0; it < nst && ok; ++it, ++g) {
                 const int s = g % PG_ST;
-                if (g >= PG_ST) ok = dg_wait_warp(&empty[s], (g / PG_ST - 1) & 1, &bad);
+                if (g >= PG_ST) ok = dg_wait_warp(&empty[s], (g / PG_ST - 1) & 1, &give);
                 if (!ok) break;
                 unsigned char *st = dgsm + s * C::STAGE + lane * 16;
 #pragma unroll
@@ -1578,9 +1626,18 @@ template <int BN> __global__ void __launch_bounds__(DG_NT, 1) k_piece_gram(Piece
             pitem = item;
         }
         if (pitem >= 0) readout(pitem, j - 1);
+        if (!ok)   // a wait gave up: NaN in the tiles of the item before the last one tried and of all that follow
+            for (int item = max((int)blockIdx.x, pitem - (int)gridDim.x); item < items; item += gridDim.x) {
+                const int tile = item % a.tiles, i = tile / a.tiles_n * DG_M + row, c0 = tile % a.tiles_n * BN + col0;
+                if (i >= a.nx) continue;
+#pragma unroll 1
+                for (int q = 0; q < CPT && c0 + q < a.ny; ++q)
+                    atomicAdd(a.S + (int64_t)i * a.lds + c0 + q, __longlong_as_double(0x7ff8000000000000ll));
+            }
     }
     DG_FENCE_BEFORE();
     __syncthreads();
+    if (tid == 0 && a.err && give.bad) atomicExch(a.err, 1);
     if (warp == DG_CW)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_s), "r"(C::TMEM) : "memory");
 }
@@ -1614,10 +1671,10 @@ bool digit_rot_takes(int n, int m, bool in_place) {
 
 template <typename T>
 int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-              double alpha, double beta, cudaStream_t st) {
+              double alpha, double beta, cudaStream_t st, int *err) {
     RotArgs<T> a{};
     a.X = X, a.C = C, a.Y = Y, a.ldx = ldx, a.ldc = ldc, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
-    a.alpha = alpha, a.beta = beta;
+    a.alpha = alpha, a.beta = beta, a.spin = t_rot_spin, a.err = err;
     a.vec = aligned16(X) && (ldx * (int64_t)sizeof(T)) % 16 == 0;
     a.yvec = aligned16(Y) && (ldy * (int64_t)sizeof(T)) % 16 == 0;
     constexpr int NS = sizeof(T) == 8 ? 8 : 5;
@@ -1628,9 +1685,9 @@ int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int 
     return one ? launch_rot<T, NS, 64, 1, true>(a, in_place, st) : launch_rot<T, NS, 64, 1, false>(a, in_place, st);
 }
 template int digit_rot<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
-                               double, double, cudaStream_t);
+                               double, double, cudaStream_t, int *);
 template int digit_rot<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
-                              double, cudaStream_t);
+                              double, cudaStream_t, int *);
 
 }  // namespace rs
 
@@ -1642,21 +1699,22 @@ int64_t piece_rot_bytes(int n, int m) {
 }
 
 int piece_gram(const float *X, int64_t ldx, int nx, const float *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, cudaStream_t st) {
+               int64_t lds, cudaStream_t st, int *err) {
     k_digit_init<<<(unsigned)std::min<int64_t>(256, ((int64_t)nx * ny + 255) / 256), 256, 0, st>>>(S, lds, nx, ny, nullptr, 0);
     RS_LAUNCH_CHECK();
     PieceGramArgs a{};
     a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.lds = lds, a.nx = nx, a.ny = ny, a.S = S, a.dV = dV;
+    a.spin = t_gram_spin, a.err = err;
     return ny <= 64 ? launch_piece_gram<64>(a, st) : launch_piece_gram<128>(a, st);
 }
 
 int piece_rot(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
-              double alpha, double beta, void *work, cudaStream_t st) {
+              double alpha, double beta, void *work, cudaStream_t st, int *err) {
     PieceArgs a{};
     a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
     a.vec = aligned16(X) && ldx % 4 == 0;
     a.yvec = aligned16(Y) && ldy % 4 == 0;
-    a.alpha = (float)alpha, a.beta = (float)beta;
+    a.alpha = (float)alpha, a.beta = (float)beta, a.spin = t_rot_spin, a.err = err;
     if (m <= 64) return launch_piece<64>(a, C, ldc, work, X == Y, st);
     return launch_piece<128>(a, C, ldc, work, X == Y, st);
 }
@@ -1676,6 +1734,20 @@ int check_work(const void *work) {
     if (!aligned16(work)) return fail(RS_EINVAL, "tensor-core call: workspace not on a 16-byte boundary");
     return RS_OK;
 }
+
+// the status word of the call's waits: the last 256 bytes of the workspace
+int clear_status(void *work, int64_t bytes, int **err, cudaStream_t st) {
+    *err = reinterpret_cast<int *>((char *)work + bytes - 256);
+    RS_CUDA(cudaMemsetAsync(*err, 0, sizeof(int), st));
+    return RS_OK;
+}
+int read_status(const int *err, cudaStream_t st) {
+    int e = 0;
+    RS_CUDA(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    RS_CUDA(cudaStreamSynchronize(st));
+    if (e) return fail(RS_ETIMEOUT, "tensor-core call: a pipeline wait timed out");
+    return RS_OK;
+}
 }  // namespace
 
 extern "C" int64_t rs_tc_workspace_bytes(int64_t rows_a, int64_t rows_b, int64_t K) {
@@ -1689,9 +1761,10 @@ extern "C" int rs_overlap_block_tc(const rs_grid *g, const float *X_dev, int64_t
     if (nx < 1 || ny < 1 || ldx < nx || ldy < ny || lds < ny) return fail(RS_EINVAL, "rs_overlap_block_tc: bad sizes");
     RS_TRY(check_work(work_dev));
     cudaStream_t st = (cudaStream_t)stream;
-    RS_TRY(piece_gram(X_dev, ldx, nx, Y_dev, ldy, ny, g->npts, g->h * g->h * g->h, S_dev, lds, st));
-    RS_CUDA(cudaStreamSynchronize(st));
-    return RS_OK;
+    int *err = nullptr;
+    RS_TRY(clear_status(work_dev, rs_tc_workspace_bytes(nx, ny, g->npts), &err, st));
+    RS_TRY(piece_gram(X_dev, ldx, nx, Y_dev, ldy, ny, g->npts, g->h * g->h * g->h, S_dev, lds, st, err));
+    return read_status(err, st);
 }
 
 extern "C" int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const double *C_dev, int64_t ldc, int m,
@@ -1700,7 +1773,14 @@ extern "C" int rs_rotate_block(const float *X_dev, int64_t ldx, int n, const dou
     if (n < 1 || m < 1 || npts < 1 || ldx < n || ldy < m || ldc < m) return fail(RS_EINVAL, "rs_rotate_block: bad sizes");
     RS_TRY(check_work(work_dev));
     cudaStream_t st = (cudaStream_t)stream;
-    RS_TRY(rotate_any(X_dev, ldx, n, C_dev, ldc, m, Y_dev, ldy, npts, 1.0, 0.0, work_dev, st));
-    RS_CUDA(cudaStreamSynchronize(st));
+    int *err = nullptr;
+    RS_TRY(clear_status(work_dev, rs_tc_workspace_bytes(npts, m, n), &err, st));
+    RS_TRY(rotate_any(X_dev, ldx, n, C_dev, ldc, m, Y_dev, ldy, npts, 1.0, 0.0, work_dev, st, err));
+    return read_status(err, st);
+}
+
+extern "C" int rs_contraction_wait_limit(int overlap_tests, int rotation_tests) {
+    t_gram_spin = overlap_tests < 0 ? DG_SPIN : overlap_tests;
+    t_rot_spin = rotation_tests < 0 ? DG_SPIN : rotation_tests;
     return RS_OK;
 }

@@ -1,5 +1,6 @@
 // FP64- and FP32-accurate contractions on the tensor cores by integer digits
-// (see digits.cu).
+// (see digits.cu).  err (here and in linalg.h): a device word that becomes 1 once
+// a bounded wait of the call has given up (its results are then NaN), or nullptr.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,7 +19,7 @@ inline int64_t digit_gram_scratch_ints(int nx, int ny) { return (int64_t)nx + ny
 // from the library's stream-ordered pool).  Asynchronous.
 template <typename T>
 int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, int *scratch, cudaStream_t st);
+               int64_t lds, int *scratch, cudaStream_t st, int *err = nullptr);
 
 // Y (m columns) = alpha X C + beta Y, X [npts][ldx] (n columns), C FP64
 // [n][ldc]; Y may be X itself (same pointer and leading dimension) when
@@ -26,18 +27,18 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
 bool digit_rot_takes(int n, int m, bool in_place);
 template <typename T>
 int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-              double alpha, double beta, cudaStream_t st);
+              double alpha, double beta, cudaStream_t st, int *err = nullptr);
 
 // S = dV X^T Y of FP32 data to FP32 accuracy by BF16 pieces, FP32 sums over at
 // most 2048 points.  Asynchronous.
 int piece_gram(const float *X, int64_t ldx, int nx, const float *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-               int64_t lds, cudaStream_t st);
+               int64_t lds, cudaStream_t st, int *err = nullptr);
 
 // FP32 rotation to FP32 accuracy by BF16 pieces (Y may be X itself, same leading
 // dimension, for m <= 1024 and beta == 0).  work: piece_rot_bytes(n, m) bytes,
 // 16-byte aligned.  Asynchronous.
 int64_t piece_rot_bytes(int n, int m);
 int piece_rot(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
-              double alpha, double beta, void *work, cudaStream_t st);
+              double alpha, double beta, void *work, cudaStream_t st, int *err = nullptr);
 
 }  // namespace rs

@@ -28,15 +28,15 @@ namespace rs {
 
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-         int64_t lds, cudaStream_t st, bool fast, int *scratch) {
+         int64_t lds, cudaStream_t st, bool fast, int *scratch, int *err) {
     if constexpr (sizeof(T) == 4)
-        if (fast) return piece_gram(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, st);
-    return digit_gram<T>(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, scratch, st);
+        if (fast) return piece_gram(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, st, err);
+    return digit_gram<T>(X, ldx, nx, Y, ldy, ny, npts, dV, S, lds, scratch, st, err);
 }
 template int gram<double>(const double *, int64_t, int, const double *, int64_t, int, int64_t, double, double *,
-                          int64_t, cudaStream_t, bool, int *);
+                          int64_t, cudaStream_t, bool, int *, int *);
 template int gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *, int64_t,
-                         cudaStream_t, bool, int *);
+                         cudaStream_t, bool, int *, int *);
 
 // ----------------------------------------------------------- k_rowmul ---
 // Y[p][0:m] = alpha * sum_k X[p][k] C[k][0:m] + beta * Y[p][0:m] for a tile of
@@ -78,8 +78,8 @@ __global__ void __launch_bounds__(R_NT) k_rowmul(const T *X, int64_t ldx, int n,
 
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-           double alpha, double beta, cudaStream_t st) {
-    if (digit_rot_takes(n, m, X == Y)) return digit_rot<T>(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, st);
+           double alpha, double beta, cudaStream_t st, int *err) {
+    if (digit_rot_takes(n, m, X == Y)) return digit_rot<T>(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, st, err);
     const size_t smem = (size_t)R_ROWS * n * sizeof(T);
     if (smem > 200 * 1024) return fail(RS_EINVAL, "rowmul: n too large");
     if (smem > 48 * 1024) RS_TRY(smem_optin((const void *)k_rowmul<T>, smem));
@@ -89,16 +89,16 @@ int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, 
     return RS_OK;
 }
 template int rowmul<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
-                            double, double, cudaStream_t);
+                            double, double, cudaStream_t, int *);
 template int rowmul<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
-                           double, cudaStream_t);
+                           double, cudaStream_t, int *);
 
 // FP32 rotation to FP32 accuracy for any placement of Y: where Y overlaps X and
 // cannot be written in place by one launch, X is copied first.
 int64_t rotate_work_bytes(int n, int m, int64_t copy_rows) { return piece_rot_bytes(n, m) + copy_rows * n * (int64_t)sizeof(float); }
 
 int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
-               double alpha, double beta, void *work, cudaStream_t st) {
+               double alpha, double beta, void *work, cudaStream_t st, int *err) {
     const bool apart = X + (npts - 1) * ldx + n <= Y || Y + (npts - 1) * ldy + m <= X;
     const bool inplace = X == Y && ldx == ldy && beta == 0.0 && m <= 1024;
     // column slices of one array, side by side
@@ -111,7 +111,7 @@ int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc,
         X = copy;
         ldx = n;
     }
-    return piece_rot(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, work, st);
+    return piece_rot(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, work, st, err);
 }
 
 // ----------------------------------------------------- small dense FP64 ---

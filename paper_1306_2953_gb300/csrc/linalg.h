@@ -14,20 +14,20 @@ namespace rs {
 // nullptr (see digits.h).
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
-         int64_t lds, cudaStream_t st, bool fast = false, int *scratch = nullptr);
+         int64_t lds, cudaStream_t st, bool fast = false, int *scratch = nullptr, int *err = nullptr);
 
 // Y = alpha X C + beta Y; X [npts][ldx] (n columns), C FP64 [n][ldc]
 // (m columns), Y [npts][ldy]; Y may alias X when beta == 0.
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-           double alpha, double beta, cudaStream_t st);
+           double alpha, double beta, cudaStream_t st, int *err = nullptr);
 
 // FP32 rotation to FP32 accuracy for any placement of Y relative to X.  work:
 // rotate_work_bytes(n, m, npts) bytes; copy_rows = 0 serves when Y is apart from
 // X, beside it in the same array, or X itself with m <= 1024.
 int64_t rotate_work_bytes(int n, int m, int64_t copy_rows);
 int rotate_any(const float *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, float *Y, int64_t ldy, int64_t npts,
-               double alpha, double beta, void *work, cudaStream_t st);
+               double alpha, double beta, void *work, cudaStream_t st, int *err = nullptr);
 
 // out[k] = sum_p A[p][k] B[p][k] (FP64, exact products, compensated sum), k < ncols <= 256.
 int coldots(int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, int ncols, int64_t npts, double *out,
@@ -84,6 +84,8 @@ struct TcWork {
     // subspace eigenvectors from FP32 Jacobi alone (the closing FP64
     // Rayleigh-Ritz fixes the final accuracy)
     bool inner = false;
+    // status word of the contractions' bounded waits (nullptr: none kept)
+    int *err = nullptr;
 };
 
 // Psi (n columns) <- Psi C in place (C FP64 n x n).

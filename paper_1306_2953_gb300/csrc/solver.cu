@@ -488,18 +488,18 @@ int copy_cols(int dtype, const void *S, int64_t lds, void *D, int64_t ldd, int n
 
 // inner-iteration contractions: FP32 mode to FP32-level accuracy
 int gram_any(int dtype, const void *X, int64_t ldx, int nx, const void *Y, int64_t ldy, int ny, int64_t npts, double dV,
-             double *S, int64_t lds, cudaStream_t st) {
+             double *S, int64_t lds, cudaStream_t st, const TcWork &tc) {
     if (dtype == RS_F64)
-        return gram<double>((const double *)X, ldx, nx, (const double *)Y, ldy, ny, npts, dV, S, lds, st);
-    return gram<float>((const float *)X, ldx, nx, (const float *)Y, ldy, ny, npts, dV, S, lds, st, true);
+        return gram<double>((const double *)X, ldx, nx, (const double *)Y, ldy, ny, npts, dV, S, lds, st, false, nullptr, tc.err);
+    return gram<float>((const float *)X, ldx, nx, (const float *)Y, ldy, ny, npts, dV, S, lds, st, true, nullptr, tc.err);
 }
 
 // (X and Y are different arrays, or column slices of one)
 int rowmul_any(int dtype, const void *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, void *Y, int64_t ldy,
                int64_t npts, double alpha, double beta, cudaStream_t st, const TcWork &tc) {
     if (dtype == RS_F64)
-        return rowmul<double>((const double *)X, ldx, n, C, ldc, m, (double *)Y, ldy, npts, alpha, beta, st);
-    return rotate_any((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, tc.p, st);
+        return rowmul<double>((const double *)X, ldx, n, C, ldc, m, (double *)Y, ldy, npts, alpha, beta, st, tc.err);
+    return rotate_any((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, tc.p, st, tc.err);
 }
 
 const char *off(const DevBuf &b, int64_t elems, int es) { return (const char *)b.p + (size_t)elems * es; }
@@ -556,7 +556,7 @@ int block_step(rs_solver *S, int b, cudaStream_t st) {
     // 3. classical Gram-Schmidt, twice, against Psi[:, :(b+1) nb]
     const int nq = (b + 1) * nb;
     for (int pass = 0; pass < 2; ++pass) {
-        RS_TRY(gram_any(dt, S->psi.p, nst, nq, Y, ldz, ny, np, S->dV, S->M, ny, st));
+        RS_TRY(gram_any(dt, S->psi.p, nst, nq, Y, ldz, ny, np, S->dV, S->M, ny, st, S->tc));
         RS_TRY(rowmul_any(dt, S->psi.p, nst, nq, S->M, ny, ny, Y, ldz, np, -1.0, 1.0, st, S->tc));
     }
     RS_TRY(coldots(dt, Y, ldz, Y, ldz, ny, np, nrm, st));
@@ -572,8 +572,8 @@ int block_step(rs_solver *S, int b, cudaStream_t st) {
 
     // 5. Rayleigh-Ritz on Z = [X, Y]
     int n = nb + ny;
-    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->Z.p, ldz, n, np, S->dV, S->G, n, st));
-    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->HZ.p, ldz, n, np, S->dV, S->A, n, st));
+    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->Z.p, ldz, n, np, S->dV, S->G, n, st, S->tc));
+    RS_TRY(gram_any(dt, S->Z.p, ldz, n, S->HZ.p, ldz, n, np, S->dV, S->A, n, st, S->tc));
     RS_TRY(symmetrize(S->G, n, n, st));
     RS_TRY(symmetrize(S->A, n, n, st));
     int bad = 1;
@@ -1050,12 +1050,14 @@ extern "C" int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void 
     S->mu = S->Yv + (size_t)n3 * n3;
     S->C = S->mu + n3;
     S->status = reinterpret_cast<int *>(S->C + (size_t)n3 * c.nb);
+    S->tc.err = S->status + 8;   // 16 words stand between C and the eigensolver's workspace
     S->eighw = reinterpret_cast<void *>(S->C + (size_t)n3 * c.nb + 8);
     S->pc = Precond::create(c.precond, c.filter_alpha, S->npts, c.nb, c.dtype);
     if (!S->pc) return bail(fail(RS_EINVAL, "rs_solver_create: preconditioner %d unavailable", c.precond));
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemcpyAsync(S->psi.p, Psi0_dev, big, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         (S->P.p && cudaMemsetAsync(S->P.p, 0, big, st) != cudaSuccess) ||
+        cudaMemsetAsync(S->tc.err, 0, sizeof(int), st) != cudaSuccess ||
         cudaMemsetAsync(S->res.p, 0, sizeof(double) * c.nst, st) != cudaSuccess)
         return bail(fail(RS_ECUDA, "rs_solver_create: copy failed"));
     if ((rc = orthonormalize_impl(S->npts, S->dV, S->psi.p, c.nst, c.nst, c.dtype, S->la.p, st, S->tc))) return bail(rc);
@@ -1067,9 +1069,10 @@ extern "C" int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void 
     return RS_OK;
 }
 
-extern "C" int rs_eigensolver_step(rs_solver *S, double *eps_dev, double *resnorm_dev, int *n_converged, void *stream) {
-    if (!S) return fail(RS_EINVAL, "rs_eigensolver_step: null solver");
-    cudaStream_t st = (cudaStream_t)stream;
+namespace {
+
+// The updates of a sweep and the Rayleigh-Ritz that closes it.
+int sweep_impl(rs_solver *S, cudaStream_t st) {
     const rs_solver_cfg &c = S->cfg;
     const bool rmm = c.method == RS_EIG_RMMDIIS;
     for (int b = 0; b < S->nblk; ++b) RS_TRY(rmm ? rmm_block_step(S, b, st) : block_step(S, b, st));
@@ -1079,15 +1082,35 @@ extern "C" int rs_eigensolver_step(rs_solver *S, double *eps_dev, double *resnor
     RS_TRY(subspace_diag_impl(S->h, S->psi.p, S->hpsi.p, c.nst, c.nst, c.dtype, c.nb, S->la.p, S->eig.as<double>(), st,
                               S->tc));
     if (!rmm) RS_TRY(rotate_inplace(S->P.p, c.nst, c.nst, w.xi, S->npts, c.dtype, st, S->tc));
+    return RS_OK;
+}
+
+}  // namespace
+
+extern "C" int rs_eigensolver_step(rs_solver *S, double *eps_dev, double *resnorm_dev, int *n_converged, void *stream) {
+    if (!S) return fail(RS_EINVAL, "rs_eigensolver_step: null solver");
+    cudaStream_t st = (cudaStream_t)stream;
+    const rs_solver_cfg &c = S->cfg;
+    // a contraction whose wait gave up leaves NaN behind, over which a later step of
+    // the sweep may stumble: its status word, which stays set, names the cause
+    int tcerr = 0;
+    const int rc = sweep_impl(S, st);
+    if (rc != RS_OK) {
+        if (cudaMemcpyAsync(&tcerr, S->tc.err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+            cudaStreamSynchronize(st) == cudaSuccess && tcerr)
+            return fail(RS_ETIMEOUT, "eigensolver: a tensor-core pipeline wait timed out");
+        return rc;
+    }
     if (eps_dev) RS_CUDA(cudaMemcpyAsync(eps_dev, S->eig.p, sizeof(double) * c.nst, cudaMemcpyDeviceToDevice, st));
     if (resnorm_dev) RS_CUDA(cudaMemcpyAsync(resnorm_dev, S->res.p, sizeof(double) * c.nst, cudaMemcpyDeviceToDevice, st));
     std::vector<double> res(c.nst);
     RS_CUDA(cudaMemcpyAsync(res.data(), S->res.p, sizeof(double) * c.nst, cudaMemcpyDeviceToHost, st));
-    // status word of the H psi ring's bounded waits (one that gave up leaves that
-    // launch's result incomplete; the contractions write NaN, found in the residuals)
+    // status words of the bounded device waits: the contractions and the H psi ring
     int ringerr = 0;
+    RS_CUDA(cudaMemcpyAsync(&tcerr, S->tc.err, sizeof(int), cudaMemcpyDeviceToHost, st));
     if (int *rw = ham_status_word(S->h)) RS_CUDA(cudaMemcpyAsync(&ringerr, rw, sizeof(int), cudaMemcpyDeviceToHost, st));
     RS_CUDA(cudaStreamSynchronize(st));
+    if (tcerr) return fail(RS_ETIMEOUT, "eigensolver: a tensor-core pipeline wait timed out");
     if (ringerr) return fail(RS_ETIMEOUT, "eigensolver: an H psi pipeline wait timed out");
     ++S->sweeps;
     const int nw = c.n_wanted > 0 ? c.n_wanted : c.nst;

@@ -48,9 +48,9 @@ namespace rs {
 
 int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, cudaStream_t st,
                    const TcWork &tc) {
-    if (dtype == RS_F64) return rowmul<double>((const double *)Psi, ld, n, C, n, n, (double *)Psi, ld, npts, 1.0, 0.0, st);
-    if (tc.p) return rotate_any((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, tc.p, st);
-    return rowmul<float>((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, st);
+    if (dtype == RS_F64) return rowmul<double>((const double *)Psi, ld, n, C, n, n, (double *)Psi, ld, npts, 1.0, 0.0, st, tc.err);
+    if (tc.p) return rotate_any((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, tc.p, st, tc.err);
+    return rowmul<float>((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, st, tc.err);
 }
 
 // Orthonormalise Psi in place; Ui (n x n) receives U^-1.  Blocking.
@@ -59,9 +59,9 @@ int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, i
     LaWork w(work, n);
     int *keys = reinterpret_cast<int *>(w.xi);   // not in use yet: scratch of the overlap
     if (dtype == RS_F64)
-        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st, false, keys));
+        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st, false, keys, tc.err));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st, tc.inner, keys));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)Psi, ld, n, npts, dV, w.U, n, st, tc.inner, keys, tc.err));
     RS_TRY(symmetrize(w.U, n, n, st));
     RS_TRY(cholesky(w.U, n, n, 1e-14, w.status, st));
     int bad = 0;
@@ -84,9 +84,9 @@ int subspace_diag_impl(rs_ham *h, void *Psi, void *HPsi, int64_t ld, int n, int 
                                   std::min(nb, n - b), dtype, st));
     int *keys = reinterpret_cast<int *>(w.xi);
     if (dtype == RS_F64)
-        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys));
+        RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys, tc.err));
     else
-        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, tc.inner, keys));
+        RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, tc.inner, keys, tc.err));
     RS_TRY(symmetrize(w.S, n, n, st));
     RS_TRY(eigh(w.S, n, n, eps_dev, w.xi, n, dtype == RS_F32 && tc.inner ? -1 : 2, w.status, w.eigw, st));
     RS_TRY(rotate_inplace(Psi, ld, n, w.xi, npts, dtype, st, tc));
