@@ -48,6 +48,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "device.h"
 #include "digits.h"
@@ -190,31 +191,35 @@ __device__ __forceinline__ int abs_key(float x) { return __float_as_int(x) & 0x7
 template <typename T> struct ExpOf;
 template <> struct ExpOf<double> {
     static constexpr int bias = 1023;
+    static constexpr int mant = 20, lo = 623, hi = 1423;   // bits below the exponent in a key; exponents taken
+    static constexpr int span = 512;                       // largest ratio of two columns of a rotation, 2^span
     static __device__ __forceinline__ int exponent(int key) { return key ? key >> 20 : bias; }
-    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 20) < 623 || (key >> 20) > 1423); }
+    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 20) < lo || (key >> 20) > hi); }
 };
 template <> struct ExpOf<float> {
     static constexpr int bias = 127;
+    static constexpr int mant = 23, lo = 64, hi = 254, span = 126;
     static __device__ __forceinline__ int exponent(int key) { return key ? key >> 23 : bias; }
-    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 23) < 64 || (key >> 23) > 254); }
+    static __device__ __forceinline__ bool plain(int key) { return key && ((key >> 23) < lo || (key >> 23) > hi); }
 };
 
 // q + 128 in every digit, q = trunc(|x| 2^(s - E)), |x| < 2^E, E = ecol - bias + 1.
 // The mantissa stands at bits 61 .. 9 (38) and is shifted right by `room` plus
-// the distance of the exponents; room = 62 - s.
+// the distance of the exponents; room = 62 - s.  sh: of an FP64 number, an exponent to
+// take off it (at bit 20).
 template <int NS> struct Bias {
     static constexpr uint64_t b = 0x8080808080808080ull >> (64 - 8 * NS);
     static constexpr int room = 62 - (8 * NS - 2);
 };
-template <int NS> __device__ __forceinline__ uint64_t biased_int(double x, int ecol) {
+template <int NS> __device__ __forceinline__ uint64_t biased_int(double x, int ecol, int sh) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int d = ((ecol + Bias<NS>::room) << 20) - (int)(hi & 0x7ff00000u);
+    const int d = ((ecol + Bias<NS>::room) << 20) + sh - (int)(hi & 0x7ff00000u);
     const uint32_t mh = (hi & 0xfffffu) | 0x100000u;
     const uint64_t l = (uint64_t)lo * 512u;
     const uint64_t m = ((uint64_t)(mh * 512u + (uint32_t)(l >> 32)) << 32) | (uint32_t)l;
     return (m >> min((uint32_t)(d >> 20), 63u)) + Bias<NS>::b;
 }
-template <int NS> __device__ __forceinline__ uint64_t biased_int(float x, int ecol) {
+template <int NS> __device__ __forceinline__ uint64_t biased_int(float x, int ecol, int) {
     const uint32_t b = __float_as_uint(x);
     const int d = ((ecol + Bias<NS>::room) << 23) - (int)(b & 0x7f800000u);
     const uint32_t mh = ((b & 0x7fffffu) | 0x800000u) << 6;
@@ -230,11 +235,12 @@ __device__ __forceinline__ uint32_t top_word(float x) { return __float_as_uint(x
 // a byte permutation and a logic operation per two digits on the integer
 // pipe, whose half rate bounds the conversion, the rest on the FP16 pipe.
 template <typename T, int NS>
-__device__ __forceinline__ void store_digits(const T (&v)[8], int ecol, unsigned char *dst, int stride) {
+__device__ __forceinline__ void store_digits(const T (&v)[8], int ecol, unsigned char *dst, int stride,
+                                             const int (&sh)[8] = {0, 0, 0, 0, 0, 0, 0, 0}) {
     uint32_t lo[8], hi[8], mul[4], add[4];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        const uint64_t u = biased_int<NS>(v[k], ecol);
+        const uint64_t u = biased_int<NS>(v[k], ecol, sh[k]);
         lo[k] = (uint32_t)u;
         hi[k] = (uint32_t)(u >> 32);
     }
@@ -694,6 +700,17 @@ template int digit_gram<double>(const double *, int64_t, int, const double *, in
 template int digit_gram<float>(const float *, int64_t, int, const float *, int64_t, int, int64_t, double, double *,
                                int64_t, int *, cudaStream_t, int *);
 
+template <typename T> int column_keys(const T *X, int64_t ldx, int n, int64_t npts, int *keys, cudaStream_t st) {
+    RS_CUDA(cudaMemsetAsync(keys, 0, sizeof(int) * (size_t)n, st));
+    const int gx = (n + 31) / 32;
+    const int rows = (int)std::max<int64_t>(1, std::min<int64_t>((npts + 63) / 64, 152 * 8 / gx));
+    k_digit_keys<T><<<dim3((unsigned)gx, (unsigned)rows), 256, 0, st>>>(X, ldx, n, X, ldx, 0, npts, gx, keys);
+    RS_LAUNCH_CHECK();
+    return RS_OK;
+}
+template int column_keys<double>(const double *, int64_t, int, int64_t, int *, cudaStream_t);
+template int column_keys<float>(const float *, int64_t, int, int64_t, int *, cudaStream_t);
+
 // ----------------------------------------------------------- rotation ---
 
 namespace {
@@ -702,6 +719,7 @@ template <typename T> struct RotArgs {
     const T *X;
     const double *C;
     T *Y;
+    const int *xk;       // keys of X's columns (their sizes), or nullptr: columns of one size
     int64_t ldx, ldc, ldy, npts;
     int n, m;
     int vec, yvec;       // X, Y rows on 16-byte boundaries
@@ -732,6 +750,14 @@ struct RotBars {
 // the key warps find the exponents of the next tile's rows (and bring the
 // rows into L2) while the converters work on this one, and the readout and
 // the stores of a tile overlap the products of the next.
+// Column sizes: an entry of X is resolved relative to the largest of its row, so a
+// small column would lose its digits beside large ones, though its row of C may
+// be as much larger (Psi U^-1 of columns that are not normalised).  So the columns are brought to
+// the size of the largest one by powers of two, 2^-a_k, and the rows of C
+// taken the other way, which changes no product: in FP64 as an addend of the
+// exponents' distance, in FP32 by a multiplication, which is exact (the factor is at
+// least 1) and on a pipe with nothing to do.  sh[k]: a_k at bit 20 (FP64), 2^-a_k
+// (FP32).  Columns more than 2^span apart: plain sums.
 // ONE: at most 256 states, so that a block is one readout and its sums need no
 // registers while the operands are converted (with them the converters spill:
 // 5.5 ms instead of 4.7 for 658 416 rows of 256 FP64 states).
@@ -743,7 +769,8 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
     extern __shared__ __align__(128) unsigned char dgsm[];
     __shared__ DgBars b;
     __shared__ RotBars rb;
-    __shared__ int ea[2][DG_M], eb[NBLK * BN];
+    __shared__ int ea[2][DG_M], eb[NBLK * BN], etop, zeros;
+    int *sh = reinterpret_cast<int *>(dgsm + DG_STAGES * C::STAGE);   // [kst * DG_K]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nb0 = blockIdx.x * NBLK;          // first column block
     const int kst = (a.n + DG_K - 1) / DG_K;    // stages per column block
@@ -755,26 +782,58 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
         }
         dg_bar_init(&rb.rd, DG_CT * (a.cluster ? gridDim.x : 1));
         dg_bar_init(&rb.sums, DG_CT);
+        etop = 0;
+        zeros = a.xk != nullptr;
     }
-    for (int i = tid; i < NBLK * BN; i += DG_NT) eb[i] = 0;
+    for (int i = tid; i < NBLK * BN; i += DG_NT) eb[i] = INT_MIN;
     dg_setup<NS>(b, C::TMEM, a.spin);
     if (a.cluster) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    // sizes of the columns of X; 0: a column of zeros, or one with entries beyond the
+    // digits' range, whose rows take plain sums: left as it is
+    auto size_of = [&](int k) {
+        const int key = a.xk && k < a.n ? __ldg(a.xk + k) : 0, e = max(key >> ExpOf<T>::mant, 1);
+        return key && e <= ExpOf<T>::hi ? e : 0;
+    };
+    for (int k = tid; k < a.n; k += DG_NT) {
+        const int e = size_of(k);
+        if (e) atomicMax(&etop, e);
+        if (a.xk && a.xk[k]) zeros = 0;   // (all columns are zero: the eigensolver's first directions)
+    }
+    __syncthreads();
+    for (int k = tid; k < kst * DG_K; k += DG_NT) {
+        const int e = size_of(k);
+        int d = e ? e - etop : 0;
+        if (d < -ExpOf<T>::span) {
+            b.plain = 1;
+            d = 0;
+        }
+        sh[k] = sizeof(T) == 8 ? d * (1 << 20) : (127 - d) << 23;
+    }
+    __syncthreads();
+    // what is added to the exponent (at bit 20) of row k of C
+    auto c_shift = [&](int v) { return sizeof(T) == 8 ? v : (127 << 20) - (v >> 3); };
     // exponents of the columns of C
     for (int blk = 0; blk < NBLK; ++blk)
         for (int w = warp; w < BN / 32 * 12; w += DG_NT / 32) {
             const int cl = (w / 12) * 32 + lane, c = (nb0 + blk) * BN + cl;
-            int k = 0;
+            int k = INT_MIN;
+            bool pl = false;
             if (c < a.m) {
 #pragma unroll 8
-                for (int q = w % 12; q < a.n; q += 12) k = max(k, abs_key(__ldg(a.C + (int64_t)q * a.ldc + c)));
+                for (int q = w % 12; q < a.n; q += 12) {
+                    const int key = abs_key(__ldg(a.C + (int64_t)q * a.ldc + c)), e = key >> 20;
+                    if (key) k = max(k, e + (c_shift(sh[q]) >> 20));
+                    pl = pl || e > ExpOf<double>::hi;
+                }
             }
-            if (k) atomicMax(&eb[blk * BN + cl], k);
+            if (pl) b.plain = 1;
+            if (k != INT_MIN) atomicMax(&eb[blk * BN + cl], k);
         }
     __syncthreads();
     for (int i = tid; i < NBLK * BN; i += DG_NT) {
-        const int k = eb[i];
-        if (ExpOf<double>::plain(k)) b.plain = 1;
-        eb[i] = ExpOf<double>::exponent(k);
+        const int e = eb[i] == INT_MIN ? ExpOf<double>::bias : eb[i];
+        if (e < ExpOf<double>::lo || e > ExpOf<double>::hi) b.plain = 1;
+        eb[i] = e;
     }
     __syncthreads();
     const bool cplain = b.plain != 0;
@@ -792,7 +851,13 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             for (int g = warp - DG_CW - 1; g < DG_M / 8; g += KW) {
                 const int r = g * 8 + (lane >> 2);
                 const T *x = a.X + (r0 + min(r, rows - 1)) * a.ldx;
-                int k = 0;
+                // largest scaled entry: as a key (FP32), with an addend to the exponent
+                // (FP64; of a zero, that stays below any exponent that is taken)
+                int k = INT_MIN;
+                auto take = [&](T v, int f) {
+                    if constexpr (sizeof(T) == 8) k = max(k, (__double2hiint(v) & 0x7fffffff) - f);
+                    else k = max(k, abs_key(v * __int_as_float(f)));
+                };
                 if (a.vec) {
                     constexpr int E = 16 / (int)sizeof(T);
                     const uint4 *xv = reinterpret_cast<const uint4 *>(x);
@@ -800,21 +865,35 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                     for (int q0 = lane & 3; q0 < nv; q0 += 32) {
                         uint4 t[8];
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) t[i] = xv[min(q0 + 4 * i, nv - 1)];
+                        for (int i = 0; i < 8; ++i)
+                            t[i] = ld_fresh(xv + min(q0 + 4 * i, nv - 1));   // in this order, ahead of the factors' reads:
+                        // with two or three in flight the key warps hold the others up (7.1 ms instead of 4.8 for 256 FP64 states)
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const T *tt = reinterpret_cast<const T *>(&t[i]);
 #pragma unroll
-                            for (int e = 0; e < E; ++e) k = max(k, abs_key(tt[e]));
+                            for (int e = 0; e < E; ++e) take(tt[e], sh[min(q0 + 4 * i, nv - 1) * E + e]);
                         }
                     }
-                    for (int q = nv * E + (lane & 3); q < a.n; q += 4) k = max(k, abs_key(x[q]));
+                    for (int q = nv * E + (lane & 3); q < a.n; q += 4) take(x[q], sh[q]);
                 } else {
 #pragma unroll 8
-                    for (int q = lane & 3; q < a.n; q += 4) k = max(k, abs_key(x[q]));
+                    for (int q = lane & 3; q < a.n; q += 4) take(x[q], sh[q]);
                 }
                 k = max(k, __shfl_xor_sync(0xffffffffu, k, 1));
                 k = max(k, __shfl_xor_sync(0xffffffffu, k, 2));
+                if (sizeof(T) == 8 && (k >> 20) < ExpOf<T>::lo) {
+                    // a row of zeros, or one for the plain sums
+                    int any = 0;
+                    if (!zeros)
+                        for (int q = lane & 3; q < a.n; q += 4) any |= abs_key(x[q]);
+                    k = any ? max(k, 1) : 0;
+                }
+                if (sizeof(T) == 8) {
+                    // (the four lanes of a row agree: one with an entry speaks for all)
+                    const int kk = max(k, __shfl_xor_sync(0xffffffffu, k, 1));
+                    k = max(kk, __shfl_xor_sync(0xffffffffu, kk, 2));
+                }
                 if ((lane & 3) == 0) ea[h][r] = ExpOf<T>::exponent(k);
                 pl = pl || ExpOf<T>::plain(k);
             }
@@ -891,6 +970,18 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
                     const int kk = k0 + 8 * bkq + k;
                     vb[k] = (c < a.m && kk < a.n) ? __ldg(a.C + (int64_t)kk * a.ldc + c) : 0.0;
                 }
+            }
+        };
+        // column factors of the eight steps kq of a stage, and the values of FP32 columns brought to one size
+        auto shifts = [&](int stage, int kq, int (&f)[8]) {
+            const int4 *p = reinterpret_cast<const int4 *>(sh + stage * DG_K + 8 * kq);
+            const int4 u = p[0], v = p[1];
+            f[0] = u.x, f[1] = u.y, f[2] = u.z, f[3] = u.w, f[4] = v.x, f[5] = v.y, f[6] = v.z, f[7] = v.w;
+        };
+        auto scale = [&](T (&v)[8], const int (&f)[8]) {
+            if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] *= __int_as_float(f[k]);
             }
         };
         // in place: tell every CTA of the row tile that this thread has read its rows
@@ -1035,15 +1126,30 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
             }
             if (!end && !plain && ok) {
                 const int s = g % DG_STAGES;
+                // read ahead of the wait (where there are registers): behind the digits'
+                // stores they would wait for those
+                int f[8], fb[8];
+                if constexpr (ONE) {
+                    shifts(kb, akq, f);
+                    shifts(kb, bkq, fb);
+                }
                 if (g >= DG_STAGES) ok = dg_wait_warp(&b.empty[s], (g / DG_STAGES - 1) & 1, &b.give);
                 const bool lasts = it + 1 == nst, more = !lasts || tile + (int)gridDim.y < ntiles;
                 const int nt = lasts ? tile + gridDim.y : tile, ni = lasts ? 0 : it + 1;
                 if (ok) {
-                    store_digits<T, NS>(va[0], ex0, adst + s * C::STAGE, C::SL_A);
+                    if constexpr (!ONE) shifts(kb, akq, f);
+                    scale(va[0], f);
+                    store_digits<T, NS>(va[0], ex0, adst + s * C::STAGE, C::SL_A, f);
                     if (more) load(0, nt, ni);
-                    store_digits<T, NS>(va[1], ex1, adst + s * C::STAGE + 128, C::SL_A);
+                    scale(va[1], f);
+                    store_digits<T, NS>(va[1], ex1, adst + s * C::STAGE + 128, C::SL_A, f);
                     if (more) load(1, nt, ni);
-                    if (hasb && g < bstages) store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B);
+                    if (hasb && g < bstages) {
+                        if constexpr (!ONE) shifts(kb, bkq, fb);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) fb[k] = -c_shift(fb[k]);
+                        store_digits<double, NS>(vb, eb[blk * BN + bcol], bdst + s * C::STAGE, C::SL_B, fb);
+                    }
                     if (more && g + 1 < bstages) load(2, nt, ni);
                     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                     dg_arrive(&b.full[s]);
@@ -1155,8 +1261,9 @@ int launch_rows(Fn fn, Args a, unsigned gx, size_t smem, bool in_place, cudaStre
 template <typename T, int NS, int BN, int NBLK, bool ONE> int launch_rot(RotArgs<T> a, bool in_place, cudaStream_t st) {
     using C = DgCfg<NS, BN, 32>;
     auto fn = k_digit_rot<T, NS, BN, NBLK, ONE>;
-    RS_TRY(smem_optin((const void *)fn, C::SMEM));
-    return launch_rows(fn, a, (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK)), C::SMEM, in_place, st);
+    const size_t smem = C::SMEM + sizeof(int) * (size_t)((a.n + DG_K - 1) / DG_K * DG_K);
+    RS_TRY(smem_optin((const void *)fn, smem));
+    return launch_rows(fn, a, (unsigned)((a.m + BN * NBLK - 1) / (BN * NBLK)), smem, in_place, st);
 }
 
 // ------------------------------------- FP32 rotation by BF16 pieces ---
@@ -1671,9 +1778,9 @@ bool digit_rot_takes(int n, int m, bool in_place) {
 
 template <typename T>
 int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-              double alpha, double beta, cudaStream_t st, int *err) {
+              double alpha, double beta, const int *xkeys, cudaStream_t st, int *err) {
     RotArgs<T> a{};
-    a.X = X, a.C = C, a.Y = Y, a.ldx = ldx, a.ldc = ldc, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
+    a.X = X, a.C = C, a.Y = Y, a.xk = xkeys, a.ldx = ldx, a.ldc = ldc, a.ldy = ldy, a.npts = npts, a.n = n, a.m = m;
     a.alpha = alpha, a.beta = beta, a.spin = t_rot_spin, a.err = err;
     a.vec = aligned16(X) && (ldx * (int64_t)sizeof(T)) % 16 == 0;
     a.yvec = aligned16(Y) && (ldy * (int64_t)sizeof(T)) % 16 == 0;
@@ -1685,9 +1792,9 @@ int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int 
     return one ? launch_rot<T, NS, 64, 1, true>(a, in_place, st) : launch_rot<T, NS, 64, 1, false>(a, in_place, st);
 }
 template int digit_rot<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
-                               double, double, cudaStream_t, int *);
+                               double, double, const int *, cudaStream_t, int *);
 template int digit_rot<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
-                              double, cudaStream_t, int *);
+                              double, const int *, cudaStream_t, int *);
 
 }  // namespace rs
 

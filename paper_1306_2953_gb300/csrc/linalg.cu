@@ -78,8 +78,9 @@ __global__ void __launch_bounds__(R_NT) k_rowmul(const T *X, int64_t ldx, int n,
 
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-           double alpha, double beta, cudaStream_t st, int *err) {
-    if (digit_rot_takes(n, m, X == Y)) return digit_rot<T>(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, st, err);
+           double alpha, double beta, const int *xkeys, cudaStream_t st, int *err) {
+    if (digit_rot_takes(n, m, X == Y))
+        return digit_rot<T>(X, ldx, n, C, ldc, m, Y, ldy, npts, alpha, beta, xkeys, st, err);
     const size_t smem = (size_t)R_ROWS * n * sizeof(T);
     if (smem > 200 * 1024) return fail(RS_EINVAL, "rowmul: n too large");
     if (smem > 48 * 1024) RS_TRY(smem_optin((const void *)k_rowmul<T>, smem));
@@ -89,9 +90,9 @@ int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, 
     return RS_OK;
 }
 template int rowmul<double>(const double *, int64_t, int, const double *, int64_t, int, double *, int64_t, int64_t,
-                            double, double, cudaStream_t, int *);
+                            double, double, const int *, cudaStream_t, int *);
 template int rowmul<float>(const float *, int64_t, int, const double *, int64_t, int, float *, int64_t, int64_t, double,
-                           double, cudaStream_t, int *);
+                           double, const int *, cudaStream_t, int *);
 
 // FP32 rotation to FP32 accuracy for any placement of Y: where Y overlaps X and
 // cannot be written in place by one launch, X is copied first.

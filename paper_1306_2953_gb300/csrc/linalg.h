@@ -11,16 +11,17 @@ namespace rs {
 
 // S = dV X^T Y (nx x ny, FP64, row stride lds); X, Y are [npts][ld] of T.
 // FP32 data: accurate like FP64, or (fast) to FP32 level; scratch: nx + ny ints or
-// nullptr (see digits.h).
+// nullptr (see digits.h; fast leaves it as it is).
 template <typename T>
 int gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny, int64_t npts, double dV, double *S,
          int64_t lds, cudaStream_t st, bool fast = false, int *scratch = nullptr, int *err = nullptr);
 
 // Y = alpha X C + beta Y; X [npts][ldx] (n columns), C FP64 [n][ldc]
-// (m columns), Y [npts][ldy]; Y may alias X when beta == 0.
+// (m columns), Y [npts][ldy]; Y may alias X when beta == 0.  xkeys: the sizes of X's columns
+// (column_keys of digits.h), or nullptr where they are of one size.
 template <typename T>
 int rowmul(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,
-           double alpha, double beta, cudaStream_t st, int *err = nullptr);
+           double alpha, double beta, const int *xkeys, cudaStream_t st, int *err = nullptr);
 
 // FP32 rotation to FP32 accuracy for any placement of Y relative to X.  work:
 // rotate_work_bytes(n, m, npts) bytes; copy_rows = 0 serves when Y is apart from
@@ -88,9 +89,10 @@ struct TcWork {
     int *err = nullptr;
 };
 
-// Psi (n columns) <- Psi C in place (C FP64 n x n).
-int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, cudaStream_t st,
-                   const TcWork &tc = TcWork());
+// Psi (n columns) <- Psi C in place (C FP64 n x n).  xkeys: as in rowmul (the FP32
+// rotations to FP32 accuracy have no use for them).
+int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, const int *xkeys,
+                   cudaStream_t st, const TcWork &tc = TcWork());
 // Psi <- Psi U^-1 with <Psi|Psi> = U^T U; w.Ui keeps U^-1.  Blocking; RS_ENOTSPD on failure.
 int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, int dtype, void *work, cudaStream_t st,
                         const TcWork &tc = TcWork());

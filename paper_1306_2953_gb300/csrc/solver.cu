@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "device.h"
+#include "digits.h"
 #include "ham.h"
 #include "learned.h"
 #include "linalg.h"
@@ -444,7 +445,7 @@ struct rs_solver {
     double dV = 0;
     int es = 8;
     int nblk = 0;
-    DevBuf psi, hpsi, P, Z, HZ, R, small, la, eig, res, tcbuf, psi64, hpsi64, rr64;
+    DevBuf psi, hpsi, P, Z, HZ, R, small, la, eig, res, tcbuf, psi64, hpsi64, rr64, pkeys;
     TcWork tc;
     std::vector<char> has_p;
     Precond *pc = nullptr;
@@ -494,11 +495,12 @@ int gram_any(int dtype, const void *X, int64_t ldx, int nx, const void *Y, int64
     return gram<float>((const float *)X, ldx, nx, (const float *)Y, ldy, ny, npts, dV, S, lds, st, true, nullptr, tc.err);
 }
 
-// (X and Y are different arrays, or column slices of one)
+// (X and Y are different arrays, or column slices of one; X's columns are normalised:
+// Psi, or the search space)
 int rowmul_any(int dtype, const void *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, void *Y, int64_t ldy,
                int64_t npts, double alpha, double beta, cudaStream_t st, const TcWork &tc) {
     if (dtype == RS_F64)
-        return rowmul<double>((const double *)X, ldx, n, C, ldc, m, (double *)Y, ldy, npts, alpha, beta, st, tc.err);
+        return rowmul<double>((const double *)X, ldx, n, C, ldc, m, (double *)Y, ldy, npts, alpha, beta, nullptr, st, tc.err);
     return rotate_any((const float *)X, ldx, n, C, ldc, m, (float *)Y, ldy, npts, alpha, beta, tc.p, st, tc.err);
 }
 
@@ -899,9 +901,10 @@ static int certify_impl(rs_solver *S, int n_smooth, double lam, double *eps_dev,
         RS_TRY(S->rr64.alloc(sizeof(double) * (4 * nn + 16) + eigh_work_bytes(n)));
     }
     DevBuf cbuf;
-    RS_TRY(cbuf.alloc(sizeof(double) * (2 * nn)));
+    RS_TRY(cbuf.alloc(sizeof(double) * (2 * nn + n)));
     double *Sm = S->rr64.as<double>(), *h = Sm + nn, *Ui = h + nn, *T = Ui + nn;
     double *Y = cbuf.as<double>(), *C = Y + nn;
+    int *keys = reinterpret_cast<int *>(C + nn);   // sizes of the columns of P and Q
     int *status = reinterpret_cast<int *>(T + nn);
     void *ew = reinterpret_cast<void *>(T + nn + 16);
     double *P = S->psi64.as<double>(), *Q = S->hpsi64.as<double>();
@@ -935,7 +938,7 @@ static int certify_impl(rs_solver *S, int n_smooth, double lam, double *eps_dev,
     // h x = eps S x (Sec. VI, Eq. 7) with S = U^T U: the Ritz vectors are
     // Psi C with C = U^-1 Y, Y the eigenvectors of U^-T h U^-1
     RS_TRY(gram<double>(P, n, n, P, n, n, S->npts, S->dV, Sm, n, st));
-    RS_TRY(gram<double>(P, n, n, Q, n, n, S->npts, S->dV, h, n, st));
+    RS_TRY(gram<double>(P, n, n, Q, n, n, S->npts, S->dV, h, n, st, false, keys));
     RS_TRY(symmetrize(Sm, n, n, st));
     RS_TRY(symmetrize(h, n, n, st));
     RS_TRY(cholesky(Sm, n, n, 1e-14, status, st));
@@ -951,8 +954,8 @@ static int certify_impl(rs_solver *S, int n_smooth, double lam, double *eps_dev,
     RS_TRY(gemm_small(n, n, n, 1.0, Ui, n, false, Y, n, false, 0.0, C, n, st));
     // the Ritz vectors and H applied to them (rotated in place), their FP64
     // residual norms ||H x_k - eps_k x_k|| with <x_k|x_k> = 1
-    RS_TRY(rowmul<double>(P, n, n, C, n, n, P, n, S->npts, 1.0, 0.0, st));
-    RS_TRY(rowmul<double>(Q, n, n, C, n, n, Q, n, S->npts, 1.0, 0.0, st));
+    RS_TRY(rowmul<double>(P, n, n, C, n, n, P, n, S->npts, 1.0, 0.0, keys, st));
+    RS_TRY(rowmul<double>(Q, n, n, C, n, n, Q, n, S->npts, 1.0, 0.0, keys + n, st));
     RS_CUDA(cudaMemsetAsync(res_dev, 0, sizeof(double) * n, st));
     k_resid_norm2<<<dim3((unsigned)((n + 255) / 256), 512), 256, 0, st>>>(P, Q, n, n, eps_dev, S->npts, res_dev);
     k_sqrt_scale<<<(n + 255) / 256, 256, 0, st>>>(res_dev, n, S->dV);
@@ -1021,7 +1024,7 @@ extern "C" int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void 
         (rc = S->res.alloc(sizeof(double) * c.nst)))
         return bail(rc);
     if (!rmm && ((rc = S->P.alloc(big)) || (rc = S->Z.alloc(zb)) || (rc = S->HZ.alloc(zb)) ||
-                 (rc = S->R.alloc((size_t)S->npts * c.nb * S->es))))
+                 (rc = S->R.alloc((size_t)S->npts * c.nb * S->es)) || (rc = S->pkeys.alloc(sizeof(int) * c.nst))))
         return bail(rc);
     if (rmm && ((rc = S->rmm_hist.alloc((size_t)(3 * (S->rmm_M + 1) + 5) * S->npts * c.nb * S->es)) ||
                 (rc = S->rmm_small.alloc(sizeof(double) * 64 * (MD_MAX + 2 * RMM_MAXK * RMM_MAXK + RMM_MAXK + 2)))))
@@ -1071,6 +1074,17 @@ extern "C" int rs_solver_create(rs_ham *h, const rs_solver_cfg *cfg, const void 
 
 namespace {
 
+// P <- P C; the directions are as different in size as the states are in convergence.
+int rotate_directions(rs_solver *S, const double *C, cudaStream_t st) {
+    const int n = S->cfg.nst;
+    int *keys = nullptr;
+    if (S->cfg.dtype == RS_F64) {
+        keys = S->pkeys.as<int>();
+        RS_TRY(column_keys(S->P.as<double>(), n, n, S->npts, keys, st));
+    }
+    return rotate_inplace(S->P.p, n, n, C, S->npts, S->cfg.dtype, keys, st, S->tc);
+}
+
 // The updates of a sweep and the Rayleigh-Ritz that closes it.
 int sweep_impl(rs_solver *S, cudaStream_t st) {
     const rs_solver_cfg &c = S->cfg;
@@ -1078,10 +1092,10 @@ int sweep_impl(rs_solver *S, cudaStream_t st) {
     for (int b = 0; b < S->nblk; ++b) RS_TRY(rmm ? rmm_block_step(S, b, st) : block_step(S, b, st));
     RS_TRY(orthonormalize_impl(S->npts, S->dV, S->psi.p, c.nst, c.nst, c.dtype, S->la.p, st, S->tc));
     LaWork w(S->la.p, c.nst);
-    if (!rmm) RS_TRY(rotate_inplace(S->P.p, c.nst, c.nst, w.Ui, S->npts, c.dtype, st, S->tc));
+    if (!rmm) RS_TRY(rotate_directions(S, w.Ui, st));
     RS_TRY(subspace_diag_impl(S->h, S->psi.p, S->hpsi.p, c.nst, c.nst, c.dtype, c.nb, S->la.p, S->eig.as<double>(), st,
                               S->tc));
-    if (!rmm) RS_TRY(rotate_inplace(S->P.p, c.nst, c.nst, w.xi, S->npts, c.dtype, st, S->tc));
+    if (!rmm) RS_TRY(rotate_directions(S, w.xi, st));
     return RS_OK;
 }
 

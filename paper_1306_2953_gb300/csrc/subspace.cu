@@ -46,18 +46,18 @@ extern "C" int64_t rs_linalg_workspace_bytes(int nst) {
 
 namespace rs {
 
-int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, cudaStream_t st,
-                   const TcWork &tc) {
-    if (dtype == RS_F64) return rowmul<double>((const double *)Psi, ld, n, C, n, n, (double *)Psi, ld, npts, 1.0, 0.0, st, tc.err);
+int rotate_inplace(void *Psi, int64_t ld, int n, const double *C, int64_t npts, int dtype, const int *xkeys,
+                   cudaStream_t st, const TcWork &tc) {
+    if (dtype == RS_F64) return rowmul<double>((const double *)Psi, ld, n, C, n, n, (double *)Psi, ld, npts, 1.0, 0.0, xkeys, st, tc.err);
     if (tc.p) return rotate_any((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, tc.p, st, tc.err);
-    return rowmul<float>((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, st, tc.err);
+    return rowmul<float>((const float *)Psi, ld, n, C, n, n, (float *)Psi, ld, npts, 1.0, 0.0, xkeys, st, tc.err);
 }
 
 // Orthonormalise Psi in place; Ui (n x n) receives U^-1.  Blocking.
 int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, int dtype, void *work, cudaStream_t st,
                         const TcWork &tc) {
     LaWork w(work, n);
-    int *keys = reinterpret_cast<int *>(w.xi);   // not in use yet: scratch of the overlap
+    int *keys = reinterpret_cast<int *>(w.xi);   // not in use: scratch of the overlap, then the columns' sizes
     if (dtype == RS_F64)
         RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)Psi, ld, n, npts, dV, w.U, n, st, false, keys, tc.err));
     else
@@ -69,7 +69,7 @@ int orthonormalize_impl(int64_t npts, double dV, void *Psi, int64_t ld, int n, i
     RS_CUDA(cudaStreamSynchronize(st));
     if (bad) return fail(RS_ENOTSPD, "orthonormalize: overlap matrix not positive definite (pivot %d)", bad - 1);
     RS_TRY(tri_inv(w.U, n, n, w.Ui, n, st));
-    return rotate_inplace(Psi, ld, n, w.Ui, npts, dtype, st, tc);
+    return rotate_inplace(Psi, ld, n, w.Ui, npts, dtype, keys, st, tc);
 }
 
 // Subspace diagonalisation; eps (device, n) and w.xi receive the results.  Blocking.
@@ -82,15 +82,15 @@ int subspace_diag_impl(rs_ham *h, void *Psi, void *HPsi, int64_t ld, int n, int 
     for (int b = 0; b < n; b += nb)
         RS_TRY(rs_ham_apply_block(h, (const char *)Psi + (size_t)b * es, ld, (char *)HPsi + (size_t)b * es, ld,
                                   std::min(nb, n - b), dtype, st));
-    int *keys = reinterpret_cast<int *>(w.xi);
+    int *keys = reinterpret_cast<int *>(w.U);   // free here (xi receives the eigenvectors): 2 n ints
     if (dtype == RS_F64)
         RS_TRY(gram<double>((const double *)Psi, ld, n, (const double *)HPsi, ld, n, npts, dV, w.S, n, st, false, keys, tc.err));
     else
         RS_TRY(gram<float>((const float *)Psi, ld, n, (const float *)HPsi, ld, n, npts, dV, w.S, n, st, tc.inner, keys, tc.err));
     RS_TRY(symmetrize(w.S, n, n, st));
     RS_TRY(eigh(w.S, n, n, eps_dev, w.xi, n, dtype == RS_F32 && tc.inner ? -1 : 2, w.status, w.eigw, st));
-    RS_TRY(rotate_inplace(Psi, ld, n, w.xi, npts, dtype, st, tc));
-    return rotate_inplace(HPsi, ld, n, w.xi, npts, dtype, st, tc);
+    RS_TRY(rotate_inplace(Psi, ld, n, w.xi, npts, dtype, keys, st, tc));
+    return rotate_inplace(HPsi, ld, n, w.xi, npts, dtype, keys + n, st, tc);
 }
 
 }  // namespace rs

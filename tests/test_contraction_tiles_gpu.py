@@ -74,3 +74,58 @@ def test_rows_beyond_the_digits_in_many_tiles(dtype, n):
         r = slice(128 * k, min(128 * k + 128, g.npts))
         assert bool((err[r] <= (2 * (n + 8) * 2.0 ** -53 + 2 * u) * mag[r]).all())
     assert bool((err <= 64 * n * u * x.abs().amax(1)[:, None] * C.abs().amax(0)[None, :]).all())
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("scales", [(1, 1e-5, 1, 1e-8), (1e-6, 1, 1e3, 1e-12), (1e20, 1e-15, 1e-3, 1)])
+@pytest.mark.parametrize("n", [4, 40, 66, 300])
+def test_rotation_of_columns_of_different_size(dtype, scales, n):
+    """Orthonormalisation of columns whose sizes differ: Psi <- Psi U^-1 multiplies
+    each by about the inverse of its size, so every one counts in full.
+    Tolerance: the digits resolve s bits below the largest entry of a row of the
+    columns brought to one size by powers of two, r_k, and of a column of U^-1 with its
+    rows taken the other way; each of the n products is off by at most 8 * 2^-s of
+    these.  The reference's sums are within n * 2^-53 of the sum of products, the
+    result is rounded once."""
+    from paper_1306_2953_gb300 import api
+    t, s, u = (torch.float64, 62, 2.0 ** -53) if dtype == "f64" else (torch.float32, 38, 2.0 ** -24)
+    g = api.Grid.box(31, 31, 32, 0.3)
+    rng = np.random.default_rng(n)
+    size = np.array([scales[k % 4] for k in range(n)])
+    P = torch.from_numpy(rng.uniform(-1, 1, (g.npts, n)) * size).to(t).cuda()
+    x = P.double().clone()
+    C = api.orthonormalize(g, P)
+    ref = x @ C
+    r = torch.exp2(torch.floor(torch.log2(x.abs().amax(0))))
+    tol = ((n + 8) * 2.0 ** -53 * (x.abs() @ C.abs()) + 2 * u * ref.abs() +
+           8 * n * 2.0 ** -s * (x.abs() / r).amax(1)[:, None] * (r[:, None] * C.abs()).amax(0)[None, :])
+    assert bool(((P.double() - ref).abs() <= tol).all())
+
+
+@pytest.mark.parametrize("dtype,scales", [("f64", (1e150, 1.0, 1e-150, 1e5)), ("f32", (1e30, 1.0, 1e-25, 1e5))])
+@pytest.mark.parametrize("n", [40, 66])
+def test_rotation_of_columns_too_far_apart_for_the_digits(dtype, scales, n):
+    """Sizes further apart than the digits' scaling reaches: plain sums.
+    Tolerance: n terms in FP64 here and in the reference, one rounding to the type."""
+    from paper_1306_2953_gb300 import api
+    t, u = (torch.float64, 2.0 ** -53) if dtype == "f64" else (torch.float32, 2.0 ** -24)
+    g = api.Grid.box(13, 12, 11, 0.3)
+    size = np.array([scales[k % 4] for k in range(n)])
+    P = torch.from_numpy(np.random.default_rng(n).uniform(-1, 1, (g.npts, n)) * size).to(t).cuda()
+    x = P.double().clone()
+    C = api.orthonormalize(g, P)
+    ref, mag = x @ C, x.abs() @ C.abs()
+    assert bool(((P.double() - ref).abs() <= (2 * (n + 8) * 2.0 ** -53 + 2 * u) * mag).all())
+
+
+def test_rotation_of_zero_rows():
+    """Rows of zeros (whole tiles and parts) stay zero, beside columns of two sizes."""
+    from paper_1306_2953_gb300 import api
+    g = api.Grid.box(31, 31, 32, 0.3)
+    x = np.random.default_rng(3).uniform(-1, 1, (g.npts, 70)) * np.array([1e-7 if k % 3 else 1.0 for k in range(70)])
+    x[1000:5000] = 0
+    P = torch.from_numpy(x).cuda()
+    C = api.orthonormalize(g, P)
+    assert not P[1000:5000].any()
+    ref = torch.from_numpy(x).cuda() @ C
+    assert (P - ref).abs().max() <= 1e-13 * ref.abs().max()
