@@ -435,6 +435,7 @@ template <typename T> struct GramArgs {
     double dV;
     int tiles_n, stages, per_cta;   // stages in all and per CTA
     int sym;                 // Y is X: only the elements j >= i are computed, and mirrored
+    int far;                 // rows 4 GB or more apart: the digit path's row strides are 32-bit numbers of bytes
     int spin;                // barrier tests before a wait gives up
     int *err;                // status word (or nullptr): 1 once one has
 };
@@ -468,12 +469,12 @@ template <typename T, int NS, int BN> __global__ void __launch_bounds__(DG_NT, 1
         const int c = isa ? m0 + i : n0 + i - DG_M;
         const int key = isa ? (c < a.nx ? a.kx[c] : 0) : (c < a.ny ? a.ky[c] : 0);
         (isa ? ea[i] : eb[i - DG_M]) = ExpOf<T>::exponent(key);
-        if (ExpOf<T>::plain(key)) b.plain = 1;
+        if (ExpOf<T>::plain(key) || a.far) b.plain = 1;
     }
     __syncthreads();
     const int64_t p0 = (int64_t)st0 * DG_K, p1 = min(a.npts, p0 + (int64_t)nst * DG_K);
     if (b.plain) {
-        // a column beyond the digits' range: plain FP64 sums of this tile and range
+        // a column beyond the digits' range, or far rows: plain FP64 sums of this tile and range
         for (int e = tid; e < DG_M * BN; e += DG_NT) {
             const int i = m0 + e / BN, j = n0 + e % BN;
             if (i >= a.nx || j >= a.ny || (a.sym && j < i)) continue;
@@ -687,7 +688,7 @@ int digit_gram(const T *X, int64_t ldx, int nx, const T *Y, int64_t ldy, int ny,
         GramArgs<T> a{};
         a.X = X, a.Y = Y, a.ldx = ldx, a.ldy = ldy, a.npts = npts, a.lds = lds, a.nx = nx, a.ny = ny;
         a.kx = keys, a.ky = sym ? keys : keys + nx;
-        a.S = S, a.dV = dV, a.sym = sym, a.spin = t_gram_spin, a.err = err;
+        a.S = S, a.dV = dV, a.sym = sym, a.far = std::max(ldx, ldy) > (int64_t)(UINT32_MAX / sizeof(T)), a.spin = t_gram_spin, a.err = err;
         const int tm = (nx + DG_M - 1) / DG_M;
         // 32 columns of Y fill half of a 64-wide tile
         const bool narrow = ny <= 32;
