@@ -626,13 +626,18 @@ __device__ __forceinline__ bool item_empty(const int (&q)[NBH]) {
 }
 
 // An FP32 value cut exactly into three BF16 pieces of 8 bits; two values to a
-// word, the first in the low half.
+// word, the first in the low half.  An infinity is its first piece alone (what is left of it
+// would be a NaN, which the next layer's relu turns into 0).
 __device__ __forceinline__ void bf16_cut(float x, float y, uint32_t (&p)[3]) {
+    auto rest = [](float v, int k) {
+        const float r = v - __uint_as_float(__float_as_uint(v) & 0xffff0000u);
+        return k > 0 || r == r ? r : 0.f;
+    };
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         p[k] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
-        x -= __uint_as_float(__float_as_uint(x) & 0xffff0000u);
-        y -= __uint_as_float(__float_as_uint(y) & 0xffff0000u);
+        x = rest(x, k);
+        y = rest(y, k);
     }
 }
 
