@@ -138,15 +138,21 @@ constexpr int CHOL_SMEM_MAX = 160;   // n x n FP64 in 200 KB
 template <typename Orig>
 __device__ __forceinline__ void chol_cta(double *A, int ld, int n, double rel, Orig orig, double *g, int *bad) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    // warp 0: pivot j, whose value is lane 0's d, and its g
+    // warp 0: pivot j, whose value is lane 0's d, and its g (by division where the
+    // reciprocal would be infinite or lose bits)
     auto pivot = [&](int j, double d) {
         double t = 0.0;
         if (lane == 0) {
             if (!(isfinite(d) && d > 0.0 && d > rel * orig(j))) *bad = j + 1;
-            t = 1.0 / d;
+            t = d > 0x1p-1020 && d < 0x1p1020 ? 1.0 / d : 0.0;
         }
         t = __shfl_sync(0xffffffffu, t, 0);
-        for (int c = j + 1 + lane; c < n; c += 32) g[(j & 1) * n + c] = A[(int64_t)j * ld + c] * t;
+        if (t != 0.0) {
+            for (int c = j + 1 + lane; c < n; c += 32) g[(j & 1) * n + c] = A[(int64_t)j * ld + c] * t;
+        } else {
+            d = __shfl_sync(0xffffffffu, d, 0);
+            for (int c = j + 1 + lane; c < n; c += 32) g[(j & 1) * n + c] = A[(int64_t)j * ld + c] / d;
+        }
     };
     if (warp == 0) pivot(0, A[0]);
     __syncthreads();
