@@ -391,8 +391,9 @@ extern "C" int rs_poisson_create(const rs_grid *g, rs_poisson **out) {
         s.e[d] = hi[d] - lo[d] + 1;
         s.N[d] = smooth_size((hi[d] - lo[d]) + (int)std::ceil(rc / g->h) + 1);
         if (s.N[d] > MAX_N) {
+            const int n = s.N[d];
             delete P;
-            return fail(RS_EINVAL, "rs_poisson_create: cube of %d points along an axis exceeds %d", P->s.N[d], MAX_N);
+            return fail(RS_EINVAL, "rs_poisson_create: cube of %d points along an axis exceeds %d", n, MAX_N);
         }
         tot *= s.N[d];
     }
