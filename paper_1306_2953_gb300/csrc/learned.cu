@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(NET_NT) k_net_last(NetGrid g, const float *__r
     }
 }
 
-// ---- one to three columns: one thread per point and state, FP32 FMA ----
+// ---- few columns and small grids: one thread per point and state, FP32 FMA ----
 
 // xhat = bf16(r / rms) and the per-column rms
 __global__ void k_net_input(const float *__restrict__ R, int64_t ldr, const double *__restrict__ rms, int nb,
@@ -1117,6 +1117,32 @@ extern "C" int rs_precond_train_tiles(float *w_dev, const float *x_dev, const ui
 
 namespace rs {
 
+// Points below which nb columns go a thread to a point and state.  The row
+// kernels win by reading each activation once for three taps, but a CTA's rows (ITEMS nb)
+// leave its last round of 256 threads part empty, and small grids do not fill the GPU.
+// us, thread per point / row kernels:
+//   points   8 052    15 915   28 872   41 625   72 344   120 681  138 507  654 520
+//   1 col.   75/77    74/82    74/87    89/105   93/125   133/161  138/167  442/454
+//   3        67/81    71/90    80/95    94/121   125/150  181/206  195/214  742/663
+//   4        70/81    82/91    99/99    140/129  211/164  315/209  340/219
+//   5        72/93    73/105   87/117   114/156  166/181  233/251  259/269
+//   6        70/97    78/113   105/121  145/153  197/185  294/272  325/288
+//   7        70/104   80/117   106/132  141/165  201/208  288/312  329/332
+//   8        73/103   90/116   119/131  176/168  246/226  378/296  420/315
+//   9        69/78    87/100   137/146  167/180  241/231  367/360  417/392
+//   11       71/83    96/107   150/157  178/189  277/250  425/396  479/433
+//   12       74/83    99/108   165/155  210/188  312/260  489/405  552/446
+//   16       77/81    128/100  163/140
+//   32       117/118  175/146  261/198
+// (8 columns, 33 429 points: 148/138; 4 columns, 20 724: 99/92; 5 and 7 columns, 154 249: 285/283, 354/348.)
+static int64_t per_point_below(int nb) {
+    if (nb <= 3) return INT64_MAX;
+    if (nb == 5 || nb == 7) return 150000;
+    if (nb == 8) return 31000;
+    if (nb >= 6 && nb <= 11) return 50000;
+    return nb <= 15 ? 18000 : nb <= 32 ? 10000 : 0;
+}
+
 int learned_apply(const rs_ham *h, const float *R, int64_t ldr, float *W, int64_t ldw, int nb, const float *wq_dev,
                   float *act, double *dots, cudaStream_t st) {
     const int64_t np = ham_npts(h);
@@ -1125,14 +1151,7 @@ int learned_apply(const rs_ham *h, const float *R, int64_t ldr, float *W, int64_
     k_rms<<<1, 64, 0, st>>>(ss, nb, 1.0 / (double)np, rms);
     if (np * nb >= (int64_t)INT32_MAX) return fail(RS_EINVAL, "learned preconditioner: npts * nb above 2^31");
     // (the scale array shares the activations' buffer: 64 floats ahead of them)
-    // Few columns do not fill the row kernels: us at 1 / 2 / 3 / 4 columns, row
-    // kernels 148 / 167 / 205 / 188 on 103 331 points and 454 / 541 / 663 / 726 on
-    // 654 520, thread per point and state 112 / 172 / 162 / 278 and 442 / 774 / 742 / 1396.
-    // Nor do 5 or 7, or 9 to 11 (a CTA's rows leave its last round half empty), until
-    // the grid has rounds enough: 5 / 7 columns 156 / 161 against 113 / 142 on 41 625 points, 250 / 309
-    // against 230 / 287 on 120 681, 283 / 348 against 285 / 354 on 154 249; 9 / 11
-    // columns 176 / 185 against 167 / 178 on 41 625, 221 / 243 against 239 / 275 on 71 387.
-    const bool per_point = nb <= 3 || (np < 150000 && (nb == 5 || nb == 7)) || (np < 50000 && nb >= 5 && nb <= 11);
+    const bool per_point = np < per_point_below(nb);
     if (per_point) {
         const int n32 = (int)np;
         float *x = act, *a1 = x + np * nb, *a2 = a1 + np * NC * nb;

@@ -6,14 +6,14 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("d", [(17, 18, 19), (27, 28, 29)])
 @pytest.mark.parametrize("nb", [4, 12, 16, 32])
-def test_infinite_activations_stay_infinite(nb):
+def test_infinite_activations_stay_infinite(nb, d):
     """One spike per column overflows the first layer's first channel: the output
     is infinite within the network's reach of three points and finite elsewhere, as the network
     in FP64 with every layer's output cast to FP32 says.  Tolerance of the finite values: FP32 sums of
     8 * 27 products and BF16 rounding of the input (2^-9, of either neighbour)."""
     from paper_1306_2953_gb300 import api
-    d = (17, 18, 19)
     g = api.Grid.box(*d, 0.3)
     H = api.Hamiltonian(g, np.zeros(g.npts))
     rng = np.random.default_rng(nb)
