@@ -33,10 +33,16 @@ int pool_of_device(cudaMemPool_t *out) {
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
+        // the first call may stand in a stream capture, which allows this thread no
+        // such call unless it asks (it enqueues nothing, so the graph is not touched)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        RS_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
         cudaMemPool_t p = nullptr;
-        RS_CUDA(cudaMemPoolCreate(&p, &props));
         uint64_t keep = 256ull << 20;
-        RS_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
+        cudaError_t e = cudaMemPoolCreate(&p, &props);
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        RS_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        RS_CUDA(e);
         pools[dev] = p;
     }
     *out = pools[dev];
