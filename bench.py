@@ -819,7 +819,6 @@ def main():
     clocks = ClockSampler(torch.cuda.current_device())
     clocks.start()
     time.sleep(0.3)
-    _lib.call("rs_ham_timing", H._h, 1)
     if world > 1:
         dist.barrier()
     torch.cuda.synchronize()
@@ -831,10 +830,16 @@ def main():
     torch.cuda.synchronize()
     if world > 1:
         dist.barrier()
-    _lib.call("rs_ham_timing", H._h, 0)
     if H.status() != 0:
         raise RuntimeError("an H psi pipeline wait gave up during the timed region: the results are incomplete")
     ms = e0.elapsed_time(e1)
+    # the launches one by one, in a pass of its own: the events between them keep
+    # each launch from overlapping the end of the one before
+    _lib.call("rs_ham_timing", H._h, 1)
+    for _ in range(args.steps):
+        step(psi, hpsi)
+    torch.cuda.synchronize()
+    _lib.call("rs_ham_timing", H._h, 0)
     pms, sms, ncalls = ctypes.c_double(), ctypes.c_double(), ctypes.c_int64()
     _lib.call("rs_ham_timing_read", H._h, ctypes.byref(pms), ctypes.byref(sms), ctypes.byref(ncalls))
     clk = clocks.stop()
@@ -901,7 +906,8 @@ def main():
                          "peak_source": peak_kind, "traffic": profiled_traffic(workload.name),
                          "algorithmic_bytes_per_launch": sb.value,
                          "stencil_ms_per_launch": sms.value / max(ncalls.value, 1),
-                         "project_ms_per_launch": pms.value / max(ncalls.value, 1)},
+                         "project_ms_per_launch": pms.value / max(ncalls.value, 1),
+                         "launch_times": "events around every launch, in a pass behind the timed one"},
             "e2e": {"value": world * bytes_per_step / e2e_s / 1e9, "unit": "GB/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": h2d, "ms_per_step": e2e_s * 1e3,
                     "pipeline": "32-state blocks from pinned host memory; copy in, H psi, copy out overlapped on 3 streams",
