@@ -232,7 +232,11 @@ int rs_ham_launch_bytes(const rs_ham *h, int nb, int dtype, int64_t *project_byt
  * blocks of points and accumulated in FP64.
  *   X_dev [npts][ldx] (nx columns), Y_dev [npts][ldy] (ny columns), dtype
  *   S_dev device double [nx][lds]
- * Asynchronous. */
+ * Every product is accurate to 9 * 2^-62 (RS_F64) or 8 * 2^-54 (RS_F32) of 2^(Ex + Ey), the
+ * powers of two above its columns' largest entries, so S_jk relative to the
+ * norms of x_j and y_k; columns with non-finite or extreme entries are summed plainly.
+ * Asynchronous; takes 4 (nx + ny) bytes from a stream-ordered pool of the library
+ * (in a captured graph: an allocation and a free node). */
 int rs_overlap_block(const rs_grid *g, const void *X_dev, int64_t ldx, int nx, const void *Y_dev, int64_t ldy,
                      int ny, double *S_dev, int64_t lds, int dtype, void *stream);
 

@@ -5,22 +5,26 @@
 //   rotation  Y = alpha X C + beta Y   (contraction over the states)
 //
 // GB300 has about 1.1 TFLOP/s of FP64 FMA against 1.9 PFLOP/s of FP16 tensor
-// throughput.  An operand value is written as an integer q = x 2^(s - E), E
-// the exponent of the largest entry of its column (overlap; of its row of X
-// and column of C in the rotation) and s = 8 NS - 2, and q as NS balanced
-// digits in base 256, |d| <= 128, each exact in FP16.  Digit products are
+// throughput.  An operand value is written as an integer q = trunc(x 2^(s - E)),
+// 2^E above the largest entry of its column (overlap; of its row of X, the columns
+// brought to one size, and of its column of C in the rotation) and s = 8 NS - 2, and q as NS
+// balanced digits in base 256, |d| <= 128, each exact in FP16.  Digit products are
 // integers of at most 2^14, so the FP32 accumulators of the tensor cores sum
 // up to 1024 of them without any rounding.  The products of weight
 // 256^-(i+j), i + j = t, have their own accumulator in tensor memory for
-// every t < NS (NS of them; those with i + j >= NS are below the digits'
-// own resolution and are left out); the accumulators are read out every 256
-// points and summed as 64-bit integers: with t + 1 pairs of digits in
-// accumulator t everything up to t = 3 is exact and a rounding of a later
-// one is below 2^-56 of the largest product.  So the result is the exact
-// sum of products of operands rounded to s bits: NS = 8 (FP64), 7 (overlap of
-// FP32 data at FP64-like accuracy) or 5 (rotation of FP32 data).  (Ozaki,
-// Ogita, Oishi and Rump 2012 give the scheme of error-free splittings of a
-// matrix product.)
+// every t < NS; the accumulators are read out every 256 points and summed as
+// 64-bit integers: with t + 1 pairs of digits in accumulator t everything up to
+// t = 3 is exact and a rounding of a later one is below 2^-56 of the largest
+// product.  NS = 8 (FP64), 7 (overlap of FP32 data at FP64-like accuracy) or 5 (rotation of
+// FP32 data).  (Ozaki, Ogita, Oishi and Rump 2012 give the scheme of error-free
+// splittings of a matrix product.)
+// Error of one product x y, in units of 2^(Ex + Ey - s): below 1 for each operand's
+// truncation and NS - 1 for the digits with i + j = NS, the first that are left out (the rest
+// is a 256th of that); signs and digits vary, so sums of many come out far below.  It is relative
+// to the largest entries, not to x y: sums of products that are all below 2^-9 (FP64,
+// s = 62; 2^-10 for FP32 overlaps against their former sums of float pairs) of the largest entries'
+// product, as of two columns that hardly meet, are less accurate relative to
+// themselves than FP64 multiply-adds.
 //
 // Kernel: 8 converter warps and one MMA warp per CTA, one CTA per SM, a 128 x
 // BN tile of the result.  Stage (32 steps of the contraction, two stages): the
@@ -44,7 +48,8 @@
 // conversion, 20 integer instructions per value on a pipe of half rate,
 // accounts for the rest, the pass that finds the column exponents for 0.4 ms.
 // Every size gains (64 x 64: 4.4 -> 0.45 ms FP64, 0.94 -> 0.41 ms FP32), so
-// there is no other path.
+// overlaps have no other path; rotations of more states or columns than
+// digit_rot_takes says take k_rowmul.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -1755,7 +1760,9 @@ template <int BN> int launch_piece_gram(PieceGramArgs a, cudaStream_t st) {
     RS_TRY(smem_optin((const void *)k_piece_gram<BN>, C::SMEM));
     a.tiles_n = (a.ny + BN - 1) / BN;
     a.tiles = (a.nx + DG_M - 1) / DG_M * a.tiles_n;
-    // chunks: enough for every SM, of at most 2048 points
+    // chunks: enough for 148 CTAs, of at most 2048 points.  (148, not this chip's
+    // 152: the chunks are the FP32 sums of a result, which stay what they were with the kernel
+    // before this one; they bind below some 300 000 points a tile, where the last 4 SMs idle.)
     const int64_t nkb = (a.npts + PG_K - 1) / PG_K;
     const int64_t want = std::max<int64_t>(1, std::min<int64_t>(nkb, (148 + a.tiles - 1) / a.tiles));
     a.kb = (int)std::min<int64_t>((nkb + want - 1) / want, 2048 / PG_K);

@@ -12,9 +12,9 @@ namespace rs {
 // Ints of scratch the overlap of nx and ny columns needs.
 inline int64_t digit_gram_scratch_ints(int nx, int ny) { return (int64_t)nx + ny; }
 
-// S (nx x ny, FP64, row stride lds) = dV X^T Y over npts points.  Accuracy:
-// the digits of an operand resolve 2^-62 (FP64) or 2^-54 (FP32) of its
-// column's largest entry.
+// S (nx x ny, FP64, row stride lds) = dV X^T Y over npts points.  Accuracy: a
+// product is off by at most 9 * 2^-62 (FP64) or 8 * 2^-54 (FP32) of 2^(Ex + Ey), the powers of two
+// above its columns' largest entries.
 // scratch: digit_gram_scratch_ints ints of device memory, or nullptr (taken
 // from the library's stream-ordered pool); it is left holding the keys of the
 // columns (see column_keys), X's and then, where Y is another block, Y's.  Asynchronous.
@@ -30,9 +30,9 @@ template <typename T> int column_keys(const T *X, int64_t ldx, int n, int64_t np
 // [n][ldc]; Y may be X itself (same pointer and leading dimension) when
 // beta == 0.  digit_rot_takes says whether the sizes are taken.  xkeys: the keys of X's
 // columns, or nullptr where they are of one size (orthonormal states, normalised
-// directions): the digits of an entry resolve 2^-62 (FP64) or 2^-38 (FP32) of the
-// largest entry of its row of X, the columns brought to one size, and of its
-// column of C, the rows taken the other way.
+// directions): a product is off by at most 9 * 2^-62 (FP64) or 6 * 2^-38 (FP32) of
+// 2^(Ex + Ec), the powers of two above the largest entry of its row of X, the columns brought to
+// one size, and of its column of C, the rows taken the other way.
 bool digit_rot_takes(int n, int m, bool in_place);
 template <typename T>
 int digit_rot(const T *X, int64_t ldx, int n, const double *C, int64_t ldc, int m, T *Y, int64_t ldy, int64_t npts,

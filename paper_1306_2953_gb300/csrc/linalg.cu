@@ -2,11 +2,12 @@
 // orthogonalisation (Eq. 6) and subspace diagonalisation (Eqs. 7-8).
 //
 // Tall-skinny contractions over grid points:
-//   digits.cu S = dV X^T Y and Y = alpha X C + beta Y as exact sums of integer
-//             digit products on the tensor cores.
+//   digits.cu S = dV X^T Y and Y = alpha X C + beta Y as sums of integer digit
+//             products on the tensor cores.
 //   k_rowmul  the rotation row by row with FP64 (FP32) FMA (each CTA owns whole
-//             rows), for in-place rotations of more than 1024 columns, whose
-//             row tiles do not fit one cluster of CTAs.
+//             rows), for rotations of more than 1536 states, whose digit sums
+//             could leave their range, and in place into more than 1024 columns,
+//             whose row tiles do not fit one cluster of CTAs.
 // Small dense kernels (n <= a few hundred, FP64 unless stated):
 //   k_chol    S = U^T U, right-looking, one CTA, status on failure
 //   k_trinv_rows  U^-1, one warp per row (n <= 256); k_trinv, one warp per
