@@ -873,7 +873,7 @@ __global__ void __launch_bounds__(DG_NT, 1) k_digit_rot(RotArgs<T> a) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
                             t[i] = ld_fresh(xv + min(q0 + 4 * i, nv - 1));   // in this order, ahead of the factors' reads:
-                        // with two or three in flight the key warps hold the others up (7.1 ms instead of 4.8 for 256 FP64 states)
+                        // with two or three in flight the key warps hold the others up (9.5 ms instead of 4.8 for 256 FP64 states)
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             const T *tt = reinterpret_cast<const T *>(&t[i]);
@@ -1762,7 +1762,7 @@ template <int BN> int launch_piece_gram(PieceGramArgs a, cudaStream_t st) {
     a.tiles = (a.nx + DG_M - 1) / DG_M * a.tiles_n;
     // chunks: enough for 148 CTAs, of at most 2048 points.  (148, not this chip's
     // 152: the chunks are the FP32 sums of a result, which stay what they were with the kernel
-    // before this one; they bind below some 300 000 points a tile, where the last 4 SMs idle.)
+    // before this one; they bind below 303 104 points divided by the tiles, where 4 SMs idle.)
     const int64_t nkb = (a.npts + PG_K - 1) / PG_K;
     const int64_t want = std::max<int64_t>(1, std::min<int64_t>(nkb, (148 + a.tiles - 1) / a.tiles));
     a.kb = (int)std::min<int64_t>((nkb + want - 1) / want, 2048 / PG_K);
